@@ -1,7 +1,7 @@
 // Halo exchange of a partitioned solve on one device: after each stage, the
 // stored state of every ghost cell is copied from the part that owns it (see
 // fvlbm_partition.cpp for which cells and why).  One launch covers every
-// message; thread (entry, component) copies one stored component.  Sources are
+// message; thread (entry, unit) copies one stored unit of a cell (16 bytes where the format has them).  Sources are
 // owned cells and destinations ghost cells, so no thread reads what another
 // writes.
 #include <cuda_runtime.h>
@@ -17,25 +17,38 @@ struct PartPtrs {
     void* p[FVLBM_MAX_PARTS];
 };
 
-// E: stored component type, C: components per cell in the blocked layout
-// (FP64: 9 doubles; FP32: 9 floats; 16-bit split: 3 floats + 3 packed words).
-template <typename E, int C>
+// Copies of one cell between two buffers of a stored format, unit u of UNITS
+// (16-byte units, then the remaining values; see PlainIO and SplitIO).
+template <typename S> struct CellCopy {
+    static constexpr int UNITS = CellIO<S>::UNITS + 1;
+    static __device__ __forceinline__ void copy(void* dst, uint32_t to, const void* src, uint32_t from, int u) {
+        typedef typename CellIO<S>::V V;
+        if (u < CellIO<S>::UNITS) ((V*)CellIO<S>::pairs(dst, to))[u * BLK] = CellIO<S>::pairs(src, from)[u * BLK];
+        else *(S*)CellIO<S>::rest(dst, to) = *CellIO<S>::rest(src, from);
+    }
+};
+template <> struct CellCopy<__half> {
+    static constexpr int UNITS = 2;
+    static __device__ __forceinline__ void copy(void* dst, uint32_t to, const void* src, uint32_t from, int u) {
+        if (u == 0) *(uint4*)CellIO<__half>::head(dst, to) = *CellIO<__half>::head(src, from);
+        else *(uint2*)CellIO<__half>::tail(dst, to) = *CellIO<__half>::tail(src, from);
+    }
+};
+
+template <typename S>
 __global__ void halo_copy_kernel(const int4* __restrict__ ent, int64_t n, PartPtrs ptr) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n * C) return;
-    const int64_t e = t / C;
-    const int c = (int)(t - e * C);
+    if (t >= n * CellCopy<S>::UNITS) return;
+    const int64_t e = t / CellCopy<S>::UNITS;
     const int4 x = ent[e];   // src part, src cell, dst part, dst cell
-    const E* src = (const E*)ptr.p[x.x];
-    E* dst = (E*)ptr.p[x.z];
-    dst[blk_index((int64_t)x.w, C) + c * BLK] = src[blk_index((int64_t)x.y, C) + c * BLK];
+    CellCopy<S>::copy(ptr.p[x.z], (uint32_t)x.w, ptr.p[x.x], (uint32_t)x.y, (int)(t - e * CellCopy<S>::UNITS));
 }
 
-template <typename E, int C>
+template <typename S>
 int launch(cudaStream_t st, const int4* ent, int64_t n, const PartPtrs& p) {
     if (n == 0) return FVLBM_OK;
     const int threads = 256;
-    halo_copy_kernel<E, C><<<(unsigned)((n * C + threads - 1) / threads), threads, 0, st>>>(ent, n, p);
+    halo_copy_kernel<S><<<(unsigned)((n * CellCopy<S>::UNITS + threads - 1) / threads), threads, 0, st>>>(ent, n, p);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? FVLBM_OK : fail(FVLBM_ERR_CUDA, "halo exchange: %s", cudaGetErrorString(e));
 }
@@ -48,10 +61,10 @@ int launch_halo_copy(int prec, void* stream, const int4* entries, int64_t n, voi
     for (int k = 0; k < n_parts; k++) p.p[k] = part_state[k];
     cudaStream_t st = (cudaStream_t)stream;
     switch (prec) {
-        case FVLBM_FP64: return launch<double, FVLBM_Q>(st, entries, n, p);
-        case FVLBM_FP32_DEV: return launch<float, FVLBM_Q>(st, entries, n, p);
+        case FVLBM_FP64: return launch<double>(st, entries, n, p);
+        case FVLBM_FP32_DEV: return launch<float>(st, entries, n, p);
         case FVLBM_FP16_DEV:
-        case FVLBM_BF16_DEV: return launch<uint32_t, 6>(st, entries, n, p);
+        case FVLBM_BF16_DEV: return launch<__half>(st, entries, n, p);
     }
     return fail(FVLBM_ERR_ARG, "halo exchange: unknown precision %d", prec);
 }

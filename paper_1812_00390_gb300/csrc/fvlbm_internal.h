@@ -115,48 +115,88 @@ struct BcParam {
 };
 
 // Per-cell arrays on the device are blocked: 32 consecutive cells per block,
-// each component of the block contiguous (see blk_index in fvlbm_device.cuh).
+// each unit of the block contiguous (see blk_index in fvlbm_device.cuh).
 constexpr int BLK_SHIFT = 5;
 constexpr int BLK = 1 << BLK_SHIFT;
 
+// Link word of one face slot of one cell:
+//   bits  0..10  fused stage: tile-local index of the neighbour (the cell
+//                itself for boundary and unused slots, so that the gradient
+//                loop needs no test: the difference is zero)
+//   bits 11..14  bit p set: direction A of pair p leaves the cell through this
+//                face and B enters it (fvlbm_device.cuh), else the reverse.  The
+//                two sides of a face hold complementary bits, which makes each
+//                (face, direction) one side's to reconstruct
+//   bits 15..17  LinkKind
+//   bits 18..31  fused stage, tile cell: row of the tile's face table that
+//                holds what enters through this face (the neighbour's outgoing
+//                values, or the ghost values of a boundary face); two-kernel
+//                stage: the same face's slot in the neighbour
+enum LinkKind : uint32_t {
+    LK_FLOW = 0,       // interior face
+    LK_OTHER = 1,      // fused stage, 1-ring cell: a face the tile's cells do not have
+    LK_WALL = 2,
+    LK_INLET = 3,
+    LK_OUTLET = 4,     // external-flow outlet
+    LK_PRESSURE = 5,   // internal-flow (pressure) outlet
+    LK_SYMMETRY = 6,
+    LK_NONE = 7,       // unused slot (the cell has fewer faces)
+};
+constexpr uint32_t LINK_NB_MASK = 0x7FFu;
+constexpr int LINK_PAIR_SHIFT = 11, LINK_KIND_SHIFT = 15, LINK_ROW_SHIFT = 18;
+constexpr uint32_t LINK_ROW_MAX = 0x3FFFu;
+
 // Fused stage: shared-memory capacity of a tile of TILE threads (compile-time
 // strides, so that every shared-memory access is a fixed offset from one
-// index): LS local cells (tile, 1-ring, 2-ring), FS local faces (the faces of
-// the tile's cells) and the instance id of each tile cell; reals of RSIZE
-// bytes.  The tile planner ends a tile early when it would not fit.
+// index): LS local cells (tile, 1-ring, 2-ring) and the face table, whose row
+// k * TILE + x holds the four values that leave local cell x through slot k,
+// and whose last GHOSTS rows hold the values that enter through the tile's
+// boundary faces; reals of RSIZE bytes.  The planner ends a tile early when
+// it would not fit.
 template <int TILE, int MAXF, int RSIZE> struct TileDims {
     static constexpr int LS = (3 * TILE) / 2 + 64;
-    static constexpr int FS = MAXF <= 4 ? 2 * TILE : (7 * TILE) / 2;
-    static constexpr size_t BYTES =
-        (size_t)RSIZE * ((size_t)FVLBM_Q * LS + (size_t)(FVLBM_Q - 1) * FS) + (size_t)4 * TILE;
+    static constexpr int GHOSTS = TILE / 2;
+    static constexpr int ROWS = MAXF * TILE + GHOSTS;
+    static constexpr size_t BYTES = (size_t)RSIZE * ((size_t)(FVLBM_Q - 1) * LS + (size_t)4 * ROWS);
+    static_assert(LS <= (int)LINK_NB_MASK + 1 && ROWS <= (int)LINK_ROW_MAX, "link word fields");
 };
-// "no local face / neighbour" in a 16-bit link field
-constexpr uint32_t LINK_NONE = 0xFFFF;
+
+// One tile of the fused stage.
+struct TileRec {
+    int32_t c0, nt;     // cells [c0, c0 + nt)
+    int32_t h0, nh;     // halo entries [h0, h0 + nh): 1-ring, then 2-ring
+    int32_t q0, n1;     // 1-ring entries [q0, q0 + n1) of the link array r1link
+    int32_t inst;       // instance of every local cell, or -1 when they differ
+    int32_t pad;
+};
 
 // Device pointers of one solver (all inside one workspace).
 struct DevView {
     int64_t n_cell;     // cells updated (internal numbering 0..n_cell-1): the owned cells
     int64_t n_grad;     // cells whose gradient the two-kernel stage computes (owned + first ghost ring)
     int64_t np;         // padded cell count (multiple of the largest tile)
-    int64_t n_face;     // face-value table length (two-kernel stage)
+    int64_t n_face;     // faces of the mesh
     int32_t maxf;       // slots per cell in the packed arrays (4 or 8)
     int32_t n_inst;
-    // geometry, blocked per cell, [maxf] (desc) and [3 maxf] (geo) components
-    const uint2* desc;  // x: kind | outmask << 8 | bc << 16;  y: link (see below)
-    const void* geo;    // T2 [3 maxf]: least-squares coefficients, face midpoint - centroid,
-                        //              face vector / area of each slot
-    // two-kernel stage: desc.y = face id; nbr = neighbour cell, blocked [maxf]
-    const int32_t* nbr;
+    // geometry, blocked per cell
+    const uint4* link;     // [maxf / 4] units of four link words
+    const void* geo;       // least-squares coefficients, face midpoint - centroid, face vector / area
+                           // of each slot (GeoRef)
+    const uint16_t* bctag; // [np][maxf] boundary tag of each slot (read for boundary slots only)
+    // two-kernel stage: neighbour cell of interior slots, ghost record of boundary slots, the cell
+    // itself for unused ones; blocked like link
+    const int4* nbr;
     const double* area;    // [np]
     const int32_t* grp;    // [np] instance of each cell
     const int32_t* iperm;  // [n_cell] internal index of each cell in the caller's order
     const InstParam* inst; // [n_inst]
     const BcParam* bc;     // [n_bc]
     // state
-    void* fa;   // S blocked [9] (or the split format): the state
+    void* fa;   // blocked (PlainIO, SplitIO): the state
     void* fb;   // same: stage state (multistage schemes) or the other buffer of a ping-pong pair
     void* rprev;// T [9][np]  AB2 previous RHS
-    void* fv;   // T [8][n_face] face values of directions 1..8 (two-kernel stage)
+    void* fv;   // two-kernel stage: Quad<T> of outgoing values per (cell, slot), blocked [maxf], then the
+                // ghost records (values that enter through boundary faces)
     double* rho;    // [np]
     double* ux;     // [np]
     double* uy;     // [np]
@@ -167,18 +207,16 @@ struct DevView {
     const int64_t* chunk;   // [n_chunk][3] (begin, end, instance)
     int64_t n_chunk;
     int32_t* flag;  // non-finite flag
-    // fused stage (one CTA per tile of at most `tile` consecutive cells);
-    // desc.y = tile-local neighbour | tile-local face << 16
+    // fused stage (one CTA per tile of at most `tile` consecutive cells)
     int32_t strategy;        // STRATEGY_TWO_KERNEL or STRATEGY_TILE
     int32_t block;           // threads per block of the two-kernel stage
     int32_t tile;            // most cells per tile (threads per CTA)
     int32_t sms;             // streaming multiprocessors of the device
     int64_t n_tiles;
-    const int64_t* tile_begin; // [n_tiles + 1] first cell of each tile
-    const int64_t* halo_ptr;   // [n_tiles + 1] into halo
+    const TileRec* tiles;      // [n_tiles]
     const int32_t* halo;       // 1-ring then 2-ring cells of each tile (global ids)
-    const int64_t* r1_ptr;     // [n_tiles + 1] 1-ring entries of each tile (running count)
-    const uint32_t* r1link;    // blocked [maxf] over 1-ring entries: local neighbour | local face << 16
+    const uint4* r1link;       // [maxf / 4][n_r1] link words of the 1-ring entries
+    int64_t n_r1;
 };
 
 enum Strategy { STRATEGY_TWO_KERNEL = 0, STRATEGY_TILE = 1 };

@@ -83,20 +83,19 @@ size_t state_bytes(int prec) {
 // cells (internal order), cut where tile and 1-ring (face neighbours outside
 // the tile) would exceed the CTA's `tile` threads, or where the local cells
 // (tile, 1-ring, 2-ring = face neighbours of the 1-ring outside tile and
-// 1-ring) or the tile's faces would exceed the kernel's shared-memory
-// capacity.  Every tile cell slot carries the local
-// index of its neighbour and the local index of its face; every 1-ring slot
-// the local index of its neighbour and, for faces shared with the tile, the
-// local face.
+// 1-ring) or the tile's boundary faces would exceed the kernel's shared-memory
+// capacity.  Every slot of a tile or 1-ring cell has a link word (see
+// fvlbm_internal.h): the local index of its neighbour, which direction of each
+// pair leaves through it, its kind and, for tile cells, the face-table row of
+// what enters.
 struct TilePlan {
     int tile = 0;
     int64_t n_tiles = 0;
-    std::vector<int64_t> begin;     // [n_tiles + 1]
-    std::vector<int64_t> halo_ptr;  // [n_tiles + 1]
+    std::vector<TileRec> rec;       // [n_tiles]
     std::vector<int32_t> halo;      // 1-ring then 2-ring of each tile
-    std::vector<int64_t> r1_ptr;    // [n_tiles + 1]
-    std::vector<uint32_t> link;     // [n_cell][maxf] local neighbour | local face << 16
-    std::vector<uint32_t> r1link;   // [1-ring entries][maxf] same fields
+    std::vector<uint32_t> link;     // [n_cell][maxf] link words of the tile cells
+    std::vector<uint32_t> r1link;   // [1-ring entries][maxf] link words
+    int64_t n_r1 = 0;               // 1-ring entries
     int32_t max_local = 0, max_faces = 0;
     int64_t short_tiles = 0;        // tiles cut below `tile` cells by the capacity
     int64_t sum_len = 0, sum_ring1 = 0, sum_local = 0;   // over the tiles
@@ -114,11 +113,11 @@ int64_t internal_nbr(const Mesh& M, int64_t i, int k) {
 }
 
 // Shared-memory capacity of the fused kernel for a tile size (TileDims).
-bool tile_dims(int tile, int maxf, int rsize, int& ls, int& fs, size_t& bytes) {
+bool tile_dims(int tile, int maxf, int rsize, int& ls, int& ghosts, size_t& bytes) {
 #define FVLBM_TD(T_)                                                                                         \
     case T_:                                                                                                 \
         ls = TileDims<T_, 4, 4>::LS;                                                                         \
-        fs = maxf <= 4 ? TileDims<T_, 4, 4>::FS : TileDims<T_, 8, 4>::FS;                                    \
+        ghosts = TileDims<T_, 4, 4>::GHOSTS;                                                                 \
         bytes = maxf <= 4 ? (rsize == 4 ? TileDims<T_, 4, 4>::BYTES : TileDims<T_, 4, 8>::BYTES)             \
                           : (rsize == 4 ? TileDims<T_, 8, 4>::BYTES : TileDims<T_, 8, 8>::BYTES);            \
         return true;
@@ -136,77 +135,58 @@ struct TileScratch {
     std::vector<int64_t> stamp;
     std::vector<int32_t> loc;
     std::vector<int64_t> r1, r2;
-    std::vector<int32_t> t_nb, t_f, r_nb, r_f;
-    std::vector<int32_t> bank_cnt, face_groups, face_row;   // bank_faces
+    std::vector<uint32_t> t_link, r_link;
     int64_t gen = 0;
 };
 
-// Face-table rows of a tile chosen for the shared-memory banks (4-byte banks,
-// 32 of them: row r lies in bank r mod 32).  A warp reaches, through one
-// slot, the faces of its 32 cells at once (phase 2 writes them, phase 3 reads
-// them); faces that share a bank there are served one after the other.  Each
-// face, in the order numbered, takes the bank that the fewest faces of its
-// warps' slot groups already hold (ties: the emptiest bank, room permitting),
-// and row bank + 32 * (faces already in that bank); face 0 keeps row 0, which
-// unused slots read (with a zero weight: it must hold finite values, and
-// every row of a face is written in full).  The rows are only addresses: the
-// arithmetic does not change.
-void bank_faces(const Mesh& M, int maxf, int64_t c0, int len, int fs, int nf, TileScratch& W) {
-    const int n1 = (int)W.r1.size();
-    const int depth = fs / BLK;   // rows per bank
-    const int n_groups = (len + n1 + BLK - 1) / BLK * maxf;
-    W.bank_cnt.assign((size_t)n_groups * BLK, 0);
-    W.face_groups.assign((size_t)nf * 2, -1);   // a face is reached through at most two slots
-    auto add = [&](int f, int g) {
-        int* fg = &W.face_groups[(size_t)f * 2];
-        if (fg[0] < 0) fg[0] = g;
-        else if (fg[0] != g) fg[1] = g;
-    };
-    for (int li = 0; li < len; li++) {
-        const int nfc = M.nf[M.perm[c0 + li]];
-        for (int k = 0; k < maxf; k++) {
-            const int g = li / BLK * maxf + k;
-            if (k < nfc) add(W.t_f[(size_t)li * maxf + k], g);
-            else W.bank_cnt[(size_t)g * BLK] = 1;
-        }
+// Direction pairs (A, B) of the link words, as in fvlbm_device.cuh.
+constexpr int PAIR_A[4] = {1, 2, 5, 6}, PAIR_B[4] = {3, 4, 7, 8};
+constexpr int EXI[FVLBM_Q] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+constexpr int EYI[FVLBM_Q] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+
+// Pair bits of slot k of cell i (internal numbers): bit p set when direction A
+// of pair p leaves the cell through the face (e.n > 0).  A pair parallel to an
+// interior face (e.n = 0, zero flux) is given to the side with the smaller
+// (cell, slot), so that the two sides always hold complementary bits.
+uint32_t pair_bits(const Mesh& M, int64_t i, int k) {
+    const Slot& S = M.slots[(size_t)M.perm[i] * MAXP + k];
+    bool first = true;
+    if (S.kind == SK_INTERIOR) {
+        const int64_t j = M.iperm[S.nb];
+        first = i < j || (i == j && k < S.nb_slot);
     }
-    for (int e = 0; e < n1; e++)
-        for (int k = 0; k < maxf; k++) {
-            const int f = W.r_f[(size_t)e * maxf + k];
-            if (f >= 0) add(f, (len + e) / BLK * maxf + k);
-        }
-    int load[BLK] = {0};
-    W.face_row.resize(nf);
-    for (int f = 0; f < nf; f++) {
-        const int* fg = &W.face_groups[(size_t)f * 2];
-        int best = 0, best_cost = -1;
-        // face 0 keeps row 0, the row unused slots read: it is written in full
-        for (int b = f == 0 ? BLK : 0; b < BLK; b++) {
-            if (load[b] >= depth) continue;
-            int c = 0;
-            for (int q = 0; q < 2; q++)
-                if (fg[q] >= 0) c += W.bank_cnt[(size_t)fg[q] * BLK + b];
-            c = c * (depth + 1) + load[b];
-            if (best_cost < 0 || c < best_cost) {
-                best_cost = c;
-                best = b;
-            }
-        }
-        for (int q = 0; q < 2; q++)
-            if (fg[q] >= 0) W.bank_cnt[(size_t)fg[q] * BLK + best]++;
-        W.face_row[f] = best + BLK * load[best]++;
+    uint32_t m = 0;
+    for (int p = 0; p < 4; p++) {
+        const bool a = (S.outmask >> (PAIR_A[p] - 1)) & 1u, b = (S.outmask >> (PAIR_B[p] - 1)) & 1u;
+        if (a || (!b && first)) m |= 1u << p;
     }
-    for (int32_t& x : W.t_f)
-        if (x >= 0) x = W.face_row[x];
-    for (int32_t& x : W.r_f)
-        if (x >= 0) x = W.face_row[x];
+    return m;
 }
 
-// Local numbering of the tile [c0, c0 + len): tile cells, 1-ring, 2-ring, and
-// the local faces of the tile cells.  False when it exceeds ls / fs, or when
-// tile and 1-ring together exceed the CTA's `threads` (the kernel gives every
-// thread at most one gradient to compute).
-bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls, int fs, TileScratch& W,
+uint32_t link_kind(const Mesh& M, const Slot& S) {
+    switch (S.kind) {
+        case SK_INTERIOR: return LK_FLOW;
+        case SK_WALL: return LK_WALL;
+        case SK_INLET: return LK_INLET;
+        case SK_OUTLET: return M.bcs[S.bc].external ? LK_OUTLET : LK_PRESSURE;
+        case SK_SYMMETRY: return LK_SYMMETRY;
+        default: return LK_NONE;
+    }
+}
+
+uint32_t link_word(uint32_t nb, uint32_t pairs, uint32_t kind, uint32_t row) {
+    return nb | pairs << LINK_PAIR_SHIFT | kind << LINK_KIND_SHIFT | row << LINK_ROW_SHIFT;
+}
+uint32_t word_nb(uint32_t w) { return w & LINK_NB_MASK; }
+uint32_t word_pairs(uint32_t w) { return (w >> LINK_PAIR_SHIFT) & 0xFu; }
+uint32_t word_kind(uint32_t w) { return (w >> LINK_KIND_SHIFT) & 7u; }
+uint32_t word_row(uint32_t w) { return w >> LINK_ROW_SHIFT; }
+
+// Link words of the tile [c0, c0 + len): local numbering tile cells, 1-ring,
+// 2-ring.  False when it exceeds ls local cells or `ghosts` boundary faces, or
+// when tile and 1-ring together exceed the CTA's `threads` (the kernel gives
+// every thread at most one gradient to compute).
+bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls, int ghosts, TileScratch& W,
               int& n_local, int& n_faces) {
     const int64_t g = ++W.gen;
     int nl = 0;
@@ -225,6 +205,8 @@ bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls,
                 W.r1.push_back(j);
             }
         }
+    const int n1 = (int)W.r1.size();
+    if (nl > ls || len + n1 > threads) return false;
     for (int64_t j : W.r1)
         for (int k = 0; k < M.nf[M.perm[j]]; k++) {
             const int64_t q = internal_nbr(M, j, k);
@@ -234,96 +216,83 @@ bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls,
                 W.r2.push_back(q);
             }
         }
-    const int n1 = (int)W.r1.size();
-    if (nl > ls || len + n1 > threads) return false;
+    if (nl > ls) return false;
     // 1-ring and 2-ring each in global order: the kernel gathers them with
-    // consecutive threads, which then share the rows of a 32-cell block
+    // consecutive threads, which then share the sectors of a 32-cell block
     std::sort(W.r1.begin(), W.r1.end());
     std::sort(W.r2.begin(), W.r2.end());
     int x = len;
     for (int64_t j : W.r1) W.loc[j] = x++;
     for (int64_t q : W.r2) W.loc[q] = x++;
-    W.t_nb.assign((size_t)len * maxf, -1);
-    W.t_f.assign((size_t)len * maxf, -1);
-    W.r_nb.assign((size_t)n1 * maxf, -1);
-    W.r_f.assign((size_t)n1 * maxf, -1);
-    // faces numbered slot by slot (all cells' slot 0, then slot 1, ...): the
-    // cells of a warp then reach their slot-k faces at mostly consecutive
-    // indices, which spreads their face-table accesses over the memory banks
-    int nf = 0;
-    for (int k = 0; k < maxf; k++) {
-        for (int li = 0; li < len; li++) {
-            const int64_t c = M.perm[c0 + li];
-            if (k >= M.nf[c]) continue;
+    W.t_link.resize((size_t)len * maxf);
+    W.r_link.resize((size_t)n1 * maxf);
+    int n_ghost = 0, n_slots = 0, inner = 0;
+    for (int li = 0; li < len; li++) {
+        const int64_t c = M.perm[c0 + li];
+        for (int k = 0; k < maxf; k++) {
+            uint32_t& w = W.t_link[(size_t)li * maxf + k];
+            if (k >= M.nf[c]) {
+                w = link_word((uint32_t)li, 0, LK_NONE, 0);   // row 0: finite, read with weight zero
+                continue;
+            }
             const Slot& S = M.slots[(size_t)c * MAXP + k];
-            const size_t x = (size_t)li * maxf + k;
+            n_slots++;
             if (S.kind == SK_INTERIOR) {
-                const int lj = W.loc[M.iperm[S.nb]];
-                W.t_nb[x] = lj;
-                if (W.t_f[x] < 0) {
-                    W.t_f[x] = nf;
-                    if (lj < len) W.t_f[(size_t)lj * maxf + S.nb_slot] = nf;
-                    else W.r_f[(size_t)(lj - len) * maxf + S.nb_slot] = nf;
-                    nf++;
-                }
+                const uint32_t lj = (uint32_t)W.loc[M.iperm[S.nb]];
+                inner += (int)lj < len;
+                w = link_word(lj, pair_bits(M, c0 + li, k), LK_FLOW, (uint32_t)S.nb_slot * threads + lj);
             } else {
-                W.t_f[x] = nf++;
+                if (n_ghost == ghosts) return false;
+                w = link_word((uint32_t)li, pair_bits(M, c0 + li, k), link_kind(M, S), (uint32_t)(maxf * threads + n_ghost++));
             }
         }
     }
-    if (nf > fs) return false;
-    bank_faces(M, maxf, c0, len, fs, nf, W);
-    for (int e = 0; e < n1; e++)
-        for (int k = 0; k < M.nf[M.perm[W.r1[e]]]; k++) {
-            const int64_t q = internal_nbr(M, W.r1[e], k);
-            if (q >= 0) W.r_nb[(size_t)e * maxf + k] = W.loc[q];
-        }
-    // Slots without a neighbour (boundary faces, unused slots) link to the
-    // cell itself, so that the kernel's gradient loop needs no test of the
-    // slot kind (the difference to itself is zero); unused slots of tile
-    // cells name face row 0, which they never write (their mask is empty) and
-    // whose values they weight by a zero face vector.
-    for (int li = 0; li < len; li++) {
-        const int nfc = M.nf[M.perm[c0 + li]];
+    for (int e = 0; e < n1; e++) {
+        const int64_t j = W.r1[e], c = M.perm[j];
         for (int k = 0; k < maxf; k++) {
-            const size_t x = (size_t)li * maxf + k;
-            if (W.t_nb[x] < 0) W.t_nb[x] = li;
-            if (k >= nfc) W.t_f[x] = 0;
+            uint32_t& w = W.r_link[(size_t)e * maxf + k];
+            const int64_t q = k < M.nf[c] ? internal_nbr(M, j, k) : -1;
+            if (q >= 0) {
+                const uint32_t lq = (uint32_t)W.loc[q];
+                w = link_word(lq, pair_bits(M, j, k), (int)lq < len ? LK_FLOW : LK_OTHER, 0);
+            } else {
+                const bool used = k < M.nf[c];
+                const uint32_t kind = used ? link_kind(M, M.slots[(size_t)c * MAXP + k]) : LK_NONE;
+                w = link_word((uint32_t)(len + e), used ? pair_bits(M, j, k) : 0, kind, 0);
+            }
         }
     }
-    for (int e = 0; e < n1; e++)
-        for (int k = 0; k < maxf; k++)
-            if (W.r_nb[(size_t)e * maxf + k] < 0) W.r_nb[(size_t)e * maxf + k] = len + e;
     n_local = nl;
-    n_faces = nf;
+    n_faces = n_slots - inner / 2;
     return true;
 }
 
-uint32_t pack_link(int nb, int f) {
-    return (uint32_t)(nb < 0 ? LINK_NONE : (uint32_t)nb) | ((uint32_t)(f < 0 ? LINK_NONE : (uint32_t)f) << 16);
+// Shared-memory wavefronts of a warp's 16-byte accesses relative to the four
+// that a conflict-free one takes: eight lanes at a time, eight 16-byte banks;
+// a group takes as many as the most distinct rows that share a bank.
+double bank_waves(const int* idx, int n) {
+    double m = 0;
+    for (int b = 0; b < n; b += 8) {
+        int v[8], cnt[8] = {0}, w = 0;
+        const int e = std::min(8, n - b);
+        for (int q = 0; q < e; q++) v[q] = idx[b + q];
+        std::sort(v, v + e);
+        for (int q = 0; q < e; q++)
+            if (q == 0 || v[q] != v[q - 1]) w = std::max(w, ++cnt[v[q] & 7]);
+        m += w;
+    }
+    return m / ((n + 7) / 8);
 }
 
-uint32_t writer_mask(const Slot& S, int64_t i, int k, int64_t j);
-
-// Shared-memory wavefronts of one warp access (4-byte banks, 32 of them):
-// the most distinct addresses that fall into one bank.
-int bank_waves(const int* idx, int n) {
-    int v[BLK];
-    for (int q = 0; q < n; q++) v[q] = idx[q];
-    std::sort(v, v + n);
-    int cnt[BLK] = {0}, m = 0;
-    for (int q = 0; q < n; q++)
-        if (q == 0 || v[q] != v[q - 1]) m = std::max(m, ++cnt[v[q] & (BLK - 1)]);
-    return m;
-}
-
-// Checks of one tile's plan (fvlbm_plan_info): every slot links to its
-// neighbour's local index (boundary and unused slots to the cell itself, unused
-// slots to face row 0), the two sides of a face name one row and no two faces
-// share one, every (face, direction) between local cells has exactly one
-// writer, and tile + 1-ring and the local cells fit the CTA; then the modelled
-// wavefronts of phase 3's face-table reads and phase 2's neighbour gathers.
-void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls, int fs, int nl,
+// Checks of one tile's plan (fvlbm_plan_info), against the mesh: every slot
+// links to its neighbour's local index (boundary and unused slots to the cell
+// itself, unused slots to row 0), what enters through an interior face is read
+// from the row that the neighbour writes there, no two boundary faces share a
+// ghost row, each (face, direction) between local cells has exactly one writer,
+// and tile + 1-ring and the local cells fit the CTA; then the modelled
+// wavefronts of the face-table accesses (a slot's own row, written and read
+// without conflict, and the neighbour's row) and of the neighbour gathers.
+void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls, int ghosts, int nl,
                  const TileScratch& W, TilePlan& P) {
     auto bad = [&](const char* what, int64_t cell) {
         if (P.violations++ == 0) {
@@ -335,58 +304,49 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
     const int n1 = (int)W.r1.size();
     if (len + n1 > threads) bad("tile and 1-ring exceed the CTA's threads", c0);
     if (nl > ls) bad("local cells exceed the shared-memory capacity", c0);
-    auto slot = [&](int64_t i, int k) -> const Slot& { return M.slots[(size_t)M.perm[i] * MAXP + k]; };
-    // a face is named by its side with the lower (cell, slot)
-    auto face_key = [&](int64_t i, int k) {
-        const Slot& S = slot(i, k);
-        if (S.kind == SK_INTERIOR) {
-            const int64_t j = M.iperm[S.nb];
-            if (j < i || (j == i && S.nb_slot < k)) return std::make_pair(j, S.nb_slot);
-        }
-        return std::make_pair(i, k);
-    };
-    std::vector<std::pair<int64_t, int>> owner((size_t)fs, std::make_pair((int64_t)-1, -1));
-    for (int li = 0; li < len; li++) {
-        const int64_t i = c0 + li;
-        const int nfc = M.nf[M.perm[i]];
+    std::vector<char> taken((size_t)ghosts, 0);
+    for (int li = 0; li < len + n1; li++) {
+        const int64_t i = li < len ? c0 + li : W.r1[li - len];
+        const int64_t c = M.perm[i];
         for (int k = 0; k < maxf; k++) {
-            const size_t x = (size_t)li * maxf + k;
-            if (k >= nfc) {
-                if (W.t_nb[x] != li || W.t_f[x] != 0) bad("unused slot not linked to itself and row 0", i);
+            const uint32_t w = li < len ? W.t_link[(size_t)li * maxf + k] : W.r_link[(size_t)(li - len) * maxf + k];
+            if (k >= M.nf[c]) {
+                if (word_kind(w) != LK_NONE || word_nb(w) != (uint32_t)li || word_row(w) != 0)
+                    bad("unused slot not linked to itself and row 0", i);
                 continue;
             }
-            const int row = W.t_f[x];
-            if (row < 0 || row >= fs) {
-                bad("face row outside the table", i);
-                continue;
+            const Slot& S = M.slots[(size_t)c * MAXP + k];
+            for (int p = 0; p < 4; p++) {
+                // the direction given to this side must not enter through the face
+                const int a = (word_pairs(w) >> p) & 1u ? PAIR_A[p] : PAIR_B[p];
+                if (EXI[a] * S.nx + EYI[a] * S.ny < 0) bad("a direction that enters marked as leaving", i);
             }
-            const auto key = face_key(i, k);
-            if (owner[row].first < 0) owner[row] = key;
-            else if (owner[row] != key) bad("two faces share a face row", i);
-            const Slot& S = slot(i, k);
             if (S.kind != SK_INTERIOR) {
-                if (W.t_nb[x] != li) bad("boundary slot not linked to itself", i);
+                if (word_nb(w) != (uint32_t)li) bad("boundary slot not linked to itself", i);
+                if (word_kind(w) != link_kind(M, S)) bad("boundary slot of the wrong kind", i);
+                if (li >= len) continue;
+                const int64_t row = (int64_t)word_row(w) - (int64_t)maxf * threads;
+                if (row < 0 || row >= ghosts) bad("ghost row outside the face table", i);
+                else if (taken[row]++) bad("two boundary faces share a ghost row", i);
                 continue;
             }
             const int64_t j = M.iperm[S.nb];
             const int lj = W.loc[j];
-            if (W.t_nb[x] != lj) bad("slot not linked to its neighbour", i);
-            int other = -2;
-            if (lj < len) other = W.t_f[(size_t)lj * maxf + S.nb_slot];
-            else if (lj < len + n1) other = W.r_f[(size_t)(lj - len) * maxf + S.nb_slot];
-            else bad("a tile cell's neighbour is not in the tile or its 1-ring", i);
-            if (other != -2 && other != row) bad("the two sides of a face name different rows", i);
-            const uint32_t mi = writer_mask(S, i, k, j), mj = writer_mask(slot(j, S.nb_slot), j, S.nb_slot, i);
-            if ((mi & mj) != 0 || (mi | mj) != 0xFFu) bad("a (face, direction) without exactly one writer", i);
-        }
-    }
-    for (int e = 0; e < n1; e++) {
-        const int64_t j = W.r1[e];
-        const int nfc = M.nf[M.perm[j]];
-        for (int k = 0; k < maxf; k++) {
-            const int64_t q = k < nfc ? internal_nbr(M, j, k) : -1;
-            const int want = q >= 0 ? W.loc[q] : len + e;
-            if (W.r_nb[(size_t)e * maxf + k] != want) bad("1-ring slot not linked to its neighbour", j);
+            if (word_nb(w) != (uint32_t)lj) bad("slot not linked to its neighbour", i);
+            if (li >= len) {
+                if (word_kind(w) != (lj < len ? LK_FLOW : LK_OTHER)) bad("a 1-ring face wrongly marked", i);
+                continue;
+            }
+            if (word_kind(w) != LK_FLOW) bad("interior slot of the wrong kind", i);
+            if (lj >= len + n1) {
+                bad("a tile cell's neighbour is not in the tile or its 1-ring", i);
+                continue;
+            }
+            if (word_row(w) != (uint32_t)(S.nb_slot * threads + lj)) bad("a face not read from the row its neighbour writes", i);
+            const uint32_t wj = lj < len ? W.t_link[(size_t)lj * maxf + S.nb_slot]
+                                         : W.r_link[(size_t)(lj - len) * maxf + S.nb_slot];
+            if (word_kind(wj) != LK_FLOW || word_nb(wj) != (uint32_t)li) bad("the two sides of a face do not link to each other", i);
+            if ((word_pairs(w) ^ word_pairs(wj)) != 0xFu) bad("a (face, direction) without exactly one writer", i);
         }
     }
     // modelled wavefronts of the warp accesses through one slot (used slots only)
@@ -396,12 +356,12 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
             int n = 0;
             bool used = k < 3;
             for (int li = w * BLK; li < std::min(len, (w + 1) * BLK); li++) {
-                idx[n++] = W.t_f[(size_t)li * maxf + k];
+                idx[n++] = (int)word_row(W.t_link[(size_t)li * maxf + k]);
                 used |= k < M.nf[M.perm[c0 + li]];
             }
             if (!used) continue;
-            P.face_groups += 1;
-            P.face_waves += bank_waves(idx, n);
+            P.face_groups += 3;
+            P.face_waves += 2 + bank_waves(idx, n);
         }
     for (int w = 0; w * BLK < len + n1; w++)
         for (int k = 0; k < maxf; k++) {
@@ -409,7 +369,7 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
             bool used = k < 3;
             for (int l = w * BLK; l < std::min(len + n1, (w + 1) * BLK); l++) {
                 const int64_t c = l < len ? c0 + l : W.r1[l - len];
-                idx[n++] = l < len ? W.t_nb[(size_t)l * maxf + k] : W.r_nb[(size_t)(l - len) * maxf + k];
+                idx[n++] = (int)word_nb(l < len ? W.t_link[(size_t)l * maxf + k] : W.r_link[(size_t)(l - len) * maxf + k]);
                 used |= k < M.nf[M.perm[c]];
             }
             if (!used) continue;
@@ -419,28 +379,26 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
 }
 
 int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify) {
-    int ls = 0, fs = 0;
+    int ls = 0, ghosts = 0;
     size_t bytes = 0;
-    if (!tile_dims(tile, maxf, 4, ls, fs, bytes)) return fail(FVLBM_ERR_ARG, "unsupported tile size %d", tile);
+    if (!tile_dims(tile, maxf, 4, ls, ghosts, bytes)) return fail(FVLBM_ERR_ARG, "unsupported tile size %d", tile);
     const int64_t n = M.n_cell;
     P = TilePlan{};
     P.tile = tile;
     P.verify = verify;
-    P.begin.push_back(0);
-    P.halo_ptr.push_back(0);
-    P.r1_ptr.push_back(0);
-    P.link.assign((size_t)n * maxf, 0xFFFFFFFFu);
+    P.link.assign((size_t)n * maxf, 0);
     TileScratch W;
     W.stamp.assign(n, 0);
     W.loc.assign(n, 0);
     // tiles cover the owned cells; ghost cells of a partition only appear in halos
     const int64_t n_own = M.n_owned;
     int64_t c0 = 0;
+    int32_t inst = 0;
     int guess = tile;   // neighbouring tiles have similar lengths: start one block above the last
     while (c0 < n_own) {
         int len = (int)std::min<int64_t>(guess, n_own - c0);
         int nl = 0, nf = 0;
-        while (!try_tile(M, maxf, c0, len, tile, ls, fs, W, nl, nf)) {
+        while (!try_tile(M, maxf, c0, len, tile, ls, ghosts, W, nl, nf)) {
             if (len == 1)
                 return fail(FVLBM_ERR_UNSUPPORTED, "cell %lld: its halo exceeds the fused stage's capacity",
                             (long long)c0);
@@ -451,23 +409,30 @@ int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify) {
         P.sum_len += len;
         P.sum_ring1 += (int64_t)W.r1.size();
         P.sum_local += nl;
-        if (verify) verify_tile(M, maxf, c0, len, tile, ls, fs, nl, W, P);
-        for (int li = 0; li < len; li++)
-            for (int k = 0; k < maxf; k++) {
-                const size_t x = (size_t)li * maxf + k;
-                if (W.t_f[x] >= 0) P.link[(size_t)(c0 + li) * maxf + k] = pack_link(W.t_nb[x], W.t_f[x]);
-            }
+        if (verify) verify_tile(M, maxf, c0, len, tile, ls, ghosts, nl, W, P);
+        std::copy(W.t_link.begin(), W.t_link.end(), P.link.begin() + (size_t)c0 * maxf);
+        // instances are contiguous in the internal order, and a face never joins two
+        while (inst + 1 < M.n_inst && c0 >= M.inst_begin[inst + 1]) inst++;
+        TileRec R{};
+        R.c0 = (int32_t)c0;
+        R.nt = len;
+        R.h0 = (int32_t)P.halo.size();
+        R.nh = (int32_t)(W.r1.size() + W.r2.size());
+        R.q0 = (int32_t)P.n_r1;
+        R.n1 = (int32_t)W.r1.size();
+        R.inst = M.n_inst == 1 || c0 + len <= M.inst_begin[inst + 1] ? inst : -1;
+        P.rec.push_back(R);
         for (int64_t j : W.r1) P.halo.push_back((int32_t)j);
         for (int64_t q : W.r2) P.halo.push_back((int32_t)q);
-        for (size_t x = 0; x < W.r_nb.size(); x++) P.r1link.push_back(pack_link(W.r_nb[x], W.r_f[x]));
+        if (P.halo.size() >= (size_t)1 << 31)
+            return fail(FVLBM_ERR_UNSUPPORTED, "fused stage: the halos exceed its 32-bit indexing; use kernel = 1");
+        P.r1link.insert(P.r1link.end(), W.r_link.begin(), W.r_link.end());
+        P.n_r1 += R.n1;
         c0 += len;
-        P.begin.push_back(c0);
-        P.halo_ptr.push_back((int64_t)P.halo.size());
-        P.r1_ptr.push_back(P.r1_ptr.back() + (int64_t)W.r1.size());
         P.max_local = std::max(P.max_local, nl);
         P.max_faces = std::max(P.max_faces, nf);
     }
-    P.n_tiles = (int64_t)P.begin.size() - 1;
+    P.n_tiles = (int64_t)P.rec.size();
     return FVLBM_OK;
 }
 
@@ -479,9 +444,10 @@ struct Layout {
     int block;
     bool pingpong;   // single-stage scheme on the fused stage: the state alternates between fa and fb
     TilePlan tp;
-    size_t off_desc, off_geo, off_nbr, off_area, off_grp, off_inst, off_bc, off_fa, off_fb, off_fc, off_rprev, off_fv,
-        off_rho, off_ux, off_uy, off_uold, off_part, off_red, off_conv, off_chunk, off_flag, off_tbegin, off_hptr,
-        off_halo, off_r1ptr, off_r1link, off_iperm, total;
+    int64_t n_ghost;   // two-kernel stage: boundary slots of owned cells (ghost records)
+    size_t off_link, off_geo, off_bctag, off_nbr, off_area, off_grp, off_inst, off_bc, off_fa, off_fb, off_fc, off_rprev,
+        off_fv, off_rho, off_ux, off_uy, off_uold, off_part, off_red, off_conv, off_chunk, off_flag, off_tiles, off_halo,
+        off_r1link, off_iperm, total;
 };
 
 constexpr size_t SMEM_LIMIT = 227 * 1024;
@@ -549,7 +515,7 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         if (rc) return rc;
         // the fused kernel indexes its blocked arrays in 32 bits
         const uint64_t lim = (uint64_t)1 << 32;
-        if ((uint64_t)L.np * 3 * L.maxf >= lim || (uint64_t)(L.tp.r1_ptr.back() + BLK) * L.maxf >= lim)
+        if ((uint64_t)L.np * 3 * L.maxf >= lim || (uint64_t)L.tp.n_r1 * L.maxf >= lim)
             return fail(FVLBM_ERR_UNSUPPORTED, "fused stage: %lld cells exceed its 32-bit indexing; use kernel = 1",
                         (long long)M.n_cell);
     }
@@ -562,25 +528,29 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         return r;
     };
     const size_t plane = (size_t)L.np, slots = plane * L.maxf;
-    const size_t n_r1 = tiled ? (size_t)round_up(L.tp.r1_ptr.back(), BLK) : 0;
-    L.off_desc = take(8 * slots);
+    L.n_ghost = 0;
+    if (two)
+        for (int64_t c = 0; c < M.n_cell; c++) {
+            if (M.iperm[c] >= M.n_owned) continue;
+            for (int k = 0; k < M.nf[c]; k++) L.n_ghost += M.slots[(size_t)c * MAXP + k].kind != SK_INTERIOR;
+        }
+    L.off_link = take(4 * slots);
     L.off_geo = take(2 * R * 3 * slots);
+    L.off_bctag = take(2 * slots);
     L.off_nbr = take(two ? 4 * slots : 0);
     L.off_area = take(8 * plane);
     L.off_grp = take(4 * plane);
     L.off_iperm = take(4 * plane);
     L.off_inst = take(sizeof(InstParam) * M.n_inst);
     L.off_bc = take(sizeof(BcParam) * std::max<size_t>(1, M.bcs.size()));
-    L.off_tbegin = take(tiled ? 8 * (size_t)(L.tp.n_tiles + 1) : 0);
-    L.off_hptr = take(tiled ? 8 * (size_t)(L.tp.n_tiles + 1) : 0);
+    L.off_tiles = take(tiled ? sizeof(TileRec) * (size_t)L.tp.n_tiles : 0);
     L.off_halo = take(tiled ? 4 * L.tp.halo.size() : 0);
-    L.off_r1ptr = take(tiled ? 8 * (size_t)(L.tp.n_tiles + 1) : 0);
-    L.off_r1link = take(tiled ? 4 * n_r1 * L.maxf : 0);
+    L.off_r1link = take(tiled ? 4 * (size_t)L.tp.n_r1 * L.maxf : 0);
     L.off_fa = take(S * plane);   // everything before this is uploaded once
     L.off_fb = (scheme == FVLBM_RK2 || scheme == FVLBM_RK4 || L.pingpong) ? take(S * plane) : 0;
     L.off_fc = (scheme == FVLBM_RK4 && tiled) ? take(S * plane) : 0;
     L.off_rprev = scheme == FVLBM_AB2 ? take(R * plane * FVLBM_Q) : 0;
-    L.off_fv = take(two ? R * (size_t)std::max<int64_t>(1, L.n_face) * (FVLBM_Q - 1) : 0);
+    L.off_fv = take(two ? 4 * R * (slots + (size_t)L.n_ghost) : 0);
     L.off_rho = take(8 * plane);
     L.off_ux = take(8 * plane);
     L.off_uy = take(8 * plane);
@@ -630,42 +600,25 @@ inline size_t blk(int64_t i, int c, int ncomp) {
     return (size_t)((i >> BLK_SHIFT) * ((int64_t)ncomp << BLK_SHIFT) + ((int64_t)c << BLK_SHIFT) + (i & (BLK - 1)));
 }
 
-// Writer mask of an interior slot: the directions whose face value this side
-// computes -- those it is upwind for (e.n > 0) and, for directions parallel
-// to the face (e.n = 0, zero flux), the side with the smaller (cell, slot) so
-// that every (face, direction) has exactly one finite writer.
-uint32_t writer_mask(const Slot& S, int64_t i, int k, int64_t j) {
-    static const int EXI[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
-    static const int EYI[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
-    uint32_t m = S.outmask;
-    const bool first = i < j || (i == j && k < S.nb_slot);
-    if (first)
-        for (int a = 1; a < FVLBM_Q; a++)
-            if (EXI[a] * S.nx + EYI[a] * S.ny == 0.0) m |= 1u << (a - 1);
-    return m;
-}
-
 template <typename T>
 void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& host) {
     const int64_t n = M.n_cell;
     const int maxf = L.maxf;
     const bool two = L.strategy == STRATEGY_TWO_KERNEL;
     unsigned char* H = host.data();
-    uint32_t* desc = (uint32_t*)(H + L.off_desc);   // pairs (x, y)
-    T* geo = (T*)(H + L.off_geo);                   // pairs of T
+    uint32_t* link = (uint32_t*)(H + L.off_link);   // units of four words
+    T* geo = (T*)(H + L.off_geo);                   // 16-byte units of 2-vectors (GeoRef)
+    uint16_t* bctag = (uint16_t*)(H + L.off_bctag);
     double* area = (double*)(H + L.off_area);
     int32_t* grp = (int32_t*)(H + L.off_grp);
     int32_t* iperm = (int32_t*)(H + L.off_iperm);
     for (int64_t c = 0; c < n; c++) iperm[c] = (int32_t)M.iperm[c];
     int32_t* nbr = two ? (int32_t*)(H + L.off_nbr) : nullptr;
-    for (size_t x = 0; x < (size_t)maxf * L.np; x++) {
-        desc[2 * x] = SK_NONE;
-        desc[2 * x + 1] = 0xFFFFFFFFu;
-        if (two) nbr[x] = -1;
-    }
-    // face ids of the two-kernel face table: both slots of an interior face share one
-    std::vector<int32_t> fid;
-    if (two) fid.assign((size_t)n * maxf, -1);
+    constexpr int PER = 16 / (2 * sizeof(T));   // 2-vectors per unit
+    const int units = maxf / PER;
+    // word of slot k, and 2-vector v of slot k
+    auto word = [&](int64_t i, int k) { return 4 * blk(i, k / 4, maxf / 4) + k % 4; };
+    auto vec = [&](int64_t i, int v, int k) { return geo + 2 * (PER * blk(i, v * units + k / PER, 3 * units) + k % PER); };
     int64_t next = 0;
     int32_t g = 0;
     for (int64_t i = 0; i < n; i++) {
@@ -673,44 +626,39 @@ void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& h
         while (g + 1 < M.n_inst && c >= M.inst_begin[g + 1]) g++;
         grp[i] = g;
         area[i] = M.area[c];
-        for (int k = 0; k < M.nf[c]; k++) {
-            const Slot& S = M.slots[(size_t)c * MAXP + k];
-            const size_t d = blk(i, k, maxf);
-            const int64_t j = S.kind == SK_INTERIOR ? M.iperm[S.nb] : -1;
-            // the directions this slot writes by reconstruction: on interior
-            // faces the upwind ones (writer_mask), on inlet and internal-outlet
-            // faces the outflow ones; the other boundary faces take ghost values
-            // for every direction, so their mask is empty
-            const bool io = S.kind == SK_INLET || (S.kind == SK_OUTLET && !M.bcs[S.bc].external);
-            const uint32_t mask = S.kind == SK_INTERIOR ? writer_mask(S, i, k, j) : (io ? S.outmask : 0u);
-            desc[2 * d] = (uint32_t)S.kind | (mask << 8) | ((uint32_t)(S.bc < 0 ? 0 : S.bc) << 16);
-            if (two) {
-                int32_t& f = fid[(size_t)i * maxf + k];
-                if (f < 0) {
-                    f = (int32_t)next++;
-                    if (j >= 0) fid[(size_t)j * maxf + S.nb_slot] = f;
-                }
-                desc[2 * d + 1] = (uint32_t)f;
-                nbr[d] = (int32_t)j;
+        for (int k = 0; k < maxf; k++) {
+            const size_t w = word(i, k);
+            if (k >= M.nf[c]) {
+                link[w] = two ? link_word(0, 0, LK_NONE, 0) : L.tp.link[(size_t)i * maxf + k];
+                if (two) nbr[w] = (int32_t)i;
+                continue;
             }
-            const size_t q0 = blk(i, 3 * k, 3 * maxf), q1 = blk(i, 3 * k + 1, 3 * maxf), q2 = blk(i, 3 * k + 2, 3 * maxf);
-            geo[2 * q0] = (T)S.cgx;
-            geo[2 * q0 + 1] = (T)S.cgy;
-            geo[2 * q1] = (T)(S.px - M.cx[c]);
-            geo[2 * q1 + 1] = (T)(S.py - M.cy[c]);
-            geo[2 * q2] = (T)(S.nx / M.area[c]);
-            geo[2 * q2 + 1] = (T)(S.ny / M.area[c]);
+            const Slot& S = M.slots[(size_t)c * MAXP + k];
+            bctag[(size_t)i * maxf + k] = (uint16_t)(S.bc < 0 ? 0 : S.bc);
+            if (two) {
+                const bool inner = S.kind == SK_INTERIOR;
+                link[w] = link_word(0, pair_bits(M, i, k), link_kind(M, S), inner ? (uint32_t)S.nb_slot : 0u);
+                nbr[w] = inner ? (int32_t)M.iperm[S.nb] : i < M.n_owned ? (int32_t)next++ : 0;
+            } else {
+                link[w] = L.tp.link[(size_t)i * maxf + k];
+            }
+            T* q = vec(i, 0, k);
+            q[0] = (T)S.cgx;
+            q[1] = (T)S.cgy;
+            q = vec(i, 1, k);
+            q[0] = (T)(S.px - M.cx[c]);
+            q[1] = (T)(S.py - M.cy[c]);
+            q = vec(i, 2, k);
+            q[0] = (T)(S.nx / M.area[c]);
+            q[1] = (T)(S.ny / M.area[c]);
         }
-        // fused stage: every slot's tile-local links (unused slots included)
-        if (!two)
-            for (int k = 0; k < maxf; k++) desc[2 * blk(i, k, maxf) + 1] = L.tp.link[(size_t)i * maxf + k];
     }
+    // 1-ring entries: unit by unit, entry by entry
     if (!two) {
         uint32_t* r1 = (uint32_t*)(H + L.off_r1link);
-        const int64_t ne = L.tp.r1_ptr.back();
-        for (int64_t e = 0; e < (int64_t)round_up(ne, BLK); e++)
-            for (int k = 0; k < maxf; k++)
-                r1[blk(e, k, maxf)] = e < ne ? L.tp.r1link[(size_t)e * maxf + k] : 0xFFFFFFFFu;
+        const int64_t ne = L.tp.n_r1;
+        for (int64_t e = 0; e < ne; e++)
+            for (int k = 0; k < maxf; k++) r1[4 * ((k / 4) * ne + e) + k % 4] = L.tp.r1link[(size_t)e * maxf + k];
     }
 }
 
@@ -871,10 +819,8 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
         if (s->prec == FVLBM_FP64) pack_geometry<double>(M, L, host);
         else pack_geometry<float>(M, L, host);
         if (L.strategy == STRATEGY_TILE) {
-            std::memcpy(host.data() + L.off_tbegin, L.tp.begin.data(), 8 * L.tp.begin.size());
-            std::memcpy(host.data() + L.off_hptr, L.tp.halo_ptr.data(), 8 * L.tp.halo_ptr.size());
+            std::memcpy(host.data() + L.off_tiles, L.tp.rec.data(), sizeof(TileRec) * L.tp.rec.size());
             std::memcpy(host.data() + L.off_halo, L.tp.halo.data(), 4 * L.tp.halo.size());
-            std::memcpy(host.data() + L.off_r1ptr, L.tp.r1_ptr.data(), 8 * L.tp.r1_ptr.size());
         }
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "fvlbm_init: out of host memory");
@@ -908,11 +854,6 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     CK(cudaMemcpyAsync(base, host.data(), L.off_fa, cudaMemcpyHostToDevice, s->stream), "upload geometry");
     CK(cudaMemcpyAsync(base + L.off_chunk, chunks.data(), chunks.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
                        s->stream), "upload chunk table");
-    // face values start at zero: directions parallel to a face (e.n = 0) are never written
-    if (L.strategy == STRATEGY_TWO_KERNEL)
-        CK(cudaMemsetAsync(base + L.off_fv, 0,
-                           real_size(s->prec) * (size_t)std::max<int64_t>(1, L.n_face) * (FVLBM_Q - 1), s->stream),
-           "clear face values");
     CK(cudaMemsetAsync(base + L.off_flag, 0, 16, s->stream), "clear flag");
 
     DevView& v = s->v;
@@ -922,9 +863,10 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     v.n_face = L.n_face;
     v.maxf = L.maxf;
     v.n_inst = M.n_inst;
-    v.desc = (const uint2*)(base + L.off_desc);
+    v.link = (const uint4*)(base + L.off_link);
     v.geo = base + L.off_geo;
-    v.nbr = (const int32_t*)(base + L.off_nbr);
+    v.bctag = (const uint16_t*)(base + L.off_bctag);
+    v.nbr = (const int4*)(base + L.off_nbr);
     v.area = (const double*)(base + L.off_area);
     v.grp = (const int32_t*)(base + L.off_grp);
     v.iperm = (const int32_t*)(base + L.off_iperm);
@@ -950,11 +892,10 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
         v.tile = L.tp.tile;
         v.sms = device_sms(p0.device);
         v.n_tiles = L.tp.n_tiles;
-        v.tile_begin = (const int64_t*)(base + L.off_tbegin);
-        v.halo_ptr = (const int64_t*)(base + L.off_hptr);
+        v.tiles = (const TileRec*)(base + L.off_tiles);
         v.halo = (const int32_t*)(base + L.off_halo);
-        v.r1_ptr = (const int64_t*)(base + L.off_r1ptr);
-        v.r1link = (const uint32_t*)(base + L.off_r1link);
+        v.r1link = (const uint4*)(base + L.off_r1link);
+        v.n_r1 = L.tp.n_r1;
     }
     s->pingpong = L.pingpong;
     s->buf[0] = v.fa;

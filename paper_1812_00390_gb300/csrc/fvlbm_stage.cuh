@@ -50,21 +50,19 @@ template <> struct BcVal<float> {
 template <typename T, bool DEV, typename NormalFn>
 __device__ __forceinline__ Ghost<T> ghost_state(uint32_t kind, const BcParam& b, T rho, T ux, T uy, NormalFn normal) {
     Ghost<T> g{rho, ux, uy, false, false, false};
-    if (kind == SK_WALL) {
+    if (kind == LK_WALL) {
         g.ux = BcVal<T>::uwx(b);
         g.uy = BcVal<T>::uwy(b);
-    } else if (kind == SK_INLET) {
+    } else if (kind == LK_INLET) {
         if (b.external) g.r = BcVal<T>::template rho<DEV>(b);
         g.ux = BcVal<T>::uix(b);
         g.uy = BcVal<T>::uiy(b);
         g.io = true;
-    } else if (kind == SK_OUTLET) {
-        if (b.external) {
-            g.zero = true;
-        } else {
-            g.r = BcVal<T>::template rho<DEV>(b);
-            g.io = true;
-        }
+    } else if (kind == LK_OUTLET) {
+        g.zero = true;
+    } else if (kind == LK_PRESSURE) {
+        g.r = BcVal<T>::template rho<DEV>(b);
+        g.io = true;
     } else {   // symmetry: the face's unit normal is needed only here
         const typename Vec2<T>::type n = normal();
         const T inv = T(1) / sqrt(n.x * n.x + n.y * n.y);
@@ -87,124 +85,144 @@ __device__ __forceinline__ T ghost_delta(const Ghost<T>& g, int a, T fa, T fe) {
 template <typename T>
 __device__ __forceinline__ bool finite_val(T x) { return isfinite(x); }
 
-// rho, u of a cell for its boundary slots (ghost states); cells with interior
-// slots only do not need them before the collision.
-template <typename T, bool DEV, int MAXF>
-__device__ __forceinline__ void boundary_moments(const uint2* d, const T* f, T& rho, T& ux, T& uy) {
-    bool bc = false;
+__device__ __forceinline__ uint32_t link_kind(uint32_t d) { return (d >> LINK_KIND_SHIFT) & 7u; }
+__device__ __forceinline__ uint32_t link_row(uint32_t d) { return d >> LINK_ROW_SHIFT; }
+__device__ __forceinline__ bool link_a_leaves(uint32_t d, int p) { return (d >> (LINK_PAIR_SHIFT + p)) & 1u; }
+__device__ __forceinline__ bool link_boundary(uint32_t d) { return link_kind(d) - LK_WALL <= LK_SYMMETRY - LK_WALL; }
+// Boundary slots whose outgoing values are reconstructed (inlets, pressure
+// outlets); on the others every face value is a ghost value (Sec. 2.4.2).
+__device__ __forceinline__ bool kind_io(uint32_t kind) { return kind == LK_INLET || kind == LK_PRESSURE; }
+
+template <typename T> __device__ __forceinline__ void to_pairs(const T* f, Pair<T>* p) {
 #pragma unroll
-    for (int k = 0; k < MAXF; k++) bc |= (d[k].x & 0xFF) > SK_INTERIOR;
-    rho = ux = uy = T(0);
-    if (bc) moments<T, DEV>(f, rho, ux, uy);
+    for (int q = 0; q < 4; q++) p[q] = make_pair2(f[dir_a(q)], f[dir_b(q)]);
+}
+template <typename T> __device__ __forceinline__ void from_pairs(const Pair<T>* p, T* f) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) split2(p[q], f[dir_a(q)], f[dir_b(q)]);
 }
 
-// Least-squares gradient (Eq. leastsquare) of f_1..f_8 of one cell from the
-// differences to its stencil values.  d: the cell's slot descriptors;
-// fnb(k, fj) fills fj[1..8] with the neighbour values across interior slot k.
-// On boundary slots it also writes the face values that are ghost values
-// (Sec. 2.4.2: all directions of walls, symmetry planes and external outlets,
-// inflow directions of inlets and internal outlets; half way to the ghost for
-// symmetry) into face(k) (stride `stride`; null: not written).
-template <typename T, bool DEV, int MAXF, typename Geo, typename Nb, typename Row>
-__device__ __forceinline__ void lsq_gradient(const uint2* d, const Geo& G, const BcParam* bcs, const T* f,
-                                             T rho, T ux, T uy, T* gx, T* gy, Nb fnb, int64_t stride, Row face) {
+// Slots (bit k) that some active thread of the warp uses: a polygon with
+// fewer faces than MAXF leaves its last slots empty, and when every cell of a
+// warp does (a warp of triangles in a 4-slot mesh), the warp skips them as a
+// whole.  Slots 0..2 are always used.
+template <int MAXF>
+__device__ __forceinline__ uint32_t warp_slots(const uint32_t* d) {
+    uint32_t u = 7u;
 #pragma unroll
-    for (int a = 0; a < FVLBM_Q - 1; a++) gx[a] = gy[a] = T(0);
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) {
-        const uint32_t kind = d[k].x & 0xFF;
-        if (kind == SK_NONE) continue;
-        const typename Vec2<T>::type c = G.cg(k);
-        if (kind == SK_INTERIOR) {
-            T fj[FVLBM_Q];
-            fnb(k, fj);
-#pragma unroll
-            for (int a = 1; a < FVLBM_Q; a++) {
-                const T dd = fj[a] - f[a];
-                gx[a - 1] += c.x * dd;
-                gy[a - 1] += c.y * dd;
-            }
-        } else {
-            // the ghost difference enters the gradient and, for every direction
-            // not reconstructed from the gradient, gives the face value at once
-            const Ghost<T> g = ghost_state<T, DEV>(kind, bcs[d[k].x >> 16], rho, ux, uy, [&] { return G.nv(k); });
-            const uint32_t mask = (d[k].x >> 8) & 0xFF;
-            T* fo = face(k);
-#pragma unroll
-            for (int a = 1; a < FVLBM_Q; a++) {
-                const T dd = ghost_delta<T, DEV>(g, a, f[a], feqs<T, DEV>(a, rho, ux, uy));
-                gx[a - 1] += c.x * dd;
-                gy[a - 1] += c.y * dd;
-                if (fo && !(g.io && ((mask >> (a - 1)) & 1u)))
-                    fo[(a - 1) * stride] = g.sym ? f[a] + T(0.5) * dd : f[a] + dd;
-            }
-        }
-    }
+    for (int k = 3; k < MAXF; k++)
+        if (link_kind(d[k]) != LK_NONE) u |= 1u << k;
+    return __reduce_or_sync(__activemask(), u);
 }
 
-// Values of one cell on its faces (Eq. lslrflux, Sec. 2.4.2) into a face
-// table with direction stride `stride`: on interior faces the directions in
-// the slot's writer mask; on inlet and internal-outlet faces the directions
-// the cell flows out through (the reconstruction f_i + grad f_i . r; every
-// other boundary face value is the ghost value, written by lsq_gradient).
-// face(k) is the slot's row in the table, or null to skip the slot.
-template <typename T, bool DEV, int MAXF, typename Geo, typename Row>
-__device__ __forceinline__ void write_faces(const uint2* d, const Geo& G, const BcParam* bcs, const T* f,
-                                            T rho, T ux, T uy, const T* gx, const T* gy, int64_t stride, Row face) {
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) {
-        const uint32_t kind = d[k].x & 0xFF;
-        if (kind == SK_NONE) continue;
-        T* fo = face(k);
-        if (!fo) continue;
-        const uint32_t mask = (d[k].x >> 8) & 0xFF;
-        const typename Vec2<T>::type r = G.rv(k);
-        if (kind == SK_INTERIOR) {
-#pragma unroll
-            for (int a = 1; a < FVLBM_Q; a++)
-                if (mask & (1u << (a - 1))) fo[(a - 1) * stride] = f[a] + gx[a - 1] * r.x + gy[a - 1] * r.y;
-        } else {
-            // inlet / internal outlet: directions the cell flows out through
-            // take the reconstruction (the others were written with the gradient)
-            const BcParam& b = bcs[d[k].x >> 16];
-            if (kind == SK_INLET || (kind == SK_OUTLET && !b.external)) {
-#pragma unroll
-                for (int a = 1; a < FVLBM_Q; a++)
-                    if ((mask >> (a - 1)) & 1u) fo[(a - 1) * stride] = f[a] + gx[a - 1] * r.x + gy[a - 1] * r.y;
-            }
-        }
-    }
-}
-
-// Flux sum of Eq. (rhs) from a face table: sum over the slots of
-// (e_a . n dl / A) f_face (deviation mode: of f_face - f_a, the same in exact
-// arithmetic because the face vectors of a closed cell sum to zero, without
-// the rounding of the FP32 face vectors acting on the constant part of g).
-// face(k, fa) fills fa[0..7] with the values of directions 1..8 on slot k.
-template <typename T, bool DEV, int MAXF, typename Face>
-__device__ __forceinline__ void flux_sum(const uint2* d, const typename Vec2<T>::type* n, const T* f, T* flux,
-                                         Face face) {
-#pragma unroll
-    for (int a = 0; a < FVLBM_Q; a++) flux[a] = T(0);
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) {
-        if ((d[k].x & 0xFF) == SK_NONE) continue;
-        T fa[FVLBM_Q - 1];
-        face(k, fa);
-#pragma unroll
-        for (int a = 1; a < FVLBM_Q; a++) {
-            const T en = T(EXA(a)) * n[k].x + T(EYA(a)) * n[k].y;
-            flux[a] += en * (DEV ? fa[a - 1] - f[a] : fa[a - 1]);
-        }
-    }
-}
-
-// cp.async copy of one 4- or 8-byte element from global to shared memory.
+// One slot's part of the least-squares gradient (Eq. leastsquare) of the eight
+// moving directions: grad += c (f_neighbour - f), half h of the pairs (2 h, 2 h + 1).
 template <typename T>
-__device__ __forceinline__ void cp_async_elem(T* dst, const T* src) {
+__device__ __forceinline__ void add_gradient(const Quad<T>& nb, const Pair<T>& cx, const Pair<T>& cy, int h,
+                                             const Pair<T>* f, Pair<T>* gx, Pair<T>* gy) {
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        const int p = 2 * h + q;
+        const Pair<T> dd = sub2(make_pair2(nb.v[2 * q], nb.v[2 * q + 1]), f[p]);
+        gx[p] = fma2(cx, dd, gx[p]);
+        gy[p] = fma2(cy, dd, gy[p]);
+    }
+}
+
+// The values that leave a cell through one face (Eq. lslrflux): of each pair
+// the direction that leaves, f + grad f . r.  FP32 computes both directions in
+// one packed operation and picks; FP64, whose units are the limit (16 cycles
+// per warp instruction and SM, whatever the active lanes), picks the operands
+// first and computes four values instead of eight.
+__device__ __forceinline__ Quad<float> leaving(uint32_t d, const Pair<float>* f, const Pair<float>* gx,
+                                               const Pair<float>* gy, const float2& r) {
+    const Pair<float> rx = make_pair2(r.x, r.x), ry = make_pair2(r.y, r.y);
+    Quad<float> o;
+#pragma unroll
+    for (int p = 0; p < 4; p++) {
+        float a, b;
+        split2(fma2(gy[p], ry, fma2(gx[p], rx, f[p])), a, b);
+        o.v[p] = link_a_leaves(d, p) ? a : b;
+    }
+    return o;
+}
+__device__ __forceinline__ Quad<double> leaving(uint32_t d, const Pair<double>* f, const Pair<double>* gx,
+                                                const Pair<double>* gy, const double2& r) {
+    Quad<double> o;
+#pragma unroll
+    for (int p = 0; p < 4; p++) {
+        const bool s = link_a_leaves(d, p);
+        o.v[p] = fma(s ? gy[p].x : gy[p].y, r.y, fma(s ? gx[p].x : gx[p].y, r.x, s ? f[p].x : f[p].y));
+    }
+    return o;
+}
+
+// One slot's part of the flux sum of Eq. (rhs): (e . n dl / A) times the face
+// value of each direction (deviation mode: minus the cell's own value, the same
+// in exact arithmetic because the face vectors of a closed cell sum to zero,
+// without the rounding of the FP32 face vectors acting on the constant part of
+// g).  out: what the cell sends through the face, in: what it receives.
+template <typename T, bool DEV>
+__device__ __forceinline__ void add_flux(uint32_t d, const typename Vec2<T>::type& n, const Quad<T>& out,
+                                         const Quad<T>& in, const Pair<T>* f, Pair<T>* flux) {
+    const T en[4] = {n.x, n.y, n.x + n.y, n.y - n.x};
+#pragma unroll
+    for (int p = 0; p < 4; p++) {
+        const bool s = link_a_leaves(d, p);
+        Pair<T> v = make_pair2(s ? out.v[p] : in.v[p], s ? in.v[p] : out.v[p]);
+        if constexpr (DEV) v = sub2(v, f[p]);
+        flux[p] = fma2(make_pair2(en[p], -en[p]), v, flux[p]);
+    }
+}
+
+// Boundary slots of one cell (Sec. 2.4): the ghost differences enter the
+// gradient; where the cell's faces are in the face table (own rows, and ghost
+// rows for what enters), the boundary face values that are ghost values are
+// written: everything on walls, symmetry planes (half way to the ghost) and
+// external outlets, what enters on inlets and pressure outlets.
+//   tag(k)  boundary tag, lsq(k) / face(k) vectors of slot k
+//   own(k, q), ghost(k, q)  store a row
+template <typename T, bool DEV, int MAXF, typename Tag, typename Lsq, typename Face, typename Own, typename In>
+__device__ __forceinline__ void boundary_slots(const uint32_t* d, const BcParam* bcs, T f0, const Pair<T>* fp,
+                                               Pair<T>* gx, Pair<T>* gy, Tag tag, Lsq lsq, Face face, Own own, In in) {
+    T f[FVLBM_Q];
+    f[0] = f0;
+    from_pairs(fp, f);
+    T rho, ux, uy;
+    moments<T, DEV>(f, rho, ux, uy);
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (!link_boundary(d[k])) continue;
+        const uint32_t kind = link_kind(d[k]);
+        const Ghost<T> g = ghost_state<T, DEV>(kind, bcs[tag(k)], rho, ux, uy, [&] { return face(k); });
+        const typename Vec2<T>::type c = lsq(k);
+        const Pair<T> cx = make_pair2(c.x, c.x), cy = make_pair2(c.y, c.y);
+        Quad<T> qo, qi;
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            const int a = dir_a(p), b = dir_b(p);
+            const T da = ghost_delta<T, DEV>(g, a, f[a], feqs<T, DEV>(a, rho, ux, uy));
+            const T db = ghost_delta<T, DEV>(g, b, f[b], feqs<T, DEV>(b, rho, ux, uy));
+            const Pair<T> dd = make_pair2(da, db);
+            gx[p] = fma2(cx, dd, gx[p]);
+            gy[p] = fma2(cy, dd, gy[p]);
+            const T va = g.sym ? f[a] + T(0.5) * da : f[a] + da, vb = g.sym ? f[b] + T(0.5) * db : f[b] + db;
+            const bool s = link_a_leaves(d[k], p);
+            qo.v[p] = s ? va : vb;
+            qi.v[p] = s ? vb : va;
+        }
+        in(k, qi);
+        if (!g.io) own(k, qo);
+    }
+}
+
+// cp.async copy of one 16- or 8-byte element from global to shared memory
+// (16 bytes: past L1).
+template <int BYTES>
+__device__ __forceinline__ void cp_async_elem(void* dst, const void* src) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-    if constexpr (sizeof(T) == 4)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(src) : "memory");
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(src) : "memory");
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(src) : "memory");
 }
@@ -213,31 +231,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"((uint32_t)bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-// Geometry of a fused-stage gradient cell: with up to 4 slots its
-// least-squares vectors in registers (loaded before the staging barrier; 8
-// slots would spill), else and for its reconstruction and face vectors from
-// global memory (through L1, which the small shared-memory footprint leaves
-// large).
-template <typename T, int MAXF> struct RegGeo {
-    typedef typename Vec2<T>::type T2;
-    static constexpr bool REGS = MAXF <= 4;
-    T2 c[REGS ? MAXF : 1];
-    GeoRef<T, MAXF> G;
-    __device__ __forceinline__ void load(const void* desc, const void* geo, uint32_t i) {
-        G = GeoRef<T, MAXF>(desc, geo, i);
-        if constexpr (REGS) {
-#pragma unroll
-            for (int k = 0; k < MAXF; k++) c[k] = G.cg(k);
-        }
-    }
-    __device__ __forceinline__ T2 cg(int k) const {
-        if constexpr (REGS) return c[k];
-        else return G.cg(k);
-    }
-    __device__ __forceinline__ T2 rv(int k) const { return G.rv(k); }
-    __device__ __forceinline__ T2 nv(int k) const { return G.nv(k); }
-};
-
 // Collision and time update of one cell (Eq. rhs, Sec. 2.3): rhs = -flux -
 // (f - f^eq) / tau, then out = base + beta dt rhs (multistage; the base state
 // is fb when use_fb, else f itself) or the AB2 combination.  Returns false
@@ -302,250 +295,187 @@ __device__ __forceinline__ bool update_cell(const DevView& v, const InstParam& P
 }
 
 // ------------------------------------------------------------------ kernels
-// Two-kernel stage, kernel 1 (Steps 1-3): per cell the gradient, then the
-// value of every (face, direction) it is the upwind side of, and every
-// direction of its boundary faces, into the face table (one writer each).
-template <typename T, typename S, int MAXF, bool DEV>
-__global__ void __launch_bounds__(256) face_values_kernel(DevView v, const S* __restrict__ fin) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= v.n_grad) return;   // owned cells and, in a partition, the first ghost ring
-    const GeoRef<T, MAXF> G(v.desc, v.geo, i);
-    const int32_t* nb = v.nbr + blk_index(i, MAXF);
-    uint2 d[MAXF];
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) d[k] = G.desc(k);
-    T f[FVLBM_Q];
-    CellIO<S>::template load<T, DEV>(fin, i, v.inst[v.grp[i]], f);
-    T rho, ux, uy;
-    boundary_moments<T, DEV, MAXF>(d, f, rho, ux, uy);
-    T gx[FVLBM_Q - 1], gy[FVLBM_Q - 1];
-    T* fv = (T*)v.fv;
-    auto row = [&](int k) { return fv + d[k].y; };
-    lsq_gradient<T, DEV, MAXF>(d, G, v.bc, f, rho, ux, uy, gx, gy, [&](int k, T* fj) {
-        const int64_t j = nb[k * BLK];
-        CellIO<S>::template load<T, DEV>(fin, j, v.inst[v.grp[j]], fj);
-    }, v.n_face, row);
-    write_faces<T, DEV, MAXF>(d, G, v.bc, f, rho, ux, uy, gx, gy, v.n_face, row);
+// Two-kernel stage.  The face table holds, for every (cell, slot), the four
+// values that leave the cell there (one side of each (face, direction) is its
+// only writer, with no test of who writes: a warp stores whole rows), then
+// the ghost records.  Row of (cell i, slot k): blk_index(i, MAXF) + k * BLK.
+template <typename T> __device__ __forceinline__ typename Vec16<T>::type* face_row(void* fv, int64_t row) {
+    return (typename Vec16<T>::type*)fv + row * QUAD_UNITS<T>;
 }
 
-// Two-kernel stage, kernel 2 (Steps 4-5): flux sum over the cell's faces,
-// collision and time update.
+// Kernel 1 (Steps 1-3): per cell the gradient, then what leaves it through
+// every face, and the ghost values of its boundary faces.
+template <typename T, typename S, int MAXF, bool DEV>
+__global__ void __launch_bounds__(256) face_values_kernel(DevView v, const S* __restrict__ fin) {
+    typedef typename Vec2<T>::type T2;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= v.n_grad) return;   // owned cells and, in a partition, the first ghost ring
+    const GeoRef<T, MAXF> G(v.geo, i);
+    uint32_t d[MAXF];
+    load_links<MAXF>(v.link, i, d);
+    int32_t nb[MAXF];
+    load_links<MAXF>((const uint4*)v.nbr, i, (uint32_t*)nb);
+    T f[FVLBM_Q];
+    CellIO<S>::template load<T, DEV>(fin, i, v.inst[v.grp[i]], f);
+    Pair<T> fp[4], gx[4], gy[4];
+    to_pairs(f, fp);
+#pragma unroll
+    for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
+    const uint32_t used = warp_slots<MAXF>(d);
+    bool bc = false;
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (k >= 3 && !((used >> k) & 1u)) continue;
+        const bool edge = link_boundary(d[k]);
+        bc |= edge;
+        const int64_t j = edge ? i : (int64_t)nb[k];
+        T fj[FVLBM_Q];
+        CellIO<S>::template load<T, DEV>(fin, j, v.inst[v.grp[j]], fj);
+        const T2 c = G.get(GEO_LSQ, k);
+        const Pair<T> cx = make_pair2(c.x, c.x), cy = make_pair2(c.y, c.y);
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+            add_gradient(Quad<T>{{fj[dir_a(2 * h)], fj[dir_b(2 * h)], fj[dir_a(2 * h + 1)], fj[dir_b(2 * h + 1)]}}, cx,
+                         cy, h, fp, gx, gy);
+    }
+    const int64_t row = blk_index(i, MAXF);
+    if (bc)
+        boundary_slots<T, DEV, MAXF>(d, v.bc, f[0], fp, gx, gy, [&](int k) { return v.bctag[i * MAXF + k]; },
+                                     [&](int k) { return G.get(GEO_LSQ, k); }, [&](int k) { return G.get(GEO_FACE, k); },
+                                     [&](int k, const Quad<T>& q) { store_quad(face_row<T>(v.fv, row + k * BLK), 1, q); },
+                                     [&](int k, const Quad<T>& q) {
+                                         if (i < v.n_cell) store_quad(face_row<T>(v.fv, v.np * MAXF + nb[k]), 1, q);
+                                     });
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (k >= 3 && !((used >> k) & 1u)) continue;
+        const uint32_t kind = link_kind(d[k]);
+        if (kind >= LK_WALL && !kind_io(kind)) continue;   // ghost values, or no face
+        store_quad(face_row<T>(v.fv, row + k * BLK), 1, leaving(d[k], fp, gx, gy, G.get(GEO_MID, k)));
+    }
+}
+
+// Kernel 2 (Steps 4-5): flux sum over the cell's faces, collision and time
+// update.
 template <typename T, typename S, int MAXF, bool DEV>
 __global__ void __launch_bounds__(256) update_kernel(DevView v, const S* __restrict__ fin, const S* fbase, S* fout,
                                                      T beta, int mode) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= v.n_cell) return;
     const InstParam& P = v.inst[v.grp[i]];
-    const GeoRef<T, MAXF> G(v.desc, v.geo, i);
-    uint2 d[MAXF];
-    typename Vec2<T>::type n[MAXF];
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) {
-        d[k] = G.desc(k);
-        n[k] = G.nv(k);
-    }
+    const GeoRef<T, MAXF> G(v.geo, i);
+    uint32_t d[MAXF];
+    load_links<MAXF>(v.link, i, d);
+    int32_t nb[MAXF];
+    load_links<MAXF>((const uint4*)v.nbr, i, (uint32_t*)nb);
     T f[FVLBM_Q];
     CellIO<S>::template load<T, DEV>(fin, i, P, f);
-    T rho, ux, uy;
-    moments<T, DEV>(f, rho, ux, uy);
-    T flux[FVLBM_Q];
-    const T* fv = (const T*)v.fv;
-    flux_sum<T, DEV, MAXF>(d, n, f, flux, [&](int k, T* fa) {
-        const T* p = fv + d[k].y;
+    Pair<T> fp[4], fx[4];
+    to_pairs(f, fp);
 #pragma unroll
-        for (int a = 0; a < FVLBM_Q - 1; a++) fa[a] = p[a * v.n_face];
-    });
-    T fb[FVLBM_Q];
+    for (int p = 0; p < 4; p++) fx[p] = make_pair2(T(0), T(0));
+    const int64_t row = blk_index(i, MAXF);
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (link_kind(d[k]) == LK_NONE) continue;
+        const int64_t from = link_boundary(d[k]) ? v.np * MAXF + nb[k]
+                                                 : blk_index((int64_t)nb[k], MAXF) + (int64_t)link_row(d[k]) * BLK;
+        add_flux<T, DEV>(d[k], G.get(GEO_FACE, k), load_quad(face_row<T>(v.fv, row + k * BLK), 1),
+                         load_quad(face_row<T>(v.fv, from), 1), fp, fx);
+    }
+    T flux[FVLBM_Q], fb[FVLBM_Q];
+    flux[0] = T(0);
+    from_pairs(fx, flux);
     const bool rk_base = mode == MODE_RK && fbase != fin;
     if (rk_base) CellIO<S>::template load<T, DEV>(fbase, i, P, fb);
+    T rho, ux, uy;
+    moments<T, DEV>(f, rho, ux, uy);
     // the FP64 two-kernel stage is bound by the FP64 units: the shorter multistage form
     if (!update_cell<T, S, DEV, sizeof(T) == 8>(v, P, i, f, rho, ux, uy, flux, fb, rk_base, fout, beta, mode))
         *v.flag = 1;
 }
 
-// Slots (bit k) that some active thread of the warp uses: a polygon with
-// fewer faces than MAXF leaves its last slots empty, and when every cell of a
-// warp does (a warp of triangles in a 4-slot mesh), the warp skips them as a
-// whole.  Slots 0..2 are always used.
-template <int MAXF>
-__device__ __forceinline__ uint32_t warp_slots(const uint2* d) {
-    uint32_t u = 7u;
-#pragma unroll
-    for (int k = 3; k < MAXF; k++)
-        if ((d[k].x & 0xFF) != SK_NONE) u |= 1u << k;
-    return __reduce_or_sync(__activemask(), u);
-}
-
-// Fused stage, phase 2 for one local cell x (a tile cell, or a 1-ring entry),
-// everything in shared memory: its least-squares gradient (Eq. leastsquare)
-// and its values on the tile's faces.  The planner links every slot without
-// a neighbour (boundary faces, unused slots) to the cell itself, and gives
-// unused slots zero geometry and an empty mask, so the loops over the slots
-// test no slot kind:
-//   1. gradient over all slots from the neighbour differences (zero for the
-//      self-linked slots);
-//   2. only for cells with boundary slots (rare): the ghost differences of
-//      Sec. 2.4.1 enter the gradient, and the boundary face values that are
-//      ghost values are written (Sec. 2.4.2);
-//   3. every slot writes the reconstruction f + grad f . (x_f - x_i)
-//      (Eq. lslrflux) for the directions in its mask: the upwind ones on
-//      interior faces, the outflow ones on inlet and internal-outlet faces,
-//      none elsewhere; a 1-ring entry writes only the faces it shares with
-//      the tile (the others carry no local face).
-template <typename T, bool DEV, int MAXF, int LS, int FS, typename Geo>
-__device__ __forceinline__ void tile_gradient_faces(const uint2* dx, const Geo& H, const BcParam* bcs, const T* fs,
-                                                    T* fvs, int x, T* f) {
-#pragma unroll
-    for (int a = 0; a < FVLBM_Q; a++) f[a] = fs[a * LS + x];
-    T gx[FVLBM_Q - 1], gy[FVLBM_Q - 1];
-#pragma unroll
-    for (int a = 0; a < FVLBM_Q - 1; a++) gx[a] = gy[a] = T(0);
-    const uint32_t used = warp_slots<MAXF>(dx);
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) {
-        if (k >= 3 && !((used >> k) & 1u)) continue;
-        const typename Vec2<T>::type c = H.cg(k);
-        const T* p = fs + (dx[k].y & 0xFFFF);
-#pragma unroll
-        for (int a = 1; a < FVLBM_Q; a++) {
-            const T dd = p[a * LS] - f[a];
-            gx[a - 1] += c.x * dd;
-            gy[a - 1] += c.y * dd;
-        }
-    }
-    bool bc = false;
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) bc |= (dx[k].x & 0xFF) > SK_INTERIOR;
-    if (bc) {
-        T rho, ux, uy;
-        moments<T, DEV>(f, rho, ux, uy);
-#pragma unroll
-        for (int k = 0; k < MAXF; k++) {
-            const uint32_t kind = dx[k].x & 0xFF;
-            if (kind <= SK_INTERIOR) continue;
-            const Ghost<T> g = ghost_state<T, DEV>(kind, bcs[dx[k].x >> 16], rho, ux, uy, [&] { return H.nv(k); });
-            const typename Vec2<T>::type c = H.cg(k);
-            const uint32_t mask = (dx[k].x >> 8) & 0xFF;
-            const uint32_t lf = dx[k].y >> 16;
-            T* fo = lf == LINK_NONE ? nullptr : fvs + lf;
-#pragma unroll
-            for (int a = 1; a < FVLBM_Q; a++) {
-                const T dd = ghost_delta<T, DEV>(g, a, f[a], feqs<T, DEV>(a, rho, ux, uy));
-                gx[a - 1] += c.x * dd;
-                gy[a - 1] += c.y * dd;
-                if (fo && !((mask >> (a - 1)) & 1u)) fo[(a - 1) * FS] = g.sym ? f[a] + T(0.5) * dd : f[a] + dd;
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < MAXF; k++) {
-        if (k >= 3 && !((used >> k) & 1u)) continue;
-        const uint32_t lf = dx[k].y >> 16;
-        const uint32_t mask = lf == LINK_NONE ? 0u : (dx[k].x >> 8) & 0xFF;
-        T* fo = fvs + (lf == LINK_NONE ? 0u : lf);
-        const typename Vec2<T>::type r = H.rv(k);
-#pragma unroll
-        for (int a = 1; a < FVLBM_Q; a++)
-            if ((mask >> (a - 1)) & 1u) fo[(a - 1) * FS] = f[a] + gx[a - 1] * r.x + gy[a - 1] * r.y;
-    }
-}
-
 // Fused stage: one CTA per tile of consecutive cells (Hilbert order; tile
 // and 1-ring together at most TILE cells), everything between the state read
 // and the state write in shared memory:
-//   phase 1  cp.async of the state of the tile, its 1-ring and its 2-ring
-//            (the 16-bit formats raw, each cell decoded by the thread that
-//            staged it) and of the instance id of each tile cell; the slot
-//            descriptors and the
-//            least-squares vectors of each thread's gradient cell into
-//            registers
+//   phase 1  the moving directions of the tile, its 1-ring and its 2-ring into
+//            shared memory (16-byte cp.async; the 16-bit formats raw, each cell
+//            decoded by the thread that staged it); links and least-squares
+//            vectors of each thread's gradient cell into registers
 //   phase 2  per tile and 1-ring cell (one per thread): the gradient
-//            (Eq. leastsquare) and its values on the tile's faces
-//            (Eq. lslrflux / Sec. 2.4.2): on interior faces the directions it
-//            writes (upwind side), on boundary faces (tile cells) every
-//            direction -- one writer per (face, direction), into a table of
-//            the tile's faces; a tile cell's thread keeps its state
-//   phase 3  per tile cell: flux sum from the face table, collision and the
-//            time update (Eq. rhs, Sec. 2.3)
+//            (Eq. leastsquare) and, per face, the four values that leave the
+//            cell there (Eq. lslrflux), as one 16-byte row of the face table (row
+//            k * TILE + x: no bank conflict); boundary cells also their ghost
+//            values (Sec. 2.4.2).  A tile cell's thread keeps its state
+//   phase 3  per tile cell: per face its own row and the neighbour's (or
+//            ghost) row give all eight face values; flux sum, collision and
+//            the time update (Eq. rhs, Sec. 2.3)
 // The global loads of each phase are issued before the barrier that precedes
 // it, so that their latency overlaps the wait, and each CTA prefetches into L2
 // the data of a tile that starts somewhat under one CTA lifetime later (pf =
-// 5/8 of the resident CTAs ahead).  The kernel is bound by shared-memory
-// traffic more than by DRAM: what a thread can hold in registers (its own
-// state, its least-squares vectors) or read through L1 (reconstruction and
-// face vectors) stays out of shared memory, whose small footprint leaves L1
-// large.  Shared-memory strides are compile-time constants (TileDims); the
-// planner keeps every tile within them.
+// 5/8 of the resident CTAs ahead).  Shared-memory strides are compile-time
+// constants (TileDims); the planner keeps every tile within them.
 template <typename T, typename S, int MAXF, bool DEV, int TILE>
 __global__ void __launch_bounds__(TILE, (sizeof(T) == 4 ? 1024 : 512) / TILE > 0 ? (sizeof(T) == 4 ? 1024 : 512) / TILE : 1)
     stage_tile_kernel(DevView v, const S* __restrict__ fin, const S* fbase, S* fout, T beta, int mode, int pf) {
-    constexpr int LS = TileDims<TILE, MAXF, sizeof(T)>::LS;
-    constexpr int FS = TileDims<TILE, MAXF, sizeof(T)>::FS;
+    typedef TileDims<TILE, MAXF, sizeof(T)> D;
     typedef typename Vec2<T>::type T2;
+    typedef typename Vec16<T>::type V;
+    constexpr int LS = D::LS, ROWS = D::ROWS;
+    constexpr int SU = 8 / Vec16<T>::N;      // 16-byte units of a cell's moving directions
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T* fs = (T*)smem_raw;            // [9][LS]  f of the local cells
-    T* fvs = fs + FVLBM_Q * LS;      // [8][FS]  face values of directions 1..8
-    int32_t* sgrp = (int32_t*)(fvs + (FVLBM_Q - 1) * FS);   // [TILE] instance of each tile cell
+    V* fs = (V*)smem_raw;         // [SU][LS]         moving directions of the local cells
+    V* tab = fs + SU * LS;        // [QUAD_UNITS][ROWS]  face table
     // cell, halo and 1-ring indices in 32 bits: the set-up keeps every array
     // of a fused-stage solver below 2^32 elements
     const uint32_t t = blockIdx.x;
-    const uint32_t c0 = (uint32_t)v.tile_begin[t];
-    const int nt = (int)((uint32_t)v.tile_begin[t + 1] - c0);
-    const uint32_t h0 = (uint32_t)v.halo_ptr[t];
-    const int nh = (int)((uint32_t)v.halo_ptr[t + 1] - h0);
-    const uint32_t q0 = (uint32_t)v.r1_ptr[t];
-    const int n1 = (int)((uint32_t)v.r1_ptr[t + 1] - q0);
+    const int4 ra = ((const int4*)(v.tiles + t))[0], rb = ((const int4*)(v.tiles + t))[1];
+    const uint32_t c0 = ra.x, h0 = ra.z, q0 = rb.x;
+    const int nt = ra.y, nh = ra.w, n1 = rb.y, inst = rb.z;
     const int l = threadIdx.x;
     const bool mine = l < nt;          // this thread owns tile cell l
     const uint32_t gi = c0 + l;
 
     // phase 1 (thread l's first local cell is local cell l).  The 16-bit split
-    // formats are staged raw (moments, packed non-equilibrium words, instance)
-    // in the face-table area, which is free until phase 2, and decoded by the
-    // thread that staged them.
+    // formats are staged raw in the face-table area, which is free until phase 2.
     constexpr bool PLAIN = sizeof(S) == sizeof(T);
-    float* rawc = (float*)fvs;                     // [3][LS]
-    uint32_t* raww = (uint32_t*)(rawc + 3 * LS);   // [3][LS]
-    int32_t* rawg = (int32_t*)(raww + 3 * LS);     // [LS]
-    static_assert(PLAIN || 7 * LS * 4 <= (FVLBM_Q - 1) * FS * (int)sizeof(T), "raw staging fits the face table");
+    uint4* rawh = (uint4*)tab;                     // [LS]
+    uint2* rawt = (uint2*)(rawh + LS);             // [LS]
+    static_assert(PLAIN || LS * 24 <= ROWS * 4 * (int)sizeof(T), "raw staging fits the face table");
+    const int n2 = nt + n1;            // gradient cells: the planner keeps nt + n1 <= TILE
     uint32_t gl = c0;
+    T f0 = T(0);
     for (int x = l; x < nt + nh; x += TILE) {
         const uint32_t gx = x < nt ? c0 + x : (uint32_t)v.halo[h0 + (x - nt)];
         if (x == l) gl = gx;
         if constexpr (PLAIN) {
-            const S* p = fin + blk_index(gx, FVLBM_Q);
+            const V* p = (const V*)CellIO<S>::pairs(fin, gx);
 #pragma unroll
-            for (int a = 0; a < FVLBM_Q; a++) cp_async_elem<T>(fs + a * LS + x, (const T*)p + a * BLK);
+            for (int u = 0; u < SU; u++) cp_async_elem<16>(fs + u * LS + x, p + u * BLK);
         } else {
-            const float* pc = CellIO<S>::cptr(fin, gx);
-            const uint32_t* pw = CellIO<S>::wptr(fin, gx);
-#pragma unroll
-            for (int q = 0; q < 3; q++) {
-                cp_async_elem<float>(rawc + q * LS + x, pc + q * BLK);
-                cp_async_elem<uint32_t>(raww + q * LS + x, pw + q * BLK);
-            }
-            cp_async_elem<int32_t>(rawg + x, v.grp + gx);
+            cp_async_elem<16>(rawh + x, CellIO<S>::head(fin, gx));
+            cp_async_elem<8>(rawt + x, CellIO<S>::tail(fin, gx));
         }
     }
-    // Phase 2 gives local cell x (tile cell, or 1-ring entry x - nt) to thread
-    // x: with the planner's bound nt + n1 <= TILE every thread has at most one.
-    // Its descriptors and local links are in flight during the wait.
-    const int n2 = nt + n1;
-    auto links = [&](int x, uint32_t g, uint2* d) {
-        const GeoRef<T, MAXF> H(v.desc, v.geo, g);
-        const uint32_t* rl = x < nt ? nullptr : v.r1link + blk_index(q0 + (uint32_t)(x - nt), MAXF);
-#pragma unroll
-        for (int k = 0; k < MAXF; k++) {
-            d[k] = H.desc(k);
-            if (x >= nt) d[k].y = rl[k * BLK];   // the 1-ring entry's local links
-        }
-    };
-    if (l < nt) cp_async_elem<int32_t>(sgrp + l, v.grp + c0 + l);
-    uint2 d[MAXF];
-    RegGeo<T, MAXF> H;
+    // phase 2 gives local cell x (tile cell, or 1-ring entry x - nt) to thread x
+    uint32_t d[MAXF];
+    T2 c[MAXF];
+    const GeoRef<T, MAXF> G(v.geo, gl);
     if (l < n2) {
-        links(l, gl, d);
-        H.load(v.desc, v.geo, gl);
+        if (mine) {
+            load_links<MAXF>(v.link, gi, d);
+        } else {
+#pragma unroll
+            for (int u = 0; u < MAXF / 4; u++) {
+                const uint4 x = v.r1link[u * v.n_r1 + q0 + (l - nt)];
+                d[4 * u] = x.x;
+                d[4 * u + 1] = x.y;
+                d[4 * u + 2] = x.z;
+                d[4 * u + 3] = x.w;
+            }
+        }
+        if constexpr (MAXF <= 4) G.load(GEO_LSQ, c);
+        if constexpr (PLAIN) f0 = (T)*CellIO<S>::rest(fin, gl);
     }
     // A CTA that starts somewhat before this one ends works on about tile
     // t + pf (pf = 5/8 of the CTAs resident on the GPU): bring that tile's
@@ -553,79 +483,116 @@ __global__ void __launch_bounds__(TILE, (sizeof(T) == 4 ? 1024 : 512) / TILE > 0
     // HBM.  The last thread does it once its own copies are in flight, so that
     // the loads of the other tile's bounds overlap them.
     if (l == TILE - 1 && pf > 0 && t + pf < v.n_tiles) {
-        const int64_t tp = t + pf;
-        const int64_t b0 = v.tile_begin[tp] >> BLK_SHIFT;
-        const int64_t nb = ((v.tile_begin[tp + 1] + BLK - 1) >> BLK_SHIFT) - b0;
+        const TileRec R = v.tiles[t + pf];
+        const int64_t b0 = R.c0 >> BLK_SHIFT;
+        const int64_t nb = ((R.c0 + R.nt + BLK - 1) >> BLK_SHIFT) - b0;
         constexpr int64_t SB = CellIO<S>::BLOCK_BYTES;
-        constexpr int64_t DB = (int64_t)MAXF * BLK * sizeof(uint2);
+        constexpr int64_t DB = (int64_t)MAXF * BLK * sizeof(uint32_t);
         constexpr int64_t GB = (int64_t)3 * MAXF * BLK * sizeof(T2);
         prefetch_l2((const unsigned char*)fin + b0 * SB, nb * SB);
         if (mode == MODE_RK && fbase != fin) prefetch_l2((const unsigned char*)fbase + b0 * SB, nb * SB);
-        prefetch_l2((const unsigned char*)v.desc + b0 * DB, nb * DB);
+        prefetch_l2((const unsigned char*)v.link + b0 * DB, nb * DB);
         prefetch_l2((const unsigned char*)v.geo + b0 * GB, nb * GB);
         // its halo list and 1-ring links (16-byte aligned cover of each range)
         auto range = [&](const void* base, int64_t begin, int64_t end) {
             const int64_t a = begin & ~(int64_t)15, e = (end + 15) & ~(int64_t)15;
             if (e > a) prefetch_l2((const unsigned char*)base + a, e - a);
         };
-        range(v.halo, 4 * v.halo_ptr[tp], 4 * v.halo_ptr[tp + 1]);
-        range(v.grp, 4 * v.tile_begin[tp], 4 * v.tile_begin[tp + 1]);   // instance ids
-        constexpr int64_t LB = (int64_t)MAXF * BLK * 4;   // bytes per block of 32 entries
-        range(v.r1link, (v.r1_ptr[tp] >> BLK_SHIFT) * LB, ((v.r1_ptr[tp + 1] + BLK - 1) >> BLK_SHIFT) * LB);
+        range(v.halo, 4 * (int64_t)R.h0, 4 * (int64_t)(R.h0 + R.nh));
+#pragma unroll
+        for (int u = 0; u < MAXF / 4; u++)
+            range(v.r1link + u * v.n_r1, 16 * (int64_t)R.q0, 16 * (int64_t)(R.q0 + R.n1));
+        if (R.inst < 0) range(v.grp, 4 * (int64_t)R.c0, 4 * (int64_t)(R.c0 + R.nt));
     }
     cp_async_wait_all();
     // a 16-bit state is decoded by the thread that staged it (its own copies
     // are complete after the wait), so one barrier serves both
-    if constexpr (PLAIN) __syncthreads();
     if constexpr (!PLAIN) {
         for (int x = l; x < nt + nh; x += TILE) {
-            const uint32_t w[3] = {raww[x], raww[LS + x], raww[2 * LS + x]};
+            const uint32_t gx = x < nt ? c0 + x : (uint32_t)v.halo[h0 + (x - nt)];
             T f[FVLBM_Q];
-            CellIO<S>::template decode<T>(rawc[x], rawc[LS + x], rawc[2 * LS + x], w, v.inst[rawg[x]], f);
+            CellIO<S>::template decode<T>(rawh[x], rawt[x], v.inst[inst >= 0 ? inst : v.grp[gx]], f);
+            if (x == l) f0 = f[0];
 #pragma unroll
-            for (int a = 0; a < FVLBM_Q; a++) fs[a * LS + x] = f[a];
+            for (int h = 0; h < 2; h++)
+                store_quad(fs + h * (SU / 2) * LS + x, LS,
+                           Quad<T>{{f[dir_a(2 * h)], f[dir_b(2 * h)], f[dir_a(2 * h + 1)], f[dir_b(2 * h + 1)]}});
         }
-        __syncthreads();
     }
+    __syncthreads();
 
     // phase 2 (a tile cell's thread keeps its state for phase 3)
-    T f[FVLBM_Q];
+    Pair<T> f[4];
     if (l < n2) {
-        tile_gradient_faces<T, DEV, MAXF, LS, FS>(d, H, v.bc, fs, fvs, l, f);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const Quad<T> q = load_quad(fs + h * (SU / 2) * LS + l, LS);
+            f[2 * h] = make_pair2(q.v[0], q.v[1]);
+            f[2 * h + 1] = make_pair2(q.v[2], q.v[3]);
+        }
+        Pair<T> gx[4], gy[4];
+#pragma unroll
+        for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
+        const uint32_t used = warp_slots<MAXF>(d);
+        bool bc = false;
+#pragma unroll
+        for (int k = 0; k < MAXF; k++) {
+            if (k >= 3 && !((used >> k) & 1u)) continue;
+            bc |= link_boundary(d[k]);
+            T2 ck;
+            if constexpr (MAXF <= 4) ck = c[k];
+            else ck = G.get(GEO_LSQ, k);
+            const Pair<T> cx = make_pair2(ck.x, ck.x), cy = make_pair2(ck.y, ck.y);
+            const V* nb = fs + (d[k] & LINK_NB_MASK);
+#pragma unroll
+            for (int h = 0; h < 2; h++) add_gradient(load_quad(nb + h * (SU / 2) * LS, LS), cx, cy, h, f, gx, gy);
+        }
+        if (bc)
+            boundary_slots<T, DEV, MAXF>(d, v.bc, f0, f, gx, gy, [&](int k) { return v.bctag[(int64_t)gl * MAXF + k]; },
+                                         [&](int k) { return G.get(GEO_LSQ, k); }, [&](int k) { return G.get(GEO_FACE, k); },
+                                         [&](int k, const Quad<T>& q) { store_quad(tab + k * TILE + l, ROWS, q); },
+                                         [&](int k, const Quad<T>& q) {
+                                             if (mine) store_quad(tab + link_row(d[k]), ROWS, q);
+                                         });
+#pragma unroll
+        for (int k = 0; k < MAXF; k++) {
+            if (k >= 3 && !((used >> k) & 1u)) continue;
+            // ghost values are in place, a 1-ring cell's other faces are not the tile's;
+            // an unused slot among used ones writes its (finite) state, read with weight zero
+            const uint32_t kind = link_kind(d[k]);
+            if (kind == LK_FLOW || kind == LK_NONE || kind_io(kind))
+                store_quad(tab + k * TILE + l, ROWS, leaving(d[k], f, gx, gy, G.get(GEO_MID, k)));
+        }
     }
     // phase 3 inputs, in flight during the wait
     T2 n[MAXF];
     T fb[FVLBM_Q];
     const bool rk_base = mode == MODE_RK && fbase != fin;
     if (mine) {
-        const GeoRef<T, MAXF> G(v.desc, v.geo, gi);
-#pragma unroll
-        for (int k = 0; k < MAXF; k++) n[k] = G.nv(k);
-        if (rk_base) CellIO<S>::template load<T, DEV>(fbase, gi, v.inst[v.grp[gi]], fb);
+        G.load(GEO_FACE, n);
+        if (rk_base) CellIO<S>::template load<T, DEV>(fbase, gi, v.inst[inst >= 0 ? inst : v.grp[gi]], fb);
     }
     __syncthreads();
 
-    // phase 3: flux of every slot from the face table, with no test of the
-    // slot kind (unused slots read face row 0 with a zero face vector)
     if (!mine) return;
-    const InstParam& P = v.inst[sgrp[l]];
-    T rho, ux, uy;
-    moments<T, DEV>(f, rho, ux, uy);
-    T flux[FVLBM_Q];
+    const InstParam& P = v.inst[inst >= 0 ? inst : v.grp[gi]];
+    Pair<T> fx[4];
 #pragma unroll
-    for (int a = 0; a < FVLBM_Q; a++) flux[a] = T(0);
+    for (int p = 0; p < 4; p++) fx[p] = make_pair2(T(0), T(0));
     const uint32_t used = warp_slots<MAXF>(d);
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
-        const T* p = fvs + (d[k].y >> 16);
-#pragma unroll
-        for (int a = 1; a < FVLBM_Q; a++) {
-            const T en = T(EXA(a)) * n[k].x + T(EYA(a)) * n[k].y;
-            flux[a] += en * (DEV ? p[(a - 1) * FS] - f[a] : p[(a - 1) * FS]);
-        }
+        add_flux<T, DEV>(d[k], n[k], load_quad(tab + k * TILE + l, ROWS), load_quad(tab + link_row(d[k]), ROWS), f, fx);
     }
-    if (!update_cell<T, S, DEV>(v, P, gi, f, rho, ux, uy, flux, fb, rk_base, fout, beta, mode))
+    T fa[FVLBM_Q], flux[FVLBM_Q];
+    fa[0] = f0;
+    from_pairs(f, fa);
+    flux[0] = T(0);
+    from_pairs(fx, flux);
+    T rho, ux, uy;
+    moments<T, DEV>(fa, rho, ux, uy);
+    if (!update_cell<T, S, DEV>(v, P, gi, fa, rho, ux, uy, flux, fb, rk_base, fout, beta, mode))
         *v.flag = 1;
 }
 
