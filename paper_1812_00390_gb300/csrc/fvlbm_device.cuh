@@ -18,6 +18,14 @@ __device__ __forceinline__ T wgt(int a) {
     return a == 0 ? T(4.0 / 9.0) : (a < 5 ? T(1.0 / 9.0) : T(1.0 / 36.0));
 }
 
+// A product that is rounded by itself.  Which of two products in a sum the
+// compiler fuses depends on the code around it; where a value is computed in
+// several kernels (stage kernels, resident loop, storage formats), the
+// operations that could fuse either way are written out, so that all give the
+// same bits.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // acc + e v for a velocity component e of -1, 0 or 1 (known when unrolled; a
 // product with 0 would be kept, since it is not 0 for an infinite v).
 template <typename T> __device__ __forceinline__ T add_e(int e, T acc, T v) {
@@ -43,25 +51,37 @@ __device__ __forceinline__ void moments(const T* f, T& r, T& ux, T& uy) {
         mx = add_e(EXA(a), mx, f[a]);
         my = add_e(EYA(a), my, f[a]);
     }
+    if constexpr (!DEV) {   // FP64 operations are dear: the diagonal differences serve both components
+        const T p = f[5] - f[7], q = f[8] - f[6];
+        mx = (f[1] - f[3]) + (p + q);
+        my = (f[2] - f[4]) + (p - q);
+    }
     r = s;
     const T inv_rho = T(1) / (DEV ? T(1) + s : s);
-    ux = mx * inv_rho;
-    uy = my * inv_rho;
+    ux = mul_rn(mx, inv_rho);
+    uy = mul_rn(my, inv_rho);
 }
+// u^2
+template <typename T> __device__ __forceinline__ T square(T ux, T uy) { return fma(ux, ux, mul_rn(uy, uy)); }
 
 // Eq. (feq).  FP64 mode: r = rho, returns f^eq.  Deviation mode: r = rho - 1,
 // returns f^eq - w = w [(rho - 1) + rho (3 e.u + 4.5 (e.u)^2 - 1.5 u^2)].
 // The polynomial is evaluated as e.u (3 + 4.5 e.u) - 1.5 u^2 (two fused
 // multiply-adds per direction once u^2 is known).
+// feq_factor * feq_value: the two factors of the product, for sums that fuse it.
+template <typename T, bool DEV> __device__ __forceinline__ T feq_factor(int a, T r) {
+    return DEV ? wgt<T>(a) : r * wgt<T>(a);
+}
+template <typename T, bool DEV>
+__device__ __forceinline__ T feq_value(int a, T r, T ux, T uy) {
+    const T eu = dot_e(a, ux, uy);
+    const T poly = fma(T(4.5), eu, T(3)), uu = square(ux, uy);
+    if (DEV) return fma(T(1) + r, fma(eu, poly, -(T(1.5) * uu)), r);
+    return fma(eu, poly, fma(T(-1.5), uu, T(1)));
+}
 template <typename T, bool DEV>
 __device__ __forceinline__ T feqs(int a, T r, T ux, T uy) {
-    const T eu = dot_e(a, ux, uy);
-    const T uu15 = T(1.5) * (ux * ux + uy * uy);
-    if (DEV) {
-        const T poly = fma(eu, fma(T(4.5), eu, T(3)), -uu15);
-        return wgt<T>(a) * fma(T(1) + r, poly, r);
-    }
-    return r * wgt<T>(a) * fma(eu, fma(T(4.5), eu, T(3)), T(1) - uu15);
+    return mul_rn(feq_factor<T, DEV>(a, r), feq_value<T, DEV>(a, r, ux, uy));
 }
 
 // Density argument of feqs for a given density.
@@ -218,6 +238,10 @@ template <typename S> struct PlainIO {
             store_quad(p + h * (UNITS / 2) * BLK, BLK,
                        Quad<S>{{(S)f[dir_a(2 * h)], (S)f[dir_b(2 * h)], (S)f[dir_a(2 * h + 1)], (S)f[dir_b(2 * h + 1)]}});
     }
+    template <typename T, bool DEV, typename I>
+    __device__ __forceinline__ static void store_rounded(void* base, I i, const InstParam& P, T* f) {
+        store<T, DEV>(base, i, P, f);   // stored as it is
+    }
     // FP64 moments of the stored state: r = sum f (FP64 mode) or sum g (deviation), j = sum e g
     __device__ static void moments64(const void* base, int64_t i, const InstParam& P, double& r, double& jx, double& jy) {
         S f[FVLBM_Q];
@@ -309,13 +333,13 @@ template <typename H> struct SplitIO {
     // f of one cell from its stored moments and non-equilibrium words
     template <typename T>
     __device__ static void decode(float dr, float jx, float jy, const uint32_t* w, const InstParam& P, T* f) {
-        const float inv_rho = 1.0f / (1.0f + dr), ux = jx * inv_rho, uy = jy * inv_rho;
+        const float inv_rho = 1.0f / (1.0f + dr), ux = mul_rn(jx, inv_rho), uy = mul_rn(jy, inv_rho);
         float n[FVLBM_Q];
         float s = 0, sx = 0, sy = 0;
 #pragma unroll
         for (int a = 3; a < FVLBM_Q; a++) {
             const uint32_t word = w[(a - 3) >> 1];
-            n[a] = h_value<H>(((a - 3) & 1) ? word >> 16 : word & 0xFFFFu) * P.inv_scale[a];
+            n[a] = mul_rn(h_value<H>(((a - 3) & 1) ? word >> 16 : word & 0xFFFFu), P.inv_scale[a]);
             s += n[a];
             sx = add_e(EXA(a), sx, n[a]);
             sy = add_e(EYA(a), sy, n[a]);
@@ -324,14 +348,14 @@ template <typename H> struct SplitIO {
         n[2] = -sy;
         n[0] = -(s + n[1] + n[2]);
 #pragma unroll
-        for (int a = 0; a < FVLBM_Q; a++) f[a] = (T)(feqs<float, true>(a, dr, ux, uy) + n[a]);
+        for (int a = 0; a < FVLBM_Q; a++) f[a] = (T)fma(wgt<float>(a), feq_value<float, true>(a, dr, ux, uy), n[a]);
     }
     template <typename T, bool DEV, typename I>
     __device__ __forceinline__ static void load(const void* base, I i, const InstParam& P, T* f) {
         decode<T>(*head(base, i), *tail(base, i), P, f);
     }
-    template <typename T, bool DEV, typename I>
-    __device__ __forceinline__ static void store(void* base, I i, const InstParam& P, const T* f) {
+    template <typename T>
+    __device__ __forceinline__ static void encode(const InstParam& P, const T* f, uint4& head_out, uint2& tail_out) {
         float dr = 0, jx = 0, jy = 0;
 #pragma unroll
         for (int a = 0; a < FVLBM_Q; a++) {
@@ -339,21 +363,39 @@ template <typename H> struct SplitIO {
             jx = add_e(EXA(a), jx, (float)f[a]);
             jy = add_e(EYA(a), jy, (float)f[a]);
         }
-        const float inv_rho = 1.0f / (1.0f + dr), ux = jx * inv_rho, uy = jy * inv_rho;
+        const float inv_rho = 1.0f / (1.0f + dr), ux = mul_rn(jx, inv_rho), uy = mul_rn(jy, inv_rho);
         float q[FVLBM_Q];
         uint32_t h = 0x811C9DC5u;
 #pragma unroll
         for (int a = 3; a < FVLBM_Q; a++) {
-            q[a] = ((float)f[a] - feqs<float, true>(a, dr, ux, uy)) * P.scale[a];
+            q[a] = fma(-wgt<float>(a), feq_value<float, true>(a, dr, ux, uy), (float)f[a]) * P.scale[a];
             h = (h ^ __float_as_uint(q[a])) * 0x01000193u;
         }
         h = mix32(h);
         uint32_t bits[FVLBM_Q];
 #pragma unroll
         for (int a = 3; a < FVLBM_Q; a++) bits[a] = h_bits_sr<H>(q[a], sr_word(h, a));
-        *(uint4*)head(base, i) = make_uint4(__float_as_uint(dr), __float_as_uint(jx), __float_as_uint(jy),
-                                            bits[3] | (bits[4] << 16));
-        *(uint2*)tail(base, i) = make_uint2(bits[5] | (bits[6] << 16), bits[7] | (bits[8] << 16));
+        head_out = make_uint4(__float_as_uint(dr), __float_as_uint(jx), __float_as_uint(jy),
+                              bits[3] | (bits[4] << 16));
+        tail_out = make_uint2(bits[5] | (bits[6] << 16), bits[7] | (bits[8] << 16));
+    }
+    template <typename T, bool DEV, typename I>
+    __device__ __forceinline__ static void store(void* base, I i, const InstParam& P, const T* f) {
+        uint4 h;
+        uint2 t;
+        encode(P, f, h, t);
+        *(uint4*)head(base, i) = h;
+        *(uint2*)tail(base, i) = t;
+    }
+    // stores f and replaces it by the value that a load would give
+    template <typename T, bool DEV, typename I>
+    __device__ __forceinline__ static void store_rounded(void* base, I i, const InstParam& P, T* f) {
+        uint4 h;
+        uint2 t;
+        encode(P, f, h, t);
+        *(uint4*)head(base, i) = h;
+        *(uint2*)tail(base, i) = t;
+        decode<T>(h, t, P, f);
     }
     __device__ static void moments64(const void* base, int64_t i, const InstParam&, double& r, double& jx, double& jy) {
         const uint4 h = *head(base, i);

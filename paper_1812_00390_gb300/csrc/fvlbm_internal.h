@@ -206,7 +206,7 @@ struct DevView {
     double* conv;   // [9][np] doubles: device staging of get_f / set_f / macros in caller order
     const int64_t* chunk;   // [n_chunk][3] (begin, end, instance)
     int64_t n_chunk;
-    int32_t* flag;  // non-finite flag
+    int32_t* flag;  // [0] non-finite flag, [1] a wait of the resident kernel ran out
     // fused stage (one CTA per tile of at most `tile` consecutive cells)
     int32_t strategy;        // STRATEGY_TWO_KERNEL or STRATEGY_TILE
     int32_t block;           // threads per block of the two-kernel stage
@@ -218,6 +218,23 @@ struct DevView {
     const uint4* r1link;       // [maxf / 4][n_r1] link words of the 1-ring entries
     int64_t n_r1;
 };
+
+// The resident plan of a small solver (fvlbm_resident.cuh): every tile has a
+// CTA of its own on the GPU for as many time steps as one launch advances.
+struct ResView {
+    int32_t tile = 0;          // threads per CTA (0: no resident plan)
+    int32_t n_tiles = 0;
+    const TileRec* tiles = nullptr;
+    const uint4* link = nullptr;       // as DevView, in this plan's tiles
+    const int32_t* halo = nullptr;
+    const int32_t* owner = nullptr;    // tile of each halo cell
+    const uint4* r1link = nullptr;
+    int64_t n_r1 = 0;
+    uint32_t* done = nullptr;          // [n_tiles] stages each tile has finished, RES_STRIDE apart
+};
+constexpr int RES_STRIDE = 8;   // one 32-byte sector per tile
+// Threads per SM that the resident kernel is built for, and its CTA sizes.
+constexpr int resident_threads(int rsize) { return rsize == 4 ? 512 : 256; }
 
 enum Strategy { STRATEGY_TWO_KERNEL = 0, STRATEGY_TILE = 1 };
 
@@ -239,6 +256,19 @@ int stage_fp16(const DevView& v, void* stream, const void* fin, const void* fbas
                void* const* ev);
 int stage_bf16(const DevView& v, void* stream, const void* fin, const void* fbase, void* fout, double beta, int mode,
                void* const* ev);
+// Resident stage loop: `stages` stages of the scheme from state fa (other
+// buffer fb; both alternate), tile counters at `epoch` before and epoch +
+// stages after.  resident_fits: whether every tile's CTA is on the GPU at once.
+int launch_resident(const DevView& v, const ResView& r, int prec, void* stream, int scheme, int64_t stages,
+                    uint32_t epoch, bool ab2_started);
+bool resident_fits(const DevView& v, const ResView& r, int prec, int scheme);
+#define FVLBM_RESIDENT_DECL(name)                                                                             \
+    int name(const DevView& v, const ResView& r, void* stream, int scheme, int64_t stages, uint32_t epoch,    \
+             bool ab2_started, int* max_ctas)
+FVLBM_RESIDENT_DECL(resident_fp64);
+FVLBM_RESIDENT_DECL(resident_fp32);
+FVLBM_RESIDENT_DECL(resident_fp16);
+FVLBM_RESIDENT_DECL(resident_bf16);
 int launch_macros(const DevView& v, int prec, void* stream);
 int launch_reduce(const DevView& v, void* stream, int what);
 // f and the macros in the caller's cell order, in a buffer the device

@@ -181,6 +181,31 @@ int launch_stage(const DevView& v, int prec, void* stream, const void* fin, cons
     return fail(FVLBM_ERR_ARG, "unknown precision %d", prec);
 }
 
+static int resident(const DevView& v, const ResView& r, int prec, void* stream, int scheme, int64_t stages,
+                    uint32_t epoch, bool ab2_started, int* max_ctas) {
+    switch (prec) {
+        case FVLBM_FP64: return resident_fp64(v, r, stream, scheme, stages, epoch, ab2_started, max_ctas);
+        case FVLBM_FP32_DEV: return resident_fp32(v, r, stream, scheme, stages, epoch, ab2_started, max_ctas);
+        case FVLBM_FP16_DEV: return resident_fp16(v, r, stream, scheme, stages, epoch, ab2_started, max_ctas);
+        case FVLBM_BF16_DEV: return resident_bf16(v, r, stream, scheme, stages, epoch, ab2_started, max_ctas);
+    }
+    return fail(FVLBM_ERR_ARG, "unknown precision %d", prec);
+}
+
+int launch_resident(const DevView& v, const ResView& r, int prec, void* stream, int scheme, int64_t stages,
+                    uint32_t epoch, bool ab2_started) {
+    return resident(v, r, prec, stream, scheme, stages, epoch, ab2_started, nullptr);
+}
+
+bool resident_fits(const DevView& v, const ResView& r, int prec, int scheme) {
+    int ctas = 0;
+    if (resident(v, r, prec, nullptr, scheme, 0, 0, false, &ctas) != FVLBM_OK) {
+        clear_error();
+        return false;
+    }
+    return ctas >= r.n_tiles;
+}
+
 int launch_init_eq(const DevView& v, int prec, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     DISPATCH_PREC(prec, init_eq_kernel<T, S, DEV><<<grid_of(v.n_cell, 256), 256, 0, st>>>(v);

@@ -53,9 +53,15 @@ struct fvlbm_solver {
     cudaGraphExec_t g1[2] = {nullptr, nullptr}, gk[2] = {nullptr, nullptr};
     bool graphs_ok = true;
     int64_t direct_steps = 0;
+    // small solvers: steps run in the resident stage loop; stages its tiles have done
+    bool resident = false;
+    ResView res{};
+    uint32_t epoch = 0;
 };
 
 static constexpr int64_t GRAPH_CHUNK = 32;
+// stages of one resident launch (a few milliseconds)
+static constexpr int64_t RESIDENT_CHUNK = 2048;
 
 namespace {
 
@@ -122,6 +128,8 @@ bool tile_dims(int tile, int maxf, int rsize, int& ls, int& ghosts, size_t& byte
                           : (rsize == 4 ? TileDims<T_, 8, 4>::BYTES : TileDims<T_, 8, 8>::BYTES);            \
         return true;
     switch (tile) {
+        FVLBM_TD(32)
+        FVLBM_TD(64)
         FVLBM_TD(128)
         FVLBM_TD(256)
         FVLBM_TD(512)
@@ -378,7 +386,8 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
         }
 }
 
-int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify) {
+// max_len: most cells of a tile (0: as many as fit).
+int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify, int max_len = 0) {
     int ls = 0, ghosts = 0;
     size_t bytes = 0;
     if (!tile_dims(tile, maxf, 4, ls, ghosts, bytes)) return fail(FVLBM_ERR_ARG, "unsupported tile size %d", tile);
@@ -394,7 +403,8 @@ int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify) {
     const int64_t n_own = M.n_owned;
     int64_t c0 = 0;
     int32_t inst = 0;
-    int guess = tile;   // neighbouring tiles have similar lengths: start one block above the last
+    if (max_len <= 0 || max_len > tile) max_len = tile;
+    int guess = max_len;   // neighbouring tiles have similar lengths: start one block above the last
     while (c0 < n_own) {
         int len = (int)std::min<int64_t>(guess, n_own - c0);
         int nl = 0, nf = 0;
@@ -404,7 +414,7 @@ int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify) {
                             (long long)c0);
             len = len > BLK ? (len - 1) / BLK * BLK : len / 2;
         }
-        guess = std::min(tile, (len + BLK) / BLK * BLK);
+        guess = std::min(max_len, (len + BLK) / BLK * BLK);
         if (len < std::min<int64_t>(tile, n_own - c0)) P.short_tiles++;
         P.sum_len += len;
         P.sum_ring1 += (int64_t)W.r1.size();
@@ -448,9 +458,14 @@ struct Layout {
     size_t off_link, off_geo, off_bctag, off_nbr, off_area, off_grp, off_inst, off_bc, off_fa, off_fb, off_fc, off_rprev,
         off_fv, off_rho, off_ux, off_uy, off_uold, off_part, off_red, off_conv, off_chunk, off_flag, off_tiles, off_halo,
         off_r1link, off_iperm, total;
+    // resident stage loop (small solvers)
+    TilePlan rp;
+    bool resident;
+    size_t off_rlink, off_rtiles, off_rhalo, off_rowner, off_rr1link, off_rdone;
 };
 
 constexpr size_t SMEM_LIMIT = 227 * 1024;
+constexpr int RES_MIN_CELLS(int rsize) { return rsize == 4 ? 32 : 8; }
 
 // Streaming multiprocessors of a device (152 on GB300 when no device answers).
 int device_sms(int device) {
@@ -464,6 +479,31 @@ int device_sms(int device) {
 constexpr int64_t PLANE_ALIGN = 1024;  // cell arrays hold whole blocks and whole tiles of the largest size
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
+
+// The resident stage loop's plan (fvlbm_resident.cuh), if the solver is small
+// enough: one tile per SM where that is possible, each as long as the SM's
+// share of the cells but not below a length at which the halo outgrows the
+// tile.
+int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P) {
+    P = TilePlan{};
+    const int64_t n = M.n_owned;
+    const int most = resident_threads(rsize), least = rsize == 4 ? 64 : 32;
+    const int64_t share = std::max<int64_t>((n + sms - 1) / sms, RES_MIN_CELLS(rsize));
+    for (int tile = least; tile <= most; tile *= 2) {
+        // a compact tile of q cells has about 4.3 sqrt(q) 1-ring cells
+        if (share + 4.3 * std::sqrt((double)share) > tile && tile < most) continue;
+        if ((n + tile - 1) / tile > (int64_t)sms * (most / tile)) continue;
+        int rc = make_tiles(M, maxf, tile, P, false, (int)std::min<int64_t>(share, tile));
+        if (rc) {
+            P = TilePlan{};
+            if (rc == FVLBM_ERR_UNSUPPORTED) continue;
+            return rc;
+        }
+        if (P.n_tiles <= sms || (tile == most && P.n_tiles <= (int64_t)sms * (most / tile))) return FVLBM_OK;
+        P = TilePlan{};
+    }
+    return FVLBM_OK;   // none: P.n_tiles == 0
+}
 
 // kernel: 1 two-kernel, 128/256/512/1024 fused with that tile size, 0
 // automatic.  The automatic choice, from measurements on GB300:
@@ -520,6 +560,14 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
                         (long long)M.n_cell);
     }
     const bool tiled = L.strategy == STRATEGY_TILE, two = !tiled;
+    // the resident loop: chosen with the automatic kernel only; parts of a
+    // partitioned mesh exchange after every stage and never use it
+    L.resident = false;
+    if (kernel == 0 && M.n_owned == M.n_cell && M.n_owned > 0) {
+        int rc = make_resident(M, L.maxf, (int)R, sms, L.rp);
+        if (rc) return rc;
+        L.resident = L.rp.n_tiles > 0;
+    }
     L.pingpong = tiled && (scheme == FVLBM_EULER || scheme == FVLBM_AB2);
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -546,8 +594,14 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
     L.off_tiles = take(tiled ? sizeof(TileRec) * (size_t)L.tp.n_tiles : 0);
     L.off_halo = take(tiled ? 4 * L.tp.halo.size() : 0);
     L.off_r1link = take(tiled ? 4 * (size_t)L.tp.n_r1 * L.maxf : 0);
+    L.off_rlink = take(L.resident ? 4 * slots : 0);
+    L.off_rtiles = take(L.resident ? sizeof(TileRec) * (size_t)L.rp.n_tiles : 0);
+    L.off_rhalo = take(L.resident ? 4 * L.rp.halo.size() : 0);
+    L.off_rowner = take(L.resident ? 4 * L.rp.halo.size() : 0);
+    L.off_rr1link = take(L.resident ? 4 * (size_t)L.rp.n_r1 * L.maxf : 0);
+    L.off_rdone = take(L.resident ? sizeof(uint32_t) * RES_STRIDE * (size_t)L.rp.n_tiles : 0);   // zeros
     L.off_fa = take(S * plane);   // everything before this is uploaded once
-    L.off_fb = (scheme == FVLBM_RK2 || scheme == FVLBM_RK4 || L.pingpong) ? take(S * plane) : 0;
+    L.off_fb = (scheme == FVLBM_RK2 || scheme == FVLBM_RK4 || L.pingpong || L.resident) ? take(S * plane) : 0;
     L.off_fc = (scheme == FVLBM_RK4 && tiled) ? take(S * plane) : 0;
     L.off_rprev = scheme == FVLBM_AB2 ? take(R * plane * FVLBM_Q) : 0;
     L.off_fv = take(two ? 4 * R * (slots + (size_t)L.n_ghost) : 0);
@@ -654,11 +708,30 @@ void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& h
         }
     }
     // 1-ring entries: unit by unit, entry by entry
+    auto pack_ring = [&](const TilePlan& P, size_t off) {
+        uint32_t* r1 = (uint32_t*)(H + off);
+        for (int64_t e = 0; e < P.n_r1; e++)
+            for (int k = 0; k < maxf; k++) r1[4 * ((k / 4) * P.n_r1 + e) + k % 4] = P.r1link[(size_t)e * maxf + k];
+    };
     if (!two) {
-        uint32_t* r1 = (uint32_t*)(H + L.off_r1link);
-        const int64_t ne = L.tp.n_r1;
-        for (int64_t e = 0; e < ne; e++)
-            for (int k = 0; k < maxf; k++) r1[4 * ((k / 4) * ne + e) + k % 4] = L.tp.r1link[(size_t)e * maxf + k];
+        pack_ring(L.tp, L.off_r1link);
+        std::memcpy(H + L.off_tiles, L.tp.rec.data(), sizeof(TileRec) * L.tp.rec.size());
+        std::memcpy(H + L.off_halo, L.tp.halo.data(), 4 * L.tp.halo.size());
+    }
+    if (L.resident) {
+        pack_ring(L.rp, L.off_rr1link);
+        std::memcpy(H + L.off_rtiles, L.rp.rec.data(), sizeof(TileRec) * L.rp.rec.size());
+        std::memcpy(H + L.off_rhalo, L.rp.halo.data(), 4 * L.rp.halo.size());
+        uint32_t* rlink = (uint32_t*)(H + L.off_rlink);
+        std::vector<int32_t> tile_of((size_t)n);
+        for (int64_t t = 0; t < L.rp.n_tiles; t++)
+            for (int32_t x = 0; x < L.rp.rec[t].nt; x++) {
+                const int64_t i = L.rp.rec[t].c0 + x;
+                tile_of[i] = (int32_t)t;
+                for (int k = 0; k < maxf; k++) rlink[word(i, k)] = L.rp.link[(size_t)i * maxf + k];
+            }
+        int32_t* owner = (int32_t*)(H + L.off_rowner);
+        for (size_t e = 0; e < L.rp.halo.size(); e++) owner[e] = tile_of[L.rp.halo[e]];
     }
 }
 
@@ -818,10 +891,6 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
         host.assign(L.off_fa, 0);
         if (s->prec == FVLBM_FP64) pack_geometry<double>(M, L, host);
         else pack_geometry<float>(M, L, host);
-        if (L.strategy == STRATEGY_TILE) {
-            std::memcpy(host.data() + L.off_tiles, L.tp.rec.data(), sizeof(TileRec) * L.tp.rec.size());
-            std::memcpy(host.data() + L.off_halo, L.tp.halo.data(), 4 * L.tp.halo.size());
-        }
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "fvlbm_init: out of host memory");
     }
@@ -890,12 +959,25 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     v.block = L.block;
     if (L.strategy == STRATEGY_TILE) {
         v.tile = L.tp.tile;
-        v.sms = device_sms(p0.device);
         v.n_tiles = L.tp.n_tiles;
         v.tiles = (const TileRec*)(base + L.off_tiles);
         v.halo = (const int32_t*)(base + L.off_halo);
         v.r1link = (const uint4*)(base + L.off_r1link);
         v.n_r1 = L.tp.n_r1;
+    }
+    v.sms = device_sms(p0.device);
+    if (L.resident) {
+        ResView& r = s->res;
+        r.tile = L.rp.tile;
+        r.n_tiles = (int32_t)L.rp.n_tiles;
+        r.tiles = (const TileRec*)(base + L.off_rtiles);
+        r.link = (const uint4*)(base + L.off_rlink);
+        r.halo = (const int32_t*)(base + L.off_rhalo);
+        r.owner = (const int32_t*)(base + L.off_rowner);
+        r.r1link = (const uint4*)(base + L.off_rr1link);
+        r.n_r1 = L.rp.n_r1;
+        r.done = (uint32_t*)(base + L.off_rdone);
+        s->resident = resident_fits(v, r, s->prec, s->scheme);
     }
     s->pingpong = L.pingpong;
     s->buf[0] = v.fa;
@@ -1095,6 +1177,21 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
     cudaStreamIsCapturing(s->stream, &cs);
     bool graphs = s->graphs_ok && s->stream != nullptr && cs == cudaStreamCaptureStatusNone &&
                   s->direct_steps > 0 && (s->scheme != FVLBM_AB2 || s->ab2_started);
+    // small solvers: chunks of whole steps in the resident loop (a caller's
+    // capture records the stages one by one)
+    if (s->resident && cs == cudaStreamCaptureStatusNone) {
+        const int ns = n_stages(s->scheme);
+        while (n > 0) {
+            const int64_t m = std::min(n, RESIDENT_CHUNK / ns);
+            int rc = launch_resident(s->v, s->res, s->prec, s->stream, s->scheme, m * ns, s->epoch, s->ab2_started);
+            if (rc) return rc;
+            s->epoch += (uint32_t)(m * ns);
+            s->ab2_started = s->scheme == FVLBM_AB2;
+            if ((m * ns) & 1) set_current(s, s->cur ^ 1);
+            n -= m;
+        }
+        return FVLBM_OK;
+    }
     auto ready = [&](int b) {
         if (s->g1[b]) return true;
         if (!build_graph(s, 1, &s->g1[b]) || !build_graph(s, GRAPH_CHUNK, &s->gk[b])) {
@@ -1127,10 +1224,11 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
 }
 
 static int sync_and_check(fvlbm_solver* s) {
-    int32_t flag = 0;
-    CK(cudaMemcpyAsync(&flag, s->v.flag, sizeof flag, cudaMemcpyDeviceToHost, s->stream), "read flag");
+    int32_t flag[2] = {0, 0};
+    CK(cudaMemcpyAsync(flag, s->v.flag, sizeof flag, cudaMemcpyDeviceToHost, s->stream), "read flag");
     CK(cudaStreamSynchronize(s->stream), "synchronise");
-    if (flag) return fail(FVLBM_ERR_DIVERGED, "a non-finite value appeared in the state");
+    if (flag[1]) return fail(FVLBM_ERR_TIMEOUT, "the resident stage loop: a tile waited too long for its neighbours");
+    if (flag[0]) return fail(FVLBM_ERR_DIVERGED, "a non-finite value appeared in the state");
     return FVLBM_OK;
 }
 

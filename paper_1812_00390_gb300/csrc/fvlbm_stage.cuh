@@ -65,11 +65,11 @@ __device__ __forceinline__ Ghost<T> ghost_state(uint32_t kind, const BcParam& b,
         g.io = true;
     } else {   // symmetry: the face's unit normal is needed only here
         const typename Vec2<T>::type n = normal();
-        const T inv = T(1) / sqrt(n.x * n.x + n.y * n.y);
-        const T nhx = n.x * inv, nhy = n.y * inv;
-        const T un = ux * nhx + uy * nhy;
-        g.ux = ux - T(2) * un * nhx;
-        g.uy = uy - T(2) * un * nhy;
+        const T inv = T(1) / sqrt(square(n.x, n.y));
+        const T nhx = mul_rn(n.x, inv), nhy = mul_rn(n.y, inv);
+        const T un2 = T(-2) * fma(ux, nhx, mul_rn(uy, nhy));
+        g.ux = fma(un2, nhx, ux);
+        g.uy = fma(un2, nhy, uy);
         g.sym = true;
     }
     return g;
@@ -79,7 +79,7 @@ __device__ __forceinline__ Ghost<T> ghost_state(uint32_t kind, const BcParam& b,
 template <typename T, bool DEV>
 __device__ __forceinline__ T ghost_delta(const Ghost<T>& g, int a, T fa, T fe) {
     if (g.zero) return T(0);
-    return feqs<T, DEV>(a, g.r, g.ux, g.uy) - (g.sym ? fa : fe);
+    return fma(feq_factor<T, DEV>(a, g.r), feq_value<T, DEV>(a, g.r, g.ux, g.uy), g.sym ? -fa : -fe);
 }
 
 template <typename T>
@@ -232,66 +232,112 @@ __device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 // Collision and time update of one cell (Eq. rhs, Sec. 2.3): rhs = -flux -
-// (f - f^eq) / tau, then out = base + beta dt rhs (multistage; the base state
-// is fb when use_fb, else f itself) or the AB2 combination.  Returns false
-// when an output is not finite.
-template <typename T, typename S, bool DEV, bool FMA_RK = false, typename I>
-__device__ __forceinline__ bool update_cell(const DevView& v, const InstParam& P, I i, const T* f, T rho, T ux,
-                                            T uy, const T* flux, const T* fb, bool use_fb, S* fout, T beta,
-                                            int mode) {
-    const T inv_tau = inst_inv_tau<T>(P);
-    const T dt = inst_dt<T>(P);
-    bool bad = false;
-    T* rp = (T*)v.rprev;
-    T out[FVLBM_Q];
-    if constexpr (FMA_RK) {
+// (f - f^eq) / tau, then out = base + beta dt rhs (multistage) or the AB2
+// combination with rp, the previous right-hand side (replaced by this one).
+// Returns false when an output is not finite.
+template <typename T, bool DEV>
+__device__ __forceinline__ bool update_values(const InstParam& P, const T* f, const Pair<T>* fp, const Pair<T>* flux,
+                                              const T* base, T* rp, T beta, int mode, T* out) {
+    T rho, ux, uy;
+    moments<T, DEV>(f, rho, ux, uy);
+    const T inv_tau = inst_inv_tau<T>(P), dt = inst_dt<T>(P);
+    const T eu[4] = {ux, uy, ux + uy, uy - ux};   // e_A . u of the pairs
+    if constexpr (!DEV) {
+        // f^eq_a = rho w_a q_a, q_a = e.u (4.5 e.u + 3) + 1 - 1.5 u^2; the units
+        // that do this are the limit, so no operation is spent that a fused
+        // multiply-add can absorb
+        const T q0 = fma(T(-1.5), square(ux, uy), T(1));
+        const T rw[3] = {rho * T(4.0 / 9.0), rho * T(1.0 / 9.0), rho * T(1.0 / 36.0)};
+        T q[FVLBM_Q], fl[FVLBM_Q];
+        q[0] = q0;
+        fl[0] = T(0);
+        from_pairs(flux, fl);
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            q[dir_a(p)] = fma(eu[p], fma(T(4.5), eu[p], T(3)), q0);
+            q[dir_b(p)] = fma(eu[p], fma(T(4.5), eu[p], T(-3)), q0);
+        }
+        const T c1 = beta * dt, c2 = c1 * inv_tau;
+#pragma unroll
+        for (int a = 0; a < FVLBM_Q; a++) {
+            const T col = fma(rw[a == 0 ? 0 : a < 5 ? 1 : 2], q[a], -f[a]);   // f^eq - f
+            if (mode == MODE_RK) {
+                // base + c1 (-flux + col / tau)
+                out[a] = fma(c2, col, a == 0 ? base[a] : fma(-c1, fl[a], base[a]));
+            } else {
+                const T rhs = fma(inv_tau, col, -fl[a]);
+                out[a] = fma(dt, mode == MODE_AB2_FIRST ? rhs : fma(T(1.5), rhs, T(-0.5) * rp[a]), f[a]);
+                rp[a] = rhs;
+            }
+        }
+    } else {
+        // Deviation modes: the collision term f^eq - f carries no mass or momentum
+        // (f^eq has the cell's rho and rho u), so directions 0..2 follow from
+        // directions 3..8 through those identities.  Evaluated directly in FP32,
+        // its nine rounding errors (about eps |g| each, |g| >> |f^eq - f|) would
+        // add a spurious mass and momentum source of about eps |g| / tau per unit
+        // time, which dominated the velocity error at small tau.  The signs are
+        // chosen so that every packed operation is one fused multiply-add: nc = f -
+        // f^eq, nr = -rhs.
+        const T uu15 = T(1.5) * square(ux, uy);
+        const Pair<T> r2 = make_pair2(rho, rho), r1 = make_pair2(T(1) + rho, T(1) + rho);
+        const Pair<T> c45 = make_pair2(T(4.5), T(4.5)), c3 = make_pair2(T(3), T(3)), cu = make_pair2(-uu15, -uu15);
+        T nc[FVLBM_Q];
+#pragma unroll
+        for (int p = 2; p < 4; p++) {
+            const Pair<T> e = make_pair2(eu[p], -eu[p]);
+            const Pair<T> q = fma2(r1, fma2(e, fma2(c45, e, c3), cu), r2);
+            split2(fma2(make_pair2(T(-1.0 / 36.0), T(-1.0 / 36.0)), q, fp[p]), nc[dir_a(p)], nc[dir_b(p)]);
+        }
+        {   // directions 3 and 4
+            const Pair<T> e = make_pair2(-ux, -uy);
+            const Pair<T> q = fma2(r1, fma2(e, fma2(c45, e, c3), cu), r2);
+            split2(fma2(make_pair2(T(-1.0 / 9.0), T(-1.0 / 9.0)), q, make_pair2(f[3], f[4])), nc[3], nc[4]);
+        }
+        nc[1] = nc[3] - nc[5] + nc[6] + nc[7] - nc[8];
+        nc[2] = nc[4] - nc[5] - nc[6] + nc[7] + nc[8];
+        nc[0] = -(nc[1] + nc[2] + nc[3] + nc[4] + nc[5] + nc[6] + nc[7] + nc[8]);
         if (mode == MODE_RK) {
-            // base + beta dt rhs = base - c1 flux + c2 (f^eq - f), c1 = beta dt,
-            // c2 = beta dt / tau: fewer FP64 operations
-            const T c1 = beta * dt, c2 = c1 * inv_tau;
+            const T c1 = -(beta * dt);
+            const Pair<T> it = make_pair2(inv_tau, inv_tau), c = make_pair2(c1, c1);
+            out[0] = fma(c1, nc[0] * inv_tau, base[0]);
+#pragma unroll
+            for (int p = 0; p < 4; p++)
+                split2(fma2(c, fma2(make_pair2(nc[dir_a(p)], nc[dir_b(p)]), it, flux[p]),
+                            make_pair2(base[dir_a(p)], base[dir_b(p)])), out[dir_a(p)], out[dir_b(p)]);
+        } else {
+            T fl[FVLBM_Q];
+            fl[0] = T(0);
+            from_pairs(flux, fl);
 #pragma unroll
             for (int a = 0; a < FVLBM_Q; a++) {
-                out[a] = fma(c2, feqs<T, DEV>(a, rho, ux, uy) - f[a], fma(-c1, flux[a], use_fb ? fb[a] : f[a]));
-                bad |= !finite_val(out[a]);
+                const T rhs = -fma(nc[a], inv_tau, fl[a]);
+                out[a] = fma(dt, mode == MODE_AB2_FIRST ? rhs : fma(T(1.5), rhs, T(-0.5) * rp[a]), f[a]);
+                rp[a] = rhs;
             }
-            CellIO<S>::template store<T, DEV>(fout, i, P, out);
-            return !bad;
         }
     }
-    // Deviation modes: the collision term f^eq - f carries no mass or momentum
-    // (f^eq has the cell's rho and rho u), so directions 0..2 follow from
-    // directions 3..8 through those identities.  Evaluated directly in FP32,
-    // its nine rounding errors (about eps |g| each, |g| >> |f^eq - f|) would
-    // add a spurious mass and momentum source of about eps |g| / tau per unit
-    // time, which dominated the velocity error at small tau.
-    T col[FVLBM_Q];
-    if constexpr (DEV) {
+    if constexpr (!DEV) {   // tests on the bits: the FP64 units have enough to do
+        bool ok = true;
 #pragma unroll
-        for (int a = 3; a < FVLBM_Q; a++) col[a] = feqs<T, DEV>(a, rho, ux, uy) - f[a];
-        col[1] = col[3] - col[5] + col[6] + col[7] - col[8];
-        col[2] = col[4] - col[5] - col[6] + col[7] + col[8];
-        col[0] = -(col[1] + col[2] + col[3] + col[4] + col[5] + col[6] + col[7] + col[8]);
-    }
-#pragma unroll
-    for (int a = 0; a < FVLBM_Q; a++) {
-        const T rhs = DEV ? -flux[a] + col[a] * inv_tau : -flux[a] - (f[a] - feqs<T, DEV>(a, rho, ux, uy)) * inv_tau;
-        if (mode == MODE_RK) {
-            out[a] = (use_fb ? fb[a] : f[a]) + beta * dt * rhs;
-        } else if (mode == MODE_AB2_FIRST) {
-            out[a] = f[a] + dt * rhs;
-            rp[a * v.np + i] = rhs;
-        } else {
-            out[a] = f[a] + dt * (T(1.5) * rhs - T(0.5) * rp[a * v.np + i]);
-            rp[a * v.np + i] = rhs;
-        }
+        for (int a = 0; a < FVLBM_Q; a++) ok &= finite_val(out[a]);
+        return ok;
     }
     // one test: the sum of the outputs is not finite when any output is not
     T sum = out[0];
 #pragma unroll
     for (int a = 1; a < FVLBM_Q; a++) sum += out[a];
-    bad = !finite_val(sum);
-    CellIO<S>::template store<T, DEV>(fout, i, P, out);
-    return !bad;
+    return finite_val(sum);
+}
+
+// The history of cell i (AB2).
+template <typename T, typename I> __device__ __forceinline__ void load_history(const DevView& v, I i, T* rp) {
+#pragma unroll
+    for (int a = 0; a < FVLBM_Q; a++) rp[a] = ((const T*)v.rprev)[a * v.np + i];
+}
+template <typename T, typename I> __device__ __forceinline__ void store_history(const DevView& v, I i, const T* rp) {
+#pragma unroll
+    for (int a = 0; a < FVLBM_Q; a++) ((T*)v.rprev)[a * v.np + i] = rp[a];
 }
 
 // ------------------------------------------------------------------ kernels
@@ -383,16 +429,55 @@ __global__ void __launch_bounds__(256) update_kernel(DevView v, const S* __restr
         add_flux<T, DEV>(d[k], G.get(GEO_FACE, k), load_quad(face_row<T>(v.fv, row + k * BLK), 1),
                          load_quad(face_row<T>(v.fv, from), 1), fp, fx);
     }
-    T flux[FVLBM_Q], fb[FVLBM_Q];
-    flux[0] = T(0);
-    from_pairs(fx, flux);
+    T fb[FVLBM_Q], rp[FVLBM_Q], out[FVLBM_Q];
     const bool rk_base = mode == MODE_RK && fbase != fin;
     if (rk_base) CellIO<S>::template load<T, DEV>(fbase, i, P, fb);
-    T rho, ux, uy;
-    moments<T, DEV>(f, rho, ux, uy);
-    // the FP64 two-kernel stage is bound by the FP64 units: the shorter multistage form
-    if (!update_cell<T, S, DEV, sizeof(T) == 8>(v, P, i, f, rho, ux, uy, flux, fb, rk_base, fout, beta, mode))
-        *v.flag = 1;
+    if (mode == MODE_AB2) load_history(v, i, rp);
+    if (!update_values<T, DEV>(P, f, fp, fx, rk_base ? fb : f, rp, beta, mode, out)) *v.flag = 1;
+    if (mode != MODE_RK) store_history(v, i, rp);
+    CellIO<S>::template store<T, DEV>(fout, i, P, out);
+}
+
+// Phase 2 of a tile for local cell l: its gradient, and what leaves it
+// through every face (and its boundary faces' ghost values) into the face
+// table.  lsq, mid, face: its geometry vectors by slot.
+template <typename T, bool DEV, int MAXF, int TILE, typename Lsq, typename Mid, typename Face>
+__device__ __forceinline__ void tile_faces(const DevView& v, const uint32_t* d, uint32_t gl, T f0, const Pair<T>* f,
+                                           const typename Vec16<T>::type* fs, typename Vec16<T>::type* tab, int l,
+                                           bool mine, Lsq lsq, Mid mid, Face face) {
+    typedef TileDims<TILE, MAXF, sizeof(T)> D;
+    typedef typename Vec2<T>::type T2;
+    constexpr int LS = D::LS, ROWS = D::ROWS, SU = 8 / Vec16<T>::N;
+    Pair<T> gx[4], gy[4];
+#pragma unroll
+    for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
+    const uint32_t used = warp_slots<MAXF>(d);
+    bool bc = false;
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (k >= 3 && !((used >> k) & 1u)) continue;
+        bc |= link_boundary(d[k]);
+        const T2 ck = lsq(k);
+        const Pair<T> cx = make_pair2(ck.x, ck.x), cy = make_pair2(ck.y, ck.y);
+        const typename Vec16<T>::type* nb = fs + (d[k] & LINK_NB_MASK);
+#pragma unroll
+        for (int h = 0; h < 2; h++) add_gradient(load_quad(nb + h * (SU / 2) * LS, LS), cx, cy, h, f, gx, gy);
+    }
+    if (bc)
+        boundary_slots<T, DEV, MAXF>(d, v.bc, f0, f, gx, gy, [&](int k) { return v.bctag[(int64_t)gl * MAXF + k]; }, lsq,
+                                     face, [&](int k, const Quad<T>& q) { store_quad(tab + k * TILE + l, ROWS, q); },
+                                     [&](int k, const Quad<T>& q) {
+                                         if (mine) store_quad(tab + link_row(d[k]), ROWS, q);
+                                     });
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (k >= 3 && !((used >> k) & 1u)) continue;
+        // ghost values are in place, a 1-ring cell's other faces are not the tile's;
+        // an unused slot among used ones writes its (finite) state, read with weight zero
+        const uint32_t kind = link_kind(d[k]);
+        if (kind == LK_FLOW || kind == LK_NONE || kind_io(kind))
+            store_quad(tab + k * TILE + l, ROWS, leaving(d[k], f, gx, gy, mid(k)));
+    }
 }
 
 // Fused stage: one CTA per tile of consecutive cells (Hilbert order; tile
@@ -415,8 +500,10 @@ __global__ void __launch_bounds__(256) update_kernel(DevView v, const S* __restr
 // the data of a tile that starts somewhat under one CTA lifetime later (pf =
 // 5/8 of the resident CTAs ahead).  Shared-memory strides are compile-time
 // constants (TileDims); the planner keeps every tile within them.
+constexpr int stage_ctas(int tile, int rsize) { return tile <= (rsize == 4 ? 1024 : 512) ? (rsize == 4 ? 1024 : 512) / tile : 1; }
+
 template <typename T, typename S, int MAXF, bool DEV, int TILE>
-__global__ void __launch_bounds__(TILE, (sizeof(T) == 4 ? 1024 : 512) / TILE > 0 ? (sizeof(T) == 4 ? 1024 : 512) / TILE : 1)
+__global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
     stage_tile_kernel(DevView v, const S* __restrict__ fin, const S* fbase, S* fout, T beta, int mode, int pf) {
     typedef TileDims<TILE, MAXF, sizeof(T)> D;
     typedef typename Vec2<T>::type T2;
@@ -530,39 +617,9 @@ __global__ void __launch_bounds__(TILE, (sizeof(T) == 4 ? 1024 : 512) / TILE > 0
             f[2 * h] = make_pair2(q.v[0], q.v[1]);
             f[2 * h + 1] = make_pair2(q.v[2], q.v[3]);
         }
-        Pair<T> gx[4], gy[4];
-#pragma unroll
-        for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
-        const uint32_t used = warp_slots<MAXF>(d);
-        bool bc = false;
-#pragma unroll
-        for (int k = 0; k < MAXF; k++) {
-            if (k >= 3 && !((used >> k) & 1u)) continue;
-            bc |= link_boundary(d[k]);
-            T2 ck;
-            if constexpr (MAXF <= 4) ck = c[k];
-            else ck = G.get(GEO_LSQ, k);
-            const Pair<T> cx = make_pair2(ck.x, ck.x), cy = make_pair2(ck.y, ck.y);
-            const V* nb = fs + (d[k] & LINK_NB_MASK);
-#pragma unroll
-            for (int h = 0; h < 2; h++) add_gradient(load_quad(nb + h * (SU / 2) * LS, LS), cx, cy, h, f, gx, gy);
-        }
-        if (bc)
-            boundary_slots<T, DEV, MAXF>(d, v.bc, f0, f, gx, gy, [&](int k) { return v.bctag[(int64_t)gl * MAXF + k]; },
-                                         [&](int k) { return G.get(GEO_LSQ, k); }, [&](int k) { return G.get(GEO_FACE, k); },
-                                         [&](int k, const Quad<T>& q) { store_quad(tab + k * TILE + l, ROWS, q); },
-                                         [&](int k, const Quad<T>& q) {
-                                             if (mine) store_quad(tab + link_row(d[k]), ROWS, q);
-                                         });
-#pragma unroll
-        for (int k = 0; k < MAXF; k++) {
-            if (k >= 3 && !((used >> k) & 1u)) continue;
-            // ghost values are in place, a 1-ring cell's other faces are not the tile's;
-            // an unused slot among used ones writes its (finite) state, read with weight zero
-            const uint32_t kind = link_kind(d[k]);
-            if (kind == LK_FLOW || kind == LK_NONE || kind_io(kind))
-                store_quad(tab + k * TILE + l, ROWS, leaving(d[k], f, gx, gy, G.get(GEO_MID, k)));
-        }
+        tile_faces<T, DEV, MAXF, TILE>(v, d, gl, f0, f, fs, tab, l, mine,
+                                       [&](int k) { return MAXF <= 4 ? c[k] : G.get(GEO_LSQ, k); },
+                                       [&](int k) { return G.get(GEO_MID, k); }, [&](int k) { return G.get(GEO_FACE, k); });
     }
     // phase 3 inputs, in flight during the wait
     T2 n[MAXF];
@@ -585,17 +642,18 @@ __global__ void __launch_bounds__(TILE, (sizeof(T) == 4 ? 1024 : 512) / TILE > 0
         if (k >= 3 && !((used >> k) & 1u)) continue;
         add_flux<T, DEV>(d[k], n[k], load_quad(tab + k * TILE + l, ROWS), load_quad(tab + link_row(d[k]), ROWS), f, fx);
     }
-    T fa[FVLBM_Q], flux[FVLBM_Q];
+    T fa[FVLBM_Q], rp[FVLBM_Q], out[FVLBM_Q];
     fa[0] = f0;
     from_pairs(f, fa);
-    flux[0] = T(0);
-    from_pairs(fx, flux);
-    T rho, ux, uy;
-    moments<T, DEV>(fa, rho, ux, uy);
-    if (!update_cell<T, S, DEV>(v, P, gi, fa, rho, ux, uy, flux, fb, rk_base, fout, beta, mode))
-        *v.flag = 1;
+    if (!rk_base) {
+#pragma unroll
+        for (int a = 0; a < FVLBM_Q; a++) fb[a] = fa[a];
+    }
+    if (mode == MODE_AB2) load_history(v, gi, rp);
+    if (!update_values<T, DEV>(P, fa, f, fx, fb, rp, beta, mode, out)) *v.flag = 1;
+    if (mode != MODE_RK) store_history(v, gi, rp);
+    CellIO<S>::template store<T, DEV>(fout, gi, P, out);
 }
-
 
 static inline unsigned grid_of(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
