@@ -227,12 +227,12 @@ struct ResView {
     const TileRec* tiles = nullptr;
     const uint4* link = nullptr;       // as DevView, in this plan's tiles
     const int32_t* halo = nullptr;
-    const int32_t* owner = nullptr;    // tile of each halo cell
     const uint4* r1link = nullptr;
     int64_t n_r1 = 0;
-    uint32_t* done = nullptr;          // [n_tiles] stages each tile has finished, RES_STRIDE apart
+    uint4* xchg = nullptr;             // [2][units][np] exchange buffer: units of three words and a tag
 };
-constexpr int RES_STRIDE = 8;   // one 32-byte sector per tile
+// 16-byte units of one cell in the exchange buffer
+constexpr int resident_units(size_t state_bytes) { return (int)(state_bytes / 12); }
 // Threads per SM that the resident kernel is built for, and its CTA sizes.
 constexpr int resident_threads(int rsize) { return rsize == 4 ? 512 : 256; }
 
@@ -256,9 +256,8 @@ int stage_fp16(const DevView& v, void* stream, const void* fin, const void* fbas
                void* const* ev);
 int stage_bf16(const DevView& v, void* stream, const void* fin, const void* fbase, void* fout, double beta, int mode,
                void* const* ev);
-// Resident stage loop: `stages` stages of the scheme from state fa (other
-// buffer fb; both alternate), tile counters at `epoch` before and epoch +
-// stages after.  resident_fits: whether every tile's CTA is on the GPU at once.
+// Resident stage loop: `stages` >= 2 stages of the scheme on state fa, with
+// tags epoch + 1 .. epoch + stages - 1, none of them used before.  resident_fits: whether every tile's CTA is on the GPU at once.
 int launch_resident(const DevView& v, const ResView& r, int prec, void* stream, int scheme, int64_t stages,
                     uint32_t epoch, bool ab2_started);
 bool resident_fits(const DevView& v, const ResView& r, int prec, int scheme);

@@ -53,7 +53,7 @@ struct fvlbm_solver {
     cudaGraphExec_t g1[2] = {nullptr, nullptr}, gk[2] = {nullptr, nullptr};
     bool graphs_ok = true;
     int64_t direct_steps = 0;
-    // small solvers: steps run in the resident stage loop; stages its tiles have done
+    // small solvers: steps run in the resident stage loop; exchange tags used so far
     bool resident = false;
     ResView res{};
     uint32_t epoch = 0;
@@ -461,7 +461,7 @@ struct Layout {
     // resident stage loop (small solvers)
     TilePlan rp;
     bool resident;
-    size_t off_rlink, off_rtiles, off_rhalo, off_rowner, off_rr1link, off_rdone;
+    size_t off_rlink, off_rtiles, off_rhalo, off_rr1link, off_xchg;
 };
 
 constexpr size_t SMEM_LIMIT = 227 * 1024;
@@ -597,11 +597,10 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
     L.off_rlink = take(L.resident ? 4 * slots : 0);
     L.off_rtiles = take(L.resident ? sizeof(TileRec) * (size_t)L.rp.n_tiles : 0);
     L.off_rhalo = take(L.resident ? 4 * L.rp.halo.size() : 0);
-    L.off_rowner = take(L.resident ? 4 * L.rp.halo.size() : 0);
     L.off_rr1link = take(L.resident ? 4 * (size_t)L.rp.n_r1 * L.maxf : 0);
-    L.off_rdone = take(L.resident ? sizeof(uint32_t) * RES_STRIDE * (size_t)L.rp.n_tiles : 0);   // zeros
     L.off_fa = take(S * plane);   // everything before this is uploaded once
-    L.off_fb = (scheme == FVLBM_RK2 || scheme == FVLBM_RK4 || L.pingpong || L.resident) ? take(S * plane) : 0;
+    L.off_fb = (scheme == FVLBM_RK2 || scheme == FVLBM_RK4 || L.pingpong) ? take(S * plane) : 0;
+    L.off_xchg = take(L.resident ? 2 * 16 * (size_t)resident_units(S) * plane : 0);
     L.off_fc = (scheme == FVLBM_RK4 && tiled) ? take(S * plane) : 0;
     L.off_rprev = scheme == FVLBM_AB2 ? take(R * plane * FVLBM_Q) : 0;
     L.off_fv = take(two ? 4 * R * (slots + (size_t)L.n_ghost) : 0);
@@ -723,15 +722,8 @@ void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& h
         std::memcpy(H + L.off_rtiles, L.rp.rec.data(), sizeof(TileRec) * L.rp.rec.size());
         std::memcpy(H + L.off_rhalo, L.rp.halo.data(), 4 * L.rp.halo.size());
         uint32_t* rlink = (uint32_t*)(H + L.off_rlink);
-        std::vector<int32_t> tile_of((size_t)n);
-        for (int64_t t = 0; t < L.rp.n_tiles; t++)
-            for (int32_t x = 0; x < L.rp.rec[t].nt; x++) {
-                const int64_t i = L.rp.rec[t].c0 + x;
-                tile_of[i] = (int32_t)t;
-                for (int k = 0; k < maxf; k++) rlink[word(i, k)] = L.rp.link[(size_t)i * maxf + k];
-            }
-        int32_t* owner = (int32_t*)(H + L.off_rowner);
-        for (size_t e = 0; e < L.rp.halo.size(); e++) owner[e] = tile_of[L.rp.halo[e]];
+        for (int64_t i = 0; i < n; i++)
+            for (int k = 0; k < maxf; k++) rlink[word(i, k)] = L.rp.link[(size_t)i * maxf + k];
     }
 }
 
@@ -973,10 +965,10 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
         r.tiles = (const TileRec*)(base + L.off_rtiles);
         r.link = (const uint4*)(base + L.off_rlink);
         r.halo = (const int32_t*)(base + L.off_rhalo);
-        r.owner = (const int32_t*)(base + L.off_rowner);
         r.r1link = (const uint4*)(base + L.off_rr1link);
         r.n_r1 = L.rp.n_r1;
-        r.done = (uint32_t*)(base + L.off_rdone);
+        r.xchg = (uint4*)(base + L.off_xchg);
+        CK(cudaMemsetAsync(r.xchg, 0, 2 * 16 * (size_t)resident_units(state_bytes(s->prec)) * L.np, s->stream), "clear tags");
         s->resident = resident_fits(v, r, s->prec, s->scheme);
     }
     s->pingpong = L.pingpong;
@@ -1177,20 +1169,19 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
     cudaStreamIsCapturing(s->stream, &cs);
     bool graphs = s->graphs_ok && s->stream != nullptr && cs == cudaStreamCaptureStatusNone &&
                   s->direct_steps > 0 && (s->scheme != FVLBM_AB2 || s->ab2_started);
-    // small solvers: chunks of whole steps in the resident loop (a caller's
-    // capture records the stages one by one)
+    // small solvers: chunks of whole steps, at least two stages each, in the
+    // resident loop (a caller's capture records the stages one by one)
     if (s->resident && cs == cudaStreamCaptureStatusNone) {
         const int ns = n_stages(s->scheme);
-        while (n > 0) {
-            const int64_t m = std::min(n, RESIDENT_CHUNK / ns);
+        while (n * ns >= 2) {
+            int64_t m = std::min(n, RESIDENT_CHUNK / ns);
+            if ((n - m) * ns == 1) m--;
             int rc = launch_resident(s->v, s->res, s->prec, s->stream, s->scheme, m * ns, s->epoch, s->ab2_started);
             if (rc) return rc;
             s->epoch += (uint32_t)(m * ns);
             s->ab2_started = s->scheme == FVLBM_AB2;
-            if ((m * ns) & 1) set_current(s, s->cur ^ 1);
             n -= m;
         }
-        return FVLBM_OK;
     }
     auto ready = [&](int b) {
         if (s->g1[b]) return true;

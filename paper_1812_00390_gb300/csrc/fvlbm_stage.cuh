@@ -235,12 +235,16 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // (f - f^eq) / tau, then out = base + beta dt rhs (multistage) or the AB2
 // combination with rp, the previous right-hand side (replaced by this one).
 // Returns false when an output is not finite.
+template <typename T> struct Relax {
+    T inv_tau, dt;
+    __device__ __forceinline__ explicit Relax(const InstParam& P) : inv_tau(inst_inv_tau<T>(P)), dt(inst_dt<T>(P)) {}
+};
 template <typename T, bool DEV>
-__device__ __forceinline__ bool update_values(const InstParam& P, const T* f, const Pair<T>* fp, const Pair<T>* flux,
+__device__ __forceinline__ bool update_values(const Relax<T>& P, const T* f, const Pair<T>* fp, const Pair<T>* flux,
                                               const T* base, T* rp, T beta, int mode, T* out) {
     T rho, ux, uy;
     moments<T, DEV>(f, rho, ux, uy);
-    const T inv_tau = inst_inv_tau<T>(P), dt = inst_dt<T>(P);
+    const T inv_tau = P.inv_tau, dt = P.dt;
     const T eu[4] = {ux, uy, ux + uy, uy - ux};   // e_A . u of the pairs
     if constexpr (!DEV) {
         // f^eq_a = rho w_a q_a, q_a = e.u (4.5 e.u + 3) + 1 - 1.5 u^2; the units
@@ -433,7 +437,7 @@ __global__ void __launch_bounds__(256) update_kernel(DevView v, const S* __restr
     const bool rk_base = mode == MODE_RK && fbase != fin;
     if (rk_base) CellIO<S>::template load<T, DEV>(fbase, i, P, fb);
     if (mode == MODE_AB2) load_history(v, i, rp);
-    if (!update_values<T, DEV>(P, f, fp, fx, rk_base ? fb : f, rp, beta, mode, out)) *v.flag = 1;
+    if (!update_values<T, DEV>(Relax<T>(P), f, fp, fx, rk_base ? fb : f, rp, beta, mode, out)) *v.flag = 1;
     if (mode != MODE_RK) store_history(v, i, rp);
     CellIO<S>::template store<T, DEV>(fout, i, P, out);
 }
@@ -650,7 +654,7 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
         for (int a = 0; a < FVLBM_Q; a++) fb[a] = fa[a];
     }
     if (mode == MODE_AB2) load_history(v, gi, rp);
-    if (!update_values<T, DEV>(P, fa, f, fx, fb, rp, beta, mode, out)) *v.flag = 1;
+    if (!update_values<T, DEV>(Relax<T>(P), fa, f, fx, fb, rp, beta, mode, out)) *v.flag = 1;
     if (mode != MODE_RK) store_history(v, gi, rp);
     CellIO<S>::template store<T, DEV>(fout, gi, P, out);
 }
