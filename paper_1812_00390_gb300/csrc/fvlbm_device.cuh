@@ -41,20 +41,24 @@ template <typename T> __device__ __forceinline__ T dot_e(int a, T ux, T uy) {
 
 // Density and velocity (Sec. 2.1).  FP64 mode: r = rho = sum f.  Deviation
 // mode: r = rho - 1 = sum g, kept unrounded by the 1 so that the density
-// deviation keeps FP32 relative precision.
+// deviation keeps FP32 relative precision.  FP64 sums by opposite pairs (16
+// operations instead of 18, and four lanes that hold a pair each can form the
+// same sums: see fvlbm_resident.cuh).
 template <typename T, bool DEV>
 __device__ __forceinline__ void moments(const T* f, T& r, T& ux, T& uy) {
     T s = 0, mx = 0, my = 0;
+    if constexpr (DEV) {
 #pragma unroll
-    for (int a = 0; a < FVLBM_Q; a++) {
-        s += f[a];
-        mx = add_e(EXA(a), mx, f[a]);
-        my = add_e(EYA(a), my, f[a]);
-    }
-    if constexpr (!DEV) {   // FP64 operations are dear: the diagonal differences serve both components
-        const T p = f[5] - f[7], q = f[8] - f[6];
-        mx = (f[1] - f[3]) + (p + q);
-        my = (f[2] - f[4]) + (p - q);
+        for (int a = 0; a < FVLBM_Q; a++) {
+            s += f[a];
+            mx = add_e(EXA(a), mx, f[a]);
+            my = add_e(EYA(a), my, f[a]);
+        }
+    } else {
+        const T d2 = f[5] - f[7], d3 = f[6] - f[8];
+        s = f[0] + (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
+        mx = (f[1] - f[3]) + (d2 - d3);
+        my = (f[2] - f[4]) + (d2 + d3);
     }
     r = s;
     const T inv_rho = T(1) / (DEV ? T(1) + s : s);

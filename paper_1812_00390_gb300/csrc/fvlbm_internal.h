@@ -222,19 +222,33 @@ struct DevView {
 // The resident plan of a small solver (fvlbm_resident.cuh): every tile has a
 // CTA of its own on the GPU for as many time steps as one launch advances.
 struct ResView {
-    int32_t tile = 0;          // threads per CTA (0: no resident plan)
+    int32_t tile = 0;          // most tile and 1-ring cells of a tile (0: no resident plan)
     int32_t n_tiles = 0;
     const TileRec* tiles = nullptr;
     const uint4* link = nullptr;       // as DevView, in this plan's tiles
     const int32_t* halo = nullptr;
     const uint4* r1link = nullptr;
     int64_t n_r1 = 0;
-    uint4* xchg = nullptr;             // [2][units][np] exchange buffer: units of three words and a tag
+    uint4* xchg = nullptr;             // [2][units][np] (FP64 [2][np][units]) exchange buffer: units of three
+                                       // words and a tag
 };
-// 16-byte units of one cell in the exchange buffer
-constexpr int resident_units(size_t state_bytes) { return (int)(state_bytes / 12); }
-// Threads per SM that the resident kernel is built for, and its CTA sizes.
-constexpr int resident_threads(int rsize) { return rsize == 4 ? 512 : 256; }
+// 16-byte units of one cell in the exchange buffer (FP64: two per direction pair)
+constexpr int resident_units(size_t state_bytes) { return state_bytes == 72 ? 8 : (int)(state_bytes / 12); }
+// The resident kernel's tiles.  FP32: a thread per tile and 1-ring cell, one
+// tile per SM, or several of the largest (RES_TILE): as many as its registers
+// and shared memory allow.  FP64: four threads per cell (a direction pair each),
+// one tile per SM.
+constexpr int RES_LANES_FP64 = 4;
+constexpr int RES_TILE = 256, RES_TILE_FP64 = 64;
+constexpr int resident_ctas(int rsize, int maxf) { return rsize == 8 ? 1 : maxf <= 4 ? 3 : 2; }
+// Its shared memory: state of the local cells, face table, the geometry of the
+// gradient cells (three 2-vectors per slot) and the state the step began with.
+template <int TILE, int MAXF, int RSIZE> struct ResDims : TileDims<TILE, MAXF, RSIZE> {
+    typedef TileDims<TILE, MAXF, RSIZE> B;
+    static constexpr size_t GEO_BYTES = (size_t)3 * 2 * RSIZE * MAXF * TILE;
+    static constexpr size_t BASE_BYTES = (size_t)FVLBM_Q * RSIZE * TILE;
+    static constexpr size_t BYTES = B::BYTES + GEO_BYTES + BASE_BYTES;
+};
 
 enum Strategy { STRATEGY_TWO_KERNEL = 0, STRATEGY_TILE = 1 };
 

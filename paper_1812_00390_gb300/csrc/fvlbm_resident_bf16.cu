@@ -3,6 +3,6 @@
 
 namespace fvlbm {
 FVLBM_RESIDENT_DECL(resident_bf16) {
-    return resident_t<float, __nv_bfloat16, true>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
+    return resident_t<__nv_bfloat16>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
 }
 }  // namespace fvlbm

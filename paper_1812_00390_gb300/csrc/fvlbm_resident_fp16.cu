@@ -3,6 +3,6 @@
 
 namespace fvlbm {
 FVLBM_RESIDENT_DECL(resident_fp16) {
-    return resident_t<float, __half, true>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
+    return resident_t<__half>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
 }
 }  // namespace fvlbm

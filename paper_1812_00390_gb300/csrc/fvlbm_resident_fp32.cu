@@ -3,6 +3,6 @@
 
 namespace fvlbm {
 FVLBM_RESIDENT_DECL(resident_fp32) {
-    return resident_t<float, float, true>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
+    return resident_t<float>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
 }
 }  // namespace fvlbm

@@ -3,6 +3,6 @@
 
 namespace fvlbm {
 FVLBM_RESIDENT_DECL(resident_fp64) {
-    return resident_t<double, double, false>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
+    return resident_t<double>(v, r, (cudaStream_t)stream, scheme, stages, epoch, ab2_started, max_ctas);
 }
 }  // namespace fvlbm

@@ -128,6 +128,7 @@ bool tile_dims(int tile, int maxf, int rsize, int& ls, int& ghosts, size_t& byte
                           : (rsize == 4 ? TileDims<T_, 8, 4>::BYTES : TileDims<T_, 8, 8>::BYTES);            \
         return true;
     switch (tile) {
+        FVLBM_TD(16)
         FVLBM_TD(32)
         FVLBM_TD(64)
         FVLBM_TD(128)
@@ -481,26 +482,23 @@ constexpr int64_t PLANE_ALIGN = 1024;  // cell arrays hold whole blocks and whol
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // The resident stage loop's plan (fvlbm_resident.cuh), if the solver is small
-// enough: one tile per SM where that is possible, each as long as the SM's
-// share of the cells but not below a length at which the halo outgrows the
-// tile.
+// enough: one tile per SM, as long as the SM's share of the cells but not below
+// a length at which the halo outgrows the tile; in FP32 also two or three of the
+// largest tiles per SM.
 int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P) {
-    P = TilePlan{};
     const int64_t n = M.n_owned;
-    const int most = resident_threads(rsize), least = rsize == 4 ? 64 : 32;
-    const int64_t share = std::max<int64_t>((n + sms - 1) / sms, RES_MIN_CELLS(rsize));
-    for (int tile = least; tile <= most; tile *= 2) {
-        // a compact tile of q cells has about 4.3 sqrt(q) 1-ring cells
-        if (share + 4.3 * std::sqrt((double)share) > tile && tile < most) continue;
-        if ((n + tile - 1) / tile > (int64_t)sms * (most / tile)) continue;
-        int rc = make_tiles(M, maxf, tile, P, false, (int)std::min<int64_t>(share, tile));
-        if (rc) {
+    const int most = rsize == 8 ? RES_TILE_FP64 : RES_TILE;
+    P = TilePlan{};
+    for (int ctas = 1; ctas <= resident_ctas(rsize, maxf); ctas++) {
+        const int64_t share = std::max<int64_t>((n + ctas * sms - 1) / (ctas * sms), RES_MIN_CELLS(rsize));
+        for (int tile = ctas > 1 ? most : rsize == 8 ? 16 : 64; tile <= most; tile *= 2) {
+            // a compact tile of q cells has about 4.3 sqrt(q) 1-ring cells
+            if (share + 4.3 * std::sqrt((double)share) > tile) continue;
+            int rc = make_tiles(M, maxf, tile, P, false, (int)std::min<int64_t>(share, tile));
+            if (rc == FVLBM_OK && P.n_tiles <= (int64_t)ctas * sms) return FVLBM_OK;
             P = TilePlan{};
-            if (rc == FVLBM_ERR_UNSUPPORTED) continue;
-            return rc;
+            if (rc && rc != FVLBM_ERR_UNSUPPORTED) return rc;
         }
-        if (P.n_tiles <= sms || (tile == most && P.n_tiles <= (int64_t)sms * (most / tile))) return FVLBM_OK;
-        P = TilePlan{};
     }
     return FVLBM_OK;   // none: P.n_tiles == 0
 }

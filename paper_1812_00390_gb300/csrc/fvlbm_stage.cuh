@@ -82,13 +82,20 @@ __device__ __forceinline__ T ghost_delta(const Ghost<T>& g, int a, T fa, T fe) {
     return fma(feq_factor<T, DEV>(a, g.r), feq_value<T, DEV>(a, g.r, g.ux, g.uy), g.sym ? -fa : -fe);
 }
 
-template <typename T>
-__device__ __forceinline__ bool finite_val(T x) { return isfinite(x); }
+__device__ __forceinline__ bool finite_val(float x) { return isfinite(x); }
+// on the bits: a comparison would take the FP64 unit
+__device__ __forceinline__ bool finite_val(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
 
 __device__ __forceinline__ uint32_t link_kind(uint32_t d) { return (d >> LINK_KIND_SHIFT) & 7u; }
 __device__ __forceinline__ uint32_t link_row(uint32_t d) { return d >> LINK_ROW_SHIFT; }
 __device__ __forceinline__ bool link_a_leaves(uint32_t d, int p) { return (d >> (LINK_PAIR_SHIFT + p)) & 1u; }
 __device__ __forceinline__ bool link_boundary(uint32_t d) { return link_kind(d) - LK_WALL <= LK_SYMMETRY - LK_WALL; }
+template <int MAXF> __device__ __forceinline__ uint32_t boundary_mask(const uint32_t* d) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) m |= link_boundary(d[k]) ? 1u << k : 0u;
+    return m;
+}
 // Boundary slots whose outgoing values are reconstructed (inlets, pressure
 // outlets); on the others every face value is a ghost value (Sec. 2.4.2).
 __device__ __forceinline__ bool kind_io(uint32_t kind) { return kind == LK_INLET || kind == LK_PRESSURE; }
@@ -175,14 +182,21 @@ __device__ __forceinline__ void add_flux(uint32_t d, const typename Vec2<T>::typ
     }
 }
 
-// Boundary slots of one cell (Sec. 2.4): the ghost differences enter the
+// Boundary slots of one cell (Sec. 2.4): the ghost differences start the
 // gradient; where the cell's faces are in the face table (own rows, and ghost
 // rows for what enters), the boundary face values that are ghost values are
 // written: everything on walls, symmetry planes (half way to the ghost) and
-// external outlets, what enters on inlets and pressure outlets.
+// external outlets, what enters on inlets and pressure outlets.  It needs the
+// cell's own state only.
 //   tag(k)  boundary tag, lsq(k) / face(k) vectors of slot k
-//   own(k, q), ghost(k, q)  store a row
-template <typename T, bool DEV, int MAXF, typename Tag, typename Lsq, typename Face, typename Own, typename In>
+//   own(k, q), in(k, link word, q)  store a row
+// NEXT: each cell takes its next boundary slot, whichever that is, so that the
+// cells of a warp that have one boundary face go through the code once, not once
+// per slot number (the resident loop, where boundary warps are the critical
+// path: 2.31 -> 2.00 us per stage of a 128^2 cavity).  The streaming kernels, where
+// they are few and registers short, unroll the slots (0.277 ms per stage of
+// the 256-instance batch, 0.300 with NEXT, whose slot number costs spills).
+template <typename T, bool DEV, int MAXF, bool NEXT, typename Tag, typename Lsq, typename Face, typename Own, typename In>
 __device__ __forceinline__ void boundary_slots(const uint32_t* d, const BcParam* bcs, T f0, const Pair<T>* fp,
                                                Pair<T>* gx, Pair<T>* gy, Tag tag, Lsq lsq, Face face, Own own, In in) {
     T f[FVLBM_Q];
@@ -190,29 +204,45 @@ __device__ __forceinline__ void boundary_slots(const uint32_t* d, const BcParam*
     from_pairs(fp, f);
     T rho, ux, uy;
     moments<T, DEV>(f, rho, ux, uy);
+    T fe[FVLBM_Q];
+    if constexpr (!DEV) {   // once per cell: FP64 operations are dear, FP32 registers are
 #pragma unroll
-    for (int k = 0; k < MAXF; k++) {
-        if (!link_boundary(d[k])) continue;
-        const uint32_t kind = link_kind(d[k]);
-        const Ghost<T> g = ghost_state<T, DEV>(kind, bcs[tag(k)], rho, ux, uy, [&] { return face(k); });
+        for (int a = 1; a < FVLBM_Q; a++) fe[a] = feqs<T, DEV>(a, rho, ux, uy);
+    }
+    auto slot = [&](int k, uint32_t dk) {
+        const Ghost<T> g = ghost_state<T, DEV>(link_kind(dk), bcs[tag(k)], rho, ux, uy, [&] { return face(k); });
         const typename Vec2<T>::type c = lsq(k);
         const Pair<T> cx = make_pair2(c.x, c.x), cy = make_pair2(c.y, c.y);
+        const T part = g.sym ? T(0.5) : T(1);
         Quad<T> qo, qi;
 #pragma unroll
         for (int p = 0; p < 4; p++) {
             const int a = dir_a(p), b = dir_b(p);
-            const T da = ghost_delta<T, DEV>(g, a, f[a], feqs<T, DEV>(a, rho, ux, uy));
-            const T db = ghost_delta<T, DEV>(g, b, f[b], feqs<T, DEV>(b, rho, ux, uy));
+            const T da = ghost_delta<T, DEV>(g, a, f[a], DEV ? feqs<T, DEV>(a, rho, ux, uy) : fe[a]);
+            const T db = ghost_delta<T, DEV>(g, b, f[b], DEV ? feqs<T, DEV>(b, rho, ux, uy) : fe[b]);
             const Pair<T> dd = make_pair2(da, db);
             gx[p] = fma2(cx, dd, gx[p]);
             gy[p] = fma2(cy, dd, gy[p]);
-            const T va = g.sym ? f[a] + T(0.5) * da : f[a] + da, vb = g.sym ? f[b] + T(0.5) * db : f[b] + db;
-            const bool s = link_a_leaves(d[k], p);
+            const T va = fma(part, da, f[a]), vb = fma(part, db, f[b]);
+            const bool s = link_a_leaves(dk, p);
             qo.v[p] = s ? va : vb;
             qi.v[p] = s ? vb : va;
         }
-        in(k, qi);
+        in(k, dk, qi);
         if (!g.io) own(k, qo);
+    };
+    if constexpr (NEXT) {
+        for (uint32_t left = boundary_mask<MAXF>(d); left; left &= left - 1) {
+            const int k = __ffs(left) - 1;
+            uint32_t dk = d[0];
+#pragma unroll
+            for (int q = 1; q < MAXF; q++) dk = k == q ? d[q] : dk;
+            slot(k, dk);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < MAXF; k++)
+            if (link_boundary(d[k])) slot(k, d[k]);
     }
 }
 
@@ -232,7 +262,55 @@ __device__ __forceinline__ void prefetch_l2(const void* p, int64_t bytes) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 // Collision and time update of one cell (Eq. rhs, Sec. 2.3): rhs = -flux -
-// (f - f^eq) / tau, then out = base + beta dt rhs (multistage) or the AB2
+// (f - f^eq) / tau, in two parts.  The first needs the cell's own state only:
+//   FP64: col = f^eq - f, f^eq_a = rho w_a q_a, q_a = e.u (4.5 e.u + 3) + 1 - 1.5 u^2;
+//         the units that do this are the limit, so no operation is spent that a
+//         fused multiply-add can absorb
+//   deviation modes: col = f - f^eq (the sign that makes every packed operation
+//         one fused multiply-add).  It carries no mass or momentum (f^eq has the
+//         cell's rho and rho u), so directions 0..2 follow from directions 3..8
+//         through those identities.  Evaluated directly in FP32, its nine rounding
+//         errors (about eps |g| each, |g| >> |f^eq - f|) would add a spurious mass
+//         and momentum source of about eps |g| / tau per unit time, which
+//         dominated the velocity error at small tau.
+template <typename T, bool DEV>
+__device__ __forceinline__ void collision(const T* f, T* col) {
+    T rho, ux, uy;
+    moments<T, DEV>(f, rho, ux, uy);
+    const T eu[4] = {ux, uy, ux + uy, uy - ux};   // e_A . u of the pairs
+    if constexpr (!DEV) {
+        const T q0 = fma(T(-1.5), square(ux, uy), T(1));
+        const T rw[3] = {rho * T(4.0 / 9.0), rho * T(1.0 / 9.0), rho * T(1.0 / 36.0)};
+        col[0] = fma(rw[0], q0, -f[0]);
+#pragma unroll
+        for (int p = 0; p < 4; p++) {
+            const int a = dir_a(p), b = dir_b(p);
+            col[a] = fma(rw[p < 2 ? 1 : 2], fma(eu[p], fma(T(4.5), eu[p], T(3)), q0), -f[a]);
+            col[b] = fma(rw[p < 2 ? 1 : 2], fma(eu[p], fma(T(4.5), eu[p], T(-3)), q0), -f[b]);
+        }
+    } else {
+        const T uu15 = T(1.5) * square(ux, uy);
+        const Pair<T> r2 = make_pair2(rho, rho), r1 = make_pair2(T(1) + rho, T(1) + rho);
+        const Pair<T> c45 = make_pair2(T(4.5), T(4.5)), c3 = make_pair2(T(3), T(3)), cu = make_pair2(-uu15, -uu15);
+#pragma unroll
+        for (int p = 2; p < 4; p++) {
+            const Pair<T> e = make_pair2(eu[p], -eu[p]);
+            const Pair<T> q = fma2(r1, fma2(e, fma2(c45, e, c3), cu), r2);
+            split2(fma2(make_pair2(T(-1.0 / 36.0), T(-1.0 / 36.0)), q, make_pair2(f[dir_a(p)], f[dir_b(p)])),
+                   col[dir_a(p)], col[dir_b(p)]);
+        }
+        {   // directions 3 and 4
+            const Pair<T> e = make_pair2(-ux, -uy);
+            const Pair<T> q = fma2(r1, fma2(e, fma2(c45, e, c3), cu), r2);
+            split2(fma2(make_pair2(T(-1.0 / 9.0), T(-1.0 / 9.0)), q, make_pair2(f[3], f[4])), col[3], col[4]);
+        }
+        col[1] = col[3] - col[5] + col[6] + col[7] - col[8];
+        col[2] = col[4] - col[5] - col[6] + col[7] + col[8];
+        col[0] = -(col[1] + col[2] + col[3] + col[4] + col[5] + col[6] + col[7] + col[8]);
+    }
+}
+
+// The second part: out = base + beta dt rhs (multistage) or the AB2
 // combination with rp, the previous right-hand side (replaced by this one).
 // Returns false when an output is not finite.
 template <typename T> struct Relax {
@@ -240,85 +318,32 @@ template <typename T> struct Relax {
     __device__ __forceinline__ explicit Relax(const InstParam& P) : inv_tau(inst_inv_tau<T>(P)), dt(inst_dt<T>(P)) {}
 };
 template <typename T, bool DEV>
-__device__ __forceinline__ bool update_values(const Relax<T>& P, const T* f, const Pair<T>* fp, const Pair<T>* flux,
-                                              const T* base, T* rp, T beta, int mode, T* out) {
-    T rho, ux, uy;
-    moments<T, DEV>(f, rho, ux, uy);
+__device__ __forceinline__ bool advance(const Relax<T>& P, const T* f, const T* col, const Pair<T>* flux,
+                                        const T* base, T* rp, T beta, int mode, T* out) {
     const T inv_tau = P.inv_tau, dt = P.dt;
-    const T eu[4] = {ux, uy, ux + uy, uy - ux};   // e_A . u of the pairs
-    if constexpr (!DEV) {
-        // f^eq_a = rho w_a q_a, q_a = e.u (4.5 e.u + 3) + 1 - 1.5 u^2; the units
-        // that do this are the limit, so no operation is spent that a fused
-        // multiply-add can absorb
-        const T q0 = fma(T(-1.5), square(ux, uy), T(1));
-        const T rw[3] = {rho * T(4.0 / 9.0), rho * T(1.0 / 9.0), rho * T(1.0 / 36.0)};
-        T q[FVLBM_Q], fl[FVLBM_Q];
-        q[0] = q0;
-        fl[0] = T(0);
-        from_pairs(flux, fl);
+    T fl[FVLBM_Q];
+    fl[0] = T(0);
+    from_pairs(flux, fl);
+    if (mode == MODE_RK) {
+        const T c1 = beta * dt;
+        if constexpr (!DEV) {
+            const T c2 = c1 * inv_tau;   // base + c1 (-flux + col / tau)
 #pragma unroll
-        for (int p = 0; p < 4; p++) {
-            q[dir_a(p)] = fma(eu[p], fma(T(4.5), eu[p], T(3)), q0);
-            q[dir_b(p)] = fma(eu[p], fma(T(4.5), eu[p], T(-3)), q0);
-        }
-        const T c1 = beta * dt, c2 = c1 * inv_tau;
-#pragma unroll
-        for (int a = 0; a < FVLBM_Q; a++) {
-            const T col = fma(rw[a == 0 ? 0 : a < 5 ? 1 : 2], q[a], -f[a]);   // f^eq - f
-            if (mode == MODE_RK) {
-                // base + c1 (-flux + col / tau)
-                out[a] = fma(c2, col, a == 0 ? base[a] : fma(-c1, fl[a], base[a]));
-            } else {
-                const T rhs = fma(inv_tau, col, -fl[a]);
-                out[a] = fma(dt, mode == MODE_AB2_FIRST ? rhs : fma(T(1.5), rhs, T(-0.5) * rp[a]), f[a]);
-                rp[a] = rhs;
-            }
-        }
-    } else {
-        // Deviation modes: the collision term f^eq - f carries no mass or momentum
-        // (f^eq has the cell's rho and rho u), so directions 0..2 follow from
-        // directions 3..8 through those identities.  Evaluated directly in FP32,
-        // its nine rounding errors (about eps |g| each, |g| >> |f^eq - f|) would
-        // add a spurious mass and momentum source of about eps |g| / tau per unit
-        // time, which dominated the velocity error at small tau.  The signs are
-        // chosen so that every packed operation is one fused multiply-add: nc = f -
-        // f^eq, nr = -rhs.
-        const T uu15 = T(1.5) * square(ux, uy);
-        const Pair<T> r2 = make_pair2(rho, rho), r1 = make_pair2(T(1) + rho, T(1) + rho);
-        const Pair<T> c45 = make_pair2(T(4.5), T(4.5)), c3 = make_pair2(T(3), T(3)), cu = make_pair2(-uu15, -uu15);
-        T nc[FVLBM_Q];
-#pragma unroll
-        for (int p = 2; p < 4; p++) {
-            const Pair<T> e = make_pair2(eu[p], -eu[p]);
-            const Pair<T> q = fma2(r1, fma2(e, fma2(c45, e, c3), cu), r2);
-            split2(fma2(make_pair2(T(-1.0 / 36.0), T(-1.0 / 36.0)), q, fp[p]), nc[dir_a(p)], nc[dir_b(p)]);
-        }
-        {   // directions 3 and 4
-            const Pair<T> e = make_pair2(-ux, -uy);
-            const Pair<T> q = fma2(r1, fma2(e, fma2(c45, e, c3), cu), r2);
-            split2(fma2(make_pair2(T(-1.0 / 9.0), T(-1.0 / 9.0)), q, make_pair2(f[3], f[4])), nc[3], nc[4]);
-        }
-        nc[1] = nc[3] - nc[5] + nc[6] + nc[7] - nc[8];
-        nc[2] = nc[4] - nc[5] - nc[6] + nc[7] + nc[8];
-        nc[0] = -(nc[1] + nc[2] + nc[3] + nc[4] + nc[5] + nc[6] + nc[7] + nc[8]);
-        if (mode == MODE_RK) {
-            const T c1 = -(beta * dt);
-            const Pair<T> it = make_pair2(inv_tau, inv_tau), c = make_pair2(c1, c1);
-            out[0] = fma(c1, nc[0] * inv_tau, base[0]);
+            for (int a = 0; a < FVLBM_Q; a++) out[a] = fma(c2, col[a], a == 0 ? base[a] : fma(-c1, fl[a], base[a]));
+        } else {
+            const Pair<T> it = make_pair2(inv_tau, inv_tau), c = make_pair2(-c1, -c1);
+            out[0] = fma(-c1, mul_rn(col[0], inv_tau), base[0]);
 #pragma unroll
             for (int p = 0; p < 4; p++)
-                split2(fma2(c, fma2(make_pair2(nc[dir_a(p)], nc[dir_b(p)]), it, flux[p]),
+                split2(fma2(c, fma2(make_pair2(col[dir_a(p)], col[dir_b(p)]), it, flux[p]),
                             make_pair2(base[dir_a(p)], base[dir_b(p)])), out[dir_a(p)], out[dir_b(p)]);
-        } else {
-            T fl[FVLBM_Q];
-            fl[0] = T(0);
-            from_pairs(flux, fl);
+        }
+    } else {
 #pragma unroll
-            for (int a = 0; a < FVLBM_Q; a++) {
-                const T rhs = -fma(nc[a], inv_tau, fl[a]);
-                out[a] = fma(dt, mode == MODE_AB2_FIRST ? rhs : fma(T(1.5), rhs, T(-0.5) * rp[a]), f[a]);
-                rp[a] = rhs;
-            }
+        for (int a = 0; a < FVLBM_Q; a++) {
+            const T rhs = DEV ? -fma(col[a], inv_tau, fl[a]) : fma(inv_tau, col[a], -fl[a]);
+            out[a] = fma(dt, mode == MODE_AB2_FIRST ? rhs : fma(T(1.5), rhs, T(-0.5) * rp[a]), f[a]);
+            rp[a] = rhs;
         }
     }
     if constexpr (!DEV) {   // tests on the bits: the FP64 units have enough to do
@@ -372,13 +397,18 @@ __global__ void __launch_bounds__(256) face_values_kernel(DevView v, const S* __
 #pragma unroll
     for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
     const uint32_t used = warp_slots<MAXF>(d);
-    bool bc = false;
+    const int64_t row = blk_index(i, MAXF);
+    if (boundary_mask<MAXF>(d))
+        boundary_slots<T, DEV, MAXF, false>(d, v.bc, f[0], fp, gx, gy, [&](int k) { return v.bctag[i * MAXF + k]; },
+                                     [&](int k) { return G.get(GEO_LSQ, k); }, [&](int k) { return G.get(GEO_FACE, k); },
+                                     [&](int k, const Quad<T>& q) { store_quad(face_row<T>(v.fv, row + k * BLK), 1, q); },
+                                     [&](int k, uint32_t, const Quad<T>& q) {
+                                         if (i < v.n_cell) store_quad(face_row<T>(v.fv, v.np * MAXF + nb[k]), 1, q);
+                                     });
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
-        const bool edge = link_boundary(d[k]);
-        bc |= edge;
-        const int64_t j = edge ? i : (int64_t)nb[k];
+        const int64_t j = link_boundary(d[k]) ? i : (int64_t)nb[k];
         T fj[FVLBM_Q];
         CellIO<S>::template load<T, DEV>(fin, j, v.inst[v.grp[j]], fj);
         const T2 c = G.get(GEO_LSQ, k);
@@ -388,14 +418,6 @@ __global__ void __launch_bounds__(256) face_values_kernel(DevView v, const S* __
             add_gradient(Quad<T>{{fj[dir_a(2 * h)], fj[dir_b(2 * h)], fj[dir_a(2 * h + 1)], fj[dir_b(2 * h + 1)]}}, cx,
                          cy, h, fp, gx, gy);
     }
-    const int64_t row = blk_index(i, MAXF);
-    if (bc)
-        boundary_slots<T, DEV, MAXF>(d, v.bc, f[0], fp, gx, gy, [&](int k) { return v.bctag[i * MAXF + k]; },
-                                     [&](int k) { return G.get(GEO_LSQ, k); }, [&](int k) { return G.get(GEO_FACE, k); },
-                                     [&](int k, const Quad<T>& q) { store_quad(face_row<T>(v.fv, row + k * BLK), 1, q); },
-                                     [&](int k, const Quad<T>& q) {
-                                         if (i < v.n_cell) store_quad(face_row<T>(v.fv, v.np * MAXF + nb[k]), 1, q);
-                                     });
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
@@ -433,46 +455,52 @@ __global__ void __launch_bounds__(256) update_kernel(DevView v, const S* __restr
         add_flux<T, DEV>(d[k], G.get(GEO_FACE, k), load_quad(face_row<T>(v.fv, row + k * BLK), 1),
                          load_quad(face_row<T>(v.fv, from), 1), fp, fx);
     }
-    T fb[FVLBM_Q], rp[FVLBM_Q], out[FVLBM_Q];
+    T fb[FVLBM_Q], rp[FVLBM_Q], col[FVLBM_Q], out[FVLBM_Q];
     const bool rk_base = mode == MODE_RK && fbase != fin;
     if (rk_base) CellIO<S>::template load<T, DEV>(fbase, i, P, fb);
     if (mode == MODE_AB2) load_history(v, i, rp);
-    if (!update_values<T, DEV>(Relax<T>(P), f, fp, fx, rk_base ? fb : f, rp, beta, mode, out)) *v.flag = 1;
+    collision<T, DEV>(f, col);
+    if (!advance<T, DEV>(Relax<T>(P), f, col, fx, rk_base ? fb : f, rp, beta, mode, out)) *v.flag = 1;
     if (mode != MODE_RK) store_history(v, i, rp);
     CellIO<S>::template store<T, DEV>(fout, i, P, out);
 }
 
-// Phase 2 of a tile for local cell l: its gradient, and what leaves it
-// through every face (and its boundary faces' ghost values) into the face
-// table.  lsq, mid, face: its geometry vectors by slot.
-template <typename T, bool DEV, int MAXF, int TILE, typename Lsq, typename Mid, typename Face>
-__device__ __forceinline__ void tile_faces(const DevView& v, const uint32_t* d, uint32_t gl, T f0, const Pair<T>* f,
-                                           const typename Vec16<T>::type* fs, typename Vec16<T>::type* tab, int l,
-                                           bool mine, Lsq lsq, Mid mid, Face face) {
+// Phase 2 of a tile for local cell l, in two parts.  The first, for boundary
+// cells, needs the cell's own state only and touches rows of the face table that
+// only the cell itself reads: ghost values, and the gradient's start.
+template <typename T, bool DEV, int MAXF, int TILE, bool NEXT, typename Lsq, typename Face>
+__device__ __forceinline__ void tile_boundary(const DevView& v, const uint32_t* d, uint32_t gl, T f0, const Pair<T>* f,
+                                              Pair<T>* gx, Pair<T>* gy, typename Vec16<T>::type* tab, int l, bool mine,
+                                              Lsq lsq, Face face) {
+    constexpr int ROWS = TileDims<TILE, MAXF, sizeof(T)>::ROWS;
+#pragma unroll
+    for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
+    if (boundary_mask<MAXF>(d))
+        boundary_slots<T, DEV, MAXF, NEXT>(d, v.bc, f0, f, gx, gy, [&](int k) { return v.bctag[(int64_t)gl * MAXF + k]; }, lsq,
+                                     face, [&](int k, const Quad<T>& q) { store_quad(tab + k * TILE + l, ROWS, q); },
+                                     [&](int, uint32_t dk, const Quad<T>& q) {
+                                         if (mine) store_quad(tab + link_row(dk), ROWS, q);
+                                     });
+}
+// The second: the neighbour differences, then what leaves the cell through
+// every face into the face table.  lsq, mid: its geometry vectors by slot.
+template <typename T, bool DEV, int MAXF, int TILE, typename Lsq, typename Mid>
+__device__ __forceinline__ void tile_faces(const uint32_t* d, const Pair<T>* f, Pair<T>* gx, Pair<T>* gy,
+                                           const typename Vec16<T>::type* fs, typename Vec16<T>::type* tab, int l, Lsq lsq,
+                                           Mid mid) {
     typedef TileDims<TILE, MAXF, sizeof(T)> D;
     typedef typename Vec2<T>::type T2;
     constexpr int LS = D::LS, ROWS = D::ROWS, SU = 8 / Vec16<T>::N;
-    Pair<T> gx[4], gy[4];
-#pragma unroll
-    for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
     const uint32_t used = warp_slots<MAXF>(d);
-    bool bc = false;
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
-        bc |= link_boundary(d[k]);
         const T2 ck = lsq(k);
         const Pair<T> cx = make_pair2(ck.x, ck.x), cy = make_pair2(ck.y, ck.y);
         const typename Vec16<T>::type* nb = fs + (d[k] & LINK_NB_MASK);
 #pragma unroll
         for (int h = 0; h < 2; h++) add_gradient(load_quad(nb + h * (SU / 2) * LS, LS), cx, cy, h, f, gx, gy);
     }
-    if (bc)
-        boundary_slots<T, DEV, MAXF>(d, v.bc, f0, f, gx, gy, [&](int k) { return v.bctag[(int64_t)gl * MAXF + k]; }, lsq,
-                                     face, [&](int k, const Quad<T>& q) { store_quad(tab + k * TILE + l, ROWS, q); },
-                                     [&](int k, const Quad<T>& q) {
-                                         if (mine) store_quad(tab + link_row(d[k]), ROWS, q);
-                                     });
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
@@ -621,9 +649,11 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
             f[2 * h] = make_pair2(q.v[0], q.v[1]);
             f[2 * h + 1] = make_pair2(q.v[2], q.v[3]);
         }
-        tile_faces<T, DEV, MAXF, TILE>(v, d, gl, f0, f, fs, tab, l, mine,
-                                       [&](int k) { return MAXF <= 4 ? c[k] : G.get(GEO_LSQ, k); },
-                                       [&](int k) { return G.get(GEO_MID, k); }, [&](int k) { return G.get(GEO_FACE, k); });
+        auto lsq = [&](int k) { return MAXF <= 4 ? c[k] : G.get(GEO_LSQ, k); };
+        Pair<T> gx[4], gy[4];
+        tile_boundary<T, DEV, MAXF, TILE, false>(v, d, gl, f0, f, gx, gy, tab, l, mine, lsq,
+                                          [&](int k) { return G.get(GEO_FACE, k); });
+        tile_faces<T, DEV, MAXF, TILE>(d, f, gx, gy, fs, tab, l, lsq, [&](int k) { return G.get(GEO_MID, k); });
     }
     // phase 3 inputs, in flight during the wait
     T2 n[MAXF];
@@ -646,7 +676,7 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
         if (k >= 3 && !((used >> k) & 1u)) continue;
         add_flux<T, DEV>(d[k], n[k], load_quad(tab + k * TILE + l, ROWS), load_quad(tab + link_row(d[k]), ROWS), f, fx);
     }
-    T fa[FVLBM_Q], rp[FVLBM_Q], out[FVLBM_Q];
+    T fa[FVLBM_Q], rp[FVLBM_Q], col[FVLBM_Q], out[FVLBM_Q];
     fa[0] = f0;
     from_pairs(f, fa);
     if (!rk_base) {
@@ -654,7 +684,8 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
         for (int a = 0; a < FVLBM_Q; a++) fb[a] = fa[a];
     }
     if (mode == MODE_AB2) load_history(v, gi, rp);
-    if (!update_values<T, DEV>(Relax<T>(P), fa, f, fx, fb, rp, beta, mode, out)) *v.flag = 1;
+    collision<T, DEV>(fa, col);
+    if (!advance<T, DEV>(Relax<T>(P), fa, col, fx, fb, rp, beta, mode, out)) *v.flag = 1;
     if (mode != MODE_RK) store_history(v, gi, rp);
     CellIO<S>::template store<T, DEV>(fout, gi, P, out);
 }
