@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
     const bool warp_mine = __any_sync(0xFFFFFFFFu, mine), warp_ring_edge = __any_sync(0xFFFFFFFFu, ring1 && edge);
     const InstParam& P = v.inst[inst >= 0 ? inst : v.grp[gl]];
     const Relax<T> relax(P);
-    const double w = p < 2 ? 1.0 / 9.0 : 1.0 / 36.0;   // weight of the pair
+    const double w = lane_weight(p);
     double f0 = 0, fa = 0, fb = 0, b0 = 0, ba = 0, bb = 0, rp0 = 0, rpa = 0, rpb = 0;
     const int ia = dir_a(0) * (p == 0) + dir_a(1) * (p == 1) + dir_a(2) * (p == 2) + dir_a(3) * (p == 3);
     const int ib = dir_b(0) * (p == 0) + dir_b(1) * (p == 1) + dir_b(2) * (p == 2) + dir_b(3) * (p == 3);
@@ -369,27 +369,6 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
         rpb = hist[ib * v.np + gl];
     }
 
-    // rho, u of the four lanes' cell (every lane of the warp takes part)
-    auto cell_moments = [&](double& rho, double& ux, double& uy) {
-        const double S = fa + fb, Df = fa - fb;
-        const double s1 = S + __shfl_xor_sync(0xFFFFFFFFu, S, 1);
-        rho = f0 + (s1 + __shfl_xor_sync(0xFFFFFFFFu, s1, 2));
-        const double o = __shfl_xor_sync(0xFFFFFFFFu, Df, 1);
-        const double even = (p & 1) ? o : Df, odd = (p & 1) ? Df : o;
-        const double X = p >= 2 ? even - odd : even, Y = p >= 2 ? even + odd : odd;
-        const double mx = X + __shfl_xor_sync(0xFFFFFFFFu, X, 2), my = Y + __shfl_xor_sync(0xFFFFFFFFu, Y, 2);
-        const double inv_rho = 1.0 / rho;
-        ux = mul_rn(mx, inv_rho);
-        uy = mul_rn(my, inv_rho);
-    };
-    // e_A . u of the lane's pair, and f^eq / (rho w) of its two directions
-    auto pair_eq = [&](double ux, double uy, double& qa, double& qb, double& q0) {
-        const double diag = uy + (p == 3 ? -ux : ux);
-        const double eu = p == 0 ? ux : p == 1 ? uy : diag;
-        q0 = fma(-1.5, square(ux, uy), 1.0);
-        qa = fma(eu, fma(4.5, eu, 3.0), q0);
-        qb = fma(eu, fma(4.5, eu, -3.0), q0);
-    };
     int k = 0;            // stage of the step
     bool first = AB2 && !ab2_started;
     for (int64_t s = 0; s < stages; s++) {
@@ -409,43 +388,25 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
             q0 = __hiloint2double((int)u[5], (int)u[2]);
             return ok;
         };
-        // ghost differences (Sec. 2.4) of the lane's pair: the gradient's start, and
-        // the rows of the face table that only this cell reads
+        // ghost differences: the gradient's start, and the rows of the face table that
+        // only this cell reads
         double gax = 0, gay = 0, gbx = 0, gby = 0;
         auto boundary = [&](double rho, double ux, double uy, double qa, double qb) {
-            const double rw = rho * w, ea = mul_rn(rw, qa), eb = mul_rn(rw, qb);
-            for (uint32_t left = edges; left; left &= left - 1) {
-                const int q = __ffs(left) - 1;
-                uint32_t dq = d[0];
-#pragma unroll
-                for (int z = 1; z < MAXF; z++) dq = q == z ? d[z] : dq;
-                const double2 cq = G.get(GEO_LSQ, q);
-                const Ghost<T> g = ghost_state<T, false>(link_kind(dq), v.bc[v.bctag[(int64_t)gl * MAXF + q]], rho, ux, uy,
-                                                         [&] { return G.get(GEO_FACE, q); });
-                double ga, gb, g0, da = 0, db = 0;
-                if (!g.zero) {
-                    pair_eq(g.ux, g.uy, ga, gb, g0);
-                    const double gw = g.r * w;
-                    da = fma(gw, ga, g.sym ? -fa : -ea);
-                    db = fma(gw, gb, g.sym ? -fb : -eb);
-                }
-                gax = fma(cq.x, da, gax);
-                gay = fma(cq.y, da, gay);
-                gbx = fma(cq.x, db, gbx);
-                gby = fma(cq.y, db, gby);
-                const double part = g.sym ? 0.5 : 1.0, va = fma(part, da, fa), vb = fma(part, db, fb);
-                const bool a_leaves = link_a_leaves(dq, p);
-                if (mine) tab[link_row(dq) * 4 + p] = a_leaves ? vb : va;
-                if (!g.io) tab[(q * TILE + x) * 4 + p] = a_leaves ? va : vb;
-            }
+            lane_boundary<MAXF>(p, d, v.bc, fa, fb, rho, ux, uy, qa, qb, gax, gay, gbx, gby,
+                                [&](int q) { return v.bctag[(int64_t)gl * MAXF + q]; },
+                                [&](int q) { return G.get(GEO_LSQ, q); }, [&](int q) { return G.get(GEO_FACE, q); },
+                                [&](int q, double z) { tab[(q * TILE + x) * 4 + p] = z; },
+                                [&](int, uint32_t dq, double z) {
+                                    if (mine) tab[link_row(dq) * 4 + p] = z;
+                                });
         };
         int late = 0;
         double col0 = 0, cola = 0, colb = 0, c1 = 0, c2 = 0;
         if (mine) fs[x * 4 + p] = make_double2(fa, fb);
         if (warp_mine) {   // what needs the own state only, before the halo is there
             double rho, ux, uy, qa, qb, q0;
-            cell_moments(rho, ux, uy);
-            pair_eq(ux, uy, qa, qb, q0);
+            lanes_moments(p, f0, fa, fb, rho, ux, uy);
+            lane_eq(p, ux, uy, qa, qb, q0);
             c1 = stage_beta<T>(ns, k) * relax.dt;
             c2 = c1 * relax.inv_tau;
             if (mine) {
@@ -462,8 +423,8 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
         }
         if (warp_ring_edge) {   // 1-ring cells' boundary faces
             double rho, ux, uy, qa, qb, q0;
-            cell_moments(rho, ux, uy);
-            pair_eq(ux, uy, qa, qb, q0);
+            lanes_moments(p, f0, fa, fb, rho, ux, uy);
+            lane_eq(p, ux, uy, qa, qb, q0);
             if (ring1 && edge) boundary(rho, ux, uy, qa, qb);
         }
         for (int e = x; e < n_ring2; e += TILE) {

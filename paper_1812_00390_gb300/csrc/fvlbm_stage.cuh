@@ -246,6 +246,66 @@ __device__ __forceinline__ void boundary_slots(const uint32_t* d, const BcParam*
     }
 }
 
+// ------------------------------------------------------------------ FP64 by lanes
+// Four lanes per cell, lane p with the pair p of its moving directions.  GB300
+// has one FP64 unit per SM quarter, which takes 64 cycles for a warp's
+// instruction whatever its active lanes (about 19 per SM when all four work):
+// with a pair per lane a warp carries 8 cells through a quarter of the
+// instructions, and its chain is a quarter as long.
+__device__ __forceinline__ double lane_weight(int p) { return p < 2 ? 1.0 / 9.0 : 1.0 / 36.0; }
+// rho, u of the four lanes' cell, in the order of moments() (every lane of the
+// warp takes part)
+__device__ __forceinline__ void lanes_moments(int p, double f0, double fa, double fb, double& rho, double& ux, double& uy) {
+    const double S = fa + fb, Df = fa - fb;
+    const double s1 = S + __shfl_xor_sync(0xFFFFFFFFu, S, 1);
+    rho = f0 + (s1 + __shfl_xor_sync(0xFFFFFFFFu, s1, 2));
+    const double o = __shfl_xor_sync(0xFFFFFFFFu, Df, 1);
+    const double even = (p & 1) ? o : Df, odd = (p & 1) ? Df : o;
+    const double X = p >= 2 ? even - odd : even, Y = p >= 2 ? even + odd : odd;
+    const double mx = X + __shfl_xor_sync(0xFFFFFFFFu, X, 2), my = Y + __shfl_xor_sync(0xFFFFFFFFu, Y, 2);
+    const double inv_rho = 1.0 / rho;
+    ux = mul_rn(mx, inv_rho);
+    uy = mul_rn(my, inv_rho);
+}
+// f^eq / (rho w) of the lane's two directions and of direction 0
+__device__ __forceinline__ void lane_eq(int p, double ux, double uy, double& qa, double& qb, double& q0) {
+    const double diag = uy + (p == 3 ? -ux : ux);
+    const double eu = p == 0 ? ux : p == 1 ? uy : diag;
+    q0 = fma(-1.5, square(ux, uy), 1.0);
+    qa = fma(eu, fma(4.5, eu, 3.0), q0);
+    qb = fma(eu, fma(4.5, eu, -3.0), q0);
+}
+// boundary_slots() for the lane's pair; qa, qb: lane_eq of the cell.
+template <int MAXF, typename Tag, typename Lsq, typename Face, typename Own, typename In>
+__device__ __forceinline__ void lane_boundary(int p, const uint32_t* d, const BcParam* bcs, double fa, double fb, double rho,
+                                              double ux, double uy, double qa, double qb, double& gax, double& gay,
+                                              double& gbx, double& gby, Tag tag, Lsq lsq, Face face, Own own, In in) {
+    const double w = lane_weight(p), rw = rho * w, ea = mul_rn(rw, qa), eb = mul_rn(rw, qb);
+    for (uint32_t left = boundary_mask<MAXF>(d); left; left &= left - 1) {
+        const int k = __ffs(left) - 1;
+        uint32_t dk = d[0];
+#pragma unroll
+        for (int z = 1; z < MAXF; z++) dk = k == z ? d[z] : dk;
+        const double2 c = lsq(k);
+        const Ghost<double> g = ghost_state<double, false>(link_kind(dk), bcs[tag(k)], rho, ux, uy, [&] { return face(k); });
+        double ga, gb, g0, da = 0, db = 0;
+        if (!g.zero) {
+            lane_eq(p, g.ux, g.uy, ga, gb, g0);
+            const double gw = g.r * w;
+            da = fma(gw, ga, g.sym ? -fa : -ea);
+            db = fma(gw, gb, g.sym ? -fb : -eb);
+        }
+        gax = fma(c.x, da, gax);
+        gay = fma(c.y, da, gay);
+        gbx = fma(c.x, db, gbx);
+        gby = fma(c.y, db, gby);
+        const double part = g.sym ? 0.5 : 1.0, va = fma(part, da, fa), vb = fma(part, db, fb);
+        const bool a_leaves = link_a_leaves(dk, p);
+        in(k, dk, a_leaves ? vb : va);
+        if (!g.io) own(k, a_leaves ? va : vb);
+    }
+}
+
 // cp.async copy of one 16- or 8-byte element from global to shared memory
 // (16 bytes: past L1).
 template <int BYTES>
@@ -427,6 +487,64 @@ __global__ void __launch_bounds__(256) face_values_kernel(DevView v, const S* __
     }
 }
 
+// Kernel 1 in FP64, four lanes per cell: the same values.
+template <int MAXF>
+__global__ void __launch_bounds__(256) face_values_pairs_kernel(DevView v, const double* __restrict__ fin) {
+    const int p = threadIdx.x & 3;
+    const int64_t at = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 2;
+    const bool ours = at < v.n_grad;   // owned cells and, in a partition, the first ghost ring
+    const int64_t i = ours ? at : v.n_grad - 1;
+    const GeoRef<double, MAXF> G(v.geo, i);
+    uint32_t d[MAXF];
+    load_links<MAXF>(v.link, i, d);
+    int32_t nb[MAXF];
+    load_links<MAXF>((const uint4*)v.nbr, i, (uint32_t*)nb);
+    const double2 f = CellIO<double>::pairs(fin, i)[p * BLK];
+    const int64_t row = blk_index(i, MAXF);
+    double* fv = (double*)v.fv + p;
+    double gax = 0, gay = 0, gbx = 0, gby = 0;
+    const bool edge = boundary_mask<MAXF>(d) != 0;
+    if (__any_sync(0xFFFFFFFFu, edge)) {
+        double rho, ux, uy, qa, qb, q0;
+        lanes_moments(p, *CellIO<double>::rest(fin, i), f.x, f.y, rho, ux, uy);
+        lane_eq(p, ux, uy, qa, qb, q0);
+        if (edge)
+            lane_boundary<MAXF>(p, d, v.bc, f.x, f.y, rho, ux, uy, qa, qb, gax, gay, gbx, gby,
+                                [&](int k) { return v.bctag[i * MAXF + k]; }, [&](int k) { return G.get(GEO_LSQ, k); },
+                                [&](int k) { return G.get(GEO_FACE, k); },
+                                [&](int k, double z) { if (ours) fv[(row + k * BLK) * 4] = z; },
+                                [&](int k, uint32_t, double z) {
+                                    if (!ours || i >= v.n_cell) return;
+                                    int32_t ghost = nb[0];
+#pragma unroll
+                                    for (int x = 1; x < MAXF; x++) ghost = k == x ? nb[x] : ghost;
+                                    fv[(v.np * MAXF + ghost) * 4] = z;
+                                });
+    }
+    const uint32_t used = warp_slots<MAXF>(d);
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (k >= 3 && !((used >> k) & 1u)) continue;
+        const double2 n = CellIO<double>::pairs(fin, link_boundary(d[k]) ? i : (int64_t)nb[k])[p * BLK];
+        const double2 c = G.get(GEO_LSQ, k);
+        const double da = n.x - f.x, db = n.y - f.y;
+        gax = fma(c.x, da, gax);
+        gay = fma(c.y, da, gay);
+        gbx = fma(c.x, db, gbx);
+        gby = fma(c.y, db, gby);
+    }
+#pragma unroll
+    for (int k = 0; k < MAXF; k++) {
+        if (k >= 3 && !((used >> k) & 1u)) continue;
+        const uint32_t kind = link_kind(d[k]);
+        if (kind >= LK_WALL && !kind_io(kind)) continue;   // ghost values, or no face
+        const double2 m = G.get(GEO_MID, k);
+        const bool a = link_a_leaves(d[k], p);
+        const double z = fma(a ? gay : gby, m.y, fma(a ? gax : gbx, m.x, a ? f.x : f.y));
+        if (ours) fv[(row + k * BLK) * 4] = z;
+    }
+}
+
 // Kernel 2 (Steps 4-5): flux sum over the cell's faces, collision and time
 // update.
 template <typename T, typename S, int MAXF, bool DEV>
@@ -562,20 +680,12 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
     uint2* rawt = (uint2*)(rawh + LS);             // [LS]
     static_assert(PLAIN || LS * 24 <= ROWS * 4 * (int)sizeof(T), "raw staging fits the face table");
     const int n2 = nt + n1;            // gradient cells: the planner keeps nt + n1 <= TILE
-    uint32_t gl = c0;
-    T f0 = T(0);
-    for (int x = l; x < nt + nh; x += TILE) {
-        const uint32_t gx = x < nt ? c0 + x : (uint32_t)v.halo[h0 + (x - nt)];
-        if (x == l) gl = gx;
-        if constexpr (PLAIN) {
-            const V* p = (const V*)CellIO<S>::pairs(fin, gx);
-#pragma unroll
-            for (int u = 0; u < SU; u++) cp_async_elem<16>(fs + u * LS + x, p + u * BLK);
-        } else {
-            cp_async_elem<16>(rawh + x, CellIO<S>::head(fin, gx));
-            cp_async_elem<8>(rawt + x, CellIO<S>::tail(fin, gx));
-        }
-    }
+    // a thread stages at most two local cells (LS <= 2 TILE)
+    static_assert(LS <= 2 * TILE, "two local cells per thread");
+    const int n_local = nt + nh;
+    uint32_t gl = c0, gl2 = 0;
+    if (l < n_local) gl = mine ? gi : (uint32_t)v.halo[h0 + (l - nt)];
+    if (l + TILE < n_local) gl2 = (uint32_t)v.halo[h0 + (l + TILE - nt)];
     // phase 2 gives local cell x (tile cell, or 1-ring entry x - nt) to thread x
     uint32_t d[MAXF];
     T2 c[MAXF];
@@ -594,8 +704,22 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
             }
         }
         if constexpr (MAXF <= 4) G.load(GEO_LSQ, c);
-        if constexpr (PLAIN) f0 = (T)*CellIO<S>::rest(fin, gl);
     }
+    T f0 = T(0);
+    auto stage_cell = [&](int x, uint32_t gx) {
+        if constexpr (PLAIN) {
+            const V* p = (const V*)CellIO<S>::pairs(fin, gx);
+#pragma unroll
+            for (int u = 0; u < SU; u++) cp_async_elem<16>(fs + u * LS + x, p + u * BLK);
+        } else {
+            cp_async_elem<16>(rawh + x, CellIO<S>::head(fin, gx));
+            cp_async_elem<8>(rawt + x, CellIO<S>::tail(fin, gx));
+        }
+    };
+    if (l < n_local) stage_cell(l, gl);
+    if (l + TILE < n_local) stage_cell(l + TILE, gl2);
+    if constexpr (PLAIN)
+        if (l < n2) f0 = (T)*CellIO<S>::rest(fin, gl);
     // A CTA that starts somewhat before this one ends works on about tile
     // t + pf (pf = 5/8 of the CTAs resident on the GPU): bring that tile's
     // state and geometry into L2 now, so that its staging reads L2 rather than
@@ -627,16 +751,18 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
     // a 16-bit state is decoded by the thread that staged it (its own copies
     // are complete after the wait), so one barrier serves both
     if constexpr (!PLAIN) {
-        for (int x = l; x < nt + nh; x += TILE) {
-            const uint32_t gx = x < nt ? c0 + x : (uint32_t)v.halo[h0 + (x - nt)];
+        auto decode_cell = [&](int x, uint32_t gx, T& rest) {
             T f[FVLBM_Q];
             CellIO<S>::template decode<T>(rawh[x], rawt[x], v.inst[inst >= 0 ? inst : v.grp[gx]], f);
-            if (x == l) f0 = f[0];
+            rest = f[0];
 #pragma unroll
             for (int h = 0; h < 2; h++)
                 store_quad(fs + h * (SU / 2) * LS + x, LS,
                            Quad<T>{{f[dir_a(2 * h)], f[dir_b(2 * h)], f[dir_a(2 * h + 1)], f[dir_b(2 * h + 1)]}});
-        }
+        };
+        T none;
+        if (l < n_local) decode_cell(l, gl, f0);
+        if (l + TILE < n_local) decode_cell(l + TILE, gl2, none);
     }
     __syncthreads();
 
@@ -765,13 +891,25 @@ static int stage_t(const DevView& v, cudaStream_t st, const void* fin, const voi
     }
     const int bs = v.block > 0 ? v.block : 256;   // smaller blocks spread small meshes over all SMs
     const unsigned g = grid_of(v.n_cell, bs), gg = grid_of(v.n_grad, bs);
-    if (v.maxf == 4) face_values_kernel<T, S, 4, DEV><<<gg, bs, 0, st>>>(v, (const S*)fin);
-    else face_values_kernel<T, S, 8, DEV><<<gg, bs, 0, st>>>(v, (const S*)fin);
+    const S *in = (const S*)fin, *base = (const S*)fbase;
+    bool lanes = false;
+    if constexpr (sizeof(T) == 8) {
+        // FP64: four lanes per cell until the SMs' quarters have work enough without
+        // (us per stage, lanes / a thread per cell: 16k-cell cavity 17.3 / 20.4, 250k
+        // cells 130 / 136, the 6.7 M cell batch 2966 / 2869)
+        lanes = v.n_grad < 2048 * (int64_t)v.sms;
+        if (lanes) {
+            auto kern = v.maxf == 4 ? face_values_pairs_kernel<4> : face_values_pairs_kernel<8>;
+            kern<<<grid_of(4 * v.n_grad, 256), 256, 0, st>>>(v, in);
+        }
+    }
+    if (!lanes) {
+        auto kern = v.maxf == 4 ? face_values_kernel<T, S, 4, DEV> : face_values_kernel<T, S, 8, DEV>;
+        kern<<<gg, bs, 0, st>>>(v, in);
+    }
     if (ev) cudaEventRecord((cudaEvent_t)ev[1], st);
-    if (v.maxf == 4)
-        update_kernel<T, S, 4, DEV><<<g, bs, 0, st>>>(v, (const S*)fin, (const S*)fbase, (S*)fout, (T)beta, mode);
-    else
-        update_kernel<T, S, 8, DEV><<<g, bs, 0, st>>>(v, (const S*)fin, (const S*)fbase, (S*)fout, (T)beta, mode);
+    auto kern = v.maxf == 4 ? update_kernel<T, S, 4, DEV> : update_kernel<T, S, 8, DEV>;
+    kern<<<g, bs, 0, st>>>(v, in, base, (S*)fout, (T)beta, mode);
     if (ev) cudaEventRecord((cudaEvent_t)ev[2], st);
     return check_launch("stage kernels");
 }
