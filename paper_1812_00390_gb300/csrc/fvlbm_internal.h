@@ -197,14 +197,12 @@ struct DevView {
     void* rprev;// T [9][np]  AB2 previous RHS
     void* fv;   // two-kernel stage: Quad<T> of outgoing values per (cell, slot), blocked [maxf], then the
                 // ghost records (values that enter through boundary faces)
-    double* rho;    // [np]
-    double* ux;     // [np]
-    double* uy;     // [np]
-    double* uold;   // [2][np]
+    double* uold;   // [2][np] the residual's snapshot of u
     double* part;   // [n_chunk][3] block partial sums
     double* red;    // [n_inst][3]  per-instance sums
     double* conv;   // [9][np] doubles: device staging of get_f / set_f / macros in caller order
     const int64_t* chunk;   // [n_chunk][3] (begin, end, instance)
+    const int64_t* inst_chunk;   // [n_inst + 1] chunks of each instance
     int64_t n_chunk;
     int32_t* flag;  // [0] non-finite flag, [1] a wait of the resident kernel ran out
     // fused stage (one CTA per tile of at most `tile` consecutive cells)
@@ -282,8 +280,8 @@ FVLBM_RESIDENT_DECL(resident_fp64);
 FVLBM_RESIDENT_DECL(resident_fp32);
 FVLBM_RESIDENT_DECL(resident_fp16);
 FVLBM_RESIDENT_DECL(resident_bf16);
-int launch_macros(const DevView& v, int prec, void* stream);
-int launch_reduce(const DevView& v, void* stream, int what);
+int launch_snapshot(const DevView& v, int prec, void* stream);
+int launch_reduce(const DevView& v, int prec, void* stream, int what);
 // f and the macros in the caller's cell order, in a buffer the device
 // accesses (host memory reachable by the GPU, or device memory).
 int launch_get_f_ordered(const DevView& v, int prec, void* stream, double* f);
@@ -303,6 +301,11 @@ int solver_ref(fvlbm_solver* s, SolverRef* out);
 // the state buffer it writes); the last stage ends the step.
 int solver_n_stages(const fvlbm_solver* s);
 int solver_stage(fvlbm_solver* s, int k, void** out);
+// Whether recorded steps can stand for enqueued ones (the kernels have run
+// once, AB2 has its history), and which of two alternating buffers holds the state.
+bool solver_replayable(const fvlbm_solver* s);
+int solver_buffer(const fvlbm_solver* s);
+void solver_set_buffer(fvlbm_solver* s, int b);
 // FP64 sums of a reduction (RED_MASS: [mass, -, -]; RED_RESIDUAL: [numerator,
 // denominator, -]) per instance, 3 per instance; synchronises.
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out);

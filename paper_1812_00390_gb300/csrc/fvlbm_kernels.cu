@@ -43,17 +43,16 @@ __global__ void init_eq_kernel(DevView v) {
     CellIO<S>::template store<T, DEV>(v.fa, i, P, f);
 }
 
-// rho, u in FP64 from the stored state (Step 6).
+// u in FP64 from the stored state into the residual's snapshot.
 template <typename T, typename S, bool DEV>
-__global__ void macros_kernel(DevView v) {
+__global__ void snapshot_kernel(DevView v) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= v.n_cell) return;
     double r, mx, my;
     CellIO<S>::moments64(v.fa, i, v.inst[v.grp[i]], r, mx, my);
-    double rho = DEV ? 1.0 + r : r;
-    v.rho[i] = rho;
-    v.ux[i] = mx / rho;
-    v.uy[i] = my / rho;
+    const double rho = DEV ? 1.0 + r : r;
+    v.uold[i] = mx / rho;
+    v.uold[v.np + i] = my / rho;
 }
 
 // f and rho, u in the caller's cell order, [n_cell][9] (get / set) or
@@ -117,47 +116,59 @@ __global__ void macros_ordered_kernel(DevView v, double* __restrict__ rho_out, d
 }
 
 // Deterministic FP64 reductions: one block per chunk of one instance, fixed
-// tree order; then one thread per instance sums its chunks in order.
+// tree order; then one warp per instance sums its chunks (they are consecutive),
+// lane by lane and in a fixed tree.  rho, u come from the stored state as they
+// are summed: as arrays of their own they cost a second pass of 48 bytes per cell
+// (and every thread of the last kernel went over every chunk: 1.26 ms for a
+// residual of the 256-instance batch).
 constexpr int RED_THREADS = 256;
 
-__global__ void reduce_chunks_kernel(DevView v, int what) {
-    __shared__ double sh[3][RED_THREADS];
+template <typename T, typename S, bool DEV>
+__global__ void __launch_bounds__(RED_THREADS) reduce_chunks_kernel(DevView v, int what) {
+    __shared__ double sh[2][RED_THREADS];
     const int64_t ch = blockIdx.x;
     const int64_t b = v.chunk[3 * ch], e = v.chunk[3 * ch + 1];
-    double s0 = 0, s1 = 0, s2 = 0;
+    const InstParam& P = v.inst[v.chunk[3 * ch + 2]];
+    double s0 = 0, s1 = 0;
     for (int64_t i = b + threadIdx.x; i < e; i += RED_THREADS) {
+        double r, mx, my;
+        CellIO<S>::moments64(v.fa, i, P, r, mx, my);
+        const double rho = DEV ? 1.0 + r : r;
         if (what == RED_MASS) {
-            s0 += v.area[i] * v.rho[i];
+            s0 += v.area[i] * rho;
         } else {
-            double ox = v.uold[i], oy = v.uold[v.np + i];
-            double dx = v.ux[i] - ox, dy = v.uy[i] - oy;
+            const double ux = mx / rho, uy = my / rho, ox = v.uold[i], oy = v.uold[v.np + i];
+            const double dx = ux - ox, dy = uy - oy;
             s0 += dx * dx + dy * dy;
             s1 += ox * ox + oy * oy;
-            v.uold[i] = v.ux[i];
-            v.uold[v.np + i] = v.uy[i];
+            v.uold[i] = ux;
+            v.uold[v.np + i] = uy;
         }
     }
     sh[0][threadIdx.x] = s0;
     sh[1][threadIdx.x] = s1;
-    sh[2][threadIdx.x] = s2;
     __syncthreads();
     for (int s = RED_THREADS / 2; s > 0; s >>= 1) {
         if (threadIdx.x < s)
-            for (int q = 0; q < 3; q++) sh[q][threadIdx.x] += sh[q][threadIdx.x + s];
+            for (int q = 0; q < 2; q++) sh[q][threadIdx.x] += sh[q][threadIdx.x + s];
         __syncthreads();
     }
     if (threadIdx.x == 0)
-        for (int q = 0; q < 3; q++) v.part[3 * ch + q] = sh[q][0];
+        for (int q = 0; q < 2; q++) v.part[3 * ch + q] = sh[q][0];
 }
 
 __global__ void reduce_final_kernel(DevView v) {
-    const int inst = blockIdx.x * blockDim.x + threadIdx.x;
+    const int inst = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
     if (inst >= v.n_inst) return;
-    double s[3] = {0, 0, 0};
-    for (int64_t ch = 0; ch < v.n_chunk; ch++)
-        if (v.chunk[3 * ch + 2] == inst)
-            for (int q = 0; q < 3; q++) s[q] += v.part[3 * ch + q];
-    for (int q = 0; q < 3; q++) v.red[3 * inst + q] = s[q];
+    double s[2] = {0, 0};
+    for (int64_t ch = v.inst_chunk[inst] + lane; ch < v.inst_chunk[inst + 1]; ch += 32)
+        for (int q = 0; q < 2; q++) s[q] += v.part[3 * ch + q];
+    for (int d = 16; d > 0; d >>= 1)
+        for (int q = 0; q < 2; q++) s[q] += __shfl_down_sync(0xFFFFFFFFu, s[q], d);
+    if (lane == 0) {
+        for (int q = 0; q < 2; q++) v.red[3 * inst + q] = s[q];
+        v.red[3 * inst + 2] = 0;
+    }
 }
 
 // ------------------------------------------------------------------ launchers
@@ -212,17 +223,20 @@ int launch_init_eq(const DevView& v, int prec, void* stream) {
                   return check_launch("init kernel"));
 }
 
-int launch_macros(const DevView& v, int prec, void* stream) {
+int launch_snapshot(const DevView& v, int prec, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    DISPATCH_PREC(prec, macros_kernel<T, S, DEV><<<grid_of(v.n_cell, 256), 256, 0, st>>>(v);
-                  return check_launch("macros kernel"));
+    DISPATCH_PREC(prec, snapshot_kernel<T, S, DEV><<<grid_of(v.n_cell, 256), 256, 0, st>>>(v);
+                  return check_launch("snapshot kernel"));
 }
 
-int launch_reduce(const DevView& v, void* stream, int what) {
+template <typename T, typename S, bool DEV> static void reduce_chunks(const DevView& v, cudaStream_t st, int what) {
+    if (v.n_chunk > 0) reduce_chunks_kernel<T, S, DEV><<<(unsigned)v.n_chunk, RED_THREADS, 0, st>>>(v, what);
+    reduce_final_kernel<<<grid_of(32 * (int64_t)v.n_inst, 128), 128, 0, st>>>(v);
+}
+
+int launch_reduce(const DevView& v, int prec, void* stream, int what) {
     cudaStream_t st = (cudaStream_t)stream;
-    if (v.n_chunk > 0) reduce_chunks_kernel<<<(unsigned)v.n_chunk, RED_THREADS, 0, st>>>(v, what);
-    reduce_final_kernel<<<grid_of(v.n_inst, 128), 128, 0, st>>>(v);
-    return check_launch("reduction kernels");
+    DISPATCH_PREC(prec, reduce_chunks<T, S, DEV>(v, st, what); return check_launch("reduction kernels"));
 }
 
 }  // namespace fvlbm

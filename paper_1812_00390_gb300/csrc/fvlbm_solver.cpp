@@ -53,6 +53,7 @@ struct fvlbm_solver {
     cudaGraphExec_t g1[2] = {nullptr, nullptr}, gk[2] = {nullptr, nullptr};
     bool graphs_ok = true;
     int64_t direct_steps = 0;
+    bool staged = false;   // a stage has been launched by itself (partitioned solve)
     // small solvers: steps run in the resident stage loop; exchange tags used so far
     bool resident = false;
     ResView res{};
@@ -457,11 +458,12 @@ struct Layout {
     TilePlan tp;
     int64_t n_ghost;   // two-kernel stage: boundary slots of owned cells (ghost records)
     size_t off_link, off_geo, off_bctag, off_nbr, off_area, off_grp, off_inst, off_bc, off_fa, off_fb, off_fc, off_rprev,
-        off_fv, off_rho, off_ux, off_uy, off_uold, off_part, off_red, off_conv, off_chunk, off_flag, off_tiles, off_halo,
+        off_fv, off_uold, off_part, off_red, off_conv, off_chunk, off_flag, off_tiles, off_halo,
         off_r1link, off_iperm, total;
     // resident stage loop (small solvers)
     TilePlan rp;
     bool resident;
+    const TilePlan& res_plan() const { return rp.n_tiles > 0 ? rp : tp; }   // tp when it serves both
     size_t off_rlink, off_rtiles, off_rhalo, off_rr1link, off_xchg;
 };
 
@@ -485,7 +487,7 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // enough: one tile per SM, as long as the SM's share of the cells but not below
 // a length at which the halo outgrows the tile; in FP32 also two or three of the
 // largest tiles per SM.
-int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P) {
+int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P, bool verify) {
     const int64_t n = M.n_owned;
     const int most = rsize == 8 ? RES_TILE_FP64 : RES_TILE;
     P = TilePlan{};
@@ -494,7 +496,7 @@ int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P) {
         for (int tile = ctas > 1 ? most : rsize == 8 ? 16 : 64; tile <= most; tile *= 2) {
             // a compact tile of q cells has about 4.3 sqrt(q) 1-ring cells
             if (share + 4.3 * std::sqrt((double)share) > tile) continue;
-            int rc = make_tiles(M, maxf, tile, P, false, (int)std::min<int64_t>(share, tile));
+            int rc = make_tiles(M, maxf, tile, P, verify, (int)std::min<int64_t>(share, tile));
             if (rc == FVLBM_OK && P.n_tiles <= (int64_t)ctas * sms) return FVLBM_OK;
             P = TilePlan{};
             if (rc && rc != FVLBM_ERR_UNSUPPORTED) return rc;
@@ -540,6 +542,14 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         else tile = 128;
     }
     L.strategy = tile == 0 || tile == 1 ? STRATEGY_TWO_KERNEL : STRATEGY_TILE;
+    // the resident loop: chosen with the automatic kernel only; parts of a
+    // partitioned mesh exchange after every stage and never use it
+    L.resident = false;
+    if (kernel == 0 && M.n_owned == M.n_cell && M.n_owned > 0) {
+        int rc = make_resident(M, L.maxf, (int)R, sms, L.rp, verify);
+        if (rc) return rc;
+        L.resident = L.rp.n_tiles > 0;
+    }
     // FP64: small blocks, whose warps the SMs' quarters share more evenly (250k-cell
     // cavity 130 us per stage with 64 threads, 134 with 256)
     L.block = prec == FVLBM_FP64 ? 64 : 256;
@@ -551,7 +561,10 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         if (smem > SMEM_LIMIT)
             return fail(FVLBM_ERR_UNSUPPORTED, "fused stage with %d-cell tiles needs %zu B of shared memory (limit %zu)",
                         tile, smem, SMEM_LIMIT);
-        int rc = make_tiles(M, L.maxf, tile, L.tp, verify);
+        // the resident loop's tiles, where it has them of this size, serve both
+        int rc = FVLBM_OK;
+        if (L.resident && L.rp.tile == tile) std::swap(L.tp, L.rp);
+        else rc = make_tiles(M, L.maxf, tile, L.tp, verify);
         if (rc) return rc;
         // the fused kernel indexes its blocked arrays in 32 bits
         const uint64_t lim = (uint64_t)1 << 32;
@@ -560,14 +573,6 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
                         (long long)M.n_cell);
     }
     const bool tiled = L.strategy == STRATEGY_TILE, two = !tiled;
-    // the resident loop: chosen with the automatic kernel only; parts of a
-    // partitioned mesh exchange after every stage and never use it
-    L.resident = false;
-    if (kernel == 0 && M.n_owned == M.n_cell && M.n_owned > 0) {
-        int rc = make_resident(M, L.maxf, (int)R, sms, L.rp);
-        if (rc) return rc;
-        L.resident = L.rp.n_tiles > 0;
-    }
     L.pingpong = tiled && (scheme == FVLBM_EULER || scheme == FVLBM_AB2);
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -576,12 +581,7 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         return r;
     };
     const size_t plane = (size_t)L.np, slots = plane * L.maxf;
-    L.n_ghost = 0;
-    if (two)
-        for (int64_t c = 0; c < M.n_cell; c++) {
-            if (M.iperm[c] >= M.n_owned) continue;
-            for (int k = 0; k < M.nf[c]; k++) L.n_ghost += M.slots[(size_t)c * MAXP + k].kind != SK_INTERIOR;
-        }
+    L.n_ghost = two ? M.n_bface : 0;
     L.off_link = take(4 * slots);
     L.off_geo = take(2 * R * 3 * slots);
     L.off_bctag = take(2 * slots);
@@ -594,24 +594,22 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
     L.off_tiles = take(tiled ? sizeof(TileRec) * (size_t)L.tp.n_tiles : 0);
     L.off_halo = take(tiled ? 4 * L.tp.halo.size() : 0);
     L.off_r1link = take(tiled ? 4 * (size_t)L.tp.n_r1 * L.maxf : 0);
-    L.off_rlink = take(L.resident ? 4 * slots : 0);
-    L.off_rtiles = take(L.resident ? sizeof(TileRec) * (size_t)L.rp.n_tiles : 0);
-    L.off_rhalo = take(L.resident ? 4 * L.rp.halo.size() : 0);
-    L.off_rr1link = take(L.resident ? 4 * (size_t)L.rp.n_r1 * L.maxf : 0);
+    const bool own_plan = L.rp.n_tiles > 0;
+    L.off_rlink = own_plan ? take(4 * slots) : L.off_link;
+    L.off_rtiles = own_plan ? take(sizeof(TileRec) * (size_t)L.rp.n_tiles) : L.off_tiles;
+    L.off_rhalo = own_plan ? take(4 * L.rp.halo.size()) : L.off_halo;
+    L.off_rr1link = own_plan ? take(4 * (size_t)L.rp.n_r1 * L.maxf) : L.off_r1link;
     L.off_fa = take(S * plane);   // everything before this is uploaded once
     L.off_fb = (scheme == FVLBM_RK2 || scheme == FVLBM_RK4 || L.pingpong) ? take(S * plane) : 0;
     L.off_xchg = take(L.resident ? 2 * 16 * (size_t)resident_units(S) * plane : 0);
     L.off_fc = (scheme == FVLBM_RK4 && tiled) ? take(S * plane) : 0;
     L.off_rprev = scheme == FVLBM_AB2 ? take(R * plane * FVLBM_Q) : 0;
     L.off_fv = take(two ? 4 * R * (slots + (size_t)L.n_ghost) : 0);
-    L.off_rho = take(8 * plane);
-    L.off_ux = take(8 * plane);
-    L.off_uy = take(8 * plane);
     L.off_uold = take(16 * plane);
     L.off_part = take(24 * (size_t)std::max<int64_t>(1, L.n_chunk));
     L.off_red = take(24 * (size_t)M.n_inst);
     L.off_conv = take(8 * plane * FVLBM_Q);
-    L.off_chunk = take(24 * (size_t)std::max<int64_t>(1, L.n_chunk));
+    L.off_chunk = take(24 * (size_t)std::max<int64_t>(1, L.n_chunk) + 8 * (size_t)(M.n_inst + 1));
     L.off_flag = take(16);
     L.total = o;
     return FVLBM_OK;
@@ -679,8 +677,12 @@ void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& h
         while (g + 1 < M.n_inst && c >= M.inst_begin[g + 1]) g++;
         grp[i] = g;
         area[i] = M.area[c];
+        // this cell's words and vectors: word k at word(i, k), 2-vector v of slot k at vec(i, v, k)
+        const size_t w0 = word(i, 0);
+        T* const g0 = vec(i, 0, 0);
+        const double area_i = M.area[c], cx = M.cx[c], cy = M.cy[c];
         for (int k = 0; k < maxf; k++) {
-            const size_t w = word(i, k);
+            const size_t w = w0 + (size_t)(k / 4) * 4 * BLK + k % 4;
             if (k >= M.nf[c]) {
                 link[w] = two ? link_word(0, 0, LK_NONE, 0) : L.tp.link[(size_t)i * maxf + k];
                 if (two) nbr[w] = (int32_t)i;
@@ -695,15 +697,16 @@ void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& h
             } else {
                 link[w] = L.tp.link[(size_t)i * maxf + k];
             }
-            T* q = vec(i, 0, k);
+            T* q = g0 + 2 * ((size_t)(k / PER) * PER * BLK + k % PER);
+            const size_t next_vec = (size_t)2 * PER * BLK * units;
             q[0] = (T)S.cgx;
             q[1] = (T)S.cgy;
-            q = vec(i, 1, k);
-            q[0] = (T)(S.px - M.cx[c]);
-            q[1] = (T)(S.py - M.cy[c]);
-            q = vec(i, 2, k);
-            q[0] = (T)(S.nx / M.area[c]);
-            q[1] = (T)(S.ny / M.area[c]);
+            q += next_vec;
+            q[0] = (T)(S.px - cx);
+            q[1] = (T)(S.py - cy);
+            q += next_vec;
+            q[0] = (T)(S.nx / area_i);
+            q[1] = (T)(S.ny / area_i);
         }
     }
     // 1-ring entries: unit by unit, entry by entry
@@ -717,7 +720,7 @@ void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& h
         std::memcpy(H + L.off_tiles, L.tp.rec.data(), sizeof(TileRec) * L.tp.rec.size());
         std::memcpy(H + L.off_halo, L.tp.halo.data(), 4 * L.tp.halo.size());
     }
-    if (L.resident) {
+    if (L.rp.n_tiles > 0) {
         pack_ring(L.rp, L.off_rr1link);
         std::memcpy(H + L.off_rtiles, L.rp.rec.data(), sizeof(TileRec) * L.rp.rec.size());
         std::memcpy(H + L.off_rhalo, L.rp.halo.data(), 4 * L.rp.halo.size());
@@ -906,10 +909,14 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
         q.uix_f = (float)q.uix;
         q.uiy_f = (float)q.uiy;
     }
-    std::vector<int64_t> chunks;
-    for (int32_t k = 0; k < M.n_inst; k++)
+    std::vector<int64_t> chunks, inst_chunk(1, 0);
+    for (int32_t k = 0; k < M.n_inst; k++) {
         for (int64_t b = M.inst_begin[k]; b < M.inst_begin[k + 1]; b += CHUNK)
             chunks.insert(chunks.end(), {b, std::min(b + CHUNK, M.inst_begin[k + 1]), (int64_t)k});
+        inst_chunk.push_back((int64_t)chunks.size() / 3);
+    }
+    const int64_t n_chunk = inst_chunk.back();
+    chunks.insert(chunks.end(), inst_chunk.begin(), inst_chunk.end());
 
     unsigned char* base = (unsigned char*)s->ws;
     CK(cudaMemcpyAsync(base, host.data(), L.off_fa, cudaMemcpyHostToDevice, s->stream), "upload geometry");
@@ -937,15 +944,13 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     v.fb = L.off_fb ? base + L.off_fb : nullptr;
     v.rprev = L.off_rprev ? base + L.off_rprev : nullptr;
     v.fv = base + L.off_fv;
-    v.rho = (double*)(base + L.off_rho);
-    v.ux = (double*)(base + L.off_ux);
-    v.uy = (double*)(base + L.off_uy);
     v.uold = (double*)(base + L.off_uold);
     v.part = (double*)(base + L.off_part);
     v.red = (double*)(base + L.off_red);
     v.conv = (double*)(base + L.off_conv);
     v.chunk = (const int64_t*)(base + L.off_chunk);
-    v.n_chunk = (int64_t)chunks.size() / 3;
+    v.n_chunk = n_chunk;
+    v.inst_chunk = v.chunk + 3 * n_chunk;
     v.flag = (int32_t*)(base + L.off_flag);
     v.strategy = L.strategy;
     v.block = L.block;
@@ -960,13 +965,13 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     v.sms = device_sms(p0.device);
     if (L.resident) {
         ResView& r = s->res;
-        r.tile = L.rp.tile;
-        r.n_tiles = (int32_t)L.rp.n_tiles;
+        r.tile = L.res_plan().tile;
+        r.n_tiles = (int32_t)L.res_plan().n_tiles;
         r.tiles = (const TileRec*)(base + L.off_rtiles);
         r.link = (const uint4*)(base + L.off_rlink);
         r.halo = (const int32_t*)(base + L.off_rhalo);
         r.r1link = (const uint4*)(base + L.off_rr1link);
-        r.n_r1 = L.rp.n_r1;
+        r.n_r1 = L.res_plan().n_r1;
         r.xchg = (uint4*)(base + L.off_xchg);
         CK(cudaMemsetAsync(r.xchg, 0, 2 * 16 * (size_t)resident_units(state_bytes(s->prec)) * L.np, s->stream), "clear tags");
         s->resident = resident_fits(v, r, s->prec, s->scheme);
@@ -980,10 +985,8 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     // Step 0 and the first residual snapshot
     rc = launch_init_eq(v, s->prec, s->stream);
     if (rc) return rc;
-    rc = launch_macros(v, s->prec, s->stream);
+    rc = launch_snapshot(v, s->prec, s->stream);
     if (rc) return rc;
-    CK(cudaMemcpyAsync(v.uold, v.ux, 8 * L.np, cudaMemcpyDeviceToDevice, s->stream), "snapshot u");
-    CK(cudaMemcpyAsync(v.uold + L.np, v.uy, 8 * L.np, cudaMemcpyDeviceToDevice, s->stream), "snapshot v");
     CK(cudaStreamSynchronize(s->stream), "fvlbm_init");
     return FVLBM_OK;
 }
@@ -1260,9 +1263,7 @@ extern "C" int fvlbm_macros(fvlbm_solver* s, double* rho, double* u) {
 }
 
 static int reduce(fvlbm_solver* s, int what, std::vector<double>& out) {
-    int rc = launch_macros(s->v, s->prec, s->stream);
-    if (rc) return rc;
-    rc = launch_reduce(s->v, s->stream, what);
+    int rc = launch_reduce(s->v, s->prec, s->stream, what);
     if (rc) return rc;
     out.assign(3 * (size_t)s->n_inst, 0.0);
     CK(cudaMemcpyAsync(out.data(), s->v.red, out.size() * 8, cudaMemcpyDeviceToHost, s->stream), "read sums");
@@ -1274,8 +1275,14 @@ int solver_n_stages(const fvlbm_solver* s) { return n_stages(s->scheme); }
 int solver_stage(fvlbm_solver* s, int k, void** out) {
     if (!s || k < 0 || k >= n_stages(s->scheme)) return fail(FVLBM_ERR_ARG, "solver_stage: bad arguments");
     DeviceGuard dg(s->device);
+    s->staged = true;
     return enqueue_stage(s, k, nullptr, out);
 }
+bool solver_replayable(const fvlbm_solver* s) {
+    return s->staged && (s->scheme != FVLBM_AB2 || s->ab2_started);
+}
+int solver_buffer(const fvlbm_solver* s) { return s->cur; }
+void solver_set_buffer(fvlbm_solver* s, int b) { set_current(s, b); }
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out) {
     DeviceGuard dg(s->device);
     return reduce(s, what, out);
