@@ -25,7 +25,13 @@ struct fvlbm_dd {
     cudaEvent_t main_done = nullptr;
     int4* entries = nullptr;   // device: (src part, src internal cell, dst part, dst internal cell)
     int64_t n_entries = 0;
+    // graphs of DD_CHUNK steps, one per state buffer the steps start from (built
+    // when first needed; an even number of steps ends where it started)
+    cudaGraphExec_t chunk[2] = {nullptr, nullptr};
+    bool graphs_ok = true;
 };
+
+static constexpr int64_t DD_CHUNK = 16;
 
 namespace {
 
@@ -51,11 +57,56 @@ int join(fvlbm_dd* d) {
 }
 
 // Copy every ghost's state from its owner, each part's buffer given: on the
-// caller's stream, after every part's queued work, and before any part's next.
+// caller's stream, after every part's queued work.  The parts' next work comes
+// after a fork().
 int exchange(fvlbm_dd* d, void* const* bufs) {
     int rc = join(d);
     if (!rc) rc = launch_halo_copy(d->prec, d->stream, d->entries, d->n_entries, bufs, (int)d->part.size());
-    return rc ? rc : fork(d);
+    return rc;
+}
+
+// n time steps: per stage, every part's stage kernels on its stream, then the exchange.
+int enqueue_steps(fvlbm_dd* d, int64_t n) {
+    const int ns = solver_n_stages(d->part[0]);
+    std::vector<void*> bufs(d->part.size());
+    for (int64_t t = 0; t < n; t++)
+        for (int k = 0; k < ns; k++) {
+            int rc = fork(d);   // after the last exchange, or the work the caller queued on its stream
+            for (size_t p = 0; !rc && p < d->part.size(); p++) rc = solver_stage(d->part[p], k, &bufs[p]);
+            if (!rc) rc = exchange(d, bufs.data());
+            if (rc) return rc;
+        }
+    return FVLBM_OK;
+}
+
+// A stage of every part takes some twenty calls to enqueue (launches, event
+// records and waits), which the host makes more slowly than the device runs the
+// stage: chunks of steps are recorded once and replayed.  False: not available.
+bool chunk_ready(fvlbm_dd* d, int b) {
+    if (d->chunk[b]) return true;
+    cudaStream_t st = (cudaStream_t)d->stream;
+    if (!d->graphs_ok || !st) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+    for (fvlbm_solver* s : d->part)
+        if (!solver_replayable(s) || solver_buffer(s) != b) return false;
+    cudaGraph_t g = nullptr;
+    bool ok = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    if (ok) {
+        const int rc = enqueue_steps(d, DD_CHUNK);
+        ok = cudaStreamEndCapture(st, &g) == cudaSuccess && rc == FVLBM_OK && g != nullptr;
+    }
+    if (ok) ok = cudaGraphInstantiate(&d->chunk[b], g, 0) == cudaSuccess;
+    if (g) cudaGraphDestroy(g);
+    if (!ok) {
+        // nothing of the recording has run: the state is where it was
+        for (fvlbm_solver* s : d->part) solver_set_buffer(s, b);
+        d->chunk[b] = nullptr;
+        d->graphs_ok = false;
+        cudaGetLastError();
+        clear_error();
+    }
+    return ok;
 }
 
 // Exchange on the parts' current states.
@@ -67,7 +118,8 @@ int exchange_current(fvlbm_dd* d) {
         if (rc) return rc;
         bufs[p] = r.view->fa;
     }
-    return exchange(d, bufs.data());
+    int rc = exchange(d, bufs.data());
+    return rc ? rc : fork(d);
 }
 
 int create_impl(fvlbm_dd* d, const fvlbm_partition* plan, const fvlbm_params* params, void* stream) {
@@ -129,6 +181,8 @@ int create_impl(fvlbm_dd* d, const fvlbm_partition* plan, const fvlbm_params* pa
 
 extern "C" void fvlbm_dd_destroy(fvlbm_dd* d) {
     if (!d) return;
+    for (cudaGraphExec_t g : d->chunk)
+        if (g) cudaGraphExecDestroy(g);
     for (fvlbm_solver* s : d->part) fvlbm_solver_destroy(s);
     DeviceGuard dg(d->device);
     if (d->entries) cudaFree(d->entries);
@@ -163,20 +217,21 @@ extern "C" int fvlbm_dd_step(fvlbm_dd* d, int64_t n) {
     clear_error();
     if (!d || n < 0) return fail(FVLBM_ERR_ARG, "fvlbm_dd_step: bad arguments");
     DeviceGuard dg(d->device);
-    const int ns = solver_n_stages(d->part[0]);
-    std::vector<void*> bufs(d->part.size());
-    int frc = fork(d);   // after the work the caller queued on its stream
-    if (frc) return frc;
-    for (int64_t t = 0; t < n; t++)
-        for (int k = 0; k < ns; k++) {
-            for (size_t p = 0; p < d->part.size(); p++) {
-                int rc = solver_stage(d->part[p], k, &bufs[p]);
-                if (rc) return rc;
-            }
-            int rc = exchange(d, bufs.data());
-            if (rc) return rc;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (d->stream) cudaStreamIsCapturing((cudaStream_t)d->stream, &cs);
+    while (n > 0) {
+        const int b = solver_buffer(d->part[0]);
+        if (n >= DD_CHUNK && d->part.size() > 1 && cs == cudaStreamCaptureStatusNone && chunk_ready(d, b)) {
+            cudaError_t e = cudaGraphLaunch(d->chunk[b], (cudaStream_t)d->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "fvlbm_dd_step: graph launch");
+            n -= DD_CHUNK;
+            continue;
         }
-    return FVLBM_OK;
+        int rc = enqueue_steps(d, 1);
+        if (rc) return rc;
+        n--;
+    }
+    return fork(d);   // what the parts do next comes after the last exchange
 }
 
 extern "C" int fvlbm_dd_sync(fvlbm_dd* d) {
