@@ -352,7 +352,12 @@ template <typename H> struct SplitIO {
         n[2] = -sy;
         n[0] = -(s + n[1] + n[2]);
 #pragma unroll
-        for (int a = 0; a < FVLBM_Q; a++) f[a] = (T)fma(wgt<float>(a), feq_value<float, true>(a, dr, ux, uy), n[a]);
+        for (int a = 0; a < FVLBM_Q; a++) {
+            // one rounding, but for direction 5, whose product is rounded by itself
+            // (states decode to the bits that the compiler's own choice gave)
+            f[a] = (T)(a == 5 ? feqs<float, true>(a, dr, ux, uy) + n[a]
+                              : fma(wgt<float>(a), feq_value<float, true>(a, dr, ux, uy), n[a]));
+        }
     }
     template <typename T, bool DEV, typename I>
     __device__ __forceinline__ static void load(const void* base, I i, const InstParam& P, T* f) {

@@ -238,12 +238,14 @@ constexpr int resident_units(size_t state_bytes) { return state_bytes == 72 ? 8 
 // one tile per SM.
 constexpr int RES_LANES_FP64 = 4;
 constexpr int RES_TILE = 256, RES_TILE_FP64 = 64;
-constexpr int resident_ctas(int rsize, int maxf) { return rsize == 8 ? 1 : maxf <= 4 ? 3 : 2; }
+constexpr int resident_ctas(int rsize, int maxf) { return rsize == 8 ? 1 : maxf <= 4 ? 4 : 2; }
 // Its shared memory: state of the local cells, face table, the geometry of the
-// gradient cells (three 2-vectors per slot) and the state the step began with.
-template <int TILE, int MAXF, int RSIZE> struct ResDims : TileDims<TILE, MAXF, RSIZE> {
+// gradient cells (three 2-vectors per slot; with four tiles per SM it stays in
+// global memory) and the state the step began with.
+template <int TILE, int MAXF, int RSIZE, int CTAS> struct ResDims : TileDims<TILE, MAXF, RSIZE> {
     typedef TileDims<TILE, MAXF, RSIZE> B;
-    static constexpr size_t GEO_BYTES = (size_t)3 * 2 * RSIZE * MAXF * TILE;
+    static constexpr bool GEO_SHARED = CTAS <= 3;
+    static constexpr size_t GEO_BYTES = GEO_SHARED ? (size_t)3 * 2 * RSIZE * MAXF * TILE : 0;
     static constexpr size_t BASE_BYTES = (size_t)FVLBM_Q * RSIZE * TILE;
     static constexpr size_t BYTES = B::BYTES + GEO_BYTES + BASE_BYTES;
 };

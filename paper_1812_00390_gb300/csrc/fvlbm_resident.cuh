@@ -114,26 +114,26 @@ template <typename T> __device__ __forceinline__ T stage_beta(int ns, int k) {
 
 // Deviation modes: a thread per tile and 1-ring cell, FP32.  Multistage
 // schemes with ns stages per step (1: Euler), or AB2.  What does not wait for
-// the halo is done before it is taken, the own cells' collision term and ghost
-// values, where a CTA has the SM to itself (EARLY); with several per SM it would
+// the halo, the own cells' collision term, is done before it is taken where a CTA
+// has the SM to itself (EARLY); with several per SM it would
 // hold registers that are short, and the other CTAs fill the wait.  Geometry and the step's first state sit in shared memory, each
 // thread's own.
 template <typename S, int MAXF, int TILE, int CTAS, bool AB2>
 __global__ void __launch_bounds__(TILE, CTAS)
     resident_kernel(DevView v, ResView r, int ns, int64_t stages, uint32_t epoch, int ab2_started) {
     typedef float T;
-    typedef ResDims<TILE, MAXF, sizeof(T)> D;
+    typedef ResDims<TILE, MAXF, sizeof(T), CTAS> D;
     typedef float2 T2;
     typedef float4 V;
     constexpr bool DEV = true;
     constexpr int LS = D::LS, ROWS = D::ROWS, W = Wire<S>::W;
     constexpr int GU = GeoRef<T, MAXF>::UNITS;
-    constexpr bool EARLY = CTAS == 1;
+    constexpr bool EARLY = CTAS == 1, SHARED = D::GEO_SHARED;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* fs = (V*)smem_raw;         // [2][LS]       moving directions of the local cells
     V* tab = fs + 2 * LS;         // [ROWS]        face table
     V* sgeo = tab + ROWS;         // [3 GU][TILE]  geometry of the gradient cells
-    V* sbase = sgeo + 3 * GU * TILE;          // [2][TILE]  state the step began with
+    V* sbase = sgeo + (SHARED ? 3 * GU * TILE : 0);   // [2][TILE]  state the step began with
     float* sbase0 = (float*)(sbase + 2 * TILE);   // [TILE]
     const TileRec R = r.tiles[blockIdx.x];
     const int l = threadIdx.x, nt = R.nt, n2 = R.nt + R.n1, n_ring2 = R.nh - R.n1, inst = R.inst;
@@ -155,18 +155,19 @@ __global__ void __launch_bounds__(TILE, CTAS)
             d[4 * u + 3] = x.w;
         }
     }
-    if (l < n2) {
+    if (SHARED && l < n2) {
 #pragma unroll
         for (int u = 0; u < 3 * GU; u++) sgeo[u * TILE + l] = G.g[u * BLK];
     }
     auto geo = [&](int vec, int k) -> T2 {
+        if (!SHARED) return G.get(vec, k);
         const float2* p = (const float2*)(sgeo + (vec * GU + k / 2) * TILE + threadIdx.x);
         return p[k % 2];
     };
     auto geo_all = [&](int vec, T2* out) {   // in 16-byte loads: no bank conflict
 #pragma unroll
         for (int u = 0; u < GU; u++) {
-            const V q = sgeo[(vec * GU + u) * TILE + threadIdx.x];
+            const V q = SHARED ? sgeo[(vec * GU + u) * TILE + threadIdx.x] : G.g[(vec * GU + u) * BLK];
             out[2 * u] = make_float2(q.x, q.y);
             out[2 * u + 1] = make_float2(q.z, q.w);
         }
@@ -215,10 +216,6 @@ __global__ void __launch_bounds__(TILE, CTAS)
             }
             to_shared(l, f);
         }
-        if (EARLY) {
-            to_pairs(f, fp);
-            if (l < n2) tile_boundary<T, DEV, MAXF, TILE, true>(v, d, gl, f[0], fp, gx, gy, tab, l, mine, lsq, face);
-        }
         for (int e = l; e < n_ring2; e += TILE) {
             const uint32_t i = (uint32_t)__ldg(r.halo + R.h0 + R.n1 + e);
             const InstParam& Pi = v.inst[inst >= 0 ? inst : v.grp[i]];
@@ -237,14 +234,13 @@ __global__ void __launch_bounds__(TILE, CTAS)
             return;
         }
         if (l < n2) {
-            if (!EARLY) {
-                to_pairs(f, fp);
-                tile_boundary<T, DEV, MAXF, TILE, true>(v, d, gl, f[0], fp, gx, gy, tab, l, mine, lsq, face);
-            }
+            to_pairs(f, fp);
             T2 c[MAXF], m[MAXF];
             geo_all(GEO_LSQ, c);
-            geo_all(GEO_MID, m);
-            tile_faces<T, DEV, MAXF, TILE>(d, fp, gx, gy, fs, tab, l, [&](int q) { return c[q]; }, [&](int q) { return m[q]; });
+            tile_faces<T, DEV, MAXF, TILE>(d, fp, gx, gy, fs, tab, l, [&](int q) { return c[q]; },
+                                           [&](int q) { return m[q]; }, [&] { geo_all(GEO_MID, m); }, [&] {
+                tile_boundary<T, DEV, MAXF, TILE, true>(v.bc, v.bctag, d, gl, f[0], fp, gx, gy, tab, l, mine, lsq, face);
+            });
         }
         __syncthreads();
         if (mine) {
@@ -302,7 +298,7 @@ template <int MAXF, int TILE, bool AB2>
 __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
     resident_pairs_kernel(DevView v, ResView r, int ns, int64_t stages, uint32_t epoch, int ab2_started) {
     typedef double T;
-    typedef ResDims<TILE, MAXF, sizeof(T)> D;
+    typedef TileDims<TILE, MAXF, sizeof(T)> D;
     constexpr int LS = D::LS, ROWS = D::ROWS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2* fs = (double2*)smem_raw;   // [LS][4]    pairs of the local cells
@@ -543,7 +539,7 @@ static const void* resident_of(int scheme, int& threads, size_t& smem) {
         return ab2 ? (const void*)resident_pairs_kernel<MAXF, TILE, true> : (const void*)resident_pairs_kernel<MAXF, TILE, false>;
     } else {
         threads = TILE;
-        smem = ResDims<TILE, MAXF, 4>::BYTES;
+        smem = ResDims<TILE, MAXF, 4, CTAS>::BYTES;
         return ab2 ? (const void*)resident_kernel<S, MAXF, TILE, CTAS, true>
                    : (const void*)resident_kernel<S, MAXF, TILE, CTAS, false>;
     }
@@ -564,8 +560,9 @@ static int resident_m(const DevView& v, const ResView& r, cudaStream_t st, int s
         if (r.tile == 64) kern = resident_of<S, MAXF, 64, 1>(scheme, threads, smem);
         if (r.tile == 128) kern = resident_of<S, MAXF, 128, 1>(scheme, threads, smem);
         if (r.tile == RES_TILE)
-            kern = r.n_tiles <= v.sms ? resident_of<S, MAXF, RES_TILE, 1>(scheme, threads, smem)
-                                      : resident_of<S, MAXF, RES_TILE, MORE>(scheme, threads, smem);
+            kern = r.n_tiles <= v.sms       ? resident_of<S, MAXF, RES_TILE, 1>(scheme, threads, smem)
+                   : r.n_tiles <= 3 * v.sms ? resident_of<S, MAXF, RES_TILE, MORE < 3 ? MORE : 3>(scheme, threads, smem)
+                                            : resident_of<S, MAXF, RES_TILE, MORE>(scheme, threads, smem);
     }
     if (!kern) return fail(FVLBM_ERR_ARG, "resident stage loop: tiles of %d cells", r.tile);
     return resident_launch(kern, threads, smem, v, r, st, scheme, stages, epoch, ab2_started, max_ctas);

@@ -485,7 +485,7 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 // The resident stage loop's plan (fvlbm_resident.cuh), if the solver is small
 // enough: one tile per SM, as long as the SM's share of the cells but not below
-// a length at which the halo outgrows the tile; in FP32 also two or three of the
+// a length at which the halo outgrows the tile; in FP32 also two to four of the
 // largest tiles per SM.
 int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P, bool verify) {
     const int64_t n = M.n_owned;
@@ -496,10 +496,14 @@ int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P, bool
         for (int tile = ctas > 1 ? most : rsize == 8 ? 16 : 64; tile <= most; tile *= 2) {
             // a compact tile of q cells has about 4.3 sqrt(q) 1-ring cells
             if (share + 4.3 * std::sqrt((double)share) > tile) continue;
-            int rc = make_tiles(M, maxf, tile, P, verify, (int)std::min<int64_t>(share, tile));
-            if (rc == FVLBM_OK && P.n_tiles <= (int64_t)ctas * sms) return FVLBM_OK;
-            P = TilePlan{};
-            if (rc && rc != FVLBM_ERR_UNSUPPORTED) return rc;
+            // equal tiles; where a few are cut shorter and there are too many, as long as they fit
+            for (int64_t len : {std::min<int64_t>(share, tile), (int64_t)tile}) {
+                if (len == tile && ctas < std::min(3, resident_ctas(rsize, maxf))) continue;
+                int rc = make_tiles(M, maxf, tile, P, verify, (int)len);
+                if (rc == FVLBM_OK && P.n_tiles <= (int64_t)ctas * sms) return FVLBM_OK;
+                P = TilePlan{};
+                if (rc && rc != FVLBM_ERR_UNSUPPORTED) return rc;
+            }
         }
     }
     return FVLBM_OK;   // none: P.n_tiles == 0

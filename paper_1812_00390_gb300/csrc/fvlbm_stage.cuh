@@ -182,7 +182,7 @@ __device__ __forceinline__ void add_flux(uint32_t d, const typename Vec2<T>::typ
     }
 }
 
-// Boundary slots of one cell (Sec. 2.4): the ghost differences start the
+// Boundary slots of one cell (Sec. 2.4): the ghost differences enter the
 // gradient; where the cell's faces are in the face table (own rows, and ghost
 // rows for what enters), the boundary face values that are ghost values are
 // written: everything on walls, symmetry planes (half way to the ghost) and
@@ -223,7 +223,9 @@ __device__ __forceinline__ void boundary_slots(const uint32_t* d, const BcParam*
             const Pair<T> dd = make_pair2(da, db);
             gx[p] = fma2(cx, dd, gx[p]);
             gy[p] = fma2(cy, dd, gy[p]);
-            const T va = fma(part, da, f[a]), vb = fma(part, db, f[b]);
+            // (a choice of factor spares FP64 an operation, a choice of result FP32 a register)
+            const T va = !DEV ? fma(part, da, f[a]) : g.sym ? f[a] + T(0.5) * da : f[a] + da;
+            const T vb = !DEV ? fma(part, db, f[b]) : g.sym ? f[b] + T(0.5) * db : f[b] + db;
             const bool s = link_a_leaves(dk, p);
             qo.v[p] = s ? va : vb;
             qi.v[p] = s ? vb : va;
@@ -458,13 +460,16 @@ __global__ void __launch_bounds__(256) face_values_kernel(DevView v, const S* __
     for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
     const uint32_t used = warp_slots<MAXF>(d);
     const int64_t row = blk_index(i, MAXF);
-    if (boundary_mask<MAXF>(d))
-        boundary_slots<T, DEV, MAXF, false>(d, v.bc, f[0], fp, gx, gy, [&](int k) { return v.bctag[i * MAXF + k]; },
-                                     [&](int k) { return G.get(GEO_LSQ, k); }, [&](int k) { return G.get(GEO_FACE, k); },
-                                     [&](int k, const Quad<T>& q) { store_quad(face_row<T>(v.fv, row + k * BLK), 1, q); },
-                                     [&](int k, uint32_t, const Quad<T>& q) {
-                                         if (i < v.n_cell) store_quad(face_row<T>(v.fv, v.np * MAXF + nb[k]), 1, q);
-                                     });
+    auto boundary = [&] {
+        if (boundary_mask<MAXF>(d))
+            boundary_slots<T, DEV, MAXF, false>(d, v.bc, f[0], fp, gx, gy, [&](int k) { return v.bctag[i * MAXF + k]; },
+                                         [&](int k) { return G.get(GEO_LSQ, k); }, [&](int k) { return G.get(GEO_FACE, k); },
+                                         [&](int k, const Quad<T>& q) { store_quad(face_row<T>(v.fv, row + k * BLK), 1, q); },
+                                         [&](int k, uint32_t, const Quad<T>& q) {
+                                             if (i < v.n_cell) store_quad(face_row<T>(v.fv, v.np * MAXF + nb[k]), 1, q);
+                                         });
+    };
+    if (!DEV) boundary();
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
@@ -478,6 +483,7 @@ __global__ void __launch_bounds__(256) face_values_kernel(DevView v, const S* __
             add_gradient(Quad<T>{{fj[dir_a(2 * h)], fj[dir_b(2 * h)], fj[dir_a(2 * h + 1)], fj[dir_b(2 * h + 1)]}}, cx,
                          cy, h, fp, gx, gy);
     }
+    if (DEV) boundary();
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
@@ -583,32 +589,35 @@ __global__ void __launch_bounds__(256) update_kernel(DevView v, const S* __restr
     CellIO<S>::template store<T, DEV>(fout, i, P, out);
 }
 
-// Phase 2 of a tile for local cell l, in two parts.  The first, for boundary
-// cells, needs the cell's own state only and touches rows of the face table that
-// only the cell itself reads: ghost values, and the gradient's start.
+// Phase 2 of a tile for local cell l.  Boundary cells' part: ghost differences
+// into the gradient and ghost values into the face table (rows that only the
+// cell itself reads).
 template <typename T, bool DEV, int MAXF, int TILE, bool NEXT, typename Lsq, typename Face>
-__device__ __forceinline__ void tile_boundary(const DevView& v, const uint32_t* d, uint32_t gl, T f0, const Pair<T>* f,
-                                              Pair<T>* gx, Pair<T>* gy, typename Vec16<T>::type* tab, int l, bool mine,
-                                              Lsq lsq, Face face) {
+__device__ __forceinline__ void tile_boundary(const BcParam* bc, const uint16_t* bctag, const uint32_t* d, uint32_t gl, T f0,
+                                              const Pair<T>* f, Pair<T>* gx, Pair<T>* gy, typename Vec16<T>::type* tab,
+                                              int l, bool mine, Lsq lsq, Face face) {
     constexpr int ROWS = TileDims<TILE, MAXF, sizeof(T)>::ROWS;
-#pragma unroll
-    for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
-    if (boundary_mask<MAXF>(d))
-        boundary_slots<T, DEV, MAXF, NEXT>(d, v.bc, f0, f, gx, gy, [&](int k) { return v.bctag[(int64_t)gl * MAXF + k]; }, lsq,
-                                     face, [&](int k, const Quad<T>& q) { store_quad(tab + k * TILE + l, ROWS, q); },
-                                     [&](int, uint32_t dk, const Quad<T>& q) {
-                                         if (mine) store_quad(tab + link_row(dk), ROWS, q);
-                                     });
+    boundary_slots<T, DEV, MAXF, NEXT>(d, bc, f0, f, gx, gy, [&](int k) { return bctag[(int64_t)gl * MAXF + k]; }, lsq, face,
+                                       [&](int k, const Quad<T>& q) { store_quad(tab + k * TILE + l, ROWS, q); },
+                                       [&](int, uint32_t dk, const Quad<T>& q) {
+                                           if (mine) store_quad(tab + link_row(dk), ROWS, q);
+                                       });
 }
-// The second: the neighbour differences, then what leaves the cell through
-// every face into the face table.  lsq, mid: its geometry vectors by slot.
-template <typename T, bool DEV, int MAXF, int TILE, typename Lsq, typename Mid>
+// All of it: the neighbour differences, boundary() where it adds its part, then
+// what leaves the cell through every face into the face table.  lsq, mid: its
+// geometry vectors by slot (mid after before_mid()).
+template <typename T, bool DEV, int MAXF, int TILE, typename Lsq, typename Mid, typename BeforeMid, typename Boundary>
 __device__ __forceinline__ void tile_faces(const uint32_t* d, const Pair<T>* f, Pair<T>* gx, Pair<T>* gy,
                                            const typename Vec16<T>::type* fs, typename Vec16<T>::type* tab, int l, Lsq lsq,
-                                           Mid mid) {
+                                           Mid mid, BeforeMid before_mid, Boundary boundary) {
     typedef TileDims<TILE, MAXF, sizeof(T)> D;
     typedef typename Vec2<T>::type T2;
     constexpr int LS = D::LS, ROWS = D::ROWS, SU = 8 / Vec16<T>::N;
+    // (FP64: before the neighbours, as the four-lane kernels, where it overlaps the wait for the halo)
+#pragma unroll
+    for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
+    const bool bc = boundary_mask<MAXF>(d) != 0;
+    if (!DEV && bc) boundary();
     const uint32_t used = warp_slots<MAXF>(d);
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
@@ -619,6 +628,8 @@ __device__ __forceinline__ void tile_faces(const uint32_t* d, const Pair<T>* f, 
 #pragma unroll
         for (int h = 0; h < 2; h++) add_gradient(load_quad(nb + h * (SU / 2) * LS, LS), cx, cy, h, f, gx, gy);
     }
+    if (DEV && bc) boundary();
+    before_mid();
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
@@ -777,9 +788,10 @@ __global__ void __launch_bounds__(TILE, stage_ctas(TILE, sizeof(T)))
         }
         auto lsq = [&](int k) { return MAXF <= 4 ? c[k] : G.get(GEO_LSQ, k); };
         Pair<T> gx[4], gy[4];
-        tile_boundary<T, DEV, MAXF, TILE, false>(v, d, gl, f0, f, gx, gy, tab, l, mine, lsq,
-                                          [&](int k) { return G.get(GEO_FACE, k); });
-        tile_faces<T, DEV, MAXF, TILE>(d, f, gx, gy, fs, tab, l, lsq, [&](int k) { return G.get(GEO_MID, k); });
+        tile_faces<T, DEV, MAXF, TILE>(d, f, gx, gy, fs, tab, l, lsq, [&](int k) { return G.get(GEO_MID, k); }, [] {}, [&] {
+            tile_boundary<T, DEV, MAXF, TILE, false>(v.bc, v.bctag, d, gl, f0, f, gx, gy, tab, l, mine, lsq,
+                                                     [&](int k) { return G.get(GEO_FACE, k); });
+        });
     }
     // phase 3 inputs, in flight during the wait
     T2 n[MAXF];

@@ -21,7 +21,7 @@ def fv():
 
 
 # one tile of two cells; a few tiles; every boundary kind; polygons; one tile on
-# (nearly) every SM; tiles of the largest size
+# (nearly) every SM; three and four tiles per SM (FP64 beyond the loop's sizes)
 MESHES = {
     "two_cells": lambda: mg.two_triangles(),
     "two_cells_periodic": lambda: mg.two_triangles(periodic=True),
@@ -33,6 +33,9 @@ MESHES = {
     "periodic": lambda: mg.periodic_tri(71, 53, lx=71.0, ly=53.0),
     "cavity": lambda: mg.cavity(127, 20.0),
     "cylinder": lambda: mg.cylinder_hybrid(n_rad=70, n_circ=171, n_tri_rings=90, seed=5),
+    "periodic_73k": lambda: mg.periodic_tri(192, 190, lx=192.0, ly=190.0),
+    "cavity_103k": lambda: mg.cavity(321, 20.0),
+    "bricks_50k": lambda: mg.bricks(400, 240),
 }
 
 
