@@ -110,7 +110,8 @@ typedef struct fvlbm_params {
     int32_t kernel;    /* stage kernel: 0 = automatic (FP32 / 16-bit: fused 512-thread tiles
                           from 512 cells per SM, 256-thread tiles from 64, 128-thread tiles
                           below; FP64: two kernels from 32 cells per SM, fused 128-thread
-                          tiles below, where one launch per stage matters most);
+                          tiles below), and fvlbm_step runs small meshes in the resident
+                          loop (see there), with the same results;
                           1 = two kernels per stage (face values
                           through memory); 128, 256, 512 or 1024 = one fused kernel per stage
                           with CTAs of that many threads (a tile holds at most that many
@@ -194,12 +195,13 @@ int fvlbm_workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params* params, in
  * Eq. lslrflux stay on chip; Sec. 2.4 algorithm Steps 1-5 in one kernel).
  * The check covers what the kernel relies on: every slot names its
  * neighbour's local cell (boundary and unused slots the cell itself, unused
- * slots face row 0), both sides of a face name one face row and no two faces
- * share one, each (face, direction) between local cells has exactly one writer
- * (Sec. 2.4.2: the upwind side), and every tile fits its CTA.  The wavefront
- * figures model the shared-memory bank conflicts of the kernel's warp
- * accesses: the most distinct addresses one of the 32 banks receives, averaged
- * over the accesses (1: conflict-free).
+ * slots face row 0), what enters through a face is read from the row its
+ * neighbour writes, no two boundary faces share a ghost row, each (face,
+ * direction) between local cells has exactly one writer (Sec. 2.4.2: the upwind
+ * side), and every tile fits its CTA.  The wavefront figures model the
+ * shared-memory bank conflicts of the kernel's 16-byte warp accesses: eight lanes
+ * at a time, the most distinct rows that share a 16-byte bank, averaged over the
+ * accesses (1: conflict-free).
  *   params: host, [n_params] as for fvlbm_init.  info: host, written.
  * A failed check is counted in info->violations and described by
  * fvlbm_last_error(); the call still returns FVLBM_OK.
@@ -215,7 +217,8 @@ typedef struct fvlbm_plan_info_s {
     double mean_tile_cells;      /* cells per tile */
     double mean_ring1_cells;     /* 1-ring cells per tile (gradients recomputed) */
     double mean_local_cells;     /* tile + 1-ring + 2-ring cells per tile */
-    double face_table_waves;     /* wavefronts per warp read of the face table (phase 3) */
+    double face_table_waves;     /* wavefronts per warp access of the face table (own row written and read,
+                                    neighbour's row read) */
     double gather_waves;         /* wavefronts per warp gather of neighbour state (phase 2) */
     int64_t violations;          /* failed checks (0) */
 } fvlbm_plan_info_t;
@@ -241,6 +244,13 @@ int fvlbm_init(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_par
  * Advance every instance by n time steps (Steps 1-6, Sec. 2.4 algorithm),
  * asynchronously on the solver's stream.  A non-finite value raises a device
  * flag that the next synchronising call reports as FVLBM_ERR_DIVERGED.
+ * With params.kernel = 0, small meshes (FP32 and 16-bit up to about 110,000
+ * cells of up to four faces, FP64 up to about 5,800) run up to 2048 stages in one
+ * cooperative launch whose thread blocks exchange halo cells; the results are
+ * those of the stage kernels, bit for bit in FP32 and 16-bit precision.  Such launches of different solvers take
+ * turns on the GPU.  Every wait in them is bounded; one that runs out is reported by
+ * the next synchronising call as FVLBM_ERR_TIMEOUT.  In a stream capture by the
+ * caller the stages are recorded one by one.
  * Errors: FVLBM_ERR_ARG, _CUDA.
  */
 int fvlbm_step(fvlbm_solver* s, int64_t n);
@@ -351,7 +361,9 @@ int fvlbm_profile(fvlbm_solver* s, int64_t n, double* avg_ms, int32_t max_kinds,
  * within 3% (or 2 microseconds per step) of the fastest the automatic choice
  * (params.kernel = 0) wins, and else the first of 512, 256, 128, 1024, 1, so
  * that timing noise on small meshes does not flip the pick between equally
- * fast variants.
+ * fast variants.  The pick is a stage kernel; the resident loop that
+ * params.kernel = 0 runs on small meshes is not among the variants (and is
+ * faster there).
  *   stream       as for fvlbm_init
  *   best_kernel  host, written: the value to put in fvlbm_params.kernel
  *   ms_per_step  host [5] or NULL: median device ms per step of each variant in
@@ -368,7 +380,8 @@ int fvlbm_autotune(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n
  */
 int fvlbm_fma_peak(int32_t device, int32_t fp64, double* tflops);
 
-/* Kernels one time step launches (host, written). */
+/* Kernels one time step launches, stage by stage (the resident loop of fvlbm_step
+ * launches one for up to 2048 stages).  launches: host, written. */
 int fvlbm_launches_per_step(const fvlbm_solver* s, int64_t* launches);
 
 void fvlbm_solver_destroy(fvlbm_solver* s);
@@ -378,7 +391,8 @@ void fvlbm_solver_destroy(fvlbm_solver* s);
  * order; every fvlbm_server_poll round
  *   1. advances every active request by check_interval time steps (the
  *      residual interval of Sec. 3.2), each request on one of n_streams
- *      streams so that the kernels of different requests overlap;
+ *      streams, so that the kernels of different requests overlap (the resident
+ *      launches of small meshes take turns);
  *   2. admits queued requests, first fit in arrival order, while fewer than
  *      max_active are active and the device arena (arena_bytes, allocated once
  *      at creation) has a free block for the request's workspace;

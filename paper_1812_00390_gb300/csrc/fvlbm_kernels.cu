@@ -7,10 +7,10 @@
 //  face_values   Steps 1-3.  Per cell: rho, u (Sec. 2.1), boundary ghost /
 //                wall values (Sec. 2.4.1, Eq. wallbc), the weighted
 //                least-squares gradient of f_1..f_8 (Eq. leastsquare, with
-//                precomputed coefficients), then the face value of every
-//                (face, direction) for which this cell is the upwind side
-//                (Eq. lslrflux), and every direction of its boundary faces
-//                (Sec. 2.4.2).  Each (face, direction) has exactly one writer.
+//                precomputed coefficients), then what leaves the cell through
+//                every face (Eq. lslrflux; one direction of each opposite pair)
+//                and the ghost values of its boundary faces (Sec. 2.4.2).  Each
+//                (face, direction) has exactly one writer.
 //  update        Steps 4-5.  Per cell: flux sum -sum_m (e.n dl / A) f_m
 //                over its faces, BGK collision -(f - f^eq)/tau with f^eq of
 //                the same stage state, and out = base + beta dt RHS (or the

@@ -468,6 +468,8 @@ struct Layout {
 };
 
 constexpr size_t SMEM_LIMIT = 227 * 1024;
+// shortest tiles (FP32: 16 / 32 / 48 / 96 cells 2.06 / 1.56 / 1.61 / 1.71 us per stage of 2,048
+// triangles, 2.28 / 2.17 / 1.96 / 1.85 of 3,600 quads; FP64: 4 / 8 / 16 cells 6.2 / 5.5 / 5.4 of 512)
 constexpr int RES_MIN_CELLS(int rsize) { return rsize == 4 ? 48 : 16; }
 
 // Streaming multiprocessors of a device (152 on GB300 when no device answers).
@@ -486,7 +488,10 @@ int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // The resident stage loop's plan (fvlbm_resident.cuh), if the solver is small
 // enough: one tile per SM, as long as the SM's share of the cells but not below
 // a length at which the halo outgrows the tile; in FP32 also two to four of the
-// largest tiles per SM.
+// largest tiles per SM.  The limits are what fits on the GPU at once, below which it
+// was the faster way throughout (us per FP32 stage, here / streaming: 40k cells 3.1 /
+// 4.9, 68k 3.8 / 5.6, 78k 5.6 / 6.5, 90k 5.9 / 6.4; FP64 3.6k cells 6.6, streaming 10k
+// cells 17.5).
 int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P, bool verify) {
     const int64_t n = M.n_owned;
     const int most = rsize == 8 ? RES_TILE_FP64 : RES_TILE;
