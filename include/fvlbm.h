@@ -391,8 +391,8 @@ void fvlbm_solver_destroy(fvlbm_solver* s);
  * order; every fvlbm_server_poll round
  *   1. advances every active request by check_interval time steps (the
  *      residual interval of Sec. 3.2), each request on one of n_streams
- *      streams, so that the kernels of different requests overlap (the resident
- *      launches of small meshes take turns);
+ *      streams, so that the kernels of different requests overlap (requests that
+ *      together are at most 110,000 cells take turns in resident launches);
  *   2. admits queued requests, first fit in arrival order, while fewer than
  *      max_active are active and the device arena (arena_bytes, allocated once
  *      at creation) has a free block for the request's workspace;

@@ -198,7 +198,7 @@ struct DevView {
     void* fv;   // two-kernel stage: Quad<T> of outgoing values per (cell, slot), blocked [maxf], then the
                 // ghost records (values that enter through boundary faces)
     double* uold;   // [2][np] the residual's snapshot of u
-    double* part;   // [n_chunk][3] block partial sums
+    double* part;   // [n_chunk][RED_PARTS][2] block partial sums
     double* red;    // [n_inst][3]  per-instance sums
     double* conv;   // [9][np] doubles: device staging of get_f / set_f / macros in caller order
     const int64_t* chunk;   // [n_chunk][3] (begin, end, instance)
@@ -249,6 +249,8 @@ template <int TILE, int MAXF, int RSIZE, int CTAS> struct ResDims : TileDims<TIL
     static constexpr size_t BASE_BYTES = (size_t)FVLBM_Q * RSIZE * TILE;
     static constexpr size_t BYTES = B::BYTES + GEO_BYTES + BASE_BYTES;
 };
+
+constexpr int RED_PARTS = 4;   // blocks per chunk of a reduction
 
 enum Strategy { STRATEGY_TWO_KERNEL = 0, STRATEGY_TILE = 1 };
 
@@ -308,6 +310,8 @@ int solver_stage(fvlbm_solver* s, int k, void** out);
 bool solver_replayable(const fvlbm_solver* s);
 int solver_buffer(const fvlbm_solver* s);
 void solver_set_buffer(fvlbm_solver* s, int b);
+// Whether the next steps may take the whole GPU (the resident loop); the results are the same.
+void solver_alone(fvlbm_solver* s, bool alone);
 // FP64 sums of a reduction (RED_MASS: [mass, -, -]; RED_RESIDUAL: [numerator,
 // denominator, -]) per instance, 3 per instance; synchronises.
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out);

@@ -115,9 +115,10 @@ __global__ void macros_ordered_kernel(DevView v, double* __restrict__ rho_out, d
     }
 }
 
-// Deterministic FP64 reductions: one block per chunk of one instance, fixed
-// tree order; then one warp per instance sums its chunks (they are consecutive),
-// lane by lane and in a fixed tree.  rho, u come from the stored state as they
+// Deterministic FP64 reductions: RED_PARTS blocks per chunk of one instance (a
+// mesh of 100,000 cells is 25 chunks: by themselves they leave most SMs idle, 147 us
+// for its residual), fixed tree order; then one warp per instance sums its parts
+// (they are consecutive), lane by lane and in a fixed tree.  rho, u come from the stored state as they
 // are summed: as arrays of their own they cost a second pass of 48 bytes per cell
 // (and every thread of the last kernel went over every chunk: 1.26 ms for a
 // residual of the 256-instance batch).
@@ -126,8 +127,10 @@ constexpr int RED_THREADS = 256;
 template <typename T, typename S, bool DEV>
 __global__ void __launch_bounds__(RED_THREADS) reduce_chunks_kernel(DevView v, int what) {
     __shared__ double sh[2][RED_THREADS];
-    const int64_t ch = blockIdx.x;
-    const int64_t b = v.chunk[3 * ch], e = v.chunk[3 * ch + 1];
+    const int64_t ch = blockIdx.x / RED_PARTS;
+    const int part = blockIdx.x % RED_PARTS;
+    const int64_t first = v.chunk[3 * ch], n = v.chunk[3 * ch + 1] - first;
+    const int64_t b = first + n * part / RED_PARTS, e = first + n * (part + 1) / RED_PARTS;
     const InstParam& P = v.inst[v.chunk[3 * ch + 2]];
     double s0 = 0, s1 = 0;
     for (int64_t i = b + threadIdx.x; i < e; i += RED_THREADS) {
@@ -154,15 +157,15 @@ __global__ void __launch_bounds__(RED_THREADS) reduce_chunks_kernel(DevView v, i
         __syncthreads();
     }
     if (threadIdx.x == 0)
-        for (int q = 0; q < 2; q++) v.part[3 * ch + q] = sh[q][0];
+        for (int q = 0; q < 2; q++) v.part[2 * (int64_t)blockIdx.x + q] = sh[q][0];
 }
 
 __global__ void reduce_final_kernel(DevView v) {
     const int inst = (blockIdx.x * blockDim.x + threadIdx.x) / 32, lane = threadIdx.x & 31;
     if (inst >= v.n_inst) return;
     double s[2] = {0, 0};
-    for (int64_t ch = v.inst_chunk[inst] + lane; ch < v.inst_chunk[inst + 1]; ch += 32)
-        for (int q = 0; q < 2; q++) s[q] += v.part[3 * ch + q];
+    for (int64_t x = RED_PARTS * v.inst_chunk[inst] + lane; x < RED_PARTS * v.inst_chunk[inst + 1]; x += 32)
+        for (int q = 0; q < 2; q++) s[q] += v.part[2 * x + q];
     for (int d = 16; d > 0; d >>= 1)
         for (int q = 0; q < 2; q++) s[q] += __shfl_down_sync(0xFFFFFFFFu, s[q], d);
     if (lane == 0) {
@@ -230,7 +233,7 @@ int launch_snapshot(const DevView& v, int prec, void* stream) {
 }
 
 template <typename T, typename S, bool DEV> static void reduce_chunks(const DevView& v, cudaStream_t st, int what) {
-    if (v.n_chunk > 0) reduce_chunks_kernel<T, S, DEV><<<(unsigned)v.n_chunk, RED_THREADS, 0, st>>>(v, what);
+    if (v.n_chunk > 0) reduce_chunks_kernel<T, S, DEV><<<(unsigned)(v.n_chunk * RED_PARTS), RED_THREADS, 0, st>>>(v, what);
     reduce_final_kernel<<<grid_of(32 * (int64_t)v.n_inst, 128), 128, 0, st>>>(v);
 }
 

@@ -55,7 +55,7 @@ struct fvlbm_solver {
     int64_t direct_steps = 0;
     bool staged = false;   // a stage has been launched by itself (partitioned solve)
     // small solvers: steps run in the resident stage loop; exchange tags used so far
-    bool resident = false;
+    bool resident = false, alone = true;
     ResView res{};
     uint32_t epoch = 0;
 };
@@ -615,7 +615,7 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
     L.off_rprev = scheme == FVLBM_AB2 ? take(R * plane * FVLBM_Q) : 0;
     L.off_fv = take(two ? 4 * R * (slots + (size_t)L.n_ghost) : 0);
     L.off_uold = take(16 * plane);
-    L.off_part = take(24 * (size_t)std::max<int64_t>(1, L.n_chunk));
+    L.off_part = take(16 * RED_PARTS * (size_t)std::max<int64_t>(1, L.n_chunk));
     L.off_red = take(24 * (size_t)M.n_inst);
     L.off_conv = take(8 * plane * FVLBM_Q);
     L.off_chunk = take(24 * (size_t)std::max<int64_t>(1, L.n_chunk) + 8 * (size_t)(M.n_inst + 1));
@@ -1183,7 +1183,7 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
                   s->direct_steps > 0 && (s->scheme != FVLBM_AB2 || s->ab2_started);
     // small solvers: chunks of whole steps, at least two stages each, in the
     // resident loop (a caller's capture records the stages one by one)
-    if (s->resident && cs == cudaStreamCaptureStatusNone) {
+    if (s->resident && s->alone && cs == cudaStreamCaptureStatusNone) {
         const int ns = n_stages(s->scheme);
         while (n * ns >= 2) {
             int64_t m = std::min(n, RESIDENT_CHUNK / ns);
@@ -1292,6 +1292,7 @@ bool solver_replayable(const fvlbm_solver* s) {
 }
 int solver_buffer(const fvlbm_solver* s) { return s->cur; }
 void solver_set_buffer(fvlbm_solver* s, int b) { set_current(s, b); }
+void solver_alone(fvlbm_solver* s, bool alone) { s->alone = alone; }
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out) {
     DeviceGuard dg(s->device);
     return reduce(s, what, out);
