@@ -83,13 +83,15 @@ int enqueue_steps(fvlbm_dd* d, int64_t n) {
 // records and waits), which the host makes more slowly than the device runs the
 // stage: chunks of steps are recorded once and replayed.  False: not available.
 bool chunk_ready(fvlbm_dd* d, int b) {
+    // whether a recording may stand for the next steps is asked every time: writing
+    // f ends AB2's history, and the step after it is an Euler start that no chunk holds
+    for (fvlbm_solver* s : d->part)
+        if (!solver_replayable(s) || solver_buffer(s) != b) return false;
     if (d->chunk[b]) return true;
     cudaStream_t st = (cudaStream_t)d->stream;
     if (!d->graphs_ok || !st) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
-    for (fvlbm_solver* s : d->part)
-        if (!solver_replayable(s) || solver_buffer(s) != b) return false;
     cudaGraph_t g = nullptr;
     bool ok = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
