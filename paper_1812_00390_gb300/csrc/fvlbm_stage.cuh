@@ -112,7 +112,8 @@ template <typename T> __device__ __forceinline__ void from_pairs(const Pair<T>* 
 // Slots (bit k) that some active thread of the warp uses: a polygon with
 // fewer faces than MAXF leaves its last slots empty, and when every cell of a
 // warp does (a warp of triangles in a 4-slot mesh), the warp skips them as a
-// whole.  Slots 0..2 are always used.
+// whole.  Slots 0..2 are always used.  Taken where the warp is whole: before any branch
+// on what a cell is.
 template <int MAXF>
 __device__ __forceinline__ uint32_t warp_slots(const uint32_t* d) {
     uint32_t u = 7u;
@@ -513,6 +514,7 @@ __global__ void __launch_bounds__(256) face_values_pairs_kernel(DevView v, const
     double* fv = (double*)v.fv + p;
     double gax = 0, gay = 0, gbx = 0, gby = 0;
     const bool edge = boundary_mask<MAXF>(d) != 0;
+    const uint32_t used = warp_slots<MAXF>(d);
     if (__any_sync(0xFFFFFFFFu, edge)) {
         double rho, ux, uy, qa, qb, q0;
         lanes_moments(p, *CellIO<double>::rest(fin, i), f.x, f.y, rho, ux, uy);
@@ -530,7 +532,6 @@ __global__ void __launch_bounds__(256) face_values_pairs_kernel(DevView v, const
                                     fv[(v.np * MAXF + ghost) * 4] = z;
                                 });
     }
-    const uint32_t used = warp_slots<MAXF>(d);
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
@@ -620,8 +621,10 @@ __device__ __forceinline__ void tile_faces(const uint32_t* d, const Pair<T>* f, 
 #pragma unroll
     for (int p = 0; p < 4; p++) gx[p] = gy[p] = make_pair2(T(0), T(0));
     const bool bc = boundary_mask<MAXF>(d) != 0;
-    if (!DEV && bc) boundary();
+    // before the branch: every row that phase 3 reads for a warp has to be written here,
+    // an empty slot's among them, also should the warp not come together after it
     const uint32_t used = warp_slots<MAXF>(d);
+    if (!DEV && bc) boundary();
 #pragma unroll
     for (int k = 0; k < MAXF; k++) {
         if (k >= 3 && !((used >> k) & 1u)) continue;
