@@ -286,6 +286,13 @@ class Solver:
         if use_torch_workspace:
             self._ws = torch.empty(nbytes.value, dtype=torch.uint8, device=f"cuda:{dev}")
             ws_ptr = self._ws.data_ptr()
+            # the allocator ties the block to torch's current stream: the solver's starts
+            # after what is queued there, and the block is not given away, when this
+            # object goes, before the solver's launches are done with it
+            user = stream if hasattr(stream, "cuda_stream") else (
+                torch.cuda.ExternalStream(sh, device=dev) if sh else torch.cuda.default_stream(dev))
+            user.wait_stream(torch.cuda.current_stream(dev))
+            self._ws.record_stream(user)
         else:
             self._ws = None
             ws_ptr = None
