@@ -247,7 +247,7 @@ int fvlbm_init(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_par
  * With params.kernel = 0, small meshes (FP32 and 16-bit up to about 110,000
  * cells of up to four faces, FP64 up to about 5,800) run up to 2048 stages in one
  * cooperative launch whose thread blocks exchange halo cells; the results are
- * those of the stage kernels, bit for bit in FP32 and 16-bit precision.  Such launches of different solvers take
+ * those of the stage kernels, bit for bit in every precision.  Such launches of different solvers take
  * turns on the GPU.  Every wait in them is bounded; one that runs out is reported by
  * the next synchronising call as FVLBM_ERR_TIMEOUT.  In a stream capture by the
  * caller the stages are recorded one by one.
@@ -333,6 +333,14 @@ int fvlbm_host_transfer(fvlbm_solver* s, int32_t mode, int32_t* direct);
  * 1 for the two-kernel stage, else the fused stage's threads per CTA.
  * kernel: host, written.  Errors: FVLBM_ERR_ARG. */
 int fvlbm_stage_kernel(const fvlbm_solver* s, int32_t* kernel);
+
+/* The resident loop of this solver (see fvlbm_step), host, written, each or NULL:
+ *   tile      most tile and 1-ring cells of one of its tiles; 0: fvlbm_step runs
+ *             the stage kernels only
+ *   tiles     its tiles, one CTA each
+ *   launches  its launches so far (a call that ran the stage kernels adds none)
+ * Errors: FVLBM_ERR_ARG. */
+int fvlbm_resident_info(const fvlbm_solver* s, int32_t* tile, int32_t* tiles, int64_t* launches);
 
 /* Wait for the solver's stream; reports FVLBM_ERR_DIVERGED if flagged. */
 int fvlbm_sync(fvlbm_solver* s);

@@ -58,6 +58,7 @@ struct fvlbm_solver {
     bool resident = false, alone = true;
     ResView res{};
     uint32_t epoch = 0;
+    int64_t res_launches = 0;
 };
 
 static constexpr int64_t GRAPH_CHUNK = 32;
@@ -1190,6 +1191,7 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
             if ((n - m) * ns == 1) m--;
             int rc = launch_resident(s->v, s->res, s->prec, s->stream, s->scheme, m * ns, s->epoch, s->ab2_started);
             if (rc) return rc;
+            s->res_launches++;
             s->epoch += (uint32_t)(m * ns);
             s->ab2_started = s->scheme == FVLBM_AB2;
             n -= m;
@@ -1360,6 +1362,15 @@ extern "C" int fvlbm_stage_kernel(const fvlbm_solver* s, int32_t* kernel) {
     clear_error();
     if (!s || !kernel) return fail(FVLBM_ERR_ARG, "fvlbm_stage_kernel: null argument");
     *kernel = s->v.strategy == STRATEGY_TILE ? s->v.tile : 1;
+    return FVLBM_OK;
+}
+
+extern "C" int fvlbm_resident_info(const fvlbm_solver* s, int32_t* tile, int32_t* tiles, int64_t* launches) {
+    clear_error();
+    if (!s) return fail(FVLBM_ERR_ARG, "fvlbm_resident_info: null solver");
+    if (tile) *tile = s->resident ? s->res.tile : 0;
+    if (tiles) *tiles = s->resident ? s->res.n_tiles : 0;
+    if (launches) *launches = s->res_launches;
     return FVLBM_OK;
 }
 
