@@ -211,7 +211,8 @@ typedef struct fvlbm_plan_info_s {
     int32_t stage_kernel;        /* 1: two kernels per stage; else the fused stage's threads per CTA */
     int32_t slots;               /* face slots per cell in the packed arrays (4 or 8) */
     int64_t n_tiles;             /* fused stage: tiles (0 for two kernels) */
-    int64_t short_tiles;         /* tiles cut below the CTA size by the shared-memory capacity */
+    int64_t short_tiles;         /* tiles cut below the length asked for (the CTA size; the resident
+                                    loop: the SM's share of the cells) by the capacity */
     int32_t max_local_cells;     /* largest tile: its cells, 1-ring and 2-ring */
     int32_t max_faces;           /* largest tile: faces of its cells */
     double mean_tile_cells;      /* cells per tile */
@@ -224,6 +225,15 @@ typedef struct fvlbm_plan_info_s {
 } fvlbm_plan_info_t;
 int fvlbm_plan_info(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
                     fvlbm_plan_info_t* info);
+
+/*
+ * The same of the resident loop's plan (see fvlbm_step): stage_kernel is its tile
+ * size, 0 when fvlbm_step runs the stage kernels only.  Checked besides: who reads
+ * from a tile is read by it, on which its exchange relies.  `violations` counts the
+ * failed checks of both plans in either call.
+ */
+int fvlbm_resident_plan(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
+                        fvlbm_plan_info_t* info);
 
 /*
  * Create a solver on params[0].device and set f = f^eq(rho0, u0) (Step 0).
@@ -245,7 +255,8 @@ int fvlbm_init(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_par
  * asynchronously on the solver's stream.  A non-finite value raises a device
  * flag that the next synchronising call reports as FVLBM_ERR_DIVERGED.
  * With params.kernel = 0, small meshes (FP32 and 16-bit up to about 110,000
- * cells of up to four faces, FP64 up to about 5,800) run up to 2048 stages in one
+ * triangles, 96,000 quads or 53,000 polygons, FP64 up to about 5,700 triangles or
+ * 4,100 other cells; fvlbm_resident_plan says of each) run up to 2048 stages in one
  * cooperative launch whose thread blocks exchange halo cells; the results are
  * those of the stage kernels, bit for bit in every precision.  Such launches of different solvers take
  * turns on the GPU.  Every wait in them is bounded; one that runs out is reported by

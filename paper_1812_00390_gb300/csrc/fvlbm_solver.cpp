@@ -105,7 +105,7 @@ struct TilePlan {
     std::vector<uint32_t> r1link;   // [1-ring entries][maxf] link words
     int64_t n_r1 = 0;               // 1-ring entries
     int32_t max_local = 0, max_faces = 0;
-    int64_t short_tiles = 0;        // tiles cut below `tile` cells by the capacity
+    int64_t short_tiles = 0;        // tiles cut below the length asked for by the capacity
     int64_t sum_len = 0, sum_ring1 = 0, sum_local = 0;   // over the tiles
     // filled when the plan is verified (fvlbm_plan_info): modelled
     // shared-memory wavefronts of the warp accesses, and failed invariants
@@ -418,7 +418,7 @@ int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify, int 
             len = len > BLK ? (len - 1) / BLK * BLK : len / 2;
         }
         guess = std::min(max_len, (len + BLK) / BLK * BLK);
-        if (len < std::min<int64_t>(tile, n_own - c0)) P.short_tiles++;
+        if (len < std::min<int64_t>(max_len, n_own - c0)) P.short_tiles++;
         P.sum_len += len;
         P.sum_ring1 += (int64_t)W.r1.size();
         P.sum_local += nl;
@@ -486,6 +486,25 @@ constexpr int64_t PLANE_ALIGN = 1024;  // cell arrays hold whole blocks and whol
 
 int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
+// What the resident loop's exchange relies on besides: who reads from a tile is read
+// by it (so that a tile that has its neighbours' cells of a stage knows that they
+// have read its older ones).
+void verify_exchange(TilePlan& P) {
+    int64_t n = 0;
+    for (const TileRec& R : P.rec) n = std::max<int64_t>(n, R.c0 + R.nt);
+    std::vector<int32_t> owner((size_t)n);
+    for (size_t t = 0; t < P.rec.size(); t++)
+        std::fill_n(owner.begin() + P.rec[t].c0, P.rec[t].nt, (int32_t)t);
+    std::vector<std::pair<int32_t, int32_t>> reads;
+    for (size_t t = 0; t < P.rec.size(); t++)
+        for (int32_t h = 0; h < P.rec[t].nh; h++) reads.emplace_back((int32_t)t, owner[P.halo[P.rec[t].h0 + h]]);
+    std::sort(reads.begin(), reads.end());
+    reads.erase(std::unique(reads.begin(), reads.end()), reads.end());
+    for (const auto& r : reads)
+        if (!std::binary_search(reads.begin(), reads.end(), std::make_pair(r.second, r.first)) && P.violations++ == 0)
+            P.first_violation = "a tile reads from one that does not read from it";
+}
+
 // The resident stage loop's plan (fvlbm_resident.cuh), if the solver is small
 // enough: one tile per SM, as long as the SM's share of the cells but not below
 // a length at which the halo outgrows the tile; in FP32 also two to four of the
@@ -506,7 +525,10 @@ int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P, bool
             for (int64_t len : {std::min<int64_t>(share, tile), (int64_t)tile}) {
                 if (len == tile && ctas < std::min(3, resident_ctas(rsize, maxf))) continue;
                 int rc = make_tiles(M, maxf, tile, P, verify, (int)len);
-                if (rc == FVLBM_OK && P.n_tiles <= (int64_t)ctas * sms) return FVLBM_OK;
+                if (rc == FVLBM_OK && P.n_tiles <= (int64_t)ctas * sms) {
+                    if (verify) verify_exchange(P);
+                    return FVLBM_OK;
+                }
                 P = TilePlan{};
                 if (rc && rc != FVLBM_ERR_UNSUPPORTED) return rc;
             }
@@ -759,10 +781,12 @@ extern "C" int fvlbm_workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params*
     return FVLBM_OK;
 }
 
-extern "C" int fvlbm_plan_info(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
-                               fvlbm_plan_info_t* info) {
+// The plans fvlbm_init would build, checked: of the stage kernels (resident: of
+// the resident loop, stage_kernel = 0 when there is none).
+static int plan_report(const char* what, const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
+                       fvlbm_plan_info_t* info, bool resident) {
     clear_error();
-    if (!mesh || !info) return fail(FVLBM_ERR_ARG, "fvlbm_plan_info: null argument");
+    if (!mesh || !info) return fail(FVLBM_ERR_ARG, "%s: null argument", what);
     int rc = check_params(mesh->m, params, n_params);
     if (rc) return rc;
     Layout L;
@@ -770,30 +794,42 @@ extern "C" int fvlbm_plan_info(const fvlbm_mesh* mesh, const fvlbm_params* param
         rc = make_layout(mesh->m, params[0].precision, params[0].scheme, params[0].kernel, L,
                          device_sms(params[0].device), true);
     } catch (const std::bad_alloc&) {
-        return fail(FVLBM_ERR_OOM, "fvlbm_plan_info: out of host memory");
+        return fail(FVLBM_ERR_OOM, "%s: out of host memory", what);
     }
     if (rc) return rc;
-    const TilePlan& P = L.tp;
+    const bool tiled = resident ? L.resident : L.strategy == STRATEGY_TILE;
+    const TilePlan& P = resident && L.resident ? L.res_plan() : L.tp;
     fvlbm_plan_info_t o{};
-    const bool tiled = L.strategy == STRATEGY_TILE;
-    o.stage_kernel = tiled ? P.tile : 1;
+    o.stage_kernel = tiled ? P.tile : resident ? 0 : 1;
     o.slots = L.maxf;
-    o.n_tiles = tiled ? P.n_tiles : 0;
-    o.short_tiles = P.short_tiles;
-    o.max_local_cells = P.max_local;
-    o.max_faces = P.max_faces;
     if (tiled && P.n_tiles > 0) {
+        o.n_tiles = P.n_tiles;
+        o.short_tiles = P.short_tiles;
+        o.max_local_cells = P.max_local;
+        o.max_faces = P.max_faces;
         o.mean_tile_cells = (double)P.sum_len / P.n_tiles;
         o.mean_ring1_cells = (double)P.sum_ring1 / P.n_tiles;
         o.mean_local_cells = (double)P.sum_local / P.n_tiles;
         o.face_table_waves = P.face_groups > 0 ? P.face_waves / P.face_groups : 0;
         o.gather_waves = P.gather_groups > 0 ? P.gather_waves / P.gather_groups : 0;
     }
-    o.violations = P.violations;
+    // every plan that the solver would run counts, whichever is reported
+    o.violations = L.tp.violations + L.rp.violations;
     *info = o;
-    if (P.violations) fail(FVLBM_OK, "%lld failed plan checks; first: %s", (long long)P.violations,
-                           P.first_violation.c_str());
+    if (o.violations)
+        fail(FVLBM_OK, "%lld failed plan checks; first: %s", (long long)o.violations,
+             (L.tp.violations ? L.tp : L.rp).first_violation.c_str());
     return FVLBM_OK;
+}
+
+extern "C" int fvlbm_plan_info(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
+                               fvlbm_plan_info_t* info) {
+    return plan_report("fvlbm_plan_info", mesh, params, n_params, info, false);
+}
+
+extern "C" int fvlbm_resident_plan(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
+                                   fvlbm_plan_info_t* info) {
+    return plan_report("fvlbm_resident_plan", mesh, params, n_params, info, true);
 }
 
 static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params, void* stream,

@@ -49,6 +49,28 @@ def test_small_meshes_run_the_resident_loop(fv, name, prec):
     s.close()
 
 
+# the largest of the loop's range: four tiles per SM (two of polygons)
+LARGEST = {"quads_96k": lambda: mg.cavity(310, 20.0), "triangles_110k": lambda: mg.periodic_tri(235, 235, lx=235.0, ly=235.0),
+           "polygons_53k": lambda: mg.bricks(460, 230)}
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("name,scheme", [("quads_96k", "rk2"), ("quads_96k", "ab2"), ("triangles_110k", "rk4"),
+                                         ("polygons_53k", "rk2")])
+def test_largest_resident_meshes_equal_stage_kernels(fv, name, scheme, prec):
+    m = LARGEST[name]()
+    h, f0, out = fv.Mesh(m), start(m.n_cell, 49), []
+    for kernel in (0, 128):
+        s = fv.Solver(h, fv.make_params(0.1, cfl=0.3, scheme=scheme, precision=prec, u_max=0.1, kernel=kernel))
+        s.set_f(f0)
+        for n in (2, 21):
+            s.step(n)
+        assert s.resident_info()["launches"] == (0 if kernel else 2)
+        out.append(s.get_f())
+        s.close()
+    assert np.isfinite(out[0]).all() and np.array_equal(*out)
+
+
 FP64_MESHES = dict({k: MESHES[k] for k in ("two_cells", "two_cells_periodic", "channel_1_wide", "couette", "symmetry",
                                            "pressure_outlet", "bricks", "periodic")},
                    cavity_5k=lambda: mg.cavity(75, 20.0),
