@@ -259,8 +259,9 @@ int fvlbm_init(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_par
  * 4,100 other cells; fvlbm_resident_plan says of each) run up to 2048 stages in one
  * cooperative launch whose thread blocks exchange halo cells; the results are
  * those of the stage kernels, bit for bit in every precision.  Such launches of different solvers take
- * turns on the GPU.  Every wait in them is bounded; one that runs out is reported by
- * the next synchronising call as FVLBM_ERR_TIMEOUT.  In a stream capture by the
+ * turns on the GPU.  Every wait in them is bounded (fvlbm_resident_polls); one that runs out
+ * is reported by every synchronising call as FVLBM_ERR_TIMEOUT until fvlbm_set_f writes a
+ * new state.  In a stream capture by the
  * caller the stages are recorded one by one.
  * Errors: FVLBM_ERR_ARG, _CUDA.
  */
@@ -317,6 +318,12 @@ int fvlbm_mass_noalloc(fvlbm_solver* s, double* mass);
  * Writing also restarts AB2 history.  Synchronise. */
 int fvlbm_get_f(fvlbm_solver* s, double* f);
 int fvlbm_set_f(fvlbm_solver* s, const double* f);
+
+/* Most polls after the first (of about half a microsecond each) that one wait of the
+ * solver's resident launches makes from here on; 2^22 unless set.  A wait is for the
+ * halo of the stage before, some microseconds: what runs out is a launch that the GPU
+ * holds up, or a limit of a few polls.  Errors: FVLBM_ERR_ARG. */
+int fvlbm_resident_polls(fvlbm_solver* s, int32_t polls);
 
 /*
  * How fvlbm_set_f reads the caller's buffer.

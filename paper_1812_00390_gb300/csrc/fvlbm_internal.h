@@ -217,6 +217,10 @@ struct DevView {
     int64_t n_r1;
 };
 
+// Most polls of a wait of the resident loop, of about half a microsecond: seconds,
+// against microseconds of waiting.
+constexpr int32_t RES_POLLS = 1 << 22;
+
 // The resident plan of a small solver (fvlbm_resident.cuh): every tile has a
 // CTA of its own on the GPU for as many time steps as one launch advances.
 struct ResView {
@@ -229,6 +233,7 @@ struct ResView {
     int64_t n_r1 = 0;
     uint4* xchg = nullptr;             // [2][units][np] (FP64 [2][np][units]) exchange buffer: units of three
                                        // words and a tag
+    int32_t polls = RES_POLLS;         // most polls of one wait
 };
 // 16-byte units of one cell in the exchange buffer (FP64: two per direction pair)
 constexpr int resident_units(size_t state_bytes) { return state_bytes == 72 ? 8 : (int)(state_bytes / 12); }

@@ -22,8 +22,8 @@
 // from a tile is read by it).
 //
 // All CTAs are on the GPU at once (a cooperative launch; the set-up checks that
-// they fit), so every wait ends; should one not, it gives up after a bounded
-// number of polls, sets flag[1] and the kernel returns.
+// they fit), so every wait ends; should one not, it gives up after r.polls polls,
+// sets flag[1] and the kernel returns, as do the launches queued behind it.
 //
 // The first stage of a launch reads its halo from the state buffer, and the
 // last one writes the state buffer instead of the exchange buffer: a launch has
@@ -40,8 +40,6 @@
 
 namespace fvlbm {
 
-constexpr int RES_POLLS = 1 << 22;   // of about half a microsecond: seconds, against microseconds of waiting
-
 __device__ __forceinline__ uint4 load_unit(const uint4* p) {
     uint64_t lo, hi;
     asm volatile("{ .reg .b128 x; ld.relaxed.gpu.global.b128 x, [%2]; mov.b128 {%0, %1}, x; }"
@@ -55,8 +53,9 @@ __device__ __forceinline__ void store_unit(uint4* p, uint32_t a, uint32_t b, uin
 }
 
 // Cell `i` in one set of the exchange buffer (units `stride` apart): W words of data in W / 3 units.
-template <int W> __device__ __forceinline__ bool take_cell(const uint4* p, int64_t stride, uint32_t tag, uint32_t* w) {
-    for (int it = 0; it < RES_POLLS; it++) {
+template <int W>
+__device__ __forceinline__ bool take_cell(const uint4* p, int64_t stride, uint32_t tag, int polls, uint32_t* w) {
+    for (int it = 0;; it++) {   // the first poll is free of the limit's test
         bool ok = true;
 #pragma unroll
         for (int u = 0; u < W / 3; u++) {
@@ -67,8 +66,8 @@ template <int W> __device__ __forceinline__ bool take_cell(const uint4* p, int64
             ok &= x.w == tag;
         }
         if (ok) return true;
+        if (it >= polls) return false;
     }
-    return false;
 }
 template <int W> __device__ __forceinline__ void give_cell(uint4* p, int64_t stride, uint32_t tag, const uint32_t* w) {
 #pragma unroll
@@ -139,6 +138,7 @@ __global__ void __launch_bounds__(TILE, CTAS)
     V* sgeo = tab + ROWS;         // [3 GU][TILE]  geometry of the gradient cells
     V* sbase = sgeo + (SHARED ? 3 * GU * TILE : 0);   // [2][TILE]  state the step began with
     float* sbase0 = (float*)(sbase + 2 * TILE);   // [TILE]
+    if (__syncthreads_or(*(volatile int32_t*)(v.flag + 1))) return;   // a launch before gave up
     const TileRec R = r.tiles[blockIdx.x];
     const int l = threadIdx.x, nt = R.nt, n2 = R.nt + R.n1, n_ring2 = R.nh - R.n1, inst = R.inst;
     const bool mine = l < nt, ring1 = !mine && l < n2;
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(TILE, CTAS)
         } else if (ring1) {
             if (s > 0) {
                 uint32_t w[W];
-                late = !take_cell<W>(from + gl, v.np, tag, w);
+                late = !take_cell<W>(from + gl, v.np, tag, r.polls, w);
                 Wire<S>::unpack(P, w, f);
             }
             to_shared(l, f);
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(TILE, CTAS)
             T q[FVLBM_Q];
             if (s > 0) {
                 uint32_t w[W];
-                late |= !take_cell<W>(from + i, v.np, tag, w);
+                late |= !take_cell<W>(from + i, v.np, tag, r.polls, w);
                 Wire<S>::unpack(Pi, w, q);
             } else {
                 CellIO<S>::template load<T, DEV>(v.fa, i, Pi, q);
@@ -307,6 +307,7 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2* fs = (double2*)smem_raw;   // [LS][4]    pairs of the local cells
     double* tab = (double*)(fs + 4 * LS);   // [ROWS][4]  face table
+    if (__syncthreads_or(*(volatile int32_t*)(v.flag + 1))) return;   // a launch before gave up
     const TileRec R = r.tiles[blockIdx.x];
     const int x = threadIdx.x >> 2, p = threadIdx.x & 3, nt = R.nt, n2 = R.nt + R.n1, n_ring2 = R.nh - R.n1,
               inst = R.inst;
@@ -382,7 +383,7 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
         // take the lane's pair (and f_0) of cell i
         auto take = [&](uint32_t i, double& q0, double& qa, double& qb) {
             uint32_t u[6];
-            const bool ok = take_cell<6>(from + ((size_t)i * 8 + p * 2), 1, tag, u);
+            const bool ok = take_cell<6>(from + ((size_t)i * 8 + p * 2), 1, tag, r.polls, u);
             qa = __hiloint2double((int)u[1], (int)u[0]);
             qb = __hiloint2double((int)u[4], (int)u[3]);
             q0 = __hiloint2double((int)u[5], (int)u[2]);

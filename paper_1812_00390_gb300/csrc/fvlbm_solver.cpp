@@ -1388,6 +1388,8 @@ extern "C" int fvlbm_set_f(fvlbm_solver* s, const double* f) {
         rc = launch_set_f_ordered(s->v, s->prec, s->stream, s->v.conv);
     }
     if (rc) return rc;
+    // a wait that ran out has left the state in the middle of a call: this one replaces it
+    CK(cudaMemsetAsync(s->v.flag + 1, 0, sizeof(int32_t), s->stream), "clear flag");
     s->ab2_started = false;
     if (s->scheme == FVLBM_AB2) s->direct_steps = 0;   // the next step is an Euler start, launched directly
     CK(cudaStreamSynchronize(s->stream), "synchronise");
@@ -1407,6 +1409,13 @@ extern "C" int fvlbm_resident_info(const fvlbm_solver* s, int32_t* tile, int32_t
     if (tile) *tile = s->resident ? s->res.tile : 0;
     if (tiles) *tiles = s->resident ? s->res.n_tiles : 0;
     if (launches) *launches = s->res_launches;
+    return FVLBM_OK;
+}
+
+extern "C" int fvlbm_resident_polls(fvlbm_solver* s, int32_t polls) {
+    clear_error();
+    if (!s || polls < 0) return fail(FVLBM_ERR_ARG, "fvlbm_resident_polls: bad arguments");
+    s->res.polls = polls;
     return FVLBM_OK;
 }
 

@@ -85,7 +85,7 @@ class ServerStatsT(C.Structure):
 #: every symbol include/fvlbm.h declares
 EXPORTS = ["fvlbm_mesh_create", "fvlbm_mesh_concat", "fvlbm_mesh_destroy", "fvlbm_mesh_info",
            "fvlbm_suggest_dt", "fvlbm_workspace_bytes", "fvlbm_plan_info", "fvlbm_resident_plan", "fvlbm_init", "fvlbm_step", "fvlbm_macros",
-           "fvlbm_residual", "fvlbm_mass", "fvlbm_mass_noalloc", "fvlbm_get_f", "fvlbm_set_f", "fvlbm_host_transfer", "fvlbm_stage_kernel", "fvlbm_resident_info", "fvlbm_sync",
+           "fvlbm_residual", "fvlbm_mass", "fvlbm_mass_noalloc", "fvlbm_get_f", "fvlbm_set_f", "fvlbm_host_transfer", "fvlbm_stage_kernel", "fvlbm_resident_info", "fvlbm_resident_polls", "fvlbm_sync",
            "fvlbm_get_dt", "fvlbm_profile", "fvlbm_autotune", "fvlbm_fma_peak", "fvlbm_launches_per_step", "fvlbm_solver_destroy",
            "fvlbm_server_create", "fvlbm_server_submit", "fvlbm_server_poll", "fvlbm_server_request",
            "fvlbm_server_stats", "fvlbm_server_destroy", "fvlbm_mesh_partition", "fvlbm_partition_destroy",
@@ -132,6 +132,7 @@ def _load():
         "fvlbm_host_transfer": [P, C.c_int32, i32p],
         "fvlbm_stage_kernel": [P, i32p],
         "fvlbm_resident_info": [P, i32p, i32p, i64p],
+        "fvlbm_resident_polls": [P, C.c_int32],
         "fvlbm_solver_destroy": [P],
         "fvlbm_server_create": [C.POINTER(ServerConfigT), PP],
         "fvlbm_server_submit": [P, P, C.POINTER(ParamsT), C.c_int32, i64p],
@@ -360,6 +361,10 @@ class Solver:
         t, n, k = C.c_int32(), C.c_int32(), C.c_int64()
         _check(lib.fvlbm_resident_info(self._h, C.byref(t), C.byref(n), C.byref(k)))
         return {"tile": t.value, "tiles": n.value, "launches": k.value}
+
+    def resident_polls(self, polls: int):
+        """Most polls of one wait of the resident loop from here on."""
+        _check(lib.fvlbm_resident_polls(self._h, int(polls)))
 
     def host_transfer(self, mode: str = "auto") -> bool:
         """How set_f reads the caller's buffer: "auto" (the kernel reads it
