@@ -261,8 +261,9 @@ int fvlbm_init(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_par
  * those of the stage kernels, bit for bit in every precision.  Such launches of different solvers take
  * turns on the GPU.  Every wait in them is bounded (fvlbm_resident_polls); one that runs out
  * is reported by every synchronising call as FVLBM_ERR_TIMEOUT until fvlbm_set_f writes a
- * new state.  In a stream capture by the
- * caller the stages are recorded one by one.
+ * new state.  On a stream whose part of the GPU does
+ * not hold all of a mesh's blocks, and in a stream capture by the caller, the stages are
+ * launched or recorded one by one.
  * Errors: FVLBM_ERR_ARG, _CUDA.
  */
 int fvlbm_step(fvlbm_solver* s, int64_t n);

@@ -278,7 +278,9 @@ int stage_fp16(const DevView& v, void* stream, const void* fin, const void* fbas
 int stage_bf16(const DevView& v, void* stream, const void* fin, const void* fbase, void* fout, double beta, int mode,
                void* const* ev);
 // Resident stage loop: `stages` >= 2 stages of the scheme on state fa, with
-// tags epoch + 1 .. epoch + stages - 1, none of them used before.  resident_fits: whether every tile's CTA is on the GPU at once.
+// tags epoch + 1 .. epoch + stages - 1, none of them used before; FVLBM_ERR_UNSUPPORTED:
+// not launched, the stream's part of the GPU does not hold every tile's CTA.
+// resident_fits: whether the whole GPU does.
 int launch_resident(const DevView& v, const ResView& r, int prec, void* stream, int scheme, int64_t stages,
                     uint32_t epoch, bool ab2_started);
 bool resident_fits(const DevView& v, const ResView& r, int prec, int scheme);

@@ -530,6 +530,12 @@ static int resident_launch(const void* kern, int threads, size_t smem, const Dev
     ResView rr = r;
     void* args[] = {&vv, &rr, &ns, &stages, &epoch, &started};
     cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)r.n_tiles), dim3((unsigned)threads), args, smem, st);
+    // refused as a whole: the tiles do not all fit where the stream's launches run
+    // (fewer SMs than the device has), or cooperative launches are not to be had there
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return fail(FVLBM_ERR_UNSUPPORTED, "resident stage loop: %s", cudaGetErrorString(e));
+    }
     if (e != cudaSuccess) return fail(FVLBM_ERR_CUDA, "resident stage loop: %s", cudaGetErrorString(e));
     return FVLBM_OK;
 }

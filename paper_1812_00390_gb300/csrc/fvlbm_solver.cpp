@@ -1226,6 +1226,11 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
             int64_t m = std::min(n, RESIDENT_CHUNK / ns);
             if ((n - m) * ns == 1) m--;
             int rc = launch_resident(s->v, s->res, s->prec, s->stream, s->scheme, m * ns, s->epoch, s->ab2_started);
+            if (rc == FVLBM_ERR_UNSUPPORTED) {   // from here on the stage kernels, which need no such room
+                clear_error();
+                s->resident = false;
+                break;
+            }
             if (rc) return rc;
             s->res_launches++;
             s->epoch += (uint32_t)(m * ns);
