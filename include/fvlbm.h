@@ -258,12 +258,14 @@ int fvlbm_init(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_par
  * triangles, 96,000 quads or 53,000 polygons, FP64 up to about 5,700 triangles or
  * 4,100 other cells; fvlbm_resident_plan says of each) run up to 2048 stages in one
  * cooperative launch whose thread blocks exchange halo cells; the results are
- * those of the stage kernels, bit for bit in every precision.  Such launches of different solvers take
- * turns on the GPU.  Every wait in them is bounded (fvlbm_resident_polls); one that runs out
- * is reported by every synchronising call as FVLBM_ERR_TIMEOUT until fvlbm_set_f writes a
- * new state.  On a stream whose part of the GPU does
- * not hold all of a mesh's blocks, and in a stream capture by the caller, the stages are
- * launched or recorded one by one.
+ * those of the stage kernels, bit for bit in every precision.  Such launches of
+ * solvers on different streams share the GPU as far as their blocks fit on it and take
+ * turns beyond; a call of 32 steps or more that finds other such solvers at work, so
+ * many that turns are estimated to take longer, runs its stages by themselves, which
+ * overlap.  So does a stream whose part of the GPU does not hold all of a mesh's
+ * blocks, and a stream capture by the caller.  Every wait in a launch is bounded
+ * (fvlbm_resident_polls); one that runs out is reported by every synchronising call as
+ * FVLBM_ERR_TIMEOUT until fvlbm_set_f writes a new state.
  * Errors: FVLBM_ERR_ARG, _CUDA.
  */
 int fvlbm_step(fvlbm_solver* s, int64_t n);
@@ -418,8 +420,8 @@ void fvlbm_solver_destroy(fvlbm_solver* s);
  * order; every fvlbm_server_poll round
  *   1. advances every active request by check_interval time steps (the
  *      residual interval of Sec. 3.2), each request on one of n_streams
- *      streams, so that the kernels of different requests overlap (requests that
- *      together are at most 110,000 cells take turns in resident launches);
+ *      streams: in resident launches, or by stage kernels that overlap with those of the
+ *      other requests, whichever is estimated to be faster for the requests at hand;
  *   2. admits queued requests, first fit in arrival order, while fewer than
  *      max_active are active and the device arena (arena_bytes, allocated once
  *      at creation) has a free block for the request's workspace;

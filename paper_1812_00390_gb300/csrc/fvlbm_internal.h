@@ -280,10 +280,10 @@ int stage_bf16(const DevView& v, void* stream, const void* fin, const void* fbas
 // Resident stage loop: `stages` >= 2 stages of the scheme on state fa, with
 // tags epoch + 1 .. epoch + stages - 1, none of them used before; FVLBM_ERR_UNSUPPORTED:
 // not launched, the stream's part of the GPU does not hold every tile's CTA.
-// resident_fits: whether the whole GPU does.
+// resident_max_ctas: how many the whole GPU holds.
 int launch_resident(const DevView& v, const ResView& r, int prec, void* stream, int scheme, int64_t stages,
                     uint32_t epoch, bool ab2_started);
-bool resident_fits(const DevView& v, const ResView& r, int prec, int scheme);
+int resident_max_ctas(const DevView& v, const ResView& r, int prec, int scheme);
 #define FVLBM_RESIDENT_DECL(name)                                                                             \
     int name(const DevView& v, const ResView& r, void* stream, int scheme, int64_t stages, uint32_t epoch,    \
              bool ab2_started, int* max_ctas)
@@ -317,8 +317,23 @@ int solver_stage(fvlbm_solver* s, int k, void** out);
 bool solver_replayable(const fvlbm_solver* s);
 int solver_buffer(const fvlbm_solver* s);
 void solver_set_buffer(fvlbm_solver* s, int b);
-// Whether the next steps may take the whole GPU (the resident loop); the results are the same.
-void solver_alone(fvlbm_solver* s, bool alone);
+// What a stage costs a solver, in microseconds on a GB300: `turn` of the whole GPU in
+// the resident loop (whose launches share the GPU as far as their tiles fit), or, by
+// stage kernels, `base` of latency, which others' overlap, and `flow` of the whole GPU.
+struct StageCost {
+    double turn = 0, base = 0, flow = 0;
+    bool resident = false;
+};
+// How much less time a stage of all of them takes in stage kernels that overlap than
+// in turns; queues: how many run side by side.
+double overlap_gain(const std::vector<StageCost>& c, int queues);
+StageCost solver_cost(const fvlbm_solver* s);
+// Microseconds that the solver's first stage kernels take besides, for their graphs (0: it has them).
+double solver_overlap_setup(const fvlbm_solver* s);
+// Where the solver's next steps run (the results are the same): as fvlbm_step finds
+// best, in the resident loop, or by stage kernels.
+enum StepPath { STEP_AUTO = 0, STEP_RESIDENT = 1, STEP_STAGES = 2 };
+void solver_path(fvlbm_solver* s, StepPath path);
 // FP64 sums of a reduction (RED_MASS: [mass, -, -]; RED_RESIDUAL: [numerator,
 // denominator, -]) per instance, 3 per instance; synchronises.
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out);

@@ -211,13 +211,13 @@ int launch_resident(const DevView& v, const ResView& r, int prec, void* stream, 
     return resident(v, r, prec, stream, scheme, stages, epoch, ab2_started, nullptr);
 }
 
-bool resident_fits(const DevView& v, const ResView& r, int prec, int scheme) {
+int resident_max_ctas(const DevView& v, const ResView& r, int prec, int scheme) {
     int ctas = 0;
     if (resident(v, r, prec, nullptr, scheme, 0, 0, false, &ctas) != FVLBM_OK) {
         clear_error();
-        return false;
+        return 0;
     }
-    return ctas >= r.n_tiles;
+    return ctas;
 }
 
 int launch_init_eq(const DevView& v, int prec, void* stream) {

@@ -215,18 +215,24 @@ extern "C" int fvlbm_server_poll(fvlbm_server* s, int32_t* n_completed) {
     // the GPU works while the host prepares new requests; the launches of
     // different requests go to different streams and overlap on the device
     std::vector<int64_t> stepping = s->active;
-    // A resident launch has the GPU to itself.  Requests that together are no more
-    // cells than one such launch takes are faster in turns (four of 256 to 39k cells:
-    // 70 ms, overlapping 85); beyond, their stage kernels overlap (16 requests per
-    // second of 20k to 150k cells: 7,400 MCUPS and p99 2.1 s, in turns 6,440 and 2.6).
-    constexpr int64_t TURNS_CELLS = 110000;
-    int64_t stepping_cells = 0;
-    for (int64_t id : stepping) stepping_cells += s->req[id].n_cell;
-    const bool turns = stepping.size() == 1 || stepping_cells <= TURNS_CELLS;
+    // Small requests run in the resident loop, whose launches take turns where they do not
+    // fit side by side, or all by stage kernels, which overlap: whichever is estimated to
+    // take less for the steps that every one has left, the graphs that overlapping needs
+    // included (ms of requests of 16k quads on 8 streams, in turns / overlapping: 6 of
+    // 20,000 steps 502 / 312, of 2,000 steps 70 / 81; 16 of 256 quads, 20,000 steps 172 / 497).
+    std::vector<StageCost> cost;
+    double stages = INFINITY, setup = 0;
+    for (int64_t id : stepping) {
+        Request& r = s->req[id];
+        cost.push_back(solver_cost(r.solver));
+        stages = std::min(stages, (double)(s->cfg.max_steps - r.steps) * solver_n_stages(r.solver));
+        if (cost.back().resident) setup += solver_overlap_setup(r.solver);
+    }
+    const bool turns = overlap_gain(cost, std::min((int)s->streams.size(), 8)) * stages <= setup;
     for (int64_t id : stepping) {
         Request& r = s->req[id];
         const int64_t n = std::min<int64_t>(s->cfg.check_interval, s->cfg.max_steps - r.steps);
-        solver_alone(r.solver, turns);
+        solver_path(r.solver, turns ? STEP_RESIDENT : STEP_STAGES);
         int rc = fvlbm_step(r.solver, n);
         if (rc) r.status = rc;
         r.steps += n;

@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include <cuda_runtime.h>
@@ -55,13 +56,23 @@ struct fvlbm_solver {
     int64_t direct_steps = 0;
     bool staged = false;   // a stage has been launched by itself (partitioned solve)
     // small solvers: steps run in the resident stage loop; exchange tags used so far
-    bool resident = false, alone = true;
+    bool resident = false;
     ResView res{};
     uint32_t epoch = 0;
     int64_t res_launches = 0;
+    StepPath path = STEP_AUTO;
+    StageCost cost;
+    // who steps beside this solver (Crowd): recorded behind its last long call, which may
+    // be in flight; number of that call; whether another solver stepped meanwhile
+    cudaEvent_t stepped = nullptr;
+    bool in_flight = false, joined = false;
+    uint64_t call = 0;
 };
 
 static constexpr int64_t GRAPH_CHUNK = 32;
+// What a solver's first stage kernels take besides: both graphs captured and instantiated,
+// while its neighbours' start (requests of 2,000 steps served both ways: 4 to 14 ms each).
+static constexpr double GRAPH_SETUP_US = 6000;
 // stages of one resident launch (a few milliseconds)
 static constexpr int64_t RESIDENT_CHUNK = 2048;
 
@@ -832,6 +843,105 @@ extern "C" int fvlbm_resident_plan(const fvlbm_mesh* mesh, const fvlbm_params* p
     return plan_report("fvlbm_resident_plan", mesh, params, n_params, info, true);
 }
 
+// What a stage costs (StageCost), from measurements of 1 to 16 solvers on streams of their
+// own, us per stage of all of them, in turns / overlapping:
+//   16k quads FP32    1: 2.0 / 4.8   2: 4.0 / 5.3   3: 6.0 / 5.6   4: 7.9 / 5.9   8: 15.8 / 7.0
+//   30k hybrid        1: 3.0 / 5.4   2: 6.0 / 5.9   3: 9.1 / 6.4   4: 12.0 / 6.6  8: 23.9 / 9.0
+//   60k hybrid        1: 3.3 / 5.8   2: 6.7 / 6.7   3: 9.9 / 7.3   4: 13.3 / 8.5
+//   12k polygons      1: 2.5 / 6.9   3: 7.3 / 8.0   4: 9.7 / 8.3   8: 19.2 / 9.6
+//   4k quads FP64     1: 7.0 / 18.6  3: 21.0 / 23.4 4: 28.0 / 25.3 8: 55.9 / 34.4
+//   2k triangles FP32 1: 1.6 / 3.9   4: 1.8 / 4.5   8: 1.9 / 4.8   16: 3.6 / 9.2 (their launches fit side by side)
+static StageCost stage_cost(const DevView& v, int prec, const ResView* r, int max_ctas) {
+    StageCost c;
+    const bool fp64 = prec == FVLBM_FP64, half = prec == FVLBM_FP16_DEV || prec == FVLBM_BF16_DEV, wide = v.maxf > 4;
+    c.base = fp64 ? 17 : wide ? 6.5 : half ? 5.4 : 4.6;
+    c.flow = v.n_cell * (fp64 ? 5.5e-4 : wide ? 3e-5 : 1.9e-5);
+    if (r) {
+        const int per_sm = (r->n_tiles + v.sms - 1) / v.sms;
+        const double t = fp64 ? 7.0 : (per_sm == 1 ? 2.0 : per_sm <= 3 ? 3.2 : 6.0) + (wide ? 0.5 : 0.0);
+        c.turn = t * (half ? 1.2 : 1.0) / (max_ctas / r->n_tiles);   // so many fit side by side
+        c.resident = true;
+    }
+    return c;
+}
+
+// The solvers of the process that have a resident loop.  Its launches are faster than
+// stage kernels for one solver, but those that do not fit on the GPU together take
+// turns, and three solvers that fill it are then slower than with stage kernels, which
+// overlap.  So a long call looks who else steps: solvers on other streams whose last
+// long call is in flight, and, when its own last one was joined by others, whoever has
+// stepped since (a program that steps several solvers in rounds and waits for all has
+// none in flight when a round begins).  The states are the same either way.
+struct Crowd {
+    std::mutex m;
+    std::vector<fvlbm_solver*> members;
+    uint64_t calls = 0;
+};
+static Crowd& crowd() {
+    static Crowd* c = new Crowd;   // outlives every solver
+    return *c;
+}
+static void crowd_join(fvlbm_solver* s) {
+    Crowd& c = crowd();
+    std::lock_guard<std::mutex> lock(c.m);
+    c.members.push_back(s);
+}
+static void crowd_leave(fvlbm_solver* s) {
+    if (!s->stepped) return;
+    Crowd& c = crowd();
+    std::lock_guard<std::mutex> lock(c.m);
+    c.members.erase(std::remove(c.members.begin(), c.members.end(), s), c.members.end());
+    cudaEventDestroy(s->stepped);
+    s->stepped = nullptr;
+}
+// Whether the solver's next long call runs in the resident loop.
+static bool crowd_turns(fvlbm_solver* s) {
+    constexpr int QUEUES = 8;   // streams that CUDA runs side by side by default
+    Crowd& c = crowd();
+    std::lock_guard<std::mutex> lock(c.m);
+    const uint64_t last = s->call;
+    const bool joined = s->joined;
+    s->call = ++c.calls;
+    s->joined = false;
+    std::vector<StageCost> cost(1, s->cost);
+    // another thread may be capturing a stream: a query of these events is none of its business
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    for (fvlbm_solver* o : c.members) {
+        if (o == s || o->device != s->device || o->stream == s->stream) continue;
+        if (o->in_flight && cudaEventQuery(o->stepped) != cudaErrorNotReady) o->in_flight = false;
+        if (o->in_flight) o->joined = true;
+        if (o->in_flight || (joined && o->call > last)) cost.push_back(o->cost);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaGetLastError();   // cudaErrorNotReady
+    return overlap_gain(cost, QUEUES) <= 0;
+}
+// The solver's long call has been enqueued.
+static void crowd_stepped(fvlbm_solver* s) {
+    std::lock_guard<std::mutex> lock(crowd().m);
+    s->in_flight = cudaEventRecord(s->stepped, s->stream) == cudaSuccess;
+    if (!s->in_flight) cudaGetLastError();
+}
+
+namespace fvlbm {
+double overlap_gain(const std::vector<StageCost>& c, int queues) {
+    double turns = 0, left_base = 0, left_flow = 0, base = 0, flow = 0;
+    for (const StageCost& x : c) {
+        base = std::max(base, x.base);
+        flow += x.flow;
+        if (x.resident) {
+            turns += x.turn;
+        } else {   // runs stage kernels in any case
+            left_base = std::max(left_base, x.base);
+            left_flow += x.flow;
+        }
+    }
+    const int n = (int)c.size(), q = std::max(1, queues);
+    return turns + left_base + left_flow - (base * ((n + q - 1) / q) + flow);
+}
+}  // namespace fvlbm
+
 static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params, void* stream,
                      void* workspace, size_t workspace_bytes, fvlbm_solver* s) {
     const Mesh& M = mesh->m;
@@ -1020,7 +1130,14 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
         r.n_r1 = L.res_plan().n_r1;
         r.xchg = (uint4*)(base + L.off_xchg);
         CK(cudaMemsetAsync(r.xchg, 0, 2 * 16 * (size_t)resident_units(state_bytes(s->prec)) * L.np, s->stream), "clear tags");
-        s->resident = resident_fits(v, r, s->prec, s->scheme);
+        const int max_ctas = resident_max_ctas(v, r, s->prec, s->scheme);
+        s->resident = max_ctas >= r.n_tiles;
+        if (s->resident) s->cost = stage_cost(v, s->prec, &r, max_ctas);
+    }
+    if (!s->resident) s->cost = stage_cost(v, s->prec, nullptr, 0);
+    if (s->resident) {
+        CK(cudaEventCreateWithFlags(&s->stepped, cudaEventDisableTiming), "event");
+        crowd_join(s);
     }
     s->pingpong = L.pingpong;
     s->buf[0] = v.fa;
@@ -1039,6 +1156,7 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
 
 extern "C" void fvlbm_solver_destroy(fvlbm_solver* s) {
     if (!s) return;
+    crowd_leave(s);
     for (int b = 0; b < 2; b++) {
         if (s->g1[b]) cudaGraphExecDestroy(s->g1[b]);
         if (s->gk[b]) cudaGraphExecDestroy(s->gk[b]);
@@ -1219,8 +1337,11 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
     bool graphs = s->graphs_ok && s->stream != nullptr && cs == cudaStreamCaptureStatusNone &&
                   s->direct_steps > 0 && (s->scheme != FVLBM_AB2 || s->ab2_started);
     // small solvers: chunks of whole steps, at least two stages each, in the
-    // resident loop (a caller's capture records the stages one by one)
-    if (s->resident && s->alone && cs == cudaStreamCaptureStatusNone) {
+    // resident loop (a caller's capture records the stages one by one).  Calls shorter
+    // than a graph's steps are bound by the host's launches, of which the loop makes fewer
+    const bool in_crowd = s->resident && s->path == STEP_AUTO && s->stream && cs == cudaStreamCaptureStatusNone && n >= GRAPH_CHUNK;
+    const bool turns = s->path == STEP_AUTO ? !in_crowd || crowd_turns(s) : s->path == STEP_RESIDENT;
+    if (s->resident && turns && cs == cudaStreamCaptureStatusNone) {
         const int ns = n_stages(s->scheme);
         while (n * ns >= 2) {
             int64_t m = std::min(n, RESIDENT_CHUNK / ns);
@@ -1266,6 +1387,7 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
         if (rc) return rc;
         n--;
     }
+    if (in_crowd) crowd_stepped(s);
     return FVLBM_OK;
 }
 
@@ -1335,7 +1457,9 @@ bool solver_replayable(const fvlbm_solver* s) {
 }
 int solver_buffer(const fvlbm_solver* s) { return s->cur; }
 void solver_set_buffer(fvlbm_solver* s, int b) { set_current(s, b); }
-void solver_alone(fvlbm_solver* s, bool alone) { s->alone = alone; }
+StageCost solver_cost(const fvlbm_solver* s) { return s->cost; }
+double solver_overlap_setup(const fvlbm_solver* s) { return s->gk[0] || s->gk[1] ? 0.0 : GRAPH_SETUP_US; }
+void solver_path(fvlbm_solver* s, StepPath path) { s->path = path; }
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out) {
     DeviceGuard dg(s->device);
     return reduce(s, what, out);
