@@ -126,11 +126,6 @@ struct TilePlan {
     std::string first_violation;
 };
 
-int64_t internal_nbr(const Mesh& M, int64_t i, int k) {
-    const Slot& S = M.slots[(size_t)M.perm[i] * MAXP + k];
-    return S.kind == SK_INTERIOR ? M.iperm[S.nb] : -1;
-}
-
 // Shared-memory capacity of the fused kernel for a tile size (TileDims).
 bool tile_dims(int tile, int maxf, int rsize, int& ls, int& ghosts, size_t& bytes) {
 #define FVLBM_TD(T_)                                                                                         \
@@ -204,13 +199,45 @@ uint32_t word_pairs(uint32_t w) { return (w >> LINK_PAIR_SHIFT) & 0xFu; }
 uint32_t word_kind(uint32_t w) { return (w >> LINK_KIND_SHIFT) & 7u; }
 uint32_t word_row(uint32_t w) { return w >> LINK_ROW_SHIFT; }
 
+// What the planner asks of a mesh, by internal cell number: the mesh's own slots are
+// some kilobyte per cell, which a plan goes over several times and a solver may have
+// two plans and tries more (host time to set up a solver of 78k quads 53 ms with the
+// slots, 25 with this).
+struct Adjacency {
+    int maxf = 0;
+    std::vector<uint8_t> nf;       // [n_cell] faces
+    std::vector<int32_t> nbr;      // [n_cell][maxf] neighbour, -1 at a boundary or an unused slot
+    std::vector<uint32_t> word;    // [n_cell][maxf] pairs and kind where a link word has them, the
+                                   // face's slot in the neighbour in place of the row
+    Adjacency() = default;
+    Adjacency(const Mesh& M, int maxf_) : maxf(maxf_) {
+        const int64_t n = M.n_cell;
+        nf.resize((size_t)n);
+        nbr.assign((size_t)n * maxf, -1);
+        word.assign((size_t)n * maxf, link_word(0, 0, LK_NONE, 0));
+        for (int64_t c = 0; c < n; c++) {   // in the slots' own order
+            const int64_t i = M.iperm[c];
+            nf[i] = (uint8_t)M.nf[c];
+            for (int k = 0; k < M.nf[c]; k++) {
+                const Slot& S = M.slots[(size_t)c * MAXP + k];
+                const size_t w = (size_t)i * maxf + k;
+                const bool inner = S.kind == SK_INTERIOR;
+                if (inner) nbr[w] = (int32_t)M.iperm[S.nb];
+                word[w] = link_word(0, pair_bits(M, i, k), link_kind(M, S), inner ? (uint32_t)S.nb_slot : 0u);
+            }
+        }
+    }
+    int32_t at(int64_t i, int k) const { return nbr[(size_t)i * maxf + k]; }
+};
+
 // Link words of the tile [c0, c0 + len): local numbering tile cells, 1-ring,
 // 2-ring.  False when it exceeds ls local cells or `ghosts` boundary faces, or
 // when tile and 1-ring together exceed the CTA's `threads` (the kernel gives
 // every thread at most one gradient to compute).
-bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls, int ghosts, TileScratch& W,
+bool try_tile(const Adjacency& A, int64_t c0, int len, int threads, int ls, int ghosts, TileScratch& W,
               int& n_local, int& n_faces) {
     const int64_t g = ++W.gen;
+    const int maxf = A.maxf;
     int nl = 0;
     for (int64_t i = c0; i < c0 + len; i++) {
         W.stamp[i] = g;
@@ -219,8 +246,8 @@ bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls,
     W.r1.clear();
     W.r2.clear();
     for (int64_t i = c0; i < c0 + len; i++)
-        for (int k = 0; k < M.nf[M.perm[i]]; k++) {
-            const int64_t j = internal_nbr(M, i, k);
+        for (int k = 0; k < A.nf[i]; k++) {
+            const int64_t j = A.at(i, k);
             if (j >= 0 && W.stamp[j] != g) {
                 W.stamp[j] = g;
                 W.loc[j] = nl++;
@@ -230,8 +257,8 @@ bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls,
     const int n1 = (int)W.r1.size();
     if (nl > ls || len + n1 > threads) return false;
     for (int64_t j : W.r1)
-        for (int k = 0; k < M.nf[M.perm[j]]; k++) {
-            const int64_t q = internal_nbr(M, j, k);
+        for (int k = 0; k < A.nf[j]; k++) {
+            const int64_t q = A.at(j, k);
             if (q >= 0 && W.stamp[q] != g) {
                 W.stamp[q] = g;
                 W.loc[q] = nl++;
@@ -250,37 +277,37 @@ bool try_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int ls,
     W.r_link.resize((size_t)n1 * maxf);
     int n_ghost = 0, n_slots = 0, inner = 0;
     for (int li = 0; li < len; li++) {
-        const int64_t c = M.perm[c0 + li];
+        const int64_t i = c0 + li;
         for (int k = 0; k < maxf; k++) {
             uint32_t& w = W.t_link[(size_t)li * maxf + k];
-            if (k >= M.nf[c]) {
+            if (k >= A.nf[i]) {
                 w = link_word((uint32_t)li, 0, LK_NONE, 0);   // row 0: finite, read with weight zero
                 continue;
             }
-            const Slot& S = M.slots[(size_t)c * MAXP + k];
+            const uint32_t a = A.word[(size_t)i * maxf + k];
+            const int32_t j = A.at(i, k);
             n_slots++;
-            if (S.kind == SK_INTERIOR) {
-                const uint32_t lj = (uint32_t)W.loc[M.iperm[S.nb]];
+            if (j >= 0) {
+                const uint32_t lj = (uint32_t)W.loc[j];
                 inner += (int)lj < len;
-                w = link_word(lj, pair_bits(M, c0 + li, k), LK_FLOW, (uint32_t)S.nb_slot * threads + lj);
+                w = link_word(lj, word_pairs(a), LK_FLOW, word_row(a) * threads + lj);
             } else {
                 if (n_ghost == ghosts) return false;
-                w = link_word((uint32_t)li, pair_bits(M, c0 + li, k), link_kind(M, S), (uint32_t)(maxf * threads + n_ghost++));
+                w = link_word((uint32_t)li, word_pairs(a), word_kind(a), (uint32_t)(maxf * threads + n_ghost++));
             }
         }
     }
     for (int e = 0; e < n1; e++) {
-        const int64_t j = W.r1[e], c = M.perm[j];
+        const int64_t i = W.r1[e];
         for (int k = 0; k < maxf; k++) {
             uint32_t& w = W.r_link[(size_t)e * maxf + k];
-            const int64_t q = k < M.nf[c] ? internal_nbr(M, j, k) : -1;
+            const uint32_t a = A.word[(size_t)i * maxf + k];
+            const int32_t q = k < A.nf[i] ? A.at(i, k) : -1;
             if (q >= 0) {
                 const uint32_t lq = (uint32_t)W.loc[q];
-                w = link_word(lq, pair_bits(M, j, k), (int)lq < len ? LK_FLOW : LK_OTHER, 0);
+                w = link_word(lq, word_pairs(a), (int)lq < len ? LK_FLOW : LK_OTHER, 0);
             } else {
-                const bool used = k < M.nf[c];
-                const uint32_t kind = used ? link_kind(M, M.slots[(size_t)c * MAXP + k]) : LK_NONE;
-                w = link_word((uint32_t)(len + e), used ? pair_bits(M, j, k) : 0, kind, 0);
+                w = link_word((uint32_t)(len + e), word_pairs(a), word_kind(a), 0);   // boundary or unused slot
             }
         }
     }
@@ -400,10 +427,13 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
         }
 }
 
-// max_len: most cells of a tile (0: as many as fit).
-int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify, int max_len = 0) {
+// max_len: most cells of a tile (0: as many as fit).  max_tiles: most tiles (0: any
+// number); FVLBM_ERR_UNSUPPORTED as soon as more are sure to be needed or, an eighth of
+// the cells along, at the mean length so far a tenth more.
+int make_tiles(const Mesh& M, const Adjacency& A, int tile, TilePlan& P, bool verify, int max_len = 0, int64_t max_tiles = 0) {
     int ls = 0, ghosts = 0;
     size_t bytes = 0;
+    const int maxf = A.maxf;
     if (!tile_dims(tile, maxf, 4, ls, ghosts, bytes)) return fail(FVLBM_ERR_ARG, "unsupported tile size %d", tile);
     const int64_t n = M.n_cell;
     P = TilePlan{};
@@ -422,7 +452,7 @@ int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify, int 
     while (c0 < n_own) {
         int len = (int)std::min<int64_t>(guess, n_own - c0);
         int nl = 0, nf = 0;
-        while (!try_tile(M, maxf, c0, len, tile, ls, ghosts, W, nl, nf)) {
+        while (!try_tile(A, c0, len, tile, ls, ghosts, W, nl, nf)) {
             if (len == 1)
                 return fail(FVLBM_ERR_UNSUPPORTED, "cell %lld: its halo exceeds the fused stage's capacity",
                             (long long)c0);
@@ -453,6 +483,10 @@ int make_tiles(const Mesh& M, int maxf, int tile, TilePlan& P, bool verify, int 
         P.r1link.insert(P.r1link.end(), W.r_link.begin(), W.r_link.end());
         P.n_r1 += R.n1;
         c0 += len;
+        const int64_t made = (int64_t)P.rec.size();
+        if (max_tiles > 0 && (made + (n_own - c0 + max_len - 1) / max_len > max_tiles ||
+                              (c0 >= n_own / 8 && (double)made * n_own > 1.1 * max_tiles * c0)))
+            return fail(FVLBM_ERR_UNSUPPORTED, "more than %lld tiles", (long long)max_tiles);
         P.max_local = std::max(P.max_local, nl);
         P.max_faces = std::max(P.max_faces, nf);
     }
@@ -523,7 +557,8 @@ void verify_exchange(TilePlan& P) {
 // was the faster way throughout (us per FP32 stage, here / streaming: 40k cells 3.1 /
 // 4.9, 68k 3.8 / 5.6, 78k 5.6 / 6.5, 90k 5.9 / 6.4; FP64 3.6k cells 6.6, streaming 10k
 // cells 17.5).
-int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P, bool verify) {
+// adjacency(): the mesh's, formed when the first plan is tried.
+template <typename Get> int make_resident(const Mesh& M, int maxf, Get adjacency, int rsize, int sms, TilePlan& P, bool verify) {
     const int64_t n = M.n_owned;
     const int most = rsize == 8 ? RES_TILE_FP64 : RES_TILE;
     P = TilePlan{};
@@ -535,13 +570,14 @@ int make_resident(const Mesh& M, int maxf, int rsize, int sms, TilePlan& P, bool
             // equal tiles; where a few are cut shorter and there are too many, as long as they fit
             for (int64_t len : {std::min<int64_t>(share, tile), (int64_t)tile}) {
                 if (len == tile && ctas < std::min(3, resident_ctas(rsize, maxf))) continue;
-                int rc = make_tiles(M, maxf, tile, P, verify, (int)len);
-                if (rc == FVLBM_OK && P.n_tiles <= (int64_t)ctas * sms) {
+                int rc = make_tiles(M, adjacency(), tile, P, verify, (int)len, (int64_t)ctas * sms);
+                if (rc == FVLBM_OK) {
                     if (verify) verify_exchange(P);
                     return FVLBM_OK;
                 }
                 P = TilePlan{};
-                if (rc && rc != FVLBM_ERR_UNSUPPORTED) return rc;
+                if (rc != FVLBM_ERR_UNSUPPORTED) return rc;
+                clear_error();
             }
         }
     }
@@ -585,11 +621,16 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         else tile = 128;
     }
     L.strategy = tile == 0 || tile == 1 ? STRATEGY_TWO_KERNEL : STRATEGY_TILE;
+    Adjacency adj;
+    auto adjacency = [&]() -> const Adjacency& {
+        if (adj.maxf == 0) adj = Adjacency(M, L.maxf);
+        return adj;
+    };
     // the resident loop: chosen with the automatic kernel only; parts of a
     // partitioned mesh exchange after every stage and never use it
     L.resident = false;
     if (kernel == 0 && M.n_owned == M.n_cell && M.n_owned > 0) {
-        int rc = make_resident(M, L.maxf, (int)R, sms, L.rp, verify);
+        int rc = make_resident(M, L.maxf, adjacency, (int)R, sms, L.rp, verify);
         if (rc) return rc;
         L.resident = L.rp.n_tiles > 0;
     }
@@ -607,7 +648,7 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         // the resident loop's tiles, where it has them of this size, serve both
         int rc = FVLBM_OK;
         if (L.resident && L.rp.tile == tile) std::swap(L.tp, L.rp);
-        else rc = make_tiles(M, L.maxf, tile, L.tp, verify);
+        else rc = make_tiles(M, adjacency(), tile, L.tp, verify);
         if (rc) return rc;
         // the fused kernel indexes its blocked arrays in 32 bits
         const uint64_t lim = (uint64_t)1 << 32;
