@@ -4,6 +4,8 @@
 
 #include <cstdint>
 #include <cstddef>
+#include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -351,8 +353,14 @@ enum ReduceWhat { RED_MASS = 0, RED_RESIDUAL = 1 };
 
 }  // namespace fvlbm
 
+namespace fvlbm {
+struct Adjacency;
+}
 struct fvlbm_mesh {
     fvlbm::Mesh m;
+    // what the planner asks of it, formed by its first plan
+    mutable std::mutex plan_mutex;
+    mutable std::shared_ptr<const fvlbm::Adjacency> adjacency;
 };
 
 namespace fvlbm {

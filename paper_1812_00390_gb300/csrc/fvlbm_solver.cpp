@@ -199,17 +199,18 @@ uint32_t word_pairs(uint32_t w) { return (w >> LINK_PAIR_SHIFT) & 0xFu; }
 uint32_t word_kind(uint32_t w) { return (w >> LINK_KIND_SHIFT) & 7u; }
 uint32_t word_row(uint32_t w) { return w >> LINK_ROW_SHIFT; }
 
+}  // namespace
+
 // What the planner asks of a mesh, by internal cell number: the mesh's own slots are
 // some kilobyte per cell, which a plan goes over several times and a solver may have
 // two plans and tries more (host time to set up a solver of 78k quads 53 ms with the
-// slots, 25 with this).
-struct Adjacency {
+// slots, 29 with this).  Kept with the mesh.
+struct fvlbm::Adjacency {
     int maxf = 0;
     std::vector<uint8_t> nf;       // [n_cell] faces
     std::vector<int32_t> nbr;      // [n_cell][maxf] neighbour, -1 at a boundary or an unused slot
     std::vector<uint32_t> word;    // [n_cell][maxf] pairs and kind where a link word has them, the
                                    // face's slot in the neighbour in place of the row
-    Adjacency() = default;
     Adjacency(const Mesh& M, int maxf_) : maxf(maxf_) {
         const int64_t n = M.n_cell;
         nf.resize((size_t)n);
@@ -229,6 +230,8 @@ struct Adjacency {
     }
     int32_t at(int64_t i, int k) const { return nbr[(size_t)i * maxf + k]; }
 };
+
+namespace {
 
 // Link words of the tile [c0, c0 + len): local numbering tile cells, 1-ring,
 // 2-ring.  False when it exceeds ls local cells or `ghosts` boundary faces, or
@@ -596,7 +599,8 @@ template <typename Get> int make_resident(const Mesh& M, int maxf, Get adjacency
 //    meshes of fewer than 32 cells per SM, which are launch-bound: fused 128.
 // The two-kernel stage shrinks its blocks (down to 32 threads) so that small
 // meshes still spread over the SMs.
-int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int sms, bool verify = false) {
+int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout& L, int sms, bool verify = false) {
+    const Mesh& M = mesh.m;
     L = Layout{};
     L.np = round_up(M.n_cell, PLANE_ALIGN);
     L.n_face = M.n_face;
@@ -621,10 +625,10 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         else tile = 128;
     }
     L.strategy = tile == 0 || tile == 1 ? STRATEGY_TWO_KERNEL : STRATEGY_TILE;
-    Adjacency adj;
     auto adjacency = [&]() -> const Adjacency& {
-        if (adj.maxf == 0) adj = Adjacency(M, L.maxf);
-        return adj;
+        std::lock_guard<std::mutex> lock(mesh.plan_mutex);
+        if (!mesh.adjacency) mesh.adjacency = std::make_shared<const Adjacency>(M, L.maxf);
+        return *mesh.adjacency;
     };
     // the resident loop: chosen with the automatic kernel only; parts of a
     // partitioned mesh exchange after every stage and never use it
@@ -645,9 +649,13 @@ int make_layout(const Mesh& M, int prec, int scheme, int kernel, Layout& L, int 
         if (smem > SMEM_LIMIT)
             return fail(FVLBM_ERR_UNSUPPORTED, "fused stage with %d-cell tiles needs %zu B of shared memory (limit %zu)",
                         tile, smem, SMEM_LIMIT);
-        // the resident loop's tiles, where it has them of this size, serve both
+        // the resident loop's tiles, where they are of this size and nearly full (a tile of q
+        // cells has about 4.3 sqrt(q) 1-ring cells), serve both.  Shorter ones would make
+        // the stage kernels compute more of their halo: eight solvers of the 30k-cell hybrid
+        // side by side 12.9 us per FP32 stage of all with tiles of 99 cells, 9.0 with 180
+        const double root = 0.5 * (std::sqrt(4.3 * 4.3 + 4.0 * tile) - 4.3), full = root * root;
         int rc = FVLBM_OK;
-        if (L.resident && L.rp.tile == tile) std::swap(L.tp, L.rp);
+        if (L.resident && L.rp.tile == tile && L.rp.sum_len >= 0.85 * full * L.rp.n_tiles) std::swap(L.tp, L.rp);
         else rc = make_tiles(M, adjacency(), tile, L.tp, verify);
         if (rc) return rc;
         // the fused kernel indexes its blocked arrays in 32 bits
@@ -824,7 +832,7 @@ extern "C" int fvlbm_workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params*
     if (rc) return rc;
     Layout L;
     try {
-        rc = make_layout(mesh->m, params[0].precision, params[0].scheme, params[0].kernel, L, device_sms(params[0].device));
+        rc = make_layout(*mesh, params[0].precision, params[0].scheme, params[0].kernel, L, device_sms(params[0].device));
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "fvlbm_workspace_bytes: out of host memory");
     }
@@ -843,7 +851,7 @@ static int plan_report(const char* what, const fvlbm_mesh* mesh, const fvlbm_par
     if (rc) return rc;
     Layout L;
     try {
-        rc = make_layout(mesh->m, params[0].precision, params[0].scheme, params[0].kernel, L,
+        rc = make_layout(*mesh, params[0].precision, params[0].scheme, params[0].kernel, L,
                          device_sms(params[0].device), true);
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "%s: out of host memory", what);
@@ -1056,7 +1064,7 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     // layout, workspace
     Layout L;
     try {
-        rc = make_layout(M, s->prec, s->scheme, p0.kernel, L, device_sms(p0.device));
+        rc = make_layout(*mesh, s->prec, s->scheme, p0.kernel, L, device_sms(p0.device));
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "fvlbm_init: out of host memory");
     }
@@ -1618,7 +1626,7 @@ extern "C" int fvlbm_autotune(const fvlbm_mesh* mesh, const fvlbm_params* params
     int32_t automatic = 0;
     {
         Layout L;
-        if (make_layout(mesh->m, params[0].precision, params[0].scheme, 0, L, device_sms(params[0].device)) == FVLBM_OK)
+        if (make_layout(*mesh, params[0].precision, params[0].scheme, 0, L, device_sms(params[0].device)) == FVLBM_OK)
             automatic = L.strategy == STRATEGY_TILE ? L.tp.tile : 1;
         clear_error();
     }

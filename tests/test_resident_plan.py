@@ -46,10 +46,17 @@ def test_resident_plan_checks(fv, k):
 
 
 def test_tiles_of_the_length_asked_for_are_not_short(fv):
-    """128^2 quads on 152 SMs: every tile is an SM's share of 108 cells, none was cut by
-    the capacity; the stage kernels of the automatic choice use the same tiles."""
-    h = fv.Mesh(mg.cavity(128, 20.0))
+    """28,800 triangles on 152 SMs: every tile is an SM's share of the cells, none was cut
+    by the capacity; nearly full, they serve the stage kernels of the automatic choice too."""
+    h = fv.Mesh(mg.periodic_tri(120, 120, lx=120.0, ly=120.0))
     p = fv.make_params(0.1, scheme="rk2", precision="fp32")
     for resident in (False, True):
         i = fv.plan_info(h, p, resident=resident)
         assert i["stage_kernel"] == 256 and i["n_tiles"] == 152 and i["short_tiles"] == 0
+
+
+def test_stage_kernels_have_full_tiles_where_the_loop_has_short_ones(fv):
+    h = fv.Mesh(mg.cavity(128, 20.0))
+    auto, own = (fv.plan_info(h, fv.make_params(0.1, scheme="rk2", precision="fp32", kernel=k)) for k in (0, 256))
+    assert auto == own and auto["mean_tile_cells"] > 150
+    assert fv.plan_info(h, fv.make_params(0.1, scheme="rk2", precision="fp32"), resident=True)["mean_tile_cells"] < 110
