@@ -291,14 +291,14 @@ int fvlbm_residual(fvlbm_solver* s, double* e);
 int fvlbm_mass(fvlbm_solver* s, double* mass);
 
 /*
- * Same result as fvlbm_mass, computed without allocating anything.  The paper
+ * Same result as fvlbm_mass, bit for bit, computed without allocating anything.  The paper
  * has no counterpart; this entry point serves callers that may not allocate
  * memory while they run -- processes whose device memory is reserved up front
  * by another allocator (a framework's caching pool, a fixed serving budget),
  * and real-time loops or plugins that must not touch the device heap.
  *   s     solver (its state and geometry are the inputs)
  *   mass  host [n_instances], written
- * The block partial sums live in a fixed 96 KB array in the library's device
+ * The block partial sums live in a fixed 640 KB array in the library's device
  * memory, not in the solver's workspace.  The array is part of the library's
  * device code: under CUDA's default lazy module loading that code, with the
  * array, is loaded into a device's memory by the first call of this function

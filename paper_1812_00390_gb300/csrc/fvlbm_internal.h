@@ -295,6 +295,7 @@ FVLBM_RESIDENT_DECL(resident_fp16);
 FVLBM_RESIDENT_DECL(resident_bf16);
 int launch_snapshot(const DevView& v, int prec, void* stream);
 int launch_reduce(const DevView& v, int prec, void* stream, int what);
+int load_reduce();   // loads the reduction's kernels on the current device (CUDA loads lazily)
 // f and the macros in the caller's cell order, in a buffer the device
 // accesses (host memory reachable by the GPU, or device memory).
 int launch_get_f_ordered(const DevView& v, int prec, void* stream, double* f);

@@ -237,6 +237,21 @@ template <typename T, typename S, bool DEV> static void reduce_chunks(const DevV
     reduce_final_kernel<<<grid_of(32 * (int64_t)v.n_inst, 128), 128, 0, st>>>(v);
 }
 
+template <typename T, typename S, bool DEV> static cudaError_t load_chunks() {
+    cudaFuncAttributes a;
+    return cudaFuncGetAttributes(&a, (const void*)reduce_chunks_kernel<T, S, DEV>);
+}
+
+int load_reduce() {
+    cudaFuncAttributes a;
+    cudaError_t e = load_chunks<double, double, false>();
+    if (e == cudaSuccess) e = load_chunks<float, float, true>();
+    if (e == cudaSuccess) e = load_chunks<float, __half, true>();
+    if (e == cudaSuccess) e = load_chunks<float, __nv_bfloat16, true>();
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, (const void*)reduce_final_kernel);
+    return e == cudaSuccess ? FVLBM_OK : fail(FVLBM_ERR_CUDA, "reduction kernels: %s", cudaGetErrorString(e));
+}
+
 int launch_reduce(const DevView& v, int prec, void* stream, int what) {
     cudaStream_t st = (cudaStream_t)stream;
     DISPATCH_PREC(prec, reduce_chunks<T, S, DEV>(v, st, what); return check_launch("reduction kernels"));
