@@ -917,10 +917,11 @@ static int stage_t(const DevView& v, cudaStream_t st, const void* fin, const voi
     const S *in = (const S*)fin, *base = (const S*)fbase;
     bool lanes = false;
     if constexpr (sizeof(T) == 8) {
-        // FP64: four lanes per cell until the SMs' quarters have work enough without
-        // (us per stage, lanes / a thread per cell: 16k-cell cavity 17.3 / 20.4, 250k
-        // cells 130 / 136, the 6.7 M cell batch 2966 / 2869)
-        lanes = v.n_grad < 2048 * (int64_t)v.sms;
+        // FP64: four lanes per cell until the SMs' quarters have work enough without, 198k cells of
+        // four slots or 129k of eight (us per stage, lanes / a thread per cell: quads 16k 16.7 / 20.6,
+        // 109k 59.5 / 66.9, 194k 100.0 / 102.2, 250k 129.5 / 129.1; triangles 180k 70.9 / 72.2,
+        // 205k 80.8 / 80.0, 259k 104.5 / 100.9; polygons 116k 85.1 / 88.7, 160k 129.7 / 120.2)
+        lanes = v.n_grad < (v.maxf == 4 ? 1300 : 850) * (int64_t)v.sms;
         if (lanes) {
             auto kern = v.maxf == 4 ? face_values_pairs_kernel<4> : face_values_pairs_kernel<8>;
             kern<<<grid_of(4 * v.n_grad, 256), 256, 0, st>>>(v, in);

@@ -108,3 +108,18 @@ def test_fp64_two_kernel_stage_is_the_same_bits_as_fused_tiles_on_a_large_mesh(f
         out.append(s.get_f())
         s.close()
     assert np.isfinite(out[0]).all() and np.array_equal(*out)
+
+
+@pytest.mark.parametrize("name,make", [("quads", lambda m: mg.cavity(m, 20.0)), ("polygons", lambda m: mg.bricks(2 * m, m))])
+def test_fp64_state_is_the_same_bits_on_both_sides_of_the_lanes_limit(fv, name, make):
+    """Four lanes per cell below 1300 cells per SM (850 of polygons), a thread per cell from there."""
+    for side in ((444, 446) if name == "quads" else (358, 362)):
+        m = make(side)
+        h, f0, out = fv.Mesh(m), start(m.n_cell, 59), []
+        for kernel in (1, 256):
+            s = fv.Solver(h, fv.make_params(0.1, cfl=0.3, scheme="rk2", precision="fp64", u_max=0.1, kernel=kernel))
+            s.set_f(f0)
+            s.step(3)
+            out.append(s.get_f())
+            s.close()
+        assert np.isfinite(out[0]).all() and np.array_equal(*out)
