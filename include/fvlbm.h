@@ -298,7 +298,7 @@ int fvlbm_mass(fvlbm_solver* s, double* mass);
  * and real-time loops or plugins that must not touch the device heap.
  *   s     solver (its state and geometry are the inputs)
  *   mass  host [n_instances], written
- * The block partial sums live in a fixed 640 KB array in the library's device
+ * The block partial sums live in a fixed 608 KB array in the library's device
  * memory, not in the solver's workspace.  The array is part of the library's
  * device code: under CUDA's default lazy module loading that code, with the
  * array, is loaded into a device's memory by the first call of this function

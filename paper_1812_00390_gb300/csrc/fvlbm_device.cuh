@@ -242,10 +242,6 @@ template <typename S> struct PlainIO {
             store_quad(p + h * (UNITS / 2) * BLK, BLK,
                        Quad<S>{{(S)f[dir_a(2 * h)], (S)f[dir_b(2 * h)], (S)f[dir_a(2 * h + 1)], (S)f[dir_b(2 * h + 1)]}});
     }
-    template <typename T, bool DEV, typename I>
-    __device__ __forceinline__ static void store_rounded(void* base, I i, const InstParam& P, T* f) {
-        store<T, DEV>(base, i, P, f);   // stored as it is
-    }
     // FP64 moments of the stored state: r = sum f (FP64 mode) or sum g (deviation), j = sum e g
     __device__ static void moments64(const void* base, int64_t i, const InstParam& P, double& r, double& jx, double& jy) {
         S f[FVLBM_Q];
@@ -395,16 +391,6 @@ template <typename H> struct SplitIO {
         encode(P, f, h, t);
         *(uint4*)head(base, i) = h;
         *(uint2*)tail(base, i) = t;
-    }
-    // stores f and replaces it by the value that a load would give
-    template <typename T, bool DEV, typename I>
-    __device__ __forceinline__ static void store_rounded(void* base, I i, const InstParam& P, T* f) {
-        uint4 h;
-        uint2 t;
-        encode(P, f, h, t);
-        *(uint4*)head(base, i) = h;
-        *(uint2*)tail(base, i) = t;
-        decode<T>(h, t, P, f);
     }
     __device__ static void moments64(const void* base, int64_t i, const InstParam&, double& r, double& jx, double& jy) {
         const uint4 h = *head(base, i);

@@ -177,7 +177,6 @@ struct DevView {
     int64_t n_cell;     // cells updated (internal numbering 0..n_cell-1): the owned cells
     int64_t n_grad;     // cells whose gradient the two-kernel stage computes (owned + first ghost ring)
     int64_t np;         // padded cell count (multiple of the largest tile)
-    int64_t n_face;     // faces of the mesh
     int32_t maxf;       // slots per cell in the packed arrays (4 or 8)
     int32_t n_inst;
     // geometry, blocked per cell
@@ -201,7 +200,7 @@ struct DevView {
                 // ghost records (values that enter through boundary faces)
     double* uold;   // [2][np] the residual's snapshot of u
     double* part;   // [n_chunk][RED_PARTS][2] block partial sums
-    double* red;    // [n_inst][3]  per-instance sums
+    double* red;    // [n_inst][2]  per-instance sums
     double* conv;   // [9][np] doubles: device staging of get_f / set_f / macros in caller order
     const int64_t* chunk;   // [n_chunk][3] (begin, end, instance)
     const int64_t* inst_chunk;   // [n_inst + 1] chunks of each instance
@@ -337,8 +336,8 @@ double solver_overlap_setup(const fvlbm_solver* s);
 // best, in the resident loop, or by stage kernels.
 enum StepPath { STEP_AUTO = 0, STEP_RESIDENT = 1, STEP_STAGES = 2 };
 void solver_path(fvlbm_solver* s, StepPath path);
-// FP64 sums of a reduction (RED_MASS: [mass, -, -]; RED_RESIDUAL: [numerator,
-// denominator, -]) per instance, 3 per instance; synchronises.
+// FP64 sums of a reduction (RED_MASS: [mass, -]; RED_RESIDUAL: [numerator,
+// denominator]) per instance; synchronises.
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out);
 // Halo exchange of a partitioned solve: entry e = (src part, src internal
 // cell, dst part, dst internal cell) copies the stored state of one cell from

@@ -168,10 +168,8 @@ __global__ void reduce_final_kernel(DevView v) {
         for (int q = 0; q < 2; q++) s[q] += v.part[2 * x + q];
     for (int d = 16; d > 0; d >>= 1)
         for (int q = 0; q < 2; q++) s[q] += __shfl_down_sync(0xFFFFFFFFu, s[q], d);
-    if (lane == 0) {
-        for (int q = 0; q < 2; q++) v.red[3 * inst + q] = s[q];
-        v.red[3 * inst + 2] = 0;
-    }
+    if (lane == 0)
+        for (int q = 0; q < 2; q++) v.red[2 * inst + q] = s[q];
 }
 
 // ------------------------------------------------------------------ launchers

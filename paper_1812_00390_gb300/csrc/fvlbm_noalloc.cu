@@ -31,8 +31,8 @@ constexpr int NA_MAX_DEVICES = 64;
 
 // Partial sums and per-instance sums as the reduction of fvlbm_mass has them in the
 // solver's workspace (DevView::part, DevView::red), then the masses.  Every GPU on which the
-// module is loaded (first call there) holds these 640 KB until the process exits.
-constexpr int64_t NA_PART = 2 * RED_PARTS * NA_MAX_CHUNKS, NA_RED = 3 * NA_MAX_INST;
+// module is loaded (first call there) holds these 608 KB until the process exits.
+constexpr int64_t NA_PART = 2 * RED_PARTS * NA_MAX_CHUNKS, NA_RED = 2 * NA_MAX_INST;
 static __device__ __align__(256) double g_noalloc_scratch[NA_PART + NA_RED + NA_MAX_INST];
 
 std::mutex g_setup_mutex;
@@ -40,7 +40,7 @@ double* g_scratch_ptr[NA_MAX_DEVICES] = {};
 
 __global__ void masses_kernel(const double* red, double* mass, int n) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) mass[k] = red[3 * k];
+    if (k < n) mass[k] = red[2 * k];
 }
 
 // Device address of the scratch array on the current device, looked up once

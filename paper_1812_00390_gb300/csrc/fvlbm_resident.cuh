@@ -563,13 +563,10 @@ static int resident_m(const DevView& v, const ResView& r, cudaStream_t st, int s
     int threads = 0;
     size_t smem = 0;
     if constexpr (sizeof(S) == 8) {
-        if (r.tile == 16) kern = resident_of<S, MAXF, 16, 1>(scheme, threads, smem);
-        if (r.tile == 32) kern = resident_of<S, MAXF, 32, 1>(scheme, threads, smem);
         if (r.tile == RES_TILE_FP64) kern = resident_of<S, MAXF, RES_TILE_FP64, 1>(scheme, threads, smem);
     } else {
         constexpr int MORE = resident_ctas(4, MAXF);
-        if (r.tile == 64) kern = resident_of<S, MAXF, 64, 1>(scheme, threads, smem);
-        if (r.tile == 128) kern = resident_of<S, MAXF, 128, 1>(scheme, threads, smem);
+        if (r.tile == RES_TILE / 2) kern = resident_of<S, MAXF, RES_TILE / 2, 1>(scheme, threads, smem);
         if (r.tile == RES_TILE)
             kern = r.n_tiles <= v.sms       ? resident_of<S, MAXF, RES_TILE, 1>(scheme, threads, smem)
                    : r.n_tiles <= 3 * v.sms ? resident_of<S, MAXF, RES_TILE, MORE < 3 ? MORE : 3>(scheme, threads, smem)

@@ -136,8 +136,6 @@ bool tile_dims(int tile, int maxf, int rsize, int& ls, int& ghosts, size_t& byte
                           : (rsize == 4 ? TileDims<T_, 8, 4>::BYTES : TileDims<T_, 8, 8>::BYTES);            \
         return true;
     switch (tile) {
-        FVLBM_TD(16)
-        FVLBM_TD(32)
         FVLBM_TD(64)
         FVLBM_TD(128)
         FVLBM_TD(256)
@@ -499,7 +497,7 @@ int make_tiles(const Mesh& M, const Adjacency& A, int tile, TilePlan& P, bool ve
 
 // Offsets of every array inside the workspace (0 size when a strategy does not use it).
 struct Layout {
-    int64_t np, n_face, n_chunk;
+    int64_t np, n_chunk;
     int maxf;
     int strategy;
     int block;
@@ -567,7 +565,7 @@ template <typename Get> int make_resident(const Mesh& M, int maxf, Get adjacency
     P = TilePlan{};
     for (int ctas = 1; ctas <= resident_ctas(rsize, maxf); ctas++) {
         const int64_t share = std::max<int64_t>((n + ctas * sms - 1) / (ctas * sms), RES_MIN_CELLS(rsize));
-        for (int tile = ctas > 1 ? most : rsize == 8 ? 16 : 64; tile <= most; tile *= 2) {
+        for (int tile = ctas > 1 ? most : rsize == 8 ? RES_TILE_FP64 : RES_TILE / 2; tile <= most; tile *= 2) {
             // a compact tile of q cells has about 4.3 sqrt(q) 1-ring cells
             if (share + 4.3 * std::sqrt((double)share) > tile) continue;
             // equal tiles; where a few are cut shorter and there are too many, as long as they fit
@@ -603,7 +601,6 @@ int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout
     const Mesh& M = mesh.m;
     L = Layout{};
     L.np = round_up(M.n_cell, PLANE_ALIGN);
-    L.n_face = M.n_face;
     L.maxf = M.max_faces <= 4 ? 4 : 8;
     L.n_chunk = 0;
     for (int k = 0; k < M.n_inst; k++) L.n_chunk += (M.inst_begin[k + 1] - M.inst_begin[k] + CHUNK - 1) / CHUNK;
@@ -699,7 +696,7 @@ int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout
     L.off_fv = take(two ? 4 * R * (slots + (size_t)L.n_ghost) : 0);
     L.off_uold = take(16 * plane);
     L.off_part = take(16 * RED_PARTS * (size_t)std::max<int64_t>(1, L.n_chunk));
-    L.off_red = take(24 * (size_t)M.n_inst);
+    L.off_red = take(16 * (size_t)M.n_inst);
     L.off_conv = take(8 * plane * FVLBM_Q);
     L.off_chunk = take(24 * (size_t)std::max<int64_t>(1, L.n_chunk) + 8 * (size_t)(M.n_inst + 1));
     L.off_flag = take(16);
@@ -1133,7 +1130,6 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     v.n_cell = M.n_owned;
     v.n_grad = M.n_grad;
     v.np = L.np;
-    v.n_face = L.n_face;
     v.maxf = L.maxf;
     v.n_inst = M.n_inst;
     v.link = (const uint4*)(base + L.off_link);
@@ -1488,7 +1484,7 @@ extern "C" int fvlbm_macros(fvlbm_solver* s, double* rho, double* u) {
 static int reduce(fvlbm_solver* s, int what, std::vector<double>& out) {
     int rc = launch_reduce(s->v, s->prec, s->stream, what);
     if (rc) return rc;
-    out.assign(3 * (size_t)s->n_inst, 0.0);
+    out.assign(2 * (size_t)s->n_inst, 0.0);
     CK(cudaMemcpyAsync(out.data(), s->v.red, out.size() * 8, cudaMemcpyDeviceToHost, s->stream), "read sums");
     return sync_and_check(s);
 }
@@ -1523,7 +1519,7 @@ extern "C" int fvlbm_residual(fvlbm_solver* s, double* e) {
     int rc = reduce(s, RED_RESIDUAL, r);
     if (rc) return rc;
     for (int32_t k = 0; k < s->n_inst; k++) {
-        const double num = r[3 * k], den = r[3 * k + 1];
+        const double num = r[2 * k], den = r[2 * k + 1];
         e[k] = den == 0 ? (num == 0 ? 0.0 : INFINITY) : std::sqrt(num) / std::sqrt(den);
     }
     return FVLBM_OK;
@@ -1536,7 +1532,7 @@ extern "C" int fvlbm_mass(fvlbm_solver* s, double* mass) {
     std::vector<double> r;
     int rc = reduce(s, RED_MASS, r);
     if (rc) return rc;
-    for (int32_t k = 0; k < s->n_inst; k++) mass[k] = r[3 * k];
+    for (int32_t k = 0; k < s->n_inst; k++) mass[k] = r[2 * k];
     return FVLBM_OK;
 }
 
