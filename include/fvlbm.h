@@ -181,7 +181,10 @@ int fvlbm_suggest_dt(const fvlbm_mesh* mesh, int32_t instance, double tau, doubl
                      double u_max, int32_t scheme, double* dt);
 
 /*
- * Device bytes fvlbm_init needs when the caller supplies the workspace.
+ * Device bytes fvlbm_init needs when the caller supplies the workspace.  Of a small mesh
+ * with params.kernel = 0 they hold the resident loop's arrays (see fvlbm_step) besides,
+ * some 70 to 130 bytes per cell (FP64 260); a workspace without room for those is
+ * accepted, and fvlbm_step then runs the stage kernels.
  * params: host, [n_params] as for fvlbm_init.  bytes: host, written.
  */
 int fvlbm_workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,

@@ -310,6 +310,9 @@ struct SolverRef {
     int32_t n_inst;
 };
 int solver_ref(fvlbm_solver* s, SolverRef* out);
+// fvlbm_workspace_bytes; loop = false: without the resident loop's arrays (fvlbm_init then
+// takes the solver to the stage kernels).
+int workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params, bool loop, size_t* bytes);
 // Stages of one time step, and stage k enqueued on the solver's stream (*out:
 // the state buffer it writes); the last stage ends the step.
 int solver_n_stages(const fvlbm_solver* s);

@@ -76,6 +76,7 @@ struct Request {
     const fvlbm_mesh* mesh;
     std::vector<fvlbm_params> params;
     size_t bytes = 0, off = 0;
+    size_t least = 0;   // bytes without the resident loop's arrays (0: not asked yet)
     int stream = 0;
     fvlbm_solver* solver = nullptr;
     int state = FVLBM_REQ_QUEUED;
@@ -167,6 +168,12 @@ extern "C" int fvlbm_server_submit(fvlbm_server* s, const fvlbm_mesh* mesh, cons
     size_t bytes = 0;
     int rc = fvlbm_workspace_bytes(mesh, params, n_params, &bytes);
     if (rc) return rc;
+    size_t least = 0;
+    if (Arena::round(bytes) > s->cfg.arena_bytes) {
+        rc = workspace_bytes(mesh, params, n_params, false, &least);
+        if (rc) return rc;
+        bytes = least;
+    }
     if (Arena::round(bytes) > s->cfg.arena_bytes)
         return fail(FVLBM_ERR_OOM, "request needs %zu bytes, the arena holds %zu", bytes, s->cfg.arena_bytes);
     for (int32_t k = 0; k < n_params; k++)
@@ -176,6 +183,7 @@ extern "C" int fvlbm_server_submit(fvlbm_server* s, const fvlbm_mesh* mesh, cons
     r.mesh = mesh;
     r.params.assign(params, params + n_params);
     r.bytes = bytes;
+    r.least = least;
     r.t_submit = now_s(s->t0);
     fvlbm_mesh_info_t info;
     fvlbm_mesh_info(mesh, &info);
@@ -243,7 +251,14 @@ extern "C" int fvlbm_server_poll(fvlbm_server* s, int32_t* n_completed) {
     for (auto it = s->queue.begin(); it != s->queue.end() && (int)s->active.size() < s->cfg.max_active;) {
         Request& r = s->req[*it];
         size_t off;
-        if (!s->arena.alloc(r.bytes, &off)) {
+        bool room = s->arena.alloc(r.bytes, &off);
+        if (!room) {   // rather by stage kernels now than in the resident loop later
+            if (!r.least && workspace_bytes(r.mesh, r.params.data(), (int32_t)r.params.size(), false, &r.least))
+                r.least = r.bytes;
+            room = r.least < r.bytes && s->arena.alloc(r.least, &off);
+            if (room) r.bytes = r.least;
+        }
+        if (!room) {
             ++it;
             continue;
         }

@@ -597,7 +597,9 @@ template <typename Get> int make_resident(const Mesh& M, int maxf, Get adjacency
 //    meshes of fewer than 32 cells per SM, which are launch-bound: fused 128.
 // The two-kernel stage shrinks its blocks (down to 32 threads) so that small
 // meshes still spread over the SMs.
-int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout& L, int sms, bool verify = false) {
+// loop: false leaves the resident loop and its arrays out.
+int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout& L, int sms, bool verify = false,
+                bool loop = true) {
     const Mesh& M = mesh.m;
     L = Layout{};
     L.np = round_up(M.n_cell, PLANE_ALIGN);
@@ -630,7 +632,7 @@ int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout
     // the resident loop: chosen with the automatic kernel only; parts of a
     // partitioned mesh exchange after every stage and never use it
     L.resident = false;
-    if (kernel == 0 && M.n_owned == M.n_cell && M.n_owned > 0) {
+    if (loop && kernel == 0 && M.n_owned == M.n_cell && M.n_owned > 0) {
         int rc = make_resident(M, L.maxf, adjacency, (int)R, sms, L.rp, verify);
         if (rc) return rc;
         L.resident = L.rp.n_tiles > 0;
@@ -821,21 +823,28 @@ void pack_geometry(const Mesh& M, const Layout& L, std::vector<unsigned char>& h
 
 }  // namespace
 
-extern "C" int fvlbm_workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
-                                     size_t* bytes) {
-    clear_error();
-    if (!mesh || !bytes) return fail(FVLBM_ERR_ARG, "fvlbm_workspace_bytes: null argument");
+namespace fvlbm {
+int workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params, bool loop, size_t* bytes) {
     int rc = check_params(mesh->m, params, n_params);
     if (rc) return rc;
     Layout L;
     try {
-        rc = make_layout(*mesh, params[0].precision, params[0].scheme, params[0].kernel, L, device_sms(params[0].device));
+        rc = make_layout(*mesh, params[0].precision, params[0].scheme, params[0].kernel, L, device_sms(params[0].device),
+                         false, loop);
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "fvlbm_workspace_bytes: out of host memory");
     }
     if (rc) return rc;
     *bytes = L.total;
     return FVLBM_OK;
+}
+}  // namespace fvlbm
+
+extern "C" int fvlbm_workspace_bytes(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t n_params,
+                                     size_t* bytes) {
+    clear_error();
+    if (!mesh || !bytes) return fail(FVLBM_ERR_ARG, "fvlbm_workspace_bytes: null argument");
+    return workspace_bytes(mesh, params, n_params, true, bytes);
 }
 
 // The plans fvlbm_init would build, checked: of the stage kernels (resident: of
@@ -1062,6 +1071,9 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     Layout L;
     try {
         rc = make_layout(*mesh, s->prec, s->scheme, p0.kernel, L, device_sms(p0.device));
+        // a workspace that holds everything but the loop's arrays is enough
+        if (!rc && workspace && workspace_bytes < L.total && L.resident)
+            rc = make_layout(*mesh, s->prec, s->scheme, p0.kernel, L, device_sms(p0.device), false, false);
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "fvlbm_init: out of host memory");
     }
