@@ -114,7 +114,9 @@ def config_runs(fv, torch, dev, steps: int = 30):
     that starts from DRAM; the host enqueues the step while the flush runs);
     "from_idle_host" times the same from a synchronised host, so it adds the
     launch of one step (binding, C ABI, graph launch) to an idle GPU; "warm"
-    is the same solver replaying its graphs with the mesh resident in L2."""
+    is the same solver replaying its graphs with the mesh resident in L2.  "default"
+    is what a user who sets no kernel gets for the same steps (the resident loop where
+    it serves the mesh: resident_launches > 0)."""
     from paper_1812_00390_gb300 import meshgen as mg
     cases = [
         ("couette_32x8_euler_fp64", mg.couette(), 3 * 0.1 * 8 / 10, "euler", "fp64", (0.0, 0.0)),
@@ -154,12 +156,25 @@ def config_runs(fv, torch, dev, steps: int = 30):
         b.record(s.stream)
         s.sync()
         warm = a.elapsed_time(b) / (10 * steps)
+        d = fv.Solver(h, fv.make_params(tau, scheme=scheme, precision=prec, u0=u0))
+        d.step(32)
+        d.sync()
+        launches = d.resident_info()["launches"]
+        a.record(d.stream)
+        d.step(10 * steps)
+        b.record(d.stream)
+        d.sync()
+        default = a.elapsed_time(b) / (10 * steps)
+        launches = d.resident_info()["launches"] - launches
+        d.close()
         out[name] = {"cells": m.n_cell, "stage_kernel": best,
                      "autotune_ms_per_step": {str(k): v for k, v in tune.items()},
                      "cold_l2_mcups": m.n_cell / (cold / 1e3) / 1e6,
                      "warm_l2_mcups": m.n_cell / (warm / 1e3) / 1e6, "cold_ms_per_step": cold,
                      "warm_ms_per_step": warm,
-                     "from_idle_host_mcups": m.n_cell / (idle / 1e3) / 1e6, "from_idle_host_ms_per_step": idle}
+                     "from_idle_host_mcups": m.n_cell / (idle / 1e3) / 1e6, "from_idle_host_ms_per_step": idle,
+                     "default_mcups": m.n_cell / (default / 1e3) / 1e6, "default_ms_per_step": default,
+                     "resident_launches": launches}
         s.close()
     return out
 
@@ -169,7 +184,7 @@ def error_per_config(fv):
     against the FP64 mode of the same configuration on the GPU (which the
     tests hold to the FP64 oracle within 1e-12): max relative |u| error (of
     the largest FP64 speed) and max |rho| error, per storage precision, each
-    run with the automatic stage kernel."""
+    run with the automatic choice: in the resident loop when resident_launches > 0."""
     from paper_1812_00390_gb300 import meshgen as mg
     cav, cyl = mg.cavity(128, 20.0), mg.cylinder_hybrid()
     cases = [("cavity_128_re400", cav, 3 * 0.1 / 400, (0.0, 0.0), 10_000),
@@ -190,7 +205,8 @@ def error_per_config(fv):
             s.step(n)
             r, u = s.macros()
             row[prec] = {"max_rel_velocity": float(np.abs(u - u64).max() / np.abs(u64).max()),
-                         "max_abs_density": float(np.abs(r - r64).max()), "stage_kernel": s.stage_kernel()}
+                         "max_abs_density": float(np.abs(r - r64).max()), "stage_kernel": s.stage_kernel(),
+                         "resident_launches": s.resident_info()["launches"]}
             s.close()
         out[name] = row
     return out
