@@ -153,14 +153,20 @@ constexpr uint32_t LINK_ROW_MAX = 0x3FFFu;
 // index): LS local cells (tile, 1-ring, 2-ring) and the face table, whose row
 // k * TILE + x holds the four values that leave local cell x through slot k,
 // and whose last GHOSTS rows hold the values that enter through the tile's
-// boundary faces; reals of RSIZE bytes.  The planner ends a tile early when
-// it would not fit.
+// boundary faces; reals of RSIZE bytes.  A row is one 16-byte unit in FP32, so that
+// no offset depends on how many there are: tiles there have up to MAX_GHOSTS boundary
+// faces, and a launch whose plan has tiles of more than GHOSTS asks for the memory
+// (instances of a few cells, channels one cell wide: 30,000 meshes of two triangles 9.0 us
+// per stage, 11.9 with tiles cut at GHOSTS).  The planner ends a tile early when it would
+// not fit.
 template <int TILE, int MAXF, int RSIZE> struct TileDims {
     static constexpr int LS = (3 * TILE) / 2 + 64;
     static constexpr int GHOSTS = TILE / 2;
+    static constexpr int MAX_GHOSTS = RSIZE == 4 ? 2 * TILE : GHOSTS;
     static constexpr int ROWS = MAXF * TILE + GHOSTS;
     static constexpr size_t BYTES = (size_t)RSIZE * ((size_t)(FVLBM_Q - 1) * LS + (size_t)4 * ROWS);
-    static_assert(LS <= (int)LINK_NB_MASK + 1 && ROWS <= (int)LINK_ROW_MAX, "link word fields");
+    static constexpr size_t MAX_BYTES = BYTES + (size_t)4 * RSIZE * (MAX_GHOSTS - GHOSTS);
+    static_assert(LS <= (int)LINK_NB_MASK + 1 && MAXF * TILE + MAX_GHOSTS <= (int)LINK_ROW_MAX, "link word fields");
 };
 
 // One tile of the fused stage.
@@ -210,6 +216,7 @@ struct DevView {
     int32_t strategy;        // STRATEGY_TWO_KERNEL or STRATEGY_TILE
     int32_t block;           // threads per block of the two-kernel stage
     int32_t tile;            // most cells per tile (threads per CTA)
+    int32_t tile_ghosts;     // most boundary faces of a tile
     int32_t sms;             // streaming multiprocessors of the device
     int64_t n_tiles;
     const TileRec* tiles;      // [n_tiles]

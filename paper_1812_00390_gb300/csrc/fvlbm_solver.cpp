@@ -115,7 +115,7 @@ struct TilePlan {
     std::vector<uint32_t> link;     // [n_cell][maxf] link words of the tile cells
     std::vector<uint32_t> r1link;   // [1-ring entries][maxf] link words
     int64_t n_r1 = 0;               // 1-ring entries
-    int32_t max_local = 0, max_faces = 0;
+    int32_t max_local = 0, max_faces = 0, max_ghosts = 0;
     int64_t short_tiles = 0;        // tiles cut below the length asked for by the capacity
     int64_t sum_len = 0, sum_ring1 = 0, sum_local = 0;   // over the tiles
     // filled when the plan is verified (fvlbm_plan_info): modelled
@@ -127,11 +127,12 @@ struct TilePlan {
 };
 
 // Shared-memory capacity of the fused kernel for a tile size (TileDims).
-bool tile_dims(int tile, int maxf, int rsize, int& ls, int& ghosts, size_t& bytes) {
+// loop: in the resident loop's layout, whose face table is of fixed size.
+bool tile_dims(int tile, int maxf, int rsize, bool loop, int& ls, int& ghosts, size_t& bytes) {
 #define FVLBM_TD(T_)                                                                                         \
     case T_:                                                                                                 \
         ls = TileDims<T_, 4, 4>::LS;                                                                         \
-        ghosts = TileDims<T_, 4, 4>::GHOSTS;                                                                 \
+        ghosts = rsize == 4 && !loop ? TileDims<T_, 4, 4>::MAX_GHOSTS : TileDims<T_, 4, 4>::GHOSTS;           \
         bytes = maxf <= 4 ? (rsize == 4 ? TileDims<T_, 4, 4>::BYTES : TileDims<T_, 4, 8>::BYTES)             \
                           : (rsize == 4 ? TileDims<T_, 8, 4>::BYTES : TileDims<T_, 8, 8>::BYTES);            \
         return true;
@@ -236,7 +237,7 @@ namespace {
 // when tile and 1-ring together exceed the CTA's `threads` (the kernel gives
 // every thread at most one gradient to compute).
 bool try_tile(const Adjacency& A, int64_t c0, int len, int threads, int ls, int ghosts, TileScratch& W,
-              int& n_local, int& n_faces) {
+              int& n_local, int& n_faces, int& n_ghosts) {
     const int64_t g = ++W.gen;
     const int maxf = A.maxf;
     int nl = 0;
@@ -314,6 +315,7 @@ bool try_tile(const Adjacency& A, int64_t c0, int len, int threads, int ls, int 
     }
     n_local = nl;
     n_faces = n_slots - inner / 2;
+    n_ghosts = n_ghost;
     return true;
 }
 
@@ -431,11 +433,13 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
 // max_len: most cells of a tile (0: as many as fit).  max_tiles: most tiles (0: any
 // number); FVLBM_ERR_UNSUPPORTED as soon as more are sure to be needed or, an eighth of
 // the cells along, at the mean length so far a tenth more.
-int make_tiles(const Mesh& M, const Adjacency& A, int tile, TilePlan& P, bool verify, int max_len = 0, int64_t max_tiles = 0) {
+// loop: for the resident loop.
+int make_tiles(const Mesh& M, const Adjacency& A, int tile, int rsize, bool loop, TilePlan& P, bool verify,
+               int max_len = 0, int64_t max_tiles = 0) {
     int ls = 0, ghosts = 0;
     size_t bytes = 0;
     const int maxf = A.maxf;
-    if (!tile_dims(tile, maxf, 4, ls, ghosts, bytes)) return fail(FVLBM_ERR_ARG, "unsupported tile size %d", tile);
+    if (!tile_dims(tile, maxf, rsize, loop, ls, ghosts, bytes)) return fail(FVLBM_ERR_ARG, "unsupported tile size %d", tile);
     const int64_t n = M.n_cell;
     P = TilePlan{};
     P.tile = tile;
@@ -452,8 +456,8 @@ int make_tiles(const Mesh& M, const Adjacency& A, int tile, TilePlan& P, bool ve
     int guess = max_len;   // neighbouring tiles have similar lengths: start one block above the last
     while (c0 < n_own) {
         int len = (int)std::min<int64_t>(guess, n_own - c0);
-        int nl = 0, nf = 0;
-        while (!try_tile(A, c0, len, tile, ls, ghosts, W, nl, nf)) {
+        int nl = 0, nf = 0, ng = 0;
+        while (!try_tile(A, c0, len, tile, ls, ghosts, W, nl, nf, ng)) {
             if (len == 1)
                 return fail(FVLBM_ERR_UNSUPPORTED, "cell %lld: its halo exceeds the fused stage's capacity",
                             (long long)c0);
@@ -488,6 +492,7 @@ int make_tiles(const Mesh& M, const Adjacency& A, int tile, TilePlan& P, bool ve
         if (max_tiles > 0 && (made + (n_own - c0 + max_len - 1) / max_len > max_tiles ||
                               (c0 >= n_own / 8 && (double)made * n_own > 1.1 * max_tiles * c0)))
             return fail(FVLBM_ERR_UNSUPPORTED, "more than %lld tiles", (long long)max_tiles);
+        P.max_ghosts = std::max(P.max_ghosts, ng);
         P.max_local = std::max(P.max_local, nl);
         P.max_faces = std::max(P.max_faces, nf);
     }
@@ -571,7 +576,7 @@ template <typename Get> int make_resident(const Mesh& M, int maxf, Get adjacency
             // equal tiles; where a few are cut shorter and there are too many, as long as they fit
             for (int64_t len : {std::min<int64_t>(share, tile), (int64_t)tile}) {
                 if (len == tile && ctas < std::min(3, resident_ctas(rsize, maxf))) continue;
-                int rc = make_tiles(M, adjacency(), tile, P, verify, (int)len, (int64_t)ctas * sms);
+                int rc = make_tiles(M, adjacency(), tile, rsize, true, P, verify, (int)len, (int64_t)ctas * sms);
                 if (rc == FVLBM_OK) {
                     if (verify) verify_exchange(P);
                     return FVLBM_OK;
@@ -615,7 +620,7 @@ int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout
         auto fits = [&](int t) {
             int ls = 0, fs = 0;
             size_t smem = 0;
-            tile_dims(t, L.maxf, (int)R, ls, fs, smem);
+            tile_dims(t, L.maxf, (int)R, false, ls, fs, smem);
             return smem <= SMEM_LIMIT;
         };
         if (prec == FVLBM_FP64) tile = n < 32 * (int64_t)sms ? 128 : 1;
@@ -644,7 +649,7 @@ int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout
     if (L.strategy == STRATEGY_TILE) {
         int ls = 0, fs = 0;
         size_t smem = 0;
-        tile_dims(tile, L.maxf, (int)R, ls, fs, smem);
+        tile_dims(tile, L.maxf, (int)R, false, ls, fs, smem);
         if (smem > SMEM_LIMIT)
             return fail(FVLBM_ERR_UNSUPPORTED, "fused stage with %d-cell tiles needs %zu B of shared memory (limit %zu)",
                         tile, smem, SMEM_LIMIT);
@@ -655,7 +660,7 @@ int make_layout(const fvlbm_mesh& mesh, int prec, int scheme, int kernel, Layout
         const double root = 0.5 * (std::sqrt(4.3 * 4.3 + 4.0 * tile) - 4.3), full = root * root;
         int rc = FVLBM_OK;
         if (L.resident && L.rp.tile == tile && L.rp.sum_len >= 0.85 * full * L.rp.n_tiles) std::swap(L.tp, L.rp);
-        else rc = make_tiles(M, adjacency(), tile, L.tp, verify);
+        else rc = make_tiles(M, adjacency(), tile, (int)R, false, L.tp, verify);
         if (rc) return rc;
         // the fused kernel indexes its blocked arrays in 32 bits
         const uint64_t lim = (uint64_t)1 << 32;
@@ -1169,6 +1174,7 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     v.block = L.block;
     if (L.strategy == STRATEGY_TILE) {
         v.tile = L.tp.tile;
+        v.tile_ghosts = L.tp.max_ghosts;
         v.n_tiles = L.tp.n_tiles;
         v.tiles = (const TileRec*)(base + L.off_tiles);
         v.halo = (const int32_t*)(base + L.off_halo);

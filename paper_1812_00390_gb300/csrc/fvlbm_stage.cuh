@@ -851,10 +851,12 @@ template <typename T, typename S, int MAXF, bool DEV, int TILE>
 static int tile_launch(const DevView& v, cudaStream_t st, const void* fin, const void* fbase, void* fout,
                        double beta, int mode) {
     auto kern = stage_tile_kernel<T, S, MAXF, DEV, TILE>;
-    const size_t smem = TileDims<TILE, MAXF, sizeof(T)>::BYTES;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return fail(FVLBM_ERR_CUDA, "fused stage: %zu B shared memory: %s", smem, cudaGetErrorString(e));
+    typedef TileDims<TILE, MAXF, sizeof(T)> D;
+    constexpr size_t base = D::BYTES, most = D::MAX_BYTES;
+    const size_t smem = base + (v.tile_ghosts > D::GHOSTS ? (size_t)4 * sizeof(T) * (v.tile_ghosts - D::GHOSTS) : 0);
+    if (most > 48 * 1024) {   // the most of any plan: solvers of several threads share the attribute
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        if (e != cudaSuccess) return fail(FVLBM_ERR_CUDA, "fused stage: %zu B shared memory: %s", most, cudaGetErrorString(e));
     }
     // prefetch distance: 5/8 of the CTAs that fit on the GPU at once (queried
     // once per kernel; a function-local static is initialised once even when
@@ -863,7 +865,7 @@ static int tile_launch(const DevView& v, cudaStream_t st, const void* fin, const
     // distances let the prefetched lines age out of L2 before their tile runs.
     static const int per_sm = [&] {
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TILE, smem) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TILE, base) != cudaSuccess) {
             cudaGetLastError();
             n = 0;
         }
@@ -881,6 +883,7 @@ constexpr size_t TILE_SMEM_LIMIT = 227 * 1024;
 template <typename T, typename S, int MAXF, bool DEV, int TILE>
 static int tile_launch_if_fits(const DevView& v, cudaStream_t st, const void* fin, const void* fbase, void* fout,
                                double beta, int mode) {
+    static_assert(sizeof(T) == 8 || TileDims<TILE, MAXF, sizeof(T)>::MAX_BYTES <= TILE_SMEM_LIMIT, "every plan fits");
     if constexpr (TileDims<TILE, MAXF, sizeof(T)>::BYTES <= TILE_SMEM_LIMIT)
         return tile_launch<T, S, MAXF, DEV, TILE>(v, st, fin, fbase, fout, beta, mode);
     return fail(FVLBM_ERR_UNSUPPORTED, "tile size %d does not fit in shared memory", TILE);
