@@ -182,6 +182,7 @@ struct TileRec {
 struct DevView {
     int64_t n_cell;     // cells updated (internal numbering 0..n_cell-1): the owned cells
     int64_t n_grad;     // cells whose gradient the two-kernel stage computes (owned + first ghost ring)
+    int64_t n_bface;    // boundary faces of the cells
     int64_t np;         // padded cell count (multiple of the largest tile)
     int32_t maxf;       // slots per cell in the packed arrays (4 or 8)
     int32_t n_inst;

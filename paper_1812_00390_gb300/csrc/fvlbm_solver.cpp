@@ -1146,6 +1146,7 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     DevView& v = s->v;
     v.n_cell = M.n_owned;
     v.n_grad = M.n_grad;
+    v.n_bface = M.n_bface;
     v.np = L.np;
     v.maxf = L.maxf;
     v.n_inst = M.n_inst;

@@ -921,10 +921,13 @@ static int stage_t(const DevView& v, cudaStream_t st, const void* fin, const voi
     bool lanes = false;
     if constexpr (sizeof(T) == 8) {
         // FP64: four lanes per cell until the SMs' quarters have work enough without, 198k cells of
-        // four slots or 129k of eight (us per stage, lanes / a thread per cell: quads 16k 16.7 / 20.6,
+        // four slots or 114k of eight (us per stage, lanes / a thread per cell: quads 16k 16.7 / 20.6,
         // 109k 59.5 / 66.9, 194k 100.0 / 102.2, 250k 129.5 / 129.1; triangles 180k 70.9 / 72.2,
-        // 205k 80.8 / 80.0, 259k 104.5 / 100.9; polygons 116k 85.1 / 88.7, 160k 129.7 / 120.2)
-        lanes = v.n_grad < (v.maxf == 4 ? 1300 : 850) * (int64_t)v.sms;
+        // 205k 80.8 / 80.0, 259k 104.5 / 100.9; polygons 116k 85.1 / 88.7, 160k 129.7 / 120.2).
+        // A boundary face, whose ghost values a thread forms four times as long, outweighs eight
+        // cells (0.06 of them per cell: 246k 139.6 / 143.8, 369k 203.3 / 205.2; 0.13: 410k 247.9 / 256.6;
+        // 0.25: 768k 519 / 547)
+        lanes = v.n_grad - 8 * v.n_bface < (v.maxf == 4 ? 1300 : 750) * (int64_t)v.sms;
         if (lanes) {
             auto kern = v.maxf == 4 ? face_values_pairs_kernel<4> : face_values_pairs_kernel<8>;
             kern<<<grid_of(4 * v.n_grad, 256), 256, 0, st>>>(v, in);

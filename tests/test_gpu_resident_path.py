@@ -112,8 +112,9 @@ def test_fp64_two_kernel_stage_is_the_same_bits_as_fused_tiles_on_a_large_mesh(f
 
 @pytest.mark.parametrize("name,make", [("quads", lambda m: mg.cavity(m, 20.0)), ("polygons", lambda m: mg.bricks(2 * m, m))])
 def test_fp64_state_is_the_same_bits_on_both_sides_of_the_lanes_limit(fv, name, make):
-    """Four lanes per cell below 1300 cells per SM (850 of polygons), a thread per cell from there."""
-    for side in ((444, 446) if name == "quads" else (358, 362)):
+    """Four lanes per cell below 1300 cells per SM (750 of polygons), a boundary face counting
+    as eight cells less, a thread per cell from there."""
+    for side in ((460, 462) if name == "quads" else (362, 366)):
         m = make(side)
         h, f0, out = fv.Mesh(m), start(m.n_cell, 59), []
         for kernel in (1, 256):
