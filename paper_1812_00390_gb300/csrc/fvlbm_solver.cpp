@@ -979,9 +979,11 @@ static bool crowd_turns(fvlbm_solver* s) {
 }
 // The solver's long call has been enqueued.
 static void crowd_stepped(fvlbm_solver* s) {
+    // outside the lock: a record waits when the stream's queue is full
+    const bool ok = cudaEventRecord(s->stepped, s->stream) == cudaSuccess;
+    if (!ok) cudaGetLastError();
     std::lock_guard<std::mutex> lock(crowd().m);
-    s->in_flight = cudaEventRecord(s->stepped, s->stream) == cudaSuccess;
-    if (!s->in_flight) cudaGetLastError();
+    s->in_flight = ok;
 }
 
 namespace fvlbm {
