@@ -1,11 +1,12 @@
 // The resident stage loop: many time steps of a small solver in one launch.
 //
-// A mesh of a few hundred to some 60,000 cells gives every SM one tile or
+// A mesh of a few hundred to some 100,000 cells gives every SM a few tiles or
 // less, and a stage launched by itself is then a chain of latencies: the launch,
 // the tile's record, its halo list, its geometry, its state.  Here every tile's
-// CTA stays on the GPU for all the steps of the call.  Links and geometry stay
-// in registers, the tile's own state in registers and shared memory; only the
-// halo moves between stages, through an exchange buffer in global memory (L2).
+// CTA stays on the GPU for all the steps of the call.  Links stay in registers,
+// geometry in shared memory (FP32; FP64 in registers, and with four tiles per SM it
+// is read again), the tile's own state in both; only the halo moves between
+// stages, through an exchange buffer in global memory (L2).
 //
 // Exchange.  A cell's new state is written as 16-byte units of three data
 // words and one tag word, the number of the stage, each unit one 128-bit
@@ -29,11 +30,12 @@
 // last one writes the state buffer instead of the exchange buffer: a launch has
 // at least two stages, so that every halo has been read by then.
 //
-// The arithmetic is that of the fused stage kernel, value by value.
+// The arithmetic is that of the stage kernels, value by value, in every precision.
 //
-// Measured, us per stage, here / a launch per stage: 2,048 cells FP32 1.6 / 4.0;
-// 128^2 cavity FP32 2.0 / 4.5; 60k-cell cylinder FP32 3.2 / 5.6, FP16 4.0 / 6.5; 12k
-// polygons 2.5 / 6.6; 512 cells FP64 5.5 / 19.2.
+// Measured, us per stage, here / a launch per stage: 2,048 cells FP32 1.6 / 3.9;
+// 128^2 cavity FP32 2.0 / 4.8; 60k-cell cylinder FP32 3.3 / 5.8, FP16 4.1 / 6.2; 12k
+// polygons 2.5 / 6.9; 512 cells FP64 5.5 / 16.7, 4,096 7.0 / 18.6.  (Where the exchange buffer
+// lies in memory moves these by some 1%.)
 #pragma once
 
 #include "fvlbm_stage.cuh"

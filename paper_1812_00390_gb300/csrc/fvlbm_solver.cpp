@@ -599,7 +599,9 @@ template <typename Get> int make_resident(const Mesh& M, int maxf, Get adjacency
 //    the two-kernel stage launches two, which is what small meshes wait on;
 //  - FP64: the two-kernel stage (it spends fewer FP64 operations: no 1-ring
 //    gradients, and the FP64 mode is bound by GB300's FP64 units) except on
-//    meshes of fewer than 32 cells per SM, which are launch-bound: fused 128.
+//    meshes of fewer than 32 cells per SM: fused 128, one launch per stage.  (With four
+//    lanes per cell two kernels are faster there as well, 11.0 us per stage of 512 cells
+//    against 16.6; such meshes run in the resident loop, 5.5, but for single stages.)
 // The two-kernel stage shrinks its blocks (down to 32 threads) so that small
 // meshes still spread over the SMs.
 // loop: false leaves the resident loop and its arrays out.

@@ -195,8 +195,8 @@ __device__ __forceinline__ void add_flux(uint32_t d, const typename Vec2<T>::typ
 // cells of a warp that have one boundary face go through the code once, not once
 // per slot number (the resident loop, where boundary warps are the critical
 // path: 2.31 -> 2.00 us per stage of a 128^2 cavity).  The streaming kernels, where
-// they are few and registers short, unroll the slots (0.277 ms per stage of
-// the 256-instance batch, 0.300 with NEXT, whose slot number costs spills).
+// they are few and registers short, unroll the slots (NEXT costs 8% of a stage of the
+// 256-instance batch: its slot number spills).
 template <typename T, bool DEV, int MAXF, bool NEXT, typename Tag, typename Lsq, typename Face, typename Own, typename In>
 __device__ __forceinline__ void boundary_slots(const uint32_t* d, const BcParam* bcs, T f0, const Pair<T>* fp,
                                                Pair<T>* gx, Pair<T>* gy, Tag tag, Lsq lsq, Face face, Own own, In in) {
@@ -669,9 +669,9 @@ __device__ __forceinline__ void tile_faces(const uint32_t* d, const Pair<T>* f, 
 // constants (TileDims); the planner keeps every tile within them.
 // Bound by latency (record -> halo list -> state, the two barriers) at the 32
 // warps per SM that 64 registers allow, not by DRAM or issue: 256-instance
-// batch (6.67 M cells) 0.279 ms per FP32 stage and 0.335 per FP16 stage; with
-// single 4-byte accesses, a table of faces and scalar arithmetic, half as many
-// instructions again, 0.300 and 0.360.
+// batch (6.67 M cells) 0.281 ms per FP32 stage and 0.339 per FP16 stage (graph
+// replay); with single 4-byte accesses, a table of faces and scalar arithmetic, half
+// as many instructions again, 0.302 and 0.364.
 constexpr int stage_ctas(int tile, int rsize) { return tile <= (rsize == 4 ? 1024 : 512) ? (rsize == 4 ? 1024 : 512) / tile : 1; }
 
 template <typename T, typename S, int MAXF, bool DEV, int TILE>
