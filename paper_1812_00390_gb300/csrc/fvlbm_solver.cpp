@@ -431,8 +431,7 @@ void verify_tile(const Mesh& M, int maxf, int64_t c0, int len, int threads, int 
 }
 
 // max_len: most cells of a tile (0: as many as fit).  max_tiles: most tiles (0: any
-// number); FVLBM_ERR_UNSUPPORTED as soon as more are sure to be needed or, an eighth of
-// the cells along, at the mean length so far a tenth more.
+// number); FVLBM_ERR_UNSUPPORTED as soon as more are sure to be needed.
 // loop: for the resident loop.
 int make_tiles(const Mesh& M, const Adjacency& A, int tile, int rsize, bool loop, TilePlan& P, bool verify,
                int max_len = 0, int64_t max_tiles = 0) {
@@ -488,9 +487,7 @@ int make_tiles(const Mesh& M, const Adjacency& A, int tile, int rsize, bool loop
         P.r1link.insert(P.r1link.end(), W.r_link.begin(), W.r_link.end());
         P.n_r1 += R.n1;
         c0 += len;
-        const int64_t made = (int64_t)P.rec.size();
-        if (max_tiles > 0 && (made + (n_own - c0 + max_len - 1) / max_len > max_tiles ||
-                              (c0 >= n_own / 8 && (double)made * n_own > 1.1 * max_tiles * c0)))
+        if (max_tiles > 0 && (int64_t)P.rec.size() + (n_own - c0 + max_len - 1) / max_len > max_tiles)
             return fail(FVLBM_ERR_UNSUPPORTED, "more than %lld tiles", (long long)max_tiles);
         P.max_ghosts = std::max(P.max_ghosts, ng);
         P.max_local = std::max(P.max_local, nl);
