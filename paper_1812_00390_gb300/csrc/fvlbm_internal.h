@@ -337,9 +337,14 @@ struct StageCost {
     double turn = 0, base = 0, flow = 0;
     bool resident = false;
 };
-// How much less time a stage of all of them takes in stage kernels that overlap than
+// How much less time a stage of several solvers takes in stage kernels that overlap than
 // in turns; queues: how many run side by side.
-double overlap_gain(const std::vector<StageCost>& c, int queues);
+struct OverlapGain {
+    double turns = 0, left_base = 0, left_flow = 0, base = 0, flow = 0;
+    int n = 0;
+    void add(const StageCost& x);
+    double us(int queues) const;
+};
 StageCost solver_cost(const fvlbm_solver* s);
 // Microseconds that the solver's first stage kernels take besides, for their graphs (0: it has them).
 double solver_overlap_setup(const fvlbm_solver* s);

@@ -228,15 +228,16 @@ extern "C" int fvlbm_server_poll(fvlbm_server* s, int32_t* n_completed) {
     // take less for the steps that every one has left, the graphs that overlapping needs
     // included (ms of requests of 16k quads on 8 streams, in turns / overlapping: 6 of
     // 20,000 steps 502 / 312, of 2,000 steps 70 / 81; 16 of 256 quads, 20,000 steps 172 / 497).
-    std::vector<StageCost> cost;
+    OverlapGain gain;
     double stages = INFINITY, setup = 0;
     for (int64_t id : stepping) {
         Request& r = s->req[id];
-        cost.push_back(solver_cost(r.solver));
+        const StageCost cost = solver_cost(r.solver);
+        gain.add(cost);
         stages = std::min(stages, (double)(s->cfg.max_steps - r.steps) * solver_n_stages(r.solver));
-        if (cost.back().resident) setup += solver_overlap_setup(r.solver);
+        if (cost.resident) setup += solver_overlap_setup(r.solver);
     }
-    const bool turns = overlap_gain(cost, std::min((int)s->streams.size(), 8)) * stages <= setup;
+    const bool turns = gain.us(std::min((int)s->streams.size(), 8)) * stages <= setup;
     for (int64_t id : stepping) {
         Request& r = s->req[id];
         const int64_t n = std::min<int64_t>(s->cfg.check_interval, s->cfg.max_steps - r.steps);

@@ -937,13 +937,19 @@ struct Crowd {
     uint64_t calls = 0;
 };
 static Crowd& crowd() {
-    static Crowd* c = new Crowd;   // outlives every solver
+    alignas(Crowd) static unsigned char place[sizeof(Crowd)];
+    static Crowd* c = new (place) Crowd;   // outlives every solver
     return *c;
 }
-static void crowd_join(fvlbm_solver* s) {
+static int crowd_join(fvlbm_solver* s) {
     Crowd& c = crowd();
     std::lock_guard<std::mutex> lock(c.m);
-    c.members.push_back(s);
+    try {
+        c.members.push_back(s);
+    } catch (const std::bad_alloc&) {
+        return fail(FVLBM_ERR_OOM, "fvlbm_init: out of host memory");
+    }
+    return FVLBM_OK;
 }
 static void crowd_leave(fvlbm_solver* s) {
     if (!s->stepped) return;
@@ -962,7 +968,8 @@ static bool crowd_turns(fvlbm_solver* s) {
     const bool joined = s->joined;
     s->call = ++c.calls;
     s->joined = false;
-    std::vector<StageCost> cost(1, s->cost);
+    OverlapGain gain;
+    gain.add(s->cost);
     // another thread may be capturing a stream: a query of these events is none of its business
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
@@ -970,11 +977,11 @@ static bool crowd_turns(fvlbm_solver* s) {
         if (o == s || o->device != s->device || o->stream == s->stream) continue;
         if (o->in_flight && cudaEventQuery(o->stepped) != cudaErrorNotReady) o->in_flight = false;
         if (o->in_flight) o->joined = true;
-        if (o->in_flight || (joined && o->call > last)) cost.push_back(o->cost);
+        if (o->in_flight || (joined && o->call > last)) gain.add(o->cost);
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
     cudaGetLastError();   // cudaErrorNotReady
-    return overlap_gain(cost, QUEUES) <= 0;
+    return gain.us(QUEUES) <= 0;
 }
 // The solver's long call has been enqueued.
 static void crowd_stepped(fvlbm_solver* s) {
@@ -986,19 +993,19 @@ static void crowd_stepped(fvlbm_solver* s) {
 }
 
 namespace fvlbm {
-double overlap_gain(const std::vector<StageCost>& c, int queues) {
-    double turns = 0, left_base = 0, left_flow = 0, base = 0, flow = 0;
-    for (const StageCost& x : c) {
-        base = std::max(base, x.base);
-        flow += x.flow;
-        if (x.resident) {
-            turns += x.turn;
-        } else {   // runs stage kernels in any case
-            left_base = std::max(left_base, x.base);
-            left_flow += x.flow;
-        }
+void OverlapGain::add(const StageCost& x) {
+    n++;
+    base = std::max(base, x.base);
+    flow += x.flow;
+    if (x.resident) {
+        turns += x.turn;
+    } else {   // runs stage kernels in any case
+        left_base = std::max(left_base, x.base);
+        left_flow += x.flow;
     }
-    const int n = (int)c.size(), q = std::max(1, queues);
+}
+double OverlapGain::us(int queues) const {
+    const int q = std::max(1, queues);
     return turns + left_base + left_flow - (base * ((n + q - 1) / q) + flow);
 }
 }  // namespace fvlbm
@@ -1202,7 +1209,8 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     if (!s->resident) s->cost = stage_cost(v, s->prec, nullptr, 0);
     if (s->resident) {
         CK(cudaEventCreateWithFlags(&s->stepped, cudaEventDisableTiming), "event");
-        crowd_join(s);
+        rc = crowd_join(s);
+        if (rc) return rc;
     }
     s->pingpong = L.pingpong;
     s->buf[0] = v.fa;
