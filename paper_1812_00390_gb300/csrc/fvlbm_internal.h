@@ -337,16 +337,17 @@ struct StageCost {
     double turn = 0, base = 0, flow = 0;
     bool resident = false;
 };
-// How much less time a stage of several solvers takes in stage kernels that overlap than
-// in turns; queues: how many run side by side.
+// A stage of several solvers in turns and in stage kernels that overlap; queues: how many
+// run side by side.
 struct OverlapGain {
     double turns = 0, left_base = 0, left_flow = 0, base = 0, flow = 0;
     int n = 0;
     void add(const StageCost& x);
-    double us(int queues) const;
+    double in_turns() const { return turns + left_base + left_flow; }
+    double overlapping(int queues) const { return base * ((n + queues - 1) / queues) + flow; }
 };
 StageCost solver_cost(const fvlbm_solver* s);
-// Microseconds that the solver's first stage kernels take besides, for their graphs (0: it has them).
+// Microseconds that a fresh request's first stage kernels take besides, for their graphs (0: it has them).
 double solver_overlap_setup(const fvlbm_solver* s);
 // Where the solver's next steps run (the results are the same): as fvlbm_step finds
 // best, in the resident loop, or by stage kernels.

@@ -237,7 +237,10 @@ extern "C" int fvlbm_server_poll(fvlbm_server* s, int32_t* n_completed) {
         stages = std::min(stages, (double)(s->cfg.max_steps - r.steps) * solver_n_stages(r.solver));
         if (cost.resident) setup += solver_overlap_setup(r.solver);
     }
-    const bool turns = gain.us(std::min((int)s->streams.size(), 8)) * stages <= setup;
+    const int queues = std::max(1, std::min((int)s->streams.size(), 8));
+    const double in_turns = gain.in_turns(), overlapping = gain.overlapping(queues);
+    // (a tenth more, as the streams' requests do not stay in step)
+    const bool turns = in_turns < 1.1 * overlapping || (in_turns - overlapping) * stages <= setup;
     for (int64_t id : stepping) {
         Request& r = s->req[id];
         const int64_t n = std::min<int64_t>(s->cfg.check_interval, s->cfg.max_steps - r.steps);

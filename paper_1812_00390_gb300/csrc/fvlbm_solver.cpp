@@ -67,12 +67,16 @@ struct fvlbm_solver {
     cudaEvent_t stepped = nullptr;
     bool in_flight = false, joined = false;
     uint64_t call = 0;
+    double lost = 0;   // microseconds that its calls in turns took longer than overlapping
 };
 
 static constexpr int64_t GRAPH_CHUNK = 32;
-// What a solver's first stage kernels take besides: both graphs captured and instantiated,
-// while its neighbours' start (requests of 2,000 steps served both ways: 4 to 14 ms each).
-static constexpr double GRAPH_SETUP_US = 6000;
+// What a solver's first stage kernels take besides, for both graphs captured and
+// instantiated: the host's time (eight solvers' first 600 stages 0.5 to 1 ms each), and what
+// a fresh request pays while its neighbours start (requests of 2,000 steps served both
+// ways: 4 to 7 ms each, of 4k quads in FP64 17).
+static constexpr double GRAPH_SETUP_US = 1000;
+static double request_setup_us(int prec) { return prec == FVLBM_FP64 ? 18000 : 6000; }
 // stages of one resident launch (a few milliseconds)
 static constexpr int64_t RESIDENT_CHUNK = 2048;
 
@@ -930,7 +934,8 @@ static StageCost stage_cost(const DevView& v, int prec, const ResView* r, int ma
 // overlap.  So a long call looks who else steps: solvers on other streams whose last
 // long call is in flight, and, when its own last one was joined by others, whoever has
 // stepped since (a program that steps several solvers in rounds and waits for all has
-// none in flight when a round begins).  The states are the same either way.
+// none in flight when a round begins).  Stage kernels need graphs, so it turns to them
+// once the turns have cost as much more as those take.  The states are the same either way.
 struct Crowd {
     std::mutex m;
     std::vector<fvlbm_solver*> members;
@@ -959,8 +964,8 @@ static void crowd_leave(fvlbm_solver* s) {
     cudaEventDestroy(s->stepped);
     s->stepped = nullptr;
 }
-// Whether the solver's next long call runs in the resident loop.
-static bool crowd_turns(fvlbm_solver* s) {
+// Whether the solver's next long call, of so many stages, runs in the resident loop.
+static bool crowd_turns(fvlbm_solver* s, int64_t stages) {
     constexpr int QUEUES = 8;   // streams that CUDA runs side by side by default
     Crowd& c = crowd();
     std::lock_guard<std::mutex> lock(c.m);
@@ -981,7 +986,13 @@ static bool crowd_turns(fvlbm_solver* s) {
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
     cudaGetLastError();   // cudaErrorNotReady
-    return gain.us(QUEUES) <= 0;
+    const double more = gain.in_turns() - gain.overlapping(QUEUES);
+    if (more <= 0) return true;
+    if (!s->gk[0] && !s->gk[1] && s->lost < gain.n * GRAPH_SETUP_US) {
+        s->lost += more * stages;
+        return true;
+    }
+    return false;
 }
 // The solver's long call has been enqueued.
 static void crowd_stepped(fvlbm_solver* s) {
@@ -1003,10 +1014,6 @@ void OverlapGain::add(const StageCost& x) {
         left_base = std::max(left_base, x.base);
         left_flow += x.flow;
     }
-}
-double OverlapGain::us(int queues) const {
-    const int q = std::max(1, queues);
-    return turns + left_base + left_flow - (base * ((n + q - 1) / q) + flow);
 }
 }  // namespace fvlbm
 
@@ -1413,7 +1420,7 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
     // resident loop (a caller's capture records the stages one by one).  Calls shorter
     // than a graph's steps are bound by the host's launches, of which the loop makes fewer
     const bool in_crowd = s->resident && s->path == STEP_AUTO && s->stream && cs == cudaStreamCaptureStatusNone && n >= GRAPH_CHUNK;
-    const bool turns = s->path == STEP_AUTO ? !in_crowd || crowd_turns(s) : s->path == STEP_RESIDENT;
+    const bool turns = s->path == STEP_AUTO ? !in_crowd || crowd_turns(s, n * n_stages(s->scheme)) : s->path == STEP_RESIDENT;
     if (s->resident && turns && cs == cudaStreamCaptureStatusNone) {
         const int ns = n_stages(s->scheme);
         while (n * ns >= 2) {
@@ -1531,7 +1538,7 @@ bool solver_replayable(const fvlbm_solver* s) {
 int solver_buffer(const fvlbm_solver* s) { return s->cur; }
 void solver_set_buffer(fvlbm_solver* s, int b) { set_current(s, b); }
 StageCost solver_cost(const fvlbm_solver* s) { return s->cost; }
-double solver_overlap_setup(const fvlbm_solver* s) { return s->gk[0] || s->gk[1] ? 0.0 : GRAPH_SETUP_US; }
+double solver_overlap_setup(const fvlbm_solver* s) { return s->gk[0] || s->gk[1] ? 0.0 : request_setup_us(s->prec); }
 void solver_path(fvlbm_solver* s, StepPath path) { s->path = path; }
 int solver_sums(fvlbm_solver* s, int what, std::vector<double>& out) {
     DeviceGuard dg(s->device);
