@@ -90,6 +90,8 @@ __global__ void __launch_bounds__(ORDERED_CELLS) set_f_ordered_kernel(DevView v,
     for (int w = threadIdx.x; w < nw; w += ORDERED_CELLS) buf[w] = in[c0 * FVLBM_Q + w];
     __syncthreads();
     const int64_t c = c0 + threadIdx.x;
+    // a wait that ran out has left the state in the middle of a call: this one replaces it
+    if (c == 0) v.flag[1] = 0;
     if (c >= v.n_cell) return;
     const int64_t i = v.iperm[c];
     T f[FVLBM_Q];

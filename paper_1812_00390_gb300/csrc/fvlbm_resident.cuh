@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(TILE, CTAS)
     V* sgeo = tab + ROWS;         // [3 GU][TILE]  geometry of the gradient cells
     V* sbase = sgeo + (SHARED ? 3 * GU * TILE : 0);   // [2][TILE]  state the step began with
     float* sbase0 = (float*)(sbase + 2 * TILE);   // [TILE]
-    if (__syncthreads_or(*(volatile int32_t*)(v.flag + 1))) return;   // a launch before gave up
+    const int gone = *(volatile int32_t*)(v.flag + 1);   // a launch before gave up
     const TileRec R = r.tiles[blockIdx.x];
     const int l = threadIdx.x, nt = R.nt, n2 = R.nt + R.n1, n_ring2 = R.nh - R.n1, inst = R.inst;
     const bool mine = l < nt, ring1 = !mine && l < n2;
@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(TILE, CTAS)
     };
     auto lsq = [&](int q) { return geo(GEO_LSQ, q); };
     auto face = [&](int q) { return geo(GEO_FACE, q); };
+    if (__syncthreads_or(gone)) return;
     int k = 0;            // stage of the step
     bool first = AB2 && !ab2_started;
     for (int64_t s = 0; s < stages; s++) {
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2* fs = (double2*)smem_raw;   // [LS][4]    pairs of the local cells
     double* tab = (double*)(fs + 4 * LS);   // [ROWS][4]  face table
-    if (__syncthreads_or(*(volatile int32_t*)(v.flag + 1))) return;   // a launch before gave up
+    const int gone = *(volatile int32_t*)(v.flag + 1);   // a launch before gave up
     const TileRec R = r.tiles[blockIdx.x];
     const int x = threadIdx.x >> 2, p = threadIdx.x & 3, nt = R.nt, n2 = R.nt + R.n1, n_ring2 = R.nh - R.n1,
               inst = R.inst;
@@ -372,6 +373,7 @@ __global__ void __launch_bounds__(RES_LANES_FP64* TILE, 1)
         rpb = hist[ib * v.np + gl];
     }
 
+    if (__syncthreads_or(gone)) return;
     int k = 0;            // stage of the step
     bool first = AB2 && !ab2_started;
     for (int64_t s = 0; s < stages; s++) {

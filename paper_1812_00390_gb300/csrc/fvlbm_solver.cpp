@@ -975,17 +975,19 @@ static bool crowd_turns(fvlbm_solver* s, int64_t stages) {
     s->joined = false;
     OverlapGain gain;
     gain.add(s->cost);
-    // another thread may be capturing a stream: a query of these events is none of its business
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
     for (fvlbm_solver* o : c.members) {
         if (o == s || o->device != s->device || o->stream == s->stream) continue;
-        if (o->in_flight && cudaEventQuery(o->stepped) != cudaErrorNotReady) o->in_flight = false;
+        if (o->in_flight) {
+            // another thread may be capturing a stream: a query of this event is none of its business
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            o->in_flight = cudaEventQuery(o->stepped) == cudaErrorNotReady;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            cudaGetLastError();   // cudaErrorNotReady
+        }
         if (o->in_flight) o->joined = true;
         if (o->in_flight || (joined && o->call > last)) gain.add(o->cost);
     }
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    cudaGetLastError();   // cudaErrorNotReady
     const double more = gain.in_turns() - gain.overlapping(QUEUES);
     if (more <= 0) return true;
     if (!s->gk[0] && !s->gk[1] && s->lost < gain.n * GRAPH_SETUP_US) {
@@ -996,6 +998,10 @@ static bool crowd_turns(fvlbm_solver* s, int64_t stages) {
 }
 // The solver's long call has been enqueued.
 static void crowd_stepped(fvlbm_solver* s) {
+    {
+        std::lock_guard<std::mutex> lock(crowd().m);
+        if (crowd().members.size() < 2) return;   // nobody to know
+    }
     // outside the lock: a record waits when the stream's queue is full
     const bool ok = cudaEventRecord(s->stepped, s->stream) == cudaSuccess;
     if (!ok) cudaGetLastError();
@@ -1597,8 +1603,6 @@ extern "C" int fvlbm_set_f(fvlbm_solver* s, const double* f) {
         rc = launch_set_f_ordered(s->v, s->prec, s->stream, s->v.conv);
     }
     if (rc) return rc;
-    // a wait that ran out has left the state in the middle of a call: this one replaces it
-    CK(cudaMemsetAsync(s->v.flag + 1, 0, sizeof(int32_t), s->stream), "clear flag");
     s->ab2_started = false;
     if (s->scheme == FVLBM_AB2) s->direct_steps = 0;   // the next step is an Euler start, launched directly
     CK(cudaStreamSynchronize(s->stream), "synchronise");
