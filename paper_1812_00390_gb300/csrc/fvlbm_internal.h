@@ -335,6 +335,7 @@ void solver_set_buffer(fvlbm_solver* s, int b);
 // stage kernels, `base` of latency, which others' overlap, and `flow` of the whole GPU.
 struct StageCost {
     double turn = 0, base = 0, flow = 0;
+    double alone = 0;   // in the resident loop, nobody beside
     bool resident = false;
 };
 // A stage of several solvers in turns and in stage kernels that overlap; queues: how many

@@ -7,6 +7,7 @@
 // that reads results back (macros, residual, mass, f) synchronises and maps
 // cells back to the caller's numbering.
 #include <algorithm>
+#include <chrono>
 #include <cstdio>
 #include <cmath>
 #include <cstring>
@@ -62,10 +63,10 @@ struct fvlbm_solver {
     int64_t res_launches = 0;
     StepPath path = STEP_AUTO;
     StageCost cost;
-    // who steps beside this solver (Crowd): recorded behind its last long call, which may
-    // be in flight; number of that call; whether another solver stepped meanwhile
-    cudaEvent_t stepped = nullptr;
-    bool in_flight = false, joined = false;
+    // who steps beside this solver (Crowd): the time at which its last long call is expected
+    // to be done; number of that call; whether another solver stepped meanwhile
+    bool member = false, joined = false;
+    double busy_until = 0;
     uint64_t call = 0;
     double lost = 0;   // microseconds that its calls in turns took longer than overlapping
 };
@@ -922,7 +923,8 @@ static StageCost stage_cost(const DevView& v, int prec, const ResView* r, int ma
     if (r) {
         const int per_sm = (r->n_tiles + v.sms - 1) / v.sms;
         const double t = fp64 ? 7.0 : (per_sm == 1 ? 2.0 : per_sm <= 3 ? 3.2 : 6.0) + (wide ? 0.5 : 0.0);
-        c.turn = t * (half ? 1.2 : 1.0) / (max_ctas / r->n_tiles);   // so many fit side by side
+        c.alone = t * (half ? 1.2 : 1.0);
+        c.turn = c.alone / (max_ctas / r->n_tiles);   // so many fit side by side
         c.resident = true;
     }
     return c;
@@ -932,9 +934,10 @@ static StageCost stage_cost(const DevView& v, int prec, const ResView* r, int ma
 // stage kernels for one solver, but those that do not fit on the GPU together take
 // turns, and three solvers that fill it are then slower than with stage kernels, which
 // overlap.  So a long call looks who else steps: solvers on other streams whose last
-// long call is in flight, and, when its own last one was joined by others, whoever has
-// stepped since (a program that steps several solvers in rounds and waits for all has
-// none in flight when a round begins).  Stage kernels need graphs, so it turns to them
+// long call is not expected to be done yet, and, when its own last one was joined by others,
+// whoever has stepped since (a program that steps several solvers in rounds and waits for
+// all has none at work when a round begins).  Expected, by the host's clock and the costs
+// above: events would be exact, but recording one takes 2% of a call of 100 steps.  Stage kernels need graphs, so it turns to them
 // once the turns have cost as much more as those take.  The states are the same either way.
 struct Crowd {
     std::mutex m;
@@ -954,15 +957,23 @@ static int crowd_join(fvlbm_solver* s) {
     } catch (const std::bad_alloc&) {
         return fail(FVLBM_ERR_OOM, "fvlbm_init: out of host memory");
     }
+    s->member = true;
     return FVLBM_OK;
 }
 static void crowd_leave(fvlbm_solver* s) {
-    if (!s->stepped) return;
+    if (!s->member) return;
     Crowd& c = crowd();
     std::lock_guard<std::mutex> lock(c.m);
     c.members.erase(std::remove(c.members.begin(), c.members.end(), s), c.members.end());
-    cudaEventDestroy(s->stepped);
-    s->stepped = nullptr;
+}
+// The solver's work is done.
+static void crowd_idle(fvlbm_solver* s) {
+    if (!s->member) return;
+    std::lock_guard<std::mutex> lock(crowd().m);
+    s->busy_until = 0;
+}
+static double crowd_now() {   // microseconds
+    return std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
 // Whether the solver's next long call, of so many stages, runs in the resident loop.
 static bool crowd_turns(fvlbm_solver* s, int64_t stages) {
@@ -975,38 +986,21 @@ static bool crowd_turns(fvlbm_solver* s, int64_t stages) {
     s->joined = false;
     OverlapGain gain;
     gain.add(s->cost);
+    const double now = crowd_now();
     for (fvlbm_solver* o : c.members) {
         if (o == s || o->device != s->device || o->stream == s->stream) continue;
-        if (o->in_flight) {
-            // another thread may be capturing a stream: a query of this event is none of its business
-            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            o->in_flight = cudaEventQuery(o->stepped) == cudaErrorNotReady;
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            cudaGetLastError();   // cudaErrorNotReady
-        }
-        if (o->in_flight) o->joined = true;
-        if (o->in_flight || (joined && o->call > last)) gain.add(o->cost);
+        const bool busy = o->busy_until > now;
+        if (busy) o->joined = true;
+        if (busy || (joined && o->call > last)) gain.add(o->cost);
     }
-    const double more = gain.in_turns() - gain.overlapping(QUEUES);
-    if (more <= 0) return true;
-    if (!s->gk[0] && !s->gk[1] && s->lost < gain.n * GRAPH_SETUP_US) {
+    const double in_turns = gain.in_turns(), overlapping = gain.overlapping(QUEUES), more = in_turns - overlapping;
+    bool turns = more <= 0;
+    if (!turns && !s->gk[0] && !s->gk[1] && s->lost < gain.n * GRAPH_SETUP_US) {
         s->lost += more * stages;
-        return true;
+        turns = true;
     }
-    return false;
-}
-// The solver's long call has been enqueued.
-static void crowd_stepped(fvlbm_solver* s) {
-    {
-        std::lock_guard<std::mutex> lock(crowd().m);
-        if (crowd().members.size() < 2) return;   // nobody to know
-    }
-    // outside the lock: a record waits when the stream's queue is full
-    const bool ok = cudaEventRecord(s->stepped, s->stream) == cudaSuccess;
-    if (!ok) cudaGetLastError();
-    std::lock_guard<std::mutex> lock(crowd().m);
-    s->in_flight = ok;
+    s->busy_until = std::max(now, s->busy_until) + stages * (turns ? std::max(in_turns, s->cost.alone) : overlapping);
+    return turns;
 }
 
 namespace fvlbm {
@@ -1221,7 +1215,6 @@ static int init_impl(const fvlbm_mesh* mesh, const fvlbm_params* params, int32_t
     }
     if (!s->resident) s->cost = stage_cost(v, s->prec, nullptr, 0);
     if (s->resident) {
-        CK(cudaEventCreateWithFlags(&s->stepped, cudaEventDisableTiming), "event");
         rc = crowd_join(s);
         if (rc) return rc;
     }
@@ -1473,7 +1466,6 @@ extern "C" int fvlbm_step(fvlbm_solver* s, int64_t n) {
         if (rc) return rc;
         n--;
     }
-    if (in_crowd) crowd_stepped(s);
     return FVLBM_OK;
 }
 
@@ -1481,6 +1473,7 @@ static int sync_and_check(fvlbm_solver* s) {
     int32_t flag[2] = {0, 0};
     CK(cudaMemcpyAsync(flag, s->v.flag, sizeof flag, cudaMemcpyDeviceToHost, s->stream), "read flag");
     CK(cudaStreamSynchronize(s->stream), "synchronise");
+    crowd_idle(s);
     if (flag[1]) return fail(FVLBM_ERR_TIMEOUT, "the resident stage loop: a tile waited too long for its neighbours");
     if (flag[0]) return fail(FVLBM_ERR_DIVERGED, "a non-finite value appeared in the state");
     return FVLBM_OK;
